@@ -42,6 +42,10 @@ cudaError_t lfk::ensure_dynamic_smem(const void* kernel, int bytes) {
 namespace {
 
 constexpr int kRing = 4;
+// Mesh cells narrower than this on the screen: a raster lane walks a triangle's
+// box (lf_raster.cu).  Raster alone, a lane per pixel / per triangle: 2.0-pixel
+// cells (a prefilter's dense model) 5.1 / 2.8 ms; 2.9-pixel cells 71 / 82 us.
+constexpr double kFineCellPx = 2.5;
 constexpr int kHostSlots = LF_HOST_FRAMES_IN_FLIGHT;
 constexpr size_t kCounterBlock = 32;  // triangles, error word, work counter, bin offsets, bin entries
 constexpr int64_t kDefaultWaitNs = 2000000000;  // 2 s: far beyond any legitimate wait, even under a profiler
@@ -254,6 +258,16 @@ void use_counters(FrameArgs& a, unsigned char* block) {
   a.bin_entries_counter = reinterpret_cast<unsigned long long*>(block + 24);
 }
 
+// Whether the loaded mesh's cells are so small on this eye's screen that the
+// raster walks triangles instead of pixels (a value of speed only, so the first
+// view and the first eye of a call stand for all): cell width in eye pixels of a
+// surface seen from about the same distance by both.
+int32_t fine_mesh(const lf_ctx* c, const EyeParams& E) {
+  if (c->views_host.empty() || c->G < 2) return 0;
+  const double cell = (double)c->src_w / (c->G - 1) * E.fx / c->views_host[0].fx;
+  return cell < kFineCellPx ? 1 : 0;
+}
+
 FrameArgs frame_args(lf_ctx* c, const Layout& L) {
   FrameArgs a;
   std::memset(&a, 0, sizeof(a));
@@ -290,6 +304,7 @@ FrameArgs frame_args(lf_ctx* c, const Layout& L) {
   a.total_tiles = L.total_tiles;
   a.tile_w = c->cfg.tile_w;
   a.tile_h = c->cfg.tile_h;
+  if (!L.eyes.empty()) a.fine_mesh = fine_mesh(c, L.eyes[0]);
   if (c->lv.n_fine > 0) {
     a.tex_table = static_cast<const void* const*>(c->lv.table.p);
     a.enable_bits = static_cast<uint32_t*>(c->lv.enable.p);
@@ -767,7 +782,7 @@ lf_status lf_render_batch(lf_ctx* c, int32_t n_eyes, const lf_pose* eyes, const 
                               (int64_t)(intptr_t)c->tex.p, (int64_t)(intptr_t)c->depth.p, c->persistent_blocks,
                               c->cfg.tile_w, c->cfg.tile_h, c->cfg.timing, c->disk_mode, c->lv.n_fine,
                               (int64_t)(intptr_t)c->lv.pool.p, (int64_t)(intptr_t)c->lv.enable.p,
-                              (int64_t)(intptr_t)c->lv.visible.p};
+                              (int64_t)(intptr_t)c->lv.visible.p, fine_mesh(c, L.eyes[0])};
   for (int e = 0; e < n_eyes; ++e) { sig.push_back(intr[e].width); sig.push_back(intr[e].height); }
   cudaStream_t s = static_cast<cudaStream_t>(stream);
   if (c->cfg.timing) {
@@ -1080,6 +1095,7 @@ extern "C" lf_status lf_render_static(lf_ctx* c, const lf_pose* eye, const lf_in
   FrameArgs a = frame_args(c, none);
   a.n_eyes = 1;
   a.total_tiles = (int32_t)tiles;
+  a.fine_mesh = fine_mesh(c, P);
   a.eyes = reinterpret_cast<const EyeParams*>(base + kOffEye);
   a.eyes_f = reinterpret_cast<EyeFloat*>(base + kOffEyeF);
   a.vrecs = reinterpret_cast<ViewRec*>(base + kOffVrecs);

@@ -22,6 +22,7 @@
 // page table, per coarse view the fine views whose disks overlap it (CSR), and
 // per call the exact view selection and the drawn-view bits of each eye.
 #pragma once
+#include <cstddef>
 #include <cstdint>
 #include <cuda_bf16.h>
 #include <cuda_runtime.h>
@@ -85,24 +86,30 @@ struct __align__(16) EyeFloat {
 };
 
 struct __align__(16) ViewRec {
-  float Hm[12];         // eye pixel (x, y, 1) and 1/z -> source (u, v) homogeneous; Hm 3x3 then hv
+  // what the raster copies to shared memory per tile, 16 bytes at a time
   float cc[4];          // disk centre relative to the capture sphere centre, then r^2
+  float Hm[3][4];       // eye pixel (x, y, 1) and 1/z -> source (u, v) homogeneous, a row per component
   float inv_r;
-  int32_t tri_base;     // first set-up triangle of this (eye, view) in the pool
-  int32_t tri_count;    // its set-up triangles
+  float tex_scale;      // decode scale for FP8 textures
+  const void* tex;      // the view's first texel (a pool page for a fine view of a two-level frame)
+  // its triangles and bins, read as one int4 up to big_base
   int32_t bin_off;      // its tile bins in the offset pool (-1: none): bntx*bnty+1 entry offsets
-  int32_t bb[4];        // conservative footprint in pixels, inclusive; bb[0] > bb[2] when empty
   int16_t btx0, bty0, bntx, bnty;  // the tiles of the footprint box
   int32_t big_base;     // entries of the triangles spanning more than kBinMaxTiles tiles
   int32_t big_count;
+  int32_t tri_base;     // first set-up triangle of this (eye, view) in the pool
+  int32_t tri_count;    // its set-up triangles
+  int32_t pad;
+  int32_t bb[4];        // conservative footprint in pixels, inclusive; bb[0] > bb[2] when empty
   float Mf[12];         // camera -> eye rotation (3x3) then translation, FP32
   // oval disk (Sec. 4.4) in the eye frame, each the FP32 rounding of an FP64
   // value: plane normal n, u and v axes x, y (columns of M = R_eye^T R_i),
-  // k = n.c', u0 = x.c', v0 = y.c' (c' the disk centre), reciprocal extents
-  float ov_n[3], ov_x[3], ov_y[3], ov_k, ov_u0, ov_v0;
-  float ov_ru[2], ov_rv[2];   // 1 / e_u+, 1 / e_u-, 1 / e_v+, 1 / e_v-
-  const void* tex;            // the view's first texel (a pool page for a fine view of a two-level frame)
+  // k = n.c', u0 = x.c', v0 = y.c' (c' the disk centre), then the reciprocal
+  // extents 1 / e_u+, 1 / e_u-, 1 / e_v+, 1 / e_v-
+  float ov[16];
 };
+constexpr int kViewShadeQuads = 5;  // 16-byte pieces from cc to tex
+static_assert(offsetof(ViewRec, bin_off) == 16 * kViewShadeQuads && offsetof(ViewRec, ov) % 16 == 0, "ViewRec layout");
 
 struct __align__(16) TriRec {
   int16_t bx0, by0, bx1, by1;   // pixel-centre bounding box clipped to screen and footprint
@@ -162,6 +169,8 @@ struct FrameArgs {
   uint32_t* texel_bits;
   // persistent batch raster
   int32_t* work_counter;
+  int32_t fine_mesh;       // 1: mesh cells of a few eye pixels, a raster lane takes a triangle
+  int32_t strips_per_item; // strips of a tile that a raster warp takes at a time (set by launch_raster)
   // two-level progressive rendering (all null / 0 with one level)
   const void* const* tex_table;  // per view: its texels (a pool page for fine views; null when not resident)
   uint32_t* enable_bits;         // n_eyes x mask_words: the views each eye draws

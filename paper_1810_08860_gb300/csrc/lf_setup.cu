@@ -281,14 +281,15 @@ __global__ void __launch_bounds__(kViewSetupThreads) view_setup_kernel(FrameArgs
           KM[r * 3 + c] = Ki[r * 3 + 0] * Mc[c * 3 + 0] + Ki[r * 3 + 1] * Mc[c * 3 + 1] + Ki[r * 3 + 2] * Mc[c * 3 + 2];
       for (int r = 0; r < 3; ++r) {
         for (int c = 0; c < 3; ++c)
-          R.Hm[r * 3 + c] = KM[r * 3 + 0] * Ke[0 * 3 + c] + KM[r * 3 + 1] * Ke[1 * 3 + c] + KM[r * 3 + 2] * Ke[2 * 3 + c];
-        R.Hm[9 + r] = -(KM[r * 3 + 0] * mc[0] + KM[r * 3 + 1] * mc[1] + KM[r * 3 + 2] * mc[2]);
+          R.Hm[r][c] = KM[r * 3 + 0] * Ke[0 * 3 + c] + KM[r * 3 + 1] * Ke[1 * 3 + c] + KM[r * 3 + 2] * Ke[2 * 3 + c];
+        R.Hm[r][3] = -(KM[r * 3 + 0] * mc[0] + KM[r * 3 + 1] * mc[1] + KM[r * 3 + 2] * mc[2]);
       }
 
       // Disk (Sec. 4.1): centre relative to the sphere centre in FP32, r^2.
       for (int k = 0; k < 3; ++k) R.cc[k] = __double2float_rn(__dsub_rn((double)V.disk_c[k], A.sphere_c[k]));
       R.cc[3] = __fmul_rn(V.disk_r, V.disk_r);
       R.inv_r = __frcp_rn(V.disk_r);
+      R.tex_scale = V.tex_scale;
       if (A.disk_mode == 1) {
         // Oval disk (Sec. 4.4): its plane's normal and axes are the columns of M; the
         // centre in the eye frame and the dot products in FP64, fixed order, each
@@ -309,17 +310,17 @@ __global__ void __launch_bounds__(kViewSetupThreads) view_setup_kernel(FrameArgs
         };
 #pragma unroll
         for (int k = 0; k < 3; ++k) {
-          R.ov_x[k] = Mc[k * 3 + 0];
-          R.ov_y[k] = Mc[k * 3 + 1];
-          R.ov_n[k] = Mc[k * 3 + 2];
+          R.ov[k] = Mc[k * 3 + 2];      // n
+          R.ov[3 + k] = Mc[k * 3 + 0];  // x
+          R.ov[6 + k] = Mc[k * 3 + 1];  // y
         }
-        R.ov_k = __double2float_rn(dotc(2));
-        R.ov_u0 = __double2float_rn(dotc(0));
-        R.ov_v0 = __double2float_rn(dotc(1));
-        R.ov_ru[0] = __double2float_rn(__ddiv_rn(1.0, (double)V.disk_ext[0]));
-        R.ov_ru[1] = __double2float_rn(__ddiv_rn(1.0, (double)V.disk_ext[1]));
-        R.ov_rv[0] = __double2float_rn(__ddiv_rn(1.0, (double)V.disk_ext[2]));
-        R.ov_rv[1] = __double2float_rn(__ddiv_rn(1.0, (double)V.disk_ext[3]));
+        R.ov[9] = __double2float_rn(dotc(2));
+        R.ov[10] = __double2float_rn(dotc(0));
+        R.ov[11] = __double2float_rn(dotc(1));
+        R.ov[12] = __double2float_rn(__ddiv_rn(1.0, (double)V.disk_ext[0]));
+        R.ov[13] = __double2float_rn(__ddiv_rn(1.0, (double)V.disk_ext[1]));
+        R.ov[14] = __double2float_rn(__ddiv_rn(1.0, (double)V.disk_ext[2]));
+        R.ov[15] = __double2float_rn(__ddiv_rn(1.0, (double)V.disk_ext[3]));
       }
       // the view's texels: its page in a two-level frame, else its slice of the texture array
       const int tb = A.tex_format == LF_TEX_F32 ? 16 : A.tex_format == LF_TEX_BF16 ? 8 : 4;

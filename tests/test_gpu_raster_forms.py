@@ -1,0 +1,54 @@
+"""The raster's forms draw one image: a warp per tile or per strip, a lane per
+pixel or per triangle (fine meshes), one or several windows of gathered
+triangles, one or several rounds of views.  The reference is the inspection
+render, whose coverage is held to the oracle elsewhere; the arithmetic of every
+form is the same, so the images are compared bit for bit."""
+import math
+
+import pytest
+
+import scene
+
+pytestmark = pytest.mark.gpu
+
+# views, image size, grid, disk scale, eye size, ovals.  Cells of about 0.6-2 px (fine) and up to 64 px;
+# eyes that no tile divides, one pixel and one row; 40 wide disks: two rounds of views and several windows.
+CASES = [
+    (16, 96, 65, 1.2, (61, 47), False),
+    (16, 96, 33, 1.2, (63, 49), False),
+    (16, 64, 65, 1.2, (17, 3), True),
+    (9, 64, 9, 1.2, (257, 255), False),
+    (9, 64, 9, 1.2, (1, 1), False),
+    (9, 64, 5, 1.2, (1100, 900), True),
+    (40, 64, 33, 6.0, (90, 70), False),
+    (40, 64, 33, 6.0, (24, 20), False),
+]
+
+
+@pytest.mark.parametrize("views,size,grid,disk,eye,oval", CASES)
+@pytest.mark.parametrize("tile", [(16, 16), (32, 8), (8, 8)])
+def test_every_form_draws_the_inspection_image(views, size, grid, disk, eye, oval, tile):
+    torch = pytest.importorskip("torch")
+    import __graft_entry__
+
+    __graft_entry__.build()
+    import paper_1810_08860_gb300 as lfm
+    from paper_1810_08860_gb300 import disks
+
+    side = math.isqrt(views - 1) + 1
+    lf = scene.build_light_field(scene.sphere_scene(3, 8, forward_cone_deg=35.0), scene.cap_grid_directions(side, 40.0)[:views],
+                                 size, size, 90.0, grid, disk_scale=disk)
+    e = scene.head_pose_eyes(scene.SplitMix64(11), eye[0], eye[1], 90.0, yaw_range=(-0.1, 0.1), pitch_deg=6.0, stereo=False)[0]
+    r = lfm.Renderer(0, tile=tile)
+    r.load_views(lf)
+    r.build_meshes(lf)
+    if oval:
+        r.set_disk_ovals(disks.oval_extents(lf))
+    want = r.render_inspect(e, max_records=views)["rgba"]
+    assert eye == (1, 1) or int((want[..., 3] > 0).sum()) > 0
+    assert torch.equal(r.render([e])[0], want)
+    assert torch.equal(r.render_batch([e])[0], want)
+    tiles = -(-eye[0] // tile[0]) * -(-eye[1] // tile[1])
+    if views <= 32 and grid <= 33 and tiles <= 8192:  # lf_render_static's limits
+        assert torch.equal(r.render_static(e), want)
+    r.close()
