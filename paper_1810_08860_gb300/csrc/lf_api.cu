@@ -73,9 +73,9 @@ struct lf_ctx {
   // meshes
   int32_t G = 0;
   lf_mesh_format mesh_fmt = LF_MESH_F32_DEPTH;
-  Buffer depth, tab_a, tab_b;
+  Buffer depth, tab_a, tab_b, cluster_z;
   // per-call scratch
-  Buffer eyes, eyes_f, vrecs, masks, pool, bin_offsets, bin_entries, small, active;
+  Buffer eyes, eyes_f, vrecs, masks, pool, pool_owner, bin_offsets, bin_entries, small, active;
   EyeParams* pinned = nullptr;  // kRing slots of max_eyes
   cudaEvent_t ring_ev[kRing] = {};
   int ring_next = 0;
@@ -226,6 +226,8 @@ lf_status ensure_scratch(lf_ctx* c, int32_t n_eyes, int32_t total_tiles) {
   LF_CUDA(c, ensure(c->small, 64));
   int64_t cap = c->cfg.tri_capacity;
   LF_CUDA(c, ensure(c->pool, sizeof(TriRec) * (size_t)cap));
+  const int ncl = clusters_per_side(c->G);
+  if (ncl * ncl > kSetupPartClusters) LF_CUDA(c, ensure(c->pool_owner, sizeof(int32_t) * (size_t)cap));
   LF_CUDA(c, ensure(c->bin_offsets, sizeof(int32_t) * (size_t)bin_offsets_capacity(c, total_tiles)));
   LF_CUDA(c, ensure(c->bin_entries, sizeof(int32_t) * (size_t)bin_entries_capacity(c, total_tiles)));
   if (c->lv.n_fine > 0) {
@@ -289,10 +291,12 @@ FrameArgs frame_args(lf_ctx* c, const Layout& L) {
   a.depth = c->depth.p;
   a.tables.a = static_cast<const float*>(c->tab_a.p);
   a.tables.b = static_cast<const float*>(c->tab_b.p);
+  a.cluster_z = static_cast<const float2*>(c->cluster_z.p);
   a.vrecs = static_cast<ViewRec*>(c->vrecs.p);
   a.tile_masks = static_cast<uint32_t*>(c->masks.p);
   a.eyes_f = static_cast<EyeFloat*>(c->eyes_f.p);
   a.pool = static_cast<TriRec*>(c->pool.p);
+  a.pool_owner = static_cast<int32_t*>(c->pool_owner.p);
   a.pool_capacity = c->cfg.tri_capacity;
   a.bin_offsets = static_cast<int32_t*>(c->bin_offsets.p);
   a.bin_offsets_capacity = bin_offsets_capacity(c, L.total_tiles);
@@ -543,7 +547,7 @@ void lf_destroy(lf_ctx* ctx) {
   if (ctx->has_call && ctx->last_stream) cudaStreamSynchronize(ctx->last_stream);
   cudaDeviceSynchronize();
   if (ctx->graph) cudaGraphExecDestroy(ctx->graph);
-  for (Buffer* b : {&ctx->views, &ctx->tex, &ctx->depth, &ctx->tab_a, &ctx->tab_b, &ctx->eyes, &ctx->eyes_f,
+  for (Buffer* b : {&ctx->views, &ctx->tex, &ctx->depth, &ctx->tab_a, &ctx->tab_b, &ctx->cluster_z, &ctx->pool_owner, &ctx->eyes, &ctx->eyes_f,
                     &ctx->vrecs, &ctx->masks, &ctx->pool, &ctx->bin_offsets, &ctx->bin_entries, &ctx->small,
                     &ctx->active})
     release(*b);
@@ -604,7 +608,7 @@ lf_status lf_load_views(lf_ctx* c, int32_t n_views, const lf_pose* poses, const 
   if (c->graph) { cudaGraphExecDestroy(c->graph); c->graph = nullptr; c->graph_sig.clear(); }
   c->n_views = 0;
   c->G = 0;
-  release(c->depth); release(c->tab_a); release(c->tab_b);
+  release(c->depth); release(c->tab_a); release(c->tab_b); release(c->cluster_z);
   // one level again
   for (Buffer* b : {&c->lv.pool, &c->lv.table, &c->lv.page_of_view, &c->lv.overlap_off, &c->lv.overlap_ids,
                     &c->lv.enable, &c->lv.visible, &c->lv.stage})
@@ -714,6 +718,10 @@ lf_status lf_build_view_meshes(lf_ctx* c, int32_t grid_n, const float* depth, lf
   }
   LF_CUDA(c, launch_grid_tables(static_cast<const ViewStatic*>(c->views.p), c->n_views, c->src_w, c->src_h, grid_n,
                                 static_cast<float*>(c->tab_a.p), static_cast<float*>(c->tab_b.p), s));
+  const int ncl = clusters_per_side(grid_n);
+  LF_CUDA(c, ensure(c->cluster_z, sizeof(float2) * (size_t)c->n_views * ncl * ncl));
+  LF_CUDA(c, launch_cluster_bounds(c->depth.p, fmt, static_cast<const ViewStatic*>(c->views.p), c->n_views, grid_n,
+                                   static_cast<float2*>(c->cluster_z.p), s));
   LF_CUDA(c, cudaStreamSynchronize(s));
   c->G = grid_n;
   c->mesh_fmt = fmt;
@@ -776,7 +784,7 @@ lf_status lf_render_batch(lf_ctx* c, int32_t n_eyes, const lf_pose* eyes, const 
   std::vector<int64_t> sig = {n_eyes, L.total_tiles, c->n_views, c->G, c->tex_fmt, c->mesh_fmt,
                               (int64_t)(intptr_t)c->eyes.p, (int64_t)(intptr_t)c->eyes_f.p,
                               (int64_t)(intptr_t)c->bin_offsets.p, (int64_t)(intptr_t)c->bin_entries.p,
-                              (int64_t)(intptr_t)c->vrecs.p,
+                              (int64_t)(intptr_t)c->vrecs.p, (int64_t)(intptr_t)c->pool_owner.p, (int64_t)(intptr_t)c->cluster_z.p,
                               (int64_t)(intptr_t)c->masks.p, (int64_t)(intptr_t)c->pool.p,
                               (int64_t)(intptr_t)c->active.p, (int64_t)(intptr_t)c->small.p,
                               (int64_t)(intptr_t)c->tex.p, (int64_t)(intptr_t)c->depth.p, c->persistent_blocks,

@@ -6,14 +6,14 @@
 //                                 float4 / uchar4 / 4 x bf16 / 4 x e4m3
 //   depth grids                   n_views x G x G (float, or half + per-view origin)
 //   grid ray tables a_j, b_k      n_views x G floats each
+//   cluster depth ranges          n_views x ceil((G-1)/4)^2 float pairs
 // Per call (scratch, reused in stream order):
 //   EyeParams[n_eyes]             eye pose, intrinsics, tile range, output pointer
 //   ViewRec[n_eyes x n_views]     composed transforms, footprint, triangle segment
 //   tile masks                    per eye tile, one bit per view whose disk footprint
 //                                 overlaps the tile (ceil(n_views/32) words)
 //   EyeFloat[n_eyes]              the eye's FP32 constants (rounded once, on the device)
-//   TriRec pool                   set-up (sub-)triangles, one contiguous segment per
-//                                 (eye, view), grouped by 4x4-cell clusters
+//   TriRec pool                   set-up (sub-)triangles, in runs of one 4x4-cell cluster
 //   bin offsets / bin entries     per (eye, view): its triangles binned into the screen
 //                                 tiles of its footprint (pool indices), plus a list of
 //                                 triangles spanning more than bin_max_tiles tiles
@@ -97,8 +97,8 @@ struct __align__(16) ViewRec {
   int16_t btx0, bty0, bntx, bnty;  // the tiles of the footprint box
   int32_t big_base;     // entries of the triangles spanning more than kBinMaxTiles tiles
   int32_t big_count;
-  int32_t tri_base;     // first set-up triangle of this (eye, view) in the pool
   int32_t tri_count;    // its set-up triangles
+  int32_t parts_done;   // set-up blocks of a grid of several parts that have finished
   int32_t pad;
   int32_t bb[4];        // conservative footprint in pixels, inclusive; bb[0] > bb[2] when empty
   float Mf[12];         // camera -> eye rotation (3x3) then translation, FP32
@@ -121,7 +121,12 @@ static_assert(sizeof(TriRec) == 48, "TriRec layout");
 
 constexpr int kClusterCells = 4;         // cells per cluster side (set-up works cluster by cluster)
 constexpr int kBinMaxTiles = 16;         // the static-scratch render's cap on tiles binned per triangle
-constexpr int kMaxGridForSetup = 257;    // (G-1)/4 squared clusters must fit the set-up kernel's table
+constexpr int kMaxGridForSetup = 257;    // triangle ids and the cluster grid are sized for it
+
+constexpr int kSetupPartClusters = 256;  // clusters a triangle set-up block takes (a view of more is split into parts)
+
+// Clusters per side of a mesh grid, and whether its set-up takes several blocks per view.
+__host__ __device__ constexpr int clusters_per_side(int G) { return (G - 1 + kClusterCells - 1) / kClusterCells; }
 
 struct GridTables {
   const float* a;   // n_views x G
@@ -145,10 +150,12 @@ struct FrameArgs {
   const void* textures;
   const void* depth;
   GridTables tables;
+  const float2* cluster_z; // n_views x clusters: depth range of each cluster of cells
   ViewRec* vrecs;
   uint32_t* tile_masks;
   EyeFloat* eyes_f;
   TriRec* pool;
+  int32_t* pool_owner;     // per record its eye * n_views + view (grids set up by several blocks per view)
   int64_t pool_capacity;
   unsigned long long* pool_counter;
   int32_t* bin_offsets;
@@ -184,6 +191,8 @@ struct FrameArgs {
 // launchers (return cudaGetLastError())
 cudaError_t launch_grid_tables(const ViewStatic* views, int n_views, int src_w, int src_h, int G,
                                float* a, float* b, cudaStream_t s);
+cudaError_t launch_cluster_bounds(const void* depth, int mesh_format, const ViewStatic* views, int n_views, int G,
+                                  float2* out, cudaStream_t s);
 cudaError_t launch_convert_textures(const uint8_t* src, void* dst, int64_t n_texels, int fmt,
                                     const float* scale_per_texel_view, int64_t texels_per_view,
                                     cudaStream_t s);

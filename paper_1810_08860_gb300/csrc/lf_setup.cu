@@ -7,10 +7,14 @@
 //                        projection, disk constants, and a conservative screen
 //                        footprint of the disk, which is OR-ed into per-tile view
 //                        masks (the culling of disks against the eye, Sec. 4.2.1).
-//   tri_setup_kernel     per call, one CTA per (eye, view) with a non-empty
-//                        footprint: vertex transform and 1/256-pixel snap, near
-//                        clip, int64 triangle set-up and footprint culling, written
-//                        as one contiguous segment in triangle-id order.
+//   cluster_bounds_kernel  once per mesh build: the depth range of every cluster
+//                        of 4x4 cells.
+//   tri_setup_kernel     per call, one CTA per (eye, view, part) with a non-empty
+//                        footprint: clusters culled by their depth ranges, then
+//                        vertex transform and 1/256-pixel snap, near clip, int64
+//                        triangle set-up and footprint culling; it bins the view's
+//                        triangles when the grid is one part.
+//   bin_records_kernel, bin_scan_kernel  the binning of grids of several parts.
 //
 // Every float operation that feeds an integer decision (snapped position, depth
 // winner, disk membership) uses explicit round-to-nearest intrinsics in a fixed
@@ -326,7 +330,7 @@ __global__ void __launch_bounds__(kViewSetupThreads) view_setup_kernel(FrameArgs
       const int tb = A.tex_format == LF_TEX_F32 ? 16 : A.tex_format == LF_TEX_BF16 ? 8 : 4;
       R.tex = A.tex_table ? A.tex_table[v]
                           : static_cast<const char*>(A.textures) + (int64_t)v * A.src_w * A.src_h * tb;
-      R.tri_base = 0;
+      R.parts_done = 0;
       R.bin_off = -1;
       R.big_base = 0;
       R.big_count = 0;
@@ -421,16 +425,46 @@ cudaError_t launch_view_setup(const FrameArgs& a, cudaStream_t s) {
   return cudaGetLastError();
 }
 
+// ------------------------------------------------------------------ cluster depth bounds
+
+// Per view and cluster of kClusterCells^2 mesh cells: the smallest and largest
+// depth of its vertices, once per mesh build.  A warp per cluster.
+__global__ void cluster_bounds_kernel(const void* __restrict__ depth, int mesh_format,
+                                      const ViewStatic* __restrict__ views, int G, int ncl, int64_t n_clusters,
+                                      float2* __restrict__ out) {
+  const int64_t w = (blockIdx.x * (int64_t)blockDim.x + threadIdx.x) >> 5;
+  const int lane = threadIdx.x & 31;
+  if (w >= n_clusters) return;
+  const int64_t v = w / (ncl * ncl);
+  const int c = (int)(w - v * ncl * ncl), cy = c / ncl, cx = c - cy * ncl;
+  float lo = INFINITY, hi = -INFINITY;
+  if (lane < 25) {
+    const int k = min(cy * kClusterCells + lane / 5, G - 1), j = min(cx * kClusterCells + lane % 5, G - 1);
+    const int64_t gi = (v * G + k) * G + j;
+    const float z = mesh_format == LF_MESH_F16_OFFSET
+                        ? __fadd_rn(views[v].depth_origin, __half2float(reinterpret_cast<const __half*>(depth)[gi]))
+                        : reinterpret_cast<const float*>(depth)[gi];
+    lo = hi = z;
+  }
+#pragma unroll
+  for (int o = 16; o > 0; o >>= 1) {
+    lo = fminf(lo, __shfl_xor_sync(0xffffffffu, lo, o));
+    hi = fmaxf(hi, __shfl_xor_sync(0xffffffffu, hi, o));
+  }
+  if (lane == 0) out[w] = make_float2(lo, hi);
+}
+
+cudaError_t launch_cluster_bounds(const void* depth, int mesh_format, const ViewStatic* views, int n_views, int G,
+                                  float2* out, cudaStream_t s) {
+  const int ncl = clusters_per_side(G);
+  const int64_t n = (int64_t)n_views * ncl * ncl;
+  cluster_bounds_kernel<<<(unsigned)((n * 32 + 255) / 256), 256, 0, s>>>(depth, mesh_format, views, G, ncl, n, out);
+  return cudaGetLastError();
+}
+
 // ------------------------------------------------------------------ triangle set-up
 
-struct VtxSmem {
-  float* x;
-  float* y;
-  float* z;
-  uint8_t* oc;  // outcode: bit0..3 left/right/above/below the padded footprint, bit4 behind z_near
-};
-
-constexpr uint8_t kOcBehind = 16;
+constexpr uint32_t kOcBehind = 16;  // outcode: bit0..3 left/right/above/below the padded footprint, bit4 behind z_near
 
 struct SetupCtx {
   float fx, fy, cx, cy, zn;
@@ -471,68 +505,67 @@ __device__ bool setup_sub(const int32_t* sx, const int32_t* sy, const SetupCtx& 
   return true;
 }
 
-// Set up parent triangle `id` from vertex slots q0, q1, q2; writes up to two
-// records into out[] and returns how many were kept.  The decisions (snap,
-// clip, orientation, fill rule) are taken exactly as the oracle takes them;
-// the outcode test only drops triangles that lie wholly outside the padded
-// disk footprint, whose pixels never see this view.
-__device__ __forceinline__ int setup_parent(int id, int q0, int q1, int q2, const VtxSmem& S, const SetupCtx& C,
-                                            TriRec* out) {
-  const uint8_t o0 = S.oc[q0], o1 = S.oc[q1], o2 = S.oc[q2];
-  if (o0 & o1 & o2) return 0;  // all behind, or all beyond one side of the footprint
-  const int n_in = ((o0 & kOcBehind) == 0) + ((o1 & kOcBehind) == 0) + ((o2 & kOcBehind) == 0);
-  const float x0 = S.x[q0], y0 = S.y[q0], z0 = S.z[q0];
-  const float x1 = S.x[q1], y1 = S.y[q1], z1 = S.z[q1];
-  const float x2 = S.x[q2], y2 = S.y[q2], z2 = S.z[q2];
+// A vertex in eye space.
+struct EyeVtx {
+  float x, y, z;
+};
+
+// The snapped polygon of a parent triangle after the near clip: np vertices (0:
+// dropped, 3, or 4: two sub-triangles, a fan from the first kept vertex) and the
+// parent's FP32 inverse-depth plane.  The decisions (snap, clip) are taken
+// exactly as the oracle takes them.
+struct SetupPoly {
+  int32_t px[4], py[4];
+  int np;
+  float ia, ib, ic;
+};
+
+__device__ __forceinline__ void setup_poly(const EyeVtx& v0, const EyeVtx& v1, const EyeVtx& v2, uint32_t o0,
+                                           uint32_t o1, uint32_t o2, const SetupCtx& C, SetupPoly& P) {
+  P.np = 0;
   // FP32 inverse-depth plane of the parent (original vertex order), fixed order.
-  const float e1x = __fsub_rn(x1, x0), e1y = __fsub_rn(y1, y0), e1z = __fsub_rn(z1, z0);
-  const float e2x = __fsub_rn(x2, x0), e2y = __fsub_rn(y2, y0), e2z = __fsub_rn(z2, z0);
+  const float e1x = __fsub_rn(v1.x, v0.x), e1y = __fsub_rn(v1.y, v0.y), e1z = __fsub_rn(v1.z, v0.z);
+  const float e2x = __fsub_rn(v2.x, v0.x), e2y = __fsub_rn(v2.y, v0.y), e2z = __fsub_rn(v2.z, v0.z);
   const float nx = __fsub_rn(__fmul_rn(e1y, e2z), __fmul_rn(e1z, e2y));
   const float ny = __fsub_rn(__fmul_rn(e1z, e2x), __fmul_rn(e1x, e2z));
   const float nz = __fsub_rn(__fmul_rn(e1x, e2y), __fmul_rn(e1y, e2x));
-  const float dd = dot3_rn(nx, ny, nz, x0, y0, z0);
-  const float ia = __fdiv_rn(nx, dd), ib = __fdiv_rn(ny, dd), ic = __fdiv_rn(nz, dd);
-  if (dd == 0.0f || !isfinite(ia) || !isfinite(ib) || !isfinite(ic)) return 0;
-  int32_t px[4], py[4];
+  const float dd = dot3_rn(nx, ny, nz, v0.x, v0.y, v0.z);
+  P.ia = __fdiv_rn(nx, dd); P.ib = __fdiv_rn(ny, dd); P.ic = __fdiv_rn(nz, dd);
+  if (dd == 0.0f || !isfinite(P.ia) || !isfinite(P.ib) || !isfinite(P.ic)) return;
+  if (((o0 | o1 | o2) & kOcBehind) == 0) {
+    if (!snap_rn(v0.x, v0.y, v0.z, C.fx, C.fy, C.cx, C.cy, P.px[0], P.py[0])) return;
+    if (!snap_rn(v1.x, v1.y, v1.z, C.fx, C.fy, C.cx, C.cy, P.px[1], P.py[1])) return;
+    if (!snap_rn(v2.x, v2.y, v2.z, C.fx, C.fy, C.cx, C.cy, P.px[2], P.py[2])) return;
+    P.px[3] = P.px[2]; P.py[3] = P.py[2];
+    P.np = 3;
+    return;
+  }
+  // Sutherland-Hodgman against z >= z_near, walking v0 -> v1 -> v2 -> v0.
+  const float vx[3] = {v0.x, v1.x, v2.x}, vy[3] = {v0.y, v1.y, v2.y}, vz[3] = {v0.z, v1.z, v2.z};
+  const bool in[3] = {(o0 & kOcBehind) == 0, (o1 & kOcBehind) == 0, (o2 & kOcBehind) == 0};
   int np = 0;
-  if (n_in == 3) {
-    if (!snap_rn(x0, y0, z0, C.fx, C.fy, C.cx, C.cy, px[0], py[0])) return 0;
-    if (!snap_rn(x1, y1, z1, C.fx, C.fy, C.cx, C.cy, px[1], py[1])) return 0;
-    if (!snap_rn(x2, y2, z2, C.fx, C.fy, C.cx, C.cy, px[2], py[2])) return 0;
-    np = 3;
-  } else {
-    // Sutherland-Hodgman against z >= z_near, walking v0 -> v1 -> v2 -> v0.
-    const float vx[3] = {x0, x1, x2}, vy[3] = {y0, y1, y2}, vz[3] = {z0, z1, z2};
-    const bool in[3] = {(o0 & kOcBehind) == 0, (o1 & kOcBehind) == 0, (o2 & kOcBehind) == 0};
 #pragma unroll
-    for (int k = 0; k < 3; ++k) {
-      const int k1 = (k + 1) % 3;
-      if (in[k]) {
-        if (!snap_rn(vx[k], vy[k], vz[k], C.fx, C.fy, C.cx, C.cy, px[np], py[np])) return 0;
-        ++np;
-      }
-      if (in[k] != in[k1]) {
+  for (int k = 0; k < 3; ++k) {
+    const int k1 = (k + 1) % 3;
+#pragma unroll
+    for (int h = 0; h < 2; ++h) {  // the vertex if it is in front, then the crossing of the edge
+      float ix = vx[k], iy = vy[k], iz = vz[k];
+      if (h == 0 ? !in[k] : in[k] == in[k1]) continue;
+      if (h == 1) {
         const float tt = __fdiv_rn(__fsub_rn(C.zn, vz[k]), __fsub_rn(vz[k1], vz[k]));
-        const float ix = __fmaf_rn(tt, __fsub_rn(vx[k1], vx[k]), vx[k]);
-        const float iy = __fmaf_rn(tt, __fsub_rn(vy[k1], vy[k]), vy[k]);
-        if (!snap_rn(ix, iy, C.zn, C.fx, C.fy, C.cx, C.cy, px[np], py[np])) return 0;
-        ++np;
+        ix = __fmaf_rn(tt, __fsub_rn(vx[k1], vx[k]), vx[k]);
+        iy = __fmaf_rn(tt, __fsub_rn(vy[k1], vy[k]), vy[k]);
+        iz = C.zn;
       }
+      int32_t sx, sy;
+      if (!snap_rn(ix, iy, iz, C.fx, C.fy, C.cx, C.cy, sx, sy)) return;
+#pragma unroll
+      for (int i = 0; i < 4; ++i)  // static indexes keep the polygon in registers
+        if (i == np) { P.px[i] = sx; P.py[i] = sy; }
+      ++np;
     }
   }
-  int n = 0;
-#pragma unroll
-  for (int f = 0; f < 2; ++f) {
-    if (f + 2 >= np) break;
-    const int32_t sx[3] = {px[0], px[f + 1], px[f + 2]}, sy[3] = {py[0], py[f + 1], py[f + 2]};
-    int32_t tl;
-    TriRec& t = out[n];
-    if (!setup_sub(sx, sy, C, t, tl)) continue;
-    t.ia = ia; t.ib = ib; t.ic = ic;
-    t.id_tl = (id << 3) | tl;
-    ++n;
-  }
-  return n;
+  P.np = np;
 }
 
 // Block-wide exclusive scan of small non-negative counts (blockDim.x multiple of 32).
@@ -559,30 +592,102 @@ __device__ __forceinline__ int block_exclusive_scan(int v, int* s_warp, int& tot
 
 // ------------------------------------------------------------------ binning
 
-// Bins one (eye, view)'s n set-up triangles (pool records tri_base ..
-// tri_base + n - 1, written by this block) into the screen tiles of its
-// footprint box; the triangle set-up block calls it once its records are
-// written.  Per tile the bin holds pool indices of the triangles whose pixel
-// box overlaps it, in no particular order (the per-view depth decision does
-// not depend on order); triangles whose box spans more than A.bin_max_tiles
-// tiles go to the view's list of big ones, which every tile of the view scans
-// (only the static-scratch render caps it).  Offsets and cursors live in the
-// offset pool: [ntiles + 1 absolute entry offsets][ntiles cursors]; the
-// per-tile counts and cursors use `cnt` (cnt_cap ints of shared memory) when
-// the footprint fits, else the pool's cursor half.
+// A view's set-up triangles are binned into the screen tiles of its footprint
+// box: per tile the bin holds the pool indices of the triangles whose pixel box
+// overlaps it, in no particular order (the per-view depth decision does not
+// depend on order).  Offsets and cursors live in the offset pool: [ntiles + 1
+// absolute entry offsets][ntiles cursors].
+
+struct TileBox {
+  int tx0, ty0, ntx, nty;
+  int sw, sh;  // log2 of the tile's width and height (8, 16 or 32)
+};
+
+__device__ __forceinline__ TileBox footprint_tiles(const int32_t* bb, int tw, int th) {
+  TileBox b;
+  b.sw = __ffs(tw) - 1;
+  b.sh = __ffs(th) - 1;
+  b.tx0 = bb[0] >> b.sw;
+  b.ty0 = bb[1] >> b.sh;
+  b.ntx = (bb[2] >> b.sw) - b.tx0 + 1;
+  b.nty = (bb[3] >> b.sh) - b.ty0 + 1;
+  return b;
+}
+
+// f(tile) for each tile of the box (relative to it) that a record's pixel box
+// overlaps; returns false, without calling f, when these are more than max_tiles.
+// Shifts, not divisions: set-up of the stereo rig 25 -> 22 us.
+template <typename F>
+__device__ __forceinline__ bool for_record_tiles(int2 bb, const TileBox& b, int max_tiles, F&& f) {
+  const int x0 = max(((int)(int16_t)(bb.x & 0xffff) >> b.sw) - b.tx0, 0);
+  const int y0 = max((bb.x >> (16 + b.sh)) - b.ty0, 0);
+  const int x1 = min(((int)(int16_t)(bb.y & 0xffff) >> b.sw) - b.tx0, b.ntx - 1);
+  const int y1 = min((bb.y >> (16 + b.sh)) - b.ty0, b.nty - 1);
+  if (x0 > x1 || y0 > y1) return true;
+  if ((x1 - x0 + 1) * (y1 - y0 + 1) > max_tiles) return false;
+  for (int y = y0; y <= y1; ++y)
+    for (int x = x0; x <= x1; ++x) f(y * b.ntx + x);
+  return true;
+}
+
+// One thread: room for a view's offsets and cursors; -1 (and the error bit) when there is none.
+__device__ long long take_offsets(const FrameArgs& A, int nt) {
+  const unsigned long long o = atomicAdd(A.bin_offsets_counter, (unsigned long long)(2 * nt + 1));
+  if ((long long)o + 2 * nt + 1 <= A.bin_offsets_capacity) return (long long)o;
+  atomicOr(A.error_word, kErrPoolOverflow);
+  return -1;
+}
+
+__device__ long long take_entries(const FrameArgs& A, int need) {
+  const unsigned long long b = atomicAdd(A.bin_entries_counter, (unsigned long long)need);
+  if ((long long)b + need <= A.bin_entries_capacity) return (long long)b;
+  atomicOr(A.error_word, kErrPoolOverflow);
+  return -1;
+}
+
+// Counts -> absolute offsets (offs, nt + 1 of them) and cursors (cnt, in place)
+// by one block; `extra` entries follow the bins.  Returns the first entry, or -1
+// when the entry pool is full.
 template <int BLOCK>
-__device__ void bin_view(const FrameArgs& A, ViewRec& R, int n, int tri_base, int* cnt_smem, int cnt_cap,
+__device__ long long scan_bins(const FrameArgs& A, int* cnt, int* offs, int nt, int extra, int* s_warp, int& total) {
+  __shared__ long long s_ent;
+  const int per = (nt + BLOCK - 1) / BLOCK;  // each thread owns a contiguous run
+  const int r0 = threadIdx.x * per, r1 = min(r0 + per, nt);
+  int run = 0;
+  for (int k = r0; k < r1; ++k) run += cnt[k];
+  int o = block_exclusive_scan(run, s_warp, total);
+  if (threadIdx.x == 0) s_ent = take_entries(A, total + extra);
+  __syncthreads();
+  const long long ent = s_ent;
+  if (ent < 0) return -1;
+  for (int k = r0; k < r1; ++k) {
+    const int c = cnt[k];
+    offs[k] = (int)(ent + o);
+    cnt[k] = (int)(ent + o);
+    o += c;
+  }
+  if (threadIdx.x == 0) offs[nt] = (int)(ent + total);
+  return ent;
+}
+
+// Bins one view's records, the n_ranges ranges (first pool index, count <= 32)
+// its block has just written; a warp takes a range.  Triangles whose box spans
+// more than A.bin_max_tiles tiles go to the view's list of big ones, which every
+// tile of the view scans (only the static-scratch render caps it).  The per-tile
+// counts and cursors use `cnt` (cnt_cap ints of shared memory) when the
+// footprint fits, else the pool's cursor half.
+template <int BLOCK>
+__device__ void bin_view(const FrameArgs& A, ViewRec& R, const int2* ranges, int n_ranges, int* cnt_smem, int cnt_cap,
                          int* s_warp) {
-  __shared__ long long s_off, s_ent;
+  __shared__ long long s_off;
   __shared__ int s_big;
+  constexpr int NW = BLOCK / 32;
+  const int lane = threadIdx.x & 31, warp = threadIdx.x >> 5;
   const int tw = A.tile_w, th = A.tile_h;
-  const int tx0 = R.bb[0] / tw, ty0 = R.bb[1] / th;
-  const int ntx = R.bb[2] / tw - tx0 + 1, nty = R.bb[3] / th - ty0 + 1;
-  const int nt = ntx * nty;
+  const TileBox tb = footprint_tiles(R.bb, tw, th);
+  const int nt = tb.ntx * tb.nty;
   if (threadIdx.x == 0) {
-    const unsigned long long o = atomicAdd(A.bin_offsets_counter, (unsigned long long)(2 * nt + 1));
-    s_off = ((long long)o + 2 * nt + 1 <= A.bin_offsets_capacity) ? (long long)o : -1;
-    if (s_off < 0) atomicOr(A.error_word, kErrPoolOverflow);
+    s_off = take_offsets(A, nt);
     s_big = 0;
   }
   __syncthreads();
@@ -592,95 +697,70 @@ __device__ void bin_view(const FrameArgs& A, ViewRec& R, int n, int tri_base, in
   int* cnt = nt <= cnt_cap ? cnt_smem : curs;  // counts, then cursors
   for (int k = threadIdx.x; k < nt; k += BLOCK) cnt[k] = 0;
   __syncthreads();
-  const TriRec* tris = A.pool + tri_base;
-  auto span = [&](int t, int& x0, int& y0, int& x1, int& y1) {
-    const int2 bb = *reinterpret_cast<const int2*>(tris + t);
-    x0 = max((int)(int16_t)(bb.x & 0xffff) / tw - tx0, 0);
-    y0 = max((bb.x >> 16) / th - ty0, 0);
-    x1 = min((int)(int16_t)(bb.y & 0xffff) / tw - tx0, ntx - 1);
-    y1 = min((bb.y >> 16) / th - ty0, nty - 1);
-  };
   int my_big = 0;
-  for (int t = threadIdx.x; t < n; t += BLOCK) {
-    int x0, y0, x1, y1;
-    span(t, x0, y0, x1, y1);
-    if (x0 > x1 || y0 > y1) continue;
-    if ((x1 - x0 + 1) * (y1 - y0 + 1) > A.bin_max_tiles) { ++my_big; continue; }
-    for (int y = y0; y <= y1; ++y)
-      for (int x = x0; x <= x1; ++x) atomicAdd(&cnt[y * ntx + x], 1);
+  for (int r = warp; r < n_ranges; r += NW) {
+    if (lane >= ranges[r].y) continue;
+    const int2 bb = *reinterpret_cast<const int2*>(A.pool + ranges[r].x + lane);
+    if (!for_record_tiles(bb, tb, A.bin_max_tiles, [&](int tile) { atomicAdd(&cnt[tile], 1); })) ++my_big;
   }
   if (my_big) atomicAdd(&s_big, my_big);
   __syncthreads();
-  // exclusive scan of the counts in place; each thread owns a contiguous run
-  const int per = (nt + BLOCK - 1) / BLOCK;
-  const int r0 = threadIdx.x * per, r1 = min(r0 + per, nt);
-  int run = 0;
-  for (int k = r0; k < r1; ++k) run += cnt[k];
   int total;
-  int o = block_exclusive_scan(run, s_warp, total);
-  if (threadIdx.x == 0) {
-    const int need = total + s_big;
-    const unsigned long long b = atomicAdd(A.bin_entries_counter, (unsigned long long)need);
-    s_ent = ((long long)b + need <= A.bin_entries_capacity) ? (long long)b : -1;
-    if (s_ent < 0) atomicOr(A.error_word, kErrPoolOverflow);
-  }
-  __syncthreads();
-  const long long ent = s_ent;
+  const long long ent = scan_bins<BLOCK>(A, cnt, offs, nt, s_big, s_warp, total);
   if (ent < 0) return;
-  for (int k = r0; k < r1; ++k) {
-    const int c = cnt[k];
-    offs[k] = (int)(ent + o);
-    cnt[k] = (int)(ent + o);  // cursor
-    o += c;
-  }
-  if (threadIdx.x == 0) {
-    offs[nt] = (int)(ent + total);
-    s_big = 0;
-  }
+  __syncthreads();
+  if (threadIdx.x == 0) s_big = 0;
   __syncthreads();
   const int big_base = (int)(ent + total);
-  for (int t = threadIdx.x; t < n; t += BLOCK) {
-    int x0, y0, x1, y1;
-    span(t, x0, y0, x1, y1);
-    if (x0 > x1 || y0 > y1) continue;
-    const int idx = tri_base + t;
-    if ((x1 - x0 + 1) * (y1 - y0 + 1) > A.bin_max_tiles) {
+  for (int r = warp; r < n_ranges; r += NW) {
+    if (lane >= ranges[r].y) continue;
+    const int idx = ranges[r].x + lane;
+    const int2 bb = *reinterpret_cast<const int2*>(A.pool + idx);
+    if (!for_record_tiles(bb, tb, A.bin_max_tiles, [&](int tile) { A.bin_entries[atomicAdd(&cnt[tile], 1)] = idx; }))
       A.bin_entries[big_base + atomicAdd(&s_big, 1)] = idx;
-      continue;
-    }
-    for (int y = y0; y <= y1; ++y)
-      for (int x = x0; x <= x1; ++x) A.bin_entries[atomicAdd(&cnt[y * ntx + x], 1)] = idx;
   }
   __syncthreads();
   if (threadIdx.x == 0) {
     R.bin_off = (int32_t)s_off;
-    R.btx0 = (int16_t)tx0; R.bty0 = (int16_t)ty0;
-    R.bntx = (int16_t)ntx; R.bnty = (int16_t)nty;
+    R.btx0 = (int16_t)tb.tx0; R.bty0 = (int16_t)tb.ty0;
+    R.bntx = (int16_t)tb.ntx; R.bnty = (int16_t)tb.nty;
     R.big_base = big_base;
     R.big_count = s_big;
   }
 }
 
-// Shared-memory row stride of the vertex arrays: >= G and = 4 (mod 32), so
-// the 4x4 cells of a cluster read 16 different banks.
-__host__ __device__ inline int vertex_row_stride(int G) { return G + ((36 - G % 32) % 32); }
+constexpr int kSetupBlock = 256;
+constexpr int kPartClusters = kSetupPartClusters;
+static_assert(kPartClusters == kSetupBlock, "one thread per cluster in the first cull");
 
-// One CTA per (eye, view) whose disk footprint reaches the eye.  Per band of
-// grid rows: (1) the band's vertices go to eye space with outcodes against the
-// padded footprint; (2) warps walk the 4x4-cell clusters, skip clusters whose
-// vertices all lie beyond one side (or behind the eye), and append the
-// triangles that pass their own outcode test to a candidate list; (3) all
-// threads share the candidates for the full set-up (snap, clip, orientation,
-// fill rule).  With the whole grid in one band (the usual case) one atomic
-// reserves an upper bound of the view's records and one pass writes them;
-// with several bands pass 1 counts the records, one atomic reserves the
-// view's segment and pass 2 writes them.  The order inside a segment does not matter:
-// the raster's depth decision within a view is order-independent.  Then the
-// block bins its records into the screen tiles (bin_view), the shared memory
-// of the vertex arrays holding the per-tile counts.
-template <int BLOCK>
-__global__ void __launch_bounds__(BLOCK, 3) tri_setup_kernel(FrameArgs A, int band_rows, int cnt_cap) {
-  constexpr int NW = BLOCK / 32;
+// One block per (eye, view, part) whose disk footprint reaches the eye; a part
+// is kPartClusters clusters of 4x4 cells, the whole view for grids up to 65^2.
+// (1) A thread per cluster: the eight corners of the frustum piece that holds
+//     the cluster (its ray rectangle between its nearest and farthest depth)
+//     against the padded footprint; a cluster wholly beyond one side, or behind
+//     the near plane, is dropped without touching its vertices.  On the rig all
+//     but a few per cent go here: a view's footprint holds tens of its cells.
+// (2) A warp per listed cluster: 25 lanes transform its vertices, and each of
+//     the 32 lanes takes a triangle from their registers (shuffles), culls it by
+//     outcodes, sets it up (snap, clip, orientation, fill rule) and the warp
+//     appends the kept records to the pool.
+// (3) MULTI = false (one part): the block bins the view's records.  MULTI = true:
+//     every record notes its (eye, view) in A.pool_owner, the last part of a view
+//     to finish reserves and clears its tile counts, and the bin_* kernels below
+//     count and scatter all records of the call, a thread each.
+// Bound by the latency of its phases (dependent loads, the pool's atomic, the
+// divisions of a triangle), not by bytes (about 40 KB per view).  Against blocks
+// that staged and transformed every vertex of a view (in bands, twice, where the
+// grid did not fit shared memory), launches serialised: stereo rig 34 -> 22 us;
+// grids of 129^2 and 200^2 (256 views, a 400^2 eye, count and scatter included)
+// 208 -> 51 us and 458 -> 62 us; a prefilter's 64 renders of 256^2 meshes 5.7 ->
+// 2.3 ms.  One-part grids keep the binning in the block: with a view's blocks as a
+// cluster that counts in the leader's shared memory (distributed shared memory
+// atomics), 256 views and a 400^2 eye took 20 us instead of 29, but the stereo rig
+// 30 to 128 us instead of 22 (1 to 8 blocks per view).
+template <bool MULTI>
+__global__ void __launch_bounds__(kSetupBlock, MULTI ? 4 : 3) tri_setup_kernel(FrameArgs A, int cnt_cap) {
+  constexpr int NW = kSetupBlock / 32;
   const int v = blockIdx.x, e = blockIdx.y;
   const int lane = threadIdx.x & 31, warp = threadIdx.x >> 5;
   // the view set-up has completed (it wrote the view records read below); the
@@ -688,246 +768,227 @@ __global__ void __launch_bounds__(BLOCK, 3) tri_setup_kernel(FrameArgs A, int ba
   griddep_wait();
   griddep_release();
   ViewRec& R = A.vrecs[(int64_t)e * A.n_views + v];
-  const int bb0 = R.bb[0], bb1 = R.bb[1], bb2 = R.bb[2], bb3 = R.bb[3];
-  if (bb0 > bb2 || bb1 > bb3) return;  // disk footprint misses the eye
+  SetupCtx C;
+  C.bb0 = R.bb[0]; C.bb1 = R.bb[1]; C.bb2 = R.bb[2]; C.bb3 = R.bb[3];
+  if (C.bb0 > C.bb2 || C.bb1 > C.bb3) return;  // disk footprint misses the eye
   // a two-level frame sets up only the views the eye draws
   if (A.enable_bits && !((A.enable_bits[(int64_t)e * A.mask_words + (v >> 5)] >> (v & 31)) & 1u)) return;
   const EyeParams& E = A.eyes[e];
   const EyeFloat& EF = A.eyes_f[e];
-  const int G = A.G;
-  extern __shared__ __align__(16) unsigned char smem[];
-  const int RS = vertex_row_stride(G);
-  const int nv_band = (band_rows + 1) * RS;
-  const int n_cell = G - 1;
-  VtxSmem S;
-  S.x = reinterpret_cast<float*>(smem);
-  S.y = S.x + nv_band;
-  S.z = S.y + nv_band;
-  uint16_t* s_cand = reinterpret_cast<uint16_t*>(S.z + nv_band);  // candidate triangles of the band
-  S.oc = reinterpret_cast<uint8_t*>(s_cand + 2 * n_cell * band_rows);
+  const int G = A.G, n_cell = G - 1, ncl = clusters_per_side(G);
+  extern __shared__ __align__(16) unsigned char smem[];  // the binning's per-tile counts
   __shared__ int s_warp[NW];
-  __shared__ int s_ncand, s_pos, s_ntwo;
-  __shared__ long long s_tri_base;
-
-  SetupCtx C;
+  __shared__ uint16_t s_list[kPartClusters];
+  __shared__ int2 s_range[2 * kPartClusters];  // records written: a range per cluster, a second one after a near clip
+  __shared__ int s_nlist, s_nrange, s_total;
+  if (threadIdx.x == 0) s_nlist = s_nrange = s_total = 0;
   C.fx = EF.fx; C.fy = EF.fy; C.cx = EF.cx; C.cy = EF.cy;
   C.zn = A.z_near; C.W = E.W; C.H = E.H;
-  C.bb0 = bb0; C.bb1 = bb1; C.bb2 = bb2; C.bb3 = bb3;
   // outcode planes in the form fx*x <op> (edge - cx) * z, padded by 2 pixels
-  const float oxl = (float)bb0 - 2.0f - C.cx, oxr = (float)bb2 + 3.0f - C.cx;
-  const float oyt = (float)bb1 - 2.0f - C.cy, oyb = (float)bb3 + 3.0f - C.cy;
+  const float oxl = (float)C.bb0 - 2.0f - C.cx, oxr = (float)C.bb2 + 3.0f - C.cx;
+  const float oyt = (float)C.bb1 - 2.0f - C.cy, oyb = (float)C.bb3 + 3.0f - C.cy;
   float Mf[12];
 #pragma unroll
   for (int k = 0; k < 12; ++k) Mf[k] = R.Mf[k];
   const float* ta = A.tables.a + (int64_t)v * G;
   const float* tb = A.tables.b + (int64_t)v * G;
-  const ViewStatic& V = A.views[v];
-  const int ncl = (n_cell + kClusterCells - 1) / kClusterCells;  // clusters per side
-  const int n_bands = (n_cell + band_rows - 1) / band_rows;
+  auto to_eye = [&](float a, float b, float z) {  // grid point z (a, b, 1), fixed order
+    const float X = __fmul_rn(z, a), Y = __fmul_rn(z, b);
+    EyeVtx q;
+    q.x = __fmaf_rn(Mf[0], X, __fmaf_rn(Mf[1], Y, __fmaf_rn(Mf[2], z, Mf[9])));
+    q.y = __fmaf_rn(Mf[3], X, __fmaf_rn(Mf[4], Y, __fmaf_rn(Mf[5], z, Mf[10])));
+    q.z = __fmaf_rn(Mf[6], X, __fmaf_rn(Mf[7], Y, __fmaf_rn(Mf[8], z, Mf[11])));
+    return q;
+  };
+  auto side_bits = [&](const EyeVtx& q) -> uint32_t {
+    const float ux = C.fx * q.x, uy = C.fy * q.y;
+    return (ux < oxl * q.z ? 1u : 0u) | (ux > oxr * q.z ? 2u : 0u) | (uy < oyt * q.z ? 4u : 0u) |
+           (uy > oyb * q.z ? 8u : 0u);
+  };
+  __syncthreads();
 
-  // q / G without an integer division: (q + 1/2) / G is at least 1/(2G) away
-  // from an integer and the float product errs by under 3e-5 for q < 2^17.
-  const float inv_G = 1.0f / (float)G;
-  const float inv_ncl = 1.0f / (float)ncl;
-  auto load_band = [&](int k0, int k1) {  // vertex rows k0 .. k1 inclusive
-    const int nq = (k1 - k0 + 1) * G;
-#pragma unroll 4
-    for (int q = threadIdx.x; q < nq; q += BLOCK) {
-      const int kq = (int)(((float)q + 0.5f) * inv_G);
-      const int k = k0 + kq, j = q - kq * G;
-      const int64_t gi = ((int64_t)v * G + k) * G + j;
-      float z;
-      if (A.mesh_format == LF_MESH_F16_OFFSET)
-        z = __fadd_rn(V.depth_origin, __half2float(reinterpret_cast<const __half*>(A.depth)[gi]));
-      else
-        z = __ldg(reinterpret_cast<const float*>(A.depth) + gi);
-      const float X = __fmul_rn(z, __ldg(ta + j)), Y = __fmul_rn(z, __ldg(tb + k)), Z = z;
-      const float ex = __fmaf_rn(Mf[0], X, __fmaf_rn(Mf[1], Y, __fmaf_rn(Mf[2], Z, Mf[9])));
-      const float ey = __fmaf_rn(Mf[3], X, __fmaf_rn(Mf[4], Y, __fmaf_rn(Mf[5], Z, Mf[10])));
-      const float ez = __fmaf_rn(Mf[6], X, __fmaf_rn(Mf[7], Y, __fmaf_rn(Mf[8], Z, Mf[11])));
-      uint8_t oc = kOcBehind;
-      if (ez >= C.zn) {
-        const float ux = C.fx * ex, uy = C.fy * ey;
-        oc = (uint8_t)((ux < oxl * ez ? 1 : 0) | (ux > oxr * ez ? 2 : 0) | (uy < oyt * ez ? 4 : 0) |
-                       (uy > oyb * ez ? 8 : 0));
+  // ---- (1) clusters that can reach the footprint.  The half-spaces are linear, so
+  // what holds at the eight corners holds for every point between them.
+  {
+    const int c = blockIdx.z * kPartClusters + threadIdx.x;
+    bool keep = false;
+    if (c < ncl * ncl) {
+      const int cl_y = c / ncl, cl_x = c - cl_y * ncl;
+      const float2 zr = __ldg(A.cluster_z + (int64_t)v * ncl * ncl + c);
+      const int j = cl_x * kClusterCells, k = cl_y * kClusterCells;
+      const float a[2] = {__ldg(ta + j), __ldg(ta + min(j + kClusterCells, n_cell))};
+      const float b[2] = {__ldg(tb + k), __ldg(tb + min(k + kClusterCells, n_cell))};
+      uint32_t oc = 31u;
+#pragma unroll
+      for (int i = 0; i < 8; ++i) {
+        const EyeVtx q = to_eye(a[i & 1], b[(i >> 1) & 1], i < 4 ? zr.x : zr.y);
+        oc &= side_bits(q) | (q.z < C.zn ? kOcBehind : 0u);
       }
-      const int slot = kq * RS + j;
-      S.x[slot] = ex; S.y[slot] = ey; S.z[slot] = ez;
-      S.oc[slot] = oc;
+      keep = oc == 0u;
     }
-  };
-  // vertex slots of band-local triangle (kk, j, half)
-  auto tri_slots = [&](int kk, int j, int half, int& q0, int& q1, int& q2) {
-    const int r0 = kk * RS;
-    if (half == 0) { q0 = r0 + j; q1 = r0 + j + 1; q2 = r0 + RS + j; }
-    else { q0 = r0 + j + 1; q1 = r0 + RS + j + 1; q2 = r0 + RS + j; }
-  };
-  // Warps walk the band's clusters; surviving triangles join the candidate list.
-  auto gather = [&](int k0, int k1) {
-    if (threadIdx.x == 0) s_ncand = s_ntwo = 0;
-    __syncthreads();
-    const int cy0 = k0 / kClusterCells, cy1 = (k1 + kClusterCells - 1) / kClusterCells;
-    const int c0 = cy0 * ncl, c1 = cy1 * ncl;
-    for (int c = c0 + warp; c < c1; c += NW) {
-      const int cl_y = (int)(((float)c + 0.5f) * inv_ncl), cl_x = c - cl_y * ncl;
-      // AND of the outcodes of the cluster's (up to) 5 x 5 vertices: a bit set
-      // here is set on every vertex of every triangle of the cluster
-      uint32_t oca = 0xffu;
-      if (lane < 25) {
-        const int k = min(cl_y * kClusterCells + lane / 5, n_cell), j = min(cl_x * kClusterCells + lane % 5, n_cell);
-        oca = S.oc[(k - k0) * RS + j];
-      }
-      if (__reduce_and_sync(0xffffffffu, oca) != 0u) continue;
-      const int cell = lane >> 1, half = lane & 1;
-      const int j = cl_x * kClusterCells + (cell & 3), k = cl_y * kClusterCells + (cell >> 2);
-      bool keep = false, two = false;
-      if (j < n_cell && k < k1) {
-        int q0, q1, q2;
-        tri_slots(k - k0, j, half, q0, q1, q2);
-        const uint8_t o0 = S.oc[q0], o1 = S.oc[q1], o2 = S.oc[q2];
-        keep = (o0 & o1 & o2) == 0;
-        // exactly two vertices in front of the near plane: clipping may give two sub-triangles
-        two = keep && ((o0 & kOcBehind) == 0) + ((o1 & kOcBehind) == 0) + ((o2 & kOcBehind) == 0) == 2;
-      }
-      const uint32_t bal = __ballot_sync(0xffffffffu, keep);
-      const uint32_t bal2 = __ballot_sync(0xffffffffu, two);
-      if (lane == 0 && bal2) atomicAdd(&s_ntwo, __popc(bal2));
-      int base = 0;
-      if (lane == 0 && bal) base = atomicAdd(&s_ncand, __popc(bal));
-      base = __shfl_sync(0xffffffffu, base, 0);
-      if (keep) s_cand[base + __popc(bal & ((1u << lane) - 1u))] = (uint16_t)((((k - k0) * n_cell + j) << 1) | half);
-    }
-    __syncthreads();
-  };
-  auto setup_cand = [&](int k0, int code, TriRec* tmp) -> int {
-    const int half = code & 1, cell = code >> 1;
-    const int kk = (int)(((float)cell + 0.5f) / (float)n_cell);
-    const int j = cell - kk * n_cell;
-    int q0, q1, q2;
-    tri_slots(kk, j, half, q0, q1, q2);
-    const int id = 2 * ((k0 + kk) * n_cell + j) + half;
-    return setup_parent(id, q0, q1, q2, S, C, tmp);
-  };
-
-  if (n_bands == 1) {
-    // The whole grid in one band: one pass.  The view reserves an upper bound of
-    // its records (one per candidate, two for a candidate with exactly two
-    // vertices in front of the near plane), then writes the records it keeps
-    // compactly from the start of the reservation.
-    __syncthreads();
-    load_band(0, n_cell);
-    __syncthreads();
-    gather(0, n_cell);
-    const int nc = s_ncand;
-    if (threadIdx.x == 0) {
-      const int bound = nc + s_ntwo;
-      long long tb_ = -1;
-      if (bound > 0) {
-        const unsigned long long b = atomicAdd(A.pool_counter, (unsigned long long)bound);
-        if ((long long)b + bound <= A.pool_capacity) tb_ = (long long)b;
-        else atomicOr(A.error_word, kErrPoolOverflow);
-      }
-      s_tri_base = tb_;
-      s_pos = 0;
-    }
-    __syncthreads();
-    const long long tri_base = s_tri_base;
-    if (tri_base < 0) return;
-    for (int i = threadIdx.x; i < nc; i += BLOCK) {
-      TriRec tmp[2];
-      const int n = setup_cand(0, s_cand[i], tmp);
-      if (n) {
-        const int pos = atomicAdd(&s_pos, n);
-        for (int k = 0; k < n; ++k) A.pool[tri_base + pos + k] = tmp[k];
-      }
-    }
-    __syncthreads();  // the block's records are written and visible to all its threads
-    const int total = s_pos;
-    if (threadIdx.x == 0) {
-      R.tri_base = (int32_t)tri_base;
-      R.tri_count = total;
-    }
-    if (total > 0) bin_view<BLOCK>(A, R, total, (int)tri_base, reinterpret_cast<int*>(smem), cnt_cap, s_warp);
-    return;
-  }
-
-  // Several bands: pass 1 counts the kept records, pass 2 writes them.
-  int my_count = 0;
-  for (int bnd = 0; bnd < n_bands; ++bnd) {
-    const int k0 = bnd * band_rows, k1 = min(k0 + band_rows, n_cell);
-    __syncthreads();
-    load_band(k0, k1);
-    __syncthreads();
-    gather(k0, k1);
-    const int nc = s_ncand;
-    for (int i = threadIdx.x; i < nc; i += BLOCK) {
-      TriRec tmp[2];
-      my_count += setup_cand(k0, s_cand[i], tmp);
-    }
-  }
-  int total;
-  block_exclusive_scan(my_count, s_warp, total);
-  if (threadIdx.x == 0) {
-    long long tb_ = -1;
-    if (total > 0) {
-      const unsigned long long b = atomicAdd(A.pool_counter, (unsigned long long)total);
-      if ((long long)b + total <= A.pool_capacity) tb_ = (long long)b;
-      else atomicOr(A.error_word, kErrPoolOverflow);
-    }
-    s_tri_base = tb_;
-    s_pos = 0;
-    R.tri_base = tb_ < 0 ? 0 : (int32_t)tb_;
-    R.tri_count = tb_ < 0 ? 0 : total;
+    const uint32_t m = __ballot_sync(0xffffffffu, keep);
+    int base = 0;
+    if (lane == 0 && m) base = atomicAdd(&s_nlist, __popc(m));
+    base = __shfl_sync(0xffffffffu, base, 0);
+    if (keep) s_list[base + __popc(m & ((1u << lane) - 1u))] = (uint16_t)threadIdx.x;
   }
   __syncthreads();
-  const long long tri_base = s_tri_base;
-  if (tri_base < 0) return;
-  // Pass 2: write the records.
-  for (int bnd = 0; bnd < n_bands; ++bnd) {
-    const int k0 = bnd * band_rows, k1 = min(k0 + band_rows, n_cell);
-    __syncthreads();
-    load_band(k0, k1);
-    __syncthreads();
-    gather(k0, k1);
-    const int nc = s_ncand;
-    for (int i = threadIdx.x; i < nc; i += BLOCK) {
-      TriRec tmp[2];
-      const int n = setup_cand(k0, s_cand[i], tmp);
-      if (n) {
-        const int pos = atomicAdd(&s_pos, n);
-        for (int k = 0; k < n; ++k) A.pool[tri_base + pos + k] = tmp[k];
+
+  // ---- (2) the listed clusters' triangles
+  const int n_list = s_nlist;
+  const float z0 = A.mesh_format == LF_MESH_F16_OFFSET ? A.views[v].depth_origin : 0.0f;
+  const int cell = lane >> 1, half = lane & 1;
+  const int tcx = cell & 3, tcy = cell >> 2;  // this lane's cell in the cluster
+  // its vertices among the cluster's 5 x 5: (j,k)(j+1,k)(j,k+1) or (j+1,k)(j+1,k+1)(j,k+1)
+  const int l0 = tcy * 5 + tcx + half, l1 = half ? l0 + 5 : l0 + 1, l2 = (tcy + 1) * 5 + tcx;
+  const uint32_t below = (1u << lane) - 1u;
+  for (int i = warp; i < n_list; i += NW) {
+    const int c = blockIdx.z * kPartClusters + s_list[i];
+    const int cl_y = c / ncl, cl_x = c - cl_y * ncl;
+    const int vk = min(cl_y * kClusterCells + min(lane / 5, 4), n_cell), vj = min(cl_x * kClusterCells + lane % 5, n_cell);
+    const int64_t gi = ((int64_t)v * G + vk) * G + vj;
+    const float z = A.mesh_format == LF_MESH_F16_OFFSET
+                        ? __fadd_rn(z0, __half2float(reinterpret_cast<const __half*>(A.depth)[gi]))
+                        : __ldg(reinterpret_cast<const float*>(A.depth) + gi);
+    const EyeVtx q = to_eye(__ldg(ta + vj), __ldg(tb + vk), z);
+    const uint32_t oc = q.z >= C.zn ? side_bits(q) : kOcBehind;
+    EyeVtx p0, p1, p2;
+    p0.x = __shfl_sync(0xffffffffu, q.x, l0); p0.y = __shfl_sync(0xffffffffu, q.y, l0); p0.z = __shfl_sync(0xffffffffu, q.z, l0);
+    p1.x = __shfl_sync(0xffffffffu, q.x, l1); p1.y = __shfl_sync(0xffffffffu, q.y, l1); p1.z = __shfl_sync(0xffffffffu, q.z, l1);
+    p2.x = __shfl_sync(0xffffffffu, q.x, l2); p2.y = __shfl_sync(0xffffffffu, q.y, l2); p2.z = __shfl_sync(0xffffffffu, q.z, l2);
+    const uint32_t o0 = __shfl_sync(0xffffffffu, oc, l0), o1 = __shfl_sync(0xffffffffu, oc, l1);
+    const uint32_t o2 = __shfl_sync(0xffffffffu, oc, l2);
+    const int j = cl_x * kClusterCells + tcx, k = cl_y * kClusterCells + tcy;
+    SetupPoly P;
+    P.np = 0;
+    // the outcodes only drop triangles that lie wholly behind the near plane or outside
+    // the padded disk footprint, whose pixels never see this view
+    if (j < n_cell && k < n_cell && (o0 & o1 & o2) == 0) setup_poly(p0, p1, p2, o0, o1, o2, C, P);
+    const int id = 2 * (k * n_cell + j) + half;
+#pragma unroll
+    for (int f = 0; f < 2; ++f) {
+      if (f == 1 && !__any_sync(0xffffffffu, P.np == 4)) break;
+      TriRec t;
+      int32_t tl = 0;
+      bool kept = false;
+      if (P.np >= f + 3) {
+        const int32_t sx[3] = {P.px[0], P.px[f + 1], P.px[f + 2]}, sy[3] = {P.py[0], P.py[f + 1], P.py[f + 2]};
+        kept = setup_sub(sx, sy, C, t, tl);
+      }
+      const uint32_t m = __ballot_sync(0xffffffffu, kept);
+      if (m == 0) continue;
+      unsigned long long base = 0;
+      if (lane == 0) base = atomicAdd(A.pool_counter, (unsigned long long)__popc(m));
+      base = __shfl_sync(0xffffffffu, base, 0);
+      const int n = __popc(m);
+      const bool fits = (int64_t)base + n <= A.pool_capacity;
+      const int64_t at = (int64_t)base + __popc(m & below);
+      if (kept && at < A.pool_capacity) {
+        t.ia = P.ia; t.ib = P.ib; t.ic = P.ic;
+        t.id_tl = (id << 3) | tl;
+        A.pool[at] = t;
+        if constexpr (MULTI) A.pool_owner[at] = e * A.n_views + v;
+      }
+      if (lane == 0) {
+        if (!fits) atomicOr(A.error_word, kErrPoolOverflow);
+        atomicAdd(&s_total, n);
+        if (!MULTI && fits) s_range[atomicAdd(&s_nrange, 1)] = make_int2((int)base, n);
       }
     }
   }
-  __syncthreads();  // the block's records are written and visible to all its threads
-  bin_view<BLOCK>(A, R, total, (int)tri_base, reinterpret_cast<int*>(smem), cnt_cap, s_warp);
+  __syncthreads();  // the block's records and ranges are visible to all its threads
+
+  // ---- (3) bins
+  if constexpr (!MULTI) {
+    if (threadIdx.x == 0) R.tri_count = s_total;
+    if (s_nrange > 0) bin_view<kSetupBlock>(A, R, s_range, s_nrange, reinterpret_cast<int*>(smem), cnt_cap, s_warp);
+  } else {
+    __shared__ int s_last;
+    __shared__ long long s_off;
+    if (threadIdx.x == 0) {
+      if (s_total) atomicAdd(&R.tri_count, s_total);
+      __threadfence();
+      s_last = atomicAdd(&R.parts_done, 1) == (int)gridDim.z - 1;
+      s_off = -1;
+      if (s_last && atomicAdd(&R.tri_count, 0) > 0) {
+        const TileBox t = footprint_tiles(R.bb, A.tile_w, A.tile_h);
+        s_off = take_offsets(A, t.ntx * t.nty);
+        if (s_off >= 0) {
+          R.bin_off = (int32_t)s_off;
+          R.btx0 = (int16_t)t.tx0; R.bty0 = (int16_t)t.ty0;
+          R.bntx = (int16_t)t.ntx; R.bnty = (int16_t)t.nty;
+        }
+      }
+    }
+    __syncthreads();
+    if (s_off < 0) return;
+    const TileBox t = footprint_tiles(R.bb, A.tile_w, A.tile_h);
+    const int nt = t.ntx * t.nty;
+    int* curs = A.bin_offsets + s_off + nt + 1;
+    for (int k = threadIdx.x; k < nt; k += kSetupBlock) curs[k] = 0;
+  }
 }
 
-constexpr int kSetupBlock = 256;
-constexpr size_t kVtxBytes = 13;  // x, y, z (4 B each) + outcode
+// Records of the call, a thread each (four at a time, their loads together): pass
+// 0 counts the bins' entries, pass 1 (after bin_scan_kernel) scatters the pool
+// indices through the cursors.
+template <int PASS>
+__global__ void __launch_bounds__(256) bin_records_kernel(FrameArgs A) {
+  constexpr int U = 4;
+  griddep_wait();
+  griddep_release();
+  const int64_t n = min((int64_t)*A.pool_counter, A.pool_capacity), step = (int64_t)gridDim.x * blockDim.x;
+  const int sw = __ffs(A.tile_w) - 1, sh = __ffs(A.tile_h) - 1;
+  for (int64_t i0 = blockIdx.x * (int64_t)blockDim.x + threadIdx.x; i0 < n; i0 += U * step) {
+    int2 bb[U];
+    int4 bins[U];  // bin_off, btx0 | bty0, bntx | bnty, big_base
+#pragma unroll
+    for (int u = 0; u < U; ++u) {
+      const int64_t i = i0 + u * step;
+      bins[u].x = -1;
+      if (i >= n) continue;
+      bb[u] = *reinterpret_cast<const int2*>(A.pool + i);
+      bins[u] = *reinterpret_cast<const int4*>(&A.vrecs[A.pool_owner[i]].bin_off);
+    }
+#pragma unroll
+    for (int u = 0; u < U; ++u) {
+      if (bins[u].x < 0) continue;
+      const TileBox b = {(int16_t)(bins[u].y & 0xffff), bins[u].y >> 16, (int16_t)(bins[u].z & 0xffff), bins[u].z >> 16, sw, sh};
+      int* curs = A.bin_offsets + bins[u].x + b.ntx * b.nty + 1;
+      for_record_tiles(bb[u], b, INT32_MAX, [&](int tile) {
+        const int at = atomicAdd(&curs[tile], 1);
+        if (PASS == 1) A.bin_entries[at] = (int)(i0 + u * step);
+      });
+    }
+  }
+}
 
-// Cell rows per band: the whole grid when it fits (vertex arrays plus a 16-bit
-// candidate per triangle), else a multiple of the cluster size.
-static int setup_band_rows(int G, size_t smem_limit) {
-  const size_t per_row = kVtxBytes * (size_t)vertex_row_stride(G) + 2 * 2 * (size_t)(G - 1);
-  int rows = (int)((smem_limit - kVtxBytes * (size_t)vertex_row_stride(G)) / per_row);
-  rows = min(rows, 32767 / max(1, G - 1));  // band-local triangle codes fit 16 bits
-  if (rows >= G - 1) return G - 1;
-  rows = (rows / kClusterCells) * kClusterCells;
-  return rows < kClusterCells ? kClusterCells : rows;
+// A block per (eye, view) with records: its counts become offsets and cursors.
+__global__ void __launch_bounds__(kSetupBlock) bin_scan_kernel(FrameArgs A) {
+  __shared__ int s_warp[kSetupBlock / 32];
+  griddep_wait();
+  griddep_release();
+  ViewRec& R = A.vrecs[(int64_t)blockIdx.y * A.n_views + blockIdx.x];
+  if (R.bin_off < 0) return;
+  const int nt = (int)R.bntx * R.bnty;
+  int* offs = A.bin_offsets + R.bin_off;
+  int total;
+  const long long ent = scan_bins<kSetupBlock>(A, offs + nt + 1, offs, nt, 0, s_warp, total);
+  if (ent < 0 && threadIdx.x == 0) R.bin_off = -1;  // no room: the view has no bins (its offsets were not written)
 }
 
 cudaError_t launch_tri_setup(const FrameArgs& a, cudaStream_t s, bool pdl) {
-  const size_t limit = 96 * 1024;
-  cudaError_t err = ensure_dynamic_smem(reinterpret_cast<const void*>(tri_setup_kernel<kSetupBlock>), (int)limit + 64);
-  if (err != cudaSuccess) return err;
-  const int rows = setup_band_rows(a.G, limit);
-  const size_t vtx = (size_t)(rows + 1) * vertex_row_stride(a.G) * kVtxBytes + 2 * 2 * (size_t)(a.G - 1) * rows + 64;
-  // the binning counts reuse the vertex arrays' shared memory: at least kBinSmemTiles ints
-  const size_t bytes = std::max(vtx, sizeof(int) * (size_t)kBinSmemTiles);
-  const int cnt_cap = (int)(bytes / sizeof(int));
-  dim3 grid(a.n_views, a.n_eyes);
-  return launch_kernel(tri_setup_kernel<kSetupBlock>, grid, dim3(kSetupBlock), bytes, s, pdl, a, rows, cnt_cap);
+  const size_t bytes = sizeof(int) * (size_t)kBinSmemTiles;
+  const int ncl = clusters_per_side(a.G);
+  const int parts = (ncl * ncl + kPartClusters - 1) / kPartClusters;
+  const dim3 grid(a.n_views, a.n_eyes, parts), block(kSetupBlock);
+  if (parts == 1) return launch_kernel(tri_setup_kernel<false>, grid, block, bytes, s, pdl, a, kBinSmemTiles);
+  cudaError_t e = launch_kernel(tri_setup_kernel<true>, grid, block, 0, s, pdl, a, 0);
+  const dim3 all(152 * 8);
+  if (e == cudaSuccess) e = launch_kernel(bin_records_kernel<0>, all, dim3(256), 0, s, pdl, a);
+  if (e == cudaSuccess) e = launch_kernel(bin_scan_kernel, dim3(a.n_views, a.n_eyes), block, 0, s, pdl, a);
+  if (e == cudaSuccess) e = launch_kernel(bin_records_kernel<1>, all, dim3(256), 0, s, pdl, a);
+  return e;
 }
 
 }  // namespace lfk

@@ -2,12 +2,16 @@
 pixel or per triangle (fine meshes), one or several windows of gathered
 triangles, one or several rounds of views.  The reference is the inspection
 render, whose coverage is held to the oracle elsewhere; the arithmetic of every
-form is the same, so the images are compared bit for bit."""
+form is the same, so the images are compared bit for bit.
+
+Grids whose triangle set-up takes one block per view (up to 65^2 vertices) and
+several: coverage records against the oracle, and the triangle pool's limit."""
 import math
 
 import pytest
 
 import scene
+from tests.test_gpu_parity import _check_full_frame
 
 pytestmark = pytest.mark.gpu
 
@@ -51,4 +55,60 @@ def test_every_form_draws_the_inspection_image(views, size, grid, disk, eye, ova
     tiles = -(-eye[0] // tile[0]) * -(-eye[1] // tile[1])
     if views <= 32 and grid <= 33 and tiles <= 8192:  # lf_render_static's limits
         assert torch.equal(r.render_static(e), want)
+    r.close()
+
+
+def _cap(views, size, grid, seed=3):
+    side = math.isqrt(views - 1) + 1
+    lf = scene.build_light_field(scene.sphere_scene(seed, 8, forward_cone_deg=35.0),
+                                 scene.cap_grid_directions(side, 40.0)[:views], size, size, 90.0, grid)
+    e = scene.head_pose_eyes(scene.SplitMix64(seed), 75, 53, 90.0, yaw_range=(-0.1, 0.1), pitch_deg=6.0, stereo=False)[0]
+    return lf, e
+
+
+@pytest.mark.parametrize("grid,mesh", [(2, "f32"), (6, "f16"), (65, "f32"), (66, "f32"), (70, "f32"), (131, "f32")])
+def test_grids_of_one_and_of_several_parts_cover_as_the_oracle(grid, mesh):
+    pytest.importorskip("torch")
+    import __graft_entry__
+
+    __graft_entry__.build()
+    import paper_1810_08860_gb300 as lfm
+
+    lf, e = _cap(9, 64, grid)
+    if mesh == "f16":  # depths that FP16 offsets hold exactly: the oracle sees the same mesh
+        lf.depth = (lf.depth * 8).round().clip(8, 48) / 8
+        lf.depth = lf.depth.astype("float32")
+    r = lfm.Renderer(0)
+    r.load_views(lf)
+    r.build_meshes(lf, mesh_format=mesh)
+    _check_full_frame(r, lf, e)
+    r.close()
+
+
+@pytest.mark.parametrize("grid", [33, 66])
+def test_a_pool_that_is_too_small_is_reported_and_the_context_stays_usable(grid):
+    torch = pytest.importorskip("torch")
+    import __graft_entry__
+
+    __graft_entry__.build()
+    import paper_1810_08860_gb300 as lfm
+
+    lf, e = _cap(9, 64, grid)
+    r = lfm.Renderer(0, tri_capacity=500)
+    r.load_views(lf)
+    r.build_meshes(lf)
+    r.render([e])
+    with pytest.raises(lfm.LFError, match="CAPACITY"):
+        r.stats()
+    r.close()
+    r = lfm.Renderer(0)
+    r.load_views(lf)
+    r.build_meshes(lf)
+    img = r.render([e])[0]
+    n = r.stats()["triangles"]
+    q = lfm.Renderer(0, tri_capacity=n)  # the records that a view keeps fit exactly
+    q.load_views(lf)
+    q.build_meshes(lf)
+    assert torch.equal(q.render([e])[0], img) and q.stats()["triangles"] == n
+    q.close()
     r.close()
