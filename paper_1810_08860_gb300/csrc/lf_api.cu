@@ -1129,7 +1129,6 @@ extern "C" lf_status lf_render_static(lf_ctx* c, const lf_pose* eye, const lf_in
 namespace {
 
 constexpr int kRefineSegs[3] = {896, 9248, 867};  // W1+b1, W2+b2, W3+b3
-constexpr int kRefineSegBase[3] = {kRefineOffW1, kRefineOffW2, kRefineOffW3};
 
 float* rf_params(lf_ctx* c) { return static_cast<float*>(c->rf.state.p); }
 float* rf_grad(lf_ctx* c) { return rf_params(c) + kRefineParams; }
@@ -1236,9 +1235,9 @@ lf_status refine_backward(lf_ctx* c, int32_t n, int32_t w, int32_t h, const floa
   const int64_t n_pix = (int64_t)n * w * h;
   lf_status st = refine_hidden(c, n_pix, true);
   if (st != LF_OK) return st;
-  const int tiles_x = (w + 31) / 32, tiles_y = (h + 7) / 8;
-  const int n_tiles = tiles_x * tiles_y * n;
-  const int n_ctas = std::max(1, std::min(n_tiles, 3 * c->sm_count));  // weight-gradient CTAs: three per SM
+  int tiles_x = 0, tiles_y = 0;
+  const int n_tiles = refine_wgrad_tiles(n, h, w, &tiles_x, &tiles_y);
+  const int n_ctas = std::max(1, std::min(n_tiles, c->sm_count));  // weight-gradient CTAs: one per SM
   LF_CUDA(c, ensure(c->rf.partial, sizeof(float) * (size_t)n_ctas * (896 + 9248 + 867)));
   float* loss = static_cast<float*>(c->rf.scal.p);
   int32_t* count = reinterpret_cast<int32_t*>(loss + 1);
@@ -1272,7 +1271,7 @@ lf_status refine_backward(lf_ctx* c, int32_t n, int32_t w, int32_t h, const floa
   float* part2 = part1 + (size_t)n_ctas * kRefineSegs[0];
   float* part3 = part2 + (size_t)n_ctas * kRefineSegs[1];
   // layer 3 weights (dL/dr with a2), then dL/dz2 through layer 3's input
-  g.g_f = gr; g.a_h = a2; g.partial = part3;
+  g.g_f = gr; g.a_h = a2; g.partial = part3; g.seg = kRefineSegs[2];
   LF_CUDA(c, launch_refine_wgrad(3, g, s));
   a = conv_args(c, n, w, h);
   a.src_f = gr; a.wt = rf_w(c, kPackW3b); a.mask = a2; a.out_h = gz2;
@@ -1281,13 +1280,12 @@ lf_status refine_backward(lf_ctx* c, int32_t n, int32_t w, int32_t h, const floa
   a = conv_args(c, n, w, h);
   a.src_h = gz2; a.wt = rf_w(c, kPackW2b); a.mask = a1; a.out_h = a2;
   LF_CUDA(c, launch_refine_conv(kConvInBF16, 32, kEpiMask, a, s));
-  g.g_f = nullptr; g.g_h = gz2; g.a_h = a1; g.partial = part2;
+  g.g_f = nullptr; g.g_h = gz2; g.a_h = a1; g.partial = part2; g.seg = kRefineSegs[1];
   LF_CUDA(c, launch_refine_wgrad(2, g, s));
-  g.g_h = a2; g.a_h = nullptr; g.x = in; g.partial = part1;
+  g.g_h = a2; g.a_h = nullptr; g.x = in; g.partial = part1; g.seg = kRefineSegs[0];
   LF_CUDA(c, launch_refine_wgrad(1, g, s));
-  float* parts[3] = {part1, part2, part3};
-  for (int k = 0; k < 3; ++k)
-    LF_CUDA(c, launch_refine_reduce(parts[k], n_ctas, kRefineSegs[k], rf_grad(c) + kRefineSegBase[k], s));
+  const float* const parts[3] = {part1, part2, part3};
+  LF_CUDA(c, launch_refine_reduce(parts, n_ctas, rf_grad(c), s));
   return LF_OK;
 }
 

@@ -253,14 +253,18 @@ struct RefineWgradArgs {
   const __nv_bfloat16* g_h;    // modes 1, 2: dL/dz (32 channels)
   const __nv_bfloat16* a_h;    // modes 2, 3: the layer input (32 channels)
   const float* x;              // mode 1: the network input RGBA
-  float* partial;              // [n_ctas][segment]
-  int32_t* error;              // set (bit 8) if a wait for a chunk's MMAs gave up
-  uint64_t wait_ns;            // bound on that wait
+  float* partial;              // [n_ctas][seg]: [ky][kx][o][c], then the biases
+  int32_t seg;                 // floats of the layer's gradient
+  int32_t* error;              // set (bits 8 and on) if a wait gave up
+  uint64_t wait_ns;            // bound on each wait
 };
 
 cudaError_t launch_refine_conv(int in_mode, int cout, int epi, const RefineConvArgs& a, cudaStream_t s);
 cudaError_t launch_refine_wgrad(int mode, const RefineWgradArgs& a, cudaStream_t s);
-cudaError_t launch_refine_reduce(const float* partial, int n_rows, int seg, float* grad, cudaStream_t s);
+// The weight-gradient kernels' tiles of n H x W images: their number, and per row and column.
+int refine_wgrad_tiles(int n, int H, int W, int* tiles_x, int* tiles_y);
+// The three layers' partial rows (layer k at partial[k], seg = cin x cout x 9 + cout) summed into grad.
+cudaError_t launch_refine_reduce(const float* const partial[3], int n_rows, float* grad, cudaStream_t s);
 cudaError_t launch_refine_count(const float* x, const float* t, int64_t n_pix, int32_t* count, cudaStream_t s);
 cudaError_t launch_refine_adam(float* p, float* m, float* v, const float* g, int n, float lr, double beta1,
                                double beta2, float eps, float c1, float c2, cudaStream_t s);

@@ -24,22 +24,34 @@
 
 namespace lfk {
 
-// grad[base + i] = sum over the CTA rows b of partial[b][i], in a fixed order:
+// grad = sum over the CTA rows of the three layers' partials, in a fixed order:
 // eight interleaved sums (rows k, k + 8, k + 16, .. for k < 8) added pairwise.
-// 256 threads: 8 row phases x 32 consecutive outputs.
-__global__ void reduce_partials_kernel(const float* __restrict__ partial, int n_rows, int seg,
-                                       float* __restrict__ grad) {
+// 256 threads: 8 row phases x 32 consecutive entries of a layer's row, which is
+// [ky][kx][o][c] and then the biases; gradients are [o][c][ky][kx].  One launch for
+// the three layers.
+struct ReduceArgs {
+  const float* partial[3];
+  float* grad;
+  int n_rows;
+};
+__global__ void reduce_partials_kernel(ReduceArgs A) {
+  constexpr int kCin[3] = {3, 32, 32}, kCout[3] = {32, 32, 3}, kBase[3] = {kRefineOffW1, kRefineOffW2, kRefineOffW3};
   __shared__ float part[8][32];
-  const int lane = threadIdx.x & 31, k = threadIdx.x >> 5;
+  const int lane = threadIdx.x & 31, k = threadIdx.x >> 5, layer = blockIdx.y;
+  const int cin = kCin[layer], cout = kCout[layer], nw = 9 * cin * cout, seg = nw + cout;
   const int i = blockIdx.x * 32 + lane;
+  if (blockIdx.x * 32 >= seg) return;
   float s = 0.f;
   if (i < seg)
-    for (int b = k; b < n_rows; b += 8) s += partial[(size_t)b * seg + i];
+    for (int b = k; b < A.n_rows; b += 8) s += A.partial[layer][(size_t)b * seg + i];
   part[k][lane] = s;
   __syncthreads();
-  if (k == 0 && i < seg)
-    grad[i] = ((part[0][lane] + part[1][lane]) + (part[2][lane] + part[3][lane])) +
-              ((part[4][lane] + part[5][lane]) + (part[6][lane] + part[7][lane]));
+  if (k == 0 && i < seg) {
+    const int tap = i / (cin * cout), o = (i / cin) % cout, c = i % cin;
+    A.grad[kBase[layer] + (i < nw ? (o * cin + c) * 9 + tap : i)] =
+        ((part[0][lane] + part[1][lane]) + (part[2][lane] + part[3][lane])) +
+        ((part[4][lane] + part[5][lane]) + (part[6][lane] + part[7][lane]));
+  }
 }
 
 // Number of pixels valid (alpha > 0) in both the input and the target.
@@ -121,8 +133,9 @@ __global__ void pack_weights_kernel(const float* __restrict__ prm, __nv_bfloat16
 
 // ------------------------------------------------------------------ launchers
 
-cudaError_t launch_refine_reduce(const float* partial, int n_rows, int seg, float* grad, cudaStream_t s) {
-  reduce_partials_kernel<<<(seg + 31) / 32, 256, 0, s>>>(partial, n_rows, seg, grad);
+cudaError_t launch_refine_reduce(const float* const partial[3], int n_rows, float* grad, cudaStream_t s) {
+  const ReduceArgs a = {{partial[0], partial[1], partial[2]}, grad, n_rows};
+  reduce_partials_kernel<<<dim3((9 * 32 * 32 + 32 + 31) / 32, 3), 256, 0, s>>>(a);
   return cudaGetLastError();
 }
 

@@ -499,66 +499,105 @@ cudaError_t launch_refine_conv(int in_mode, int cout, int epi, const RefineConvA
 
 // ------------------------------------------------------------------ weight gradients
 //
-// dW[o][c][tap] = sum_p g[p][o] a[p + off(tap)][c], db[o] = sum_p g[p][o]
-// (g = dL/dz of the layer's output, a = the layer's input), as one GEMM
-// D[(tap, c)][o] over K = pixels: M = 9 x 32 rows of shifted input channels
-// plus a row of ones, whose product with g is the bias gradient (modes 2, 3:
-// 289 rows in three M-tiles of 128; mode 1, the 3-channel input: 28 rows in
-// one), N = the output channels (32; 3 padded to 16 in mode 3).  Both operands
-// are K-major, so a CTA transposes each 64-pixel chunk (32 x 2 outputs) into
-// shared memory: ldmatrix.trans turns an 8-position x 8-channel block of a
-// staged 32-channel map into one channel's 8 consecutive pixels spread over four
-// lanes, i.e. one 16-byte operand row.  The accumulators stay in TMEM over all
-// of a CTA's chunks; the CTA then writes its partial row, and the rows are
-// summed in a fixed order afterwards (deterministic).
+// dW[o][c][ky][kx] = sum_p g[p][o] a[p + (ky - 1, kx - 1)][c], db[o] = sum_p g[p][o]
+// (g = dL/dz of the layer's output, a = the layer's input), as one GEMM over
+// K = pixels whose operands are the maps as they lie in memory: both are read
+// MN-major (channels contiguous), so nothing is transposed.  A tile is 32 x 8
+// positions of a; per image row r of g
+//   D[(i, c)][(kx, o)] += sum_x a[r - 1 + i][x][c] g[r][x + 1 - kx][o]
+// with M = 128: four consecutive rows i of a (ky = i; the fourth is not used) of
+// 32 channels, and N = 96: three copies of g, each loaded by TMA with its own shift
+// (zeros outside the image).  A 32-channel map lies as [row][position][32 channels]
+// under the 64-byte swizzle, so M steps from row to row of a and N from copy to copy
+// of g.  The 3-channel maps (the network input, dL/dr) land as FP32 RGBA and two
+// warps round them to BF16 rows of 8 channels, the last five zero, without swizzle:
+// M then covers sixteen rows (three used), N = 32 four copies (three used).  The
+// same two warps sum g for the bias gradient.
 //   MODE 1: g = dL/dz1 (BF16, 32), a = the network input (FP32 RGBA, 3).  W1, b1.
 //   MODE 2: g = dL/dz2 (BF16, 32), a = a1 (BF16, 32).                        W2, b2.
 //   MODE 3: g = dL/dr  (FP32 RGBA, 3), a = a2 (BF16, 32).                    W3, b3.
+//
+// One CTA per SM, a ring of stages between a TMA warp, an MMA warp and the two
+// warps above; the accumulators stay in TMEM over all tiles of a CTA, which then
+// writes one partial row; the rows are summed in a fixed order afterwards
+// (deterministic).  Bound by the operands' way through shared memory (an MMA reads
+// 4 KB of A and 3 KB of B, 62 cycles against the 53 of its arithmetic) and by the
+// three copies of g from L2.  Against kernels that transposed chunks of 64 pixels
+// with ldmatrix and wrote every input nine times for its taps, 16 crops of 256^2:
+// 109, 67 and 93 us for W2, W1 and W3 -> 33, 32 and 23 us (training step 564 -> 370).
 
 namespace {
 
-constexpr int kWPx = 64;                         // pixels per chunk: 32 x 2 outputs
-constexpr int kWHW = 34, kWHH = 4;               // input halo of a chunk
-constexpr int kWRowB = 80;                       // staged 32-channel rows (64 B + 16 B: no bank conflicts)
-constexpr int kWThreads = 128;
+constexpr int kGTW = 32, kGTH = 8;               // tile: 32 x 8 positions
+constexpr int kG32Row = kGTW * 64;               // a row of 32 channels
+constexpr int kG8Row = kGTW * 16;                // a row of 8 channels
+constexpr int kGThreads = 128;
 
-__device__ __forceinline__ void c_ldsm_x4_t(uint32_t addr, uint32_t (&r)[4]) {
-  asm volatile("ldmatrix.sync.aligned.m8n8.x4.trans.shared.b16 {%0,%1,%2,%3}, [%4];\n"
-               : "=r"(r[0]), "=r"(r[1]), "=r"(r[2]), "=r"(r[3]) : "r"(addr));
+template <int MODE>
+struct WgradShape {
+  static constexpr int OC = MODE == 3 ? 8 : 32;          // channels of g as held
+  static constexpr int KX = MODE == 3 ? 4 : 3;           // copies of g held (three loaded)
+  static constexpr int N = KX * OC;
+  static constexpr int COUT = MODE == 3 ? 3 : 32, CIN = MODE == 1 ? 3 : 32;
+  static constexpr int kARow = MODE == 1 ? kG8Row : kG32Row, kAB = (kGTH + 2) * kARow;
+  static constexpr int kGRow = MODE == 3 ? kG8Row : kG32Row, kGCopy = kGTH * kGRow, kGB = KX * kGCopy;
+  static constexpr int FW = MODE == 1 ? kGTW : kGTW + 2, FH = MODE == 1 ? kGTH + 2 : kGTH;  // FP32 RGBA positions
+  static constexpr int kFB = MODE == 2 ? 0 : (FW * FH * 16 + 511) / 512 * 512;
+  static constexpr int kStageB = kAB + kGB + kFB;
+  static constexpr int kTx = MODE == 1 ? kGB + FW * FH * 16 : MODE == 2 ? kAB + kGB : kAB + FW * FH * 16;
+  static constexpr int kStages = MODE == 3 ? 5 : 3;
+  // The unused accumulator rows take what lies behind a tile's rows of a: the stage's g
+  static_assert((kGTH - 1) * kARow + (MODE == 1 ? 16 : 4) * kARow <= kStageB, "MMAs read within the stage");
+  static_assert(kStageB % 512 == 0, "stages start on a swizzle atom");
+  static constexpr int kBarOff = kStages * kStageB;
+  static constexpr int kSmem = 1024 + kBarOff + (3 * kStages + 1) * 8 + 16;  // 1024: the base is rounded up
+  static_assert(kSmem <= 224 * 1024, "fits one CTA's shared memory");
+};
+
+// kind::f16, FP32 accumulator, BF16 A and B, both MN-major.
+__host__ __device__ constexpr uint32_t g_idesc(int M, int N) { return c_idesc(M, N) | (1u << 15) | (1u << 16); }
+
+__device__ __forceinline__ void g_tma4(const CUtensorMap* m, uint32_t dst, uint64_t* bar, int c0, int c1, int c2, int c3) {
+  asm volatile(
+      "cp.async.bulk.tensor.4d.shared::cluster.global.mbarrier::complete_tx::bytes [%0], [%1, {%2, %3, %4, %5}], [%6];" ::
+          "r"(dst), "l"(reinterpret_cast<uint64_t>(m)), "r"(c0), "r"(c1), "r"(c2), "r"(c3), "r"(c_su32(bar))
+      : "memory");
+}
+// MN-major operands: 32-channel rows under the 64-byte swizzle (next 32 elements of M or N `mn` bytes on, 8
+// positions 512 bytes), and 8-channel rows without (next 8 elements `mn` bytes on, 8 positions 128 bytes).
+__device__ __forceinline__ uint64_t g_desc32(uint32_t addr, uint32_t mn) { return c_desc(addr, mn, 512) | (4ull << 61); }
+__device__ __forceinline__ uint64_t g_desc8(uint32_t addr, uint32_t mn) { return c_desc(addr, 128, mn); }
+
+__device__ __forceinline__ void g_arrive(uint64_t* bar) {
+  asm volatile("mbarrier.arrive.shared::cta.b64 _, [%0];" ::"r"(c_su32(bar)) : "memory");
 }
 
 }  // namespace
 
 template <int MODE>
-__global__ void __launch_bounds__(kWThreads) wgrad_tc_kernel(RefineWgradArgs A) {
-  constexpr int MR = MODE == 1 ? 128 : 384;                     // A rows (M), zero beyond the data
-  constexpr int MT = MR / 128;
-  constexpr int ONES = MODE == 1 ? 27 : 288;                    // the row of ones (bias gradient)
-  constexpr int N = MODE == 3 ? 16 : 32;
-  constexpr int COUT = MODE == 3 ? 3 : 32;
-  constexpr int SEG = MODE == 1 ? 864 + 32 : (MODE == 2 ? 9216 + 32 : 864 + 3);
-  constexpr int kLboA = MR * 16, kLboB = N * 16;                // bytes between 8-pixel K groups
-  constexpr int kAB = 8 * kLboA, kBB = 8 * kLboB;               // 64 pixels = 8 K groups
-  constexpr int kHaloB = kWHW * kWHH * kWRowB;                  // modes 2, 3: 32-channel input halo
-  constexpr int kGB = kWPx * kWRowB;                            // modes 1, 2: 32-channel g
-  extern __shared__ __align__(128) unsigned char sm[];
-  unsigned char* sa = sm;                 // A: [8 K groups][MR rows][16 B]
-  unsigned char* sb = sa + kAB;           // B: [8 K groups][N rows][16 B]
-  unsigned char* sh = sb + kBB;           // staged input halo (FP32 RGBA in mode 1)
-  unsigned char* sg = sh + kHaloB;        // staged g (FP32 RGBA in mode 3)
-  uint64_t* bar = reinterpret_cast<uint64_t*>(sg + kGB);
-  uint32_t* tslot = reinterpret_cast<uint32_t*>(bar + 1);
-  __shared__ int s_abort;
+__global__ void __launch_bounds__(kGThreads) wgrad_tc_kernel(RefineWgradArgs A, const __grid_constant__ CUtensorMap amap,
+                                                             const __grid_constant__ CUtensorMap gmap) {
+  using S = WgradShape<MODE>;
+  extern __shared__ __align__(128) unsigned char sm_raw[];
+  unsigned char* sm = sm_raw + ((1024u - (c_su32(sm_raw) & 1023u)) & 1023u);  // stages start on a swizzle atom
+  uint64_t* full = reinterpret_cast<uint64_t*>(sm + S::kBarOff);  // a stage's copies landed
+  uint64_t* ready = full + S::kStages;                             // its FP32 map is rounded (modes 1, 3)
+  uint64_t* empty = ready + S::kStages;                            // its MMAs and its readers are done
+  uint64_t* done = empty + S::kStages;                             // all MMAs of the CTA are complete
+  uint32_t* tslot = reinterpret_cast<uint32_t*>(done + 1);
+  __shared__ volatile int s_abort;
+  __shared__ float s_bias[64][8];
   const int tid = threadIdx.x, warp = tid >> 5, lane = tid & 31;
-  const int H = A.H, W = A.W;
+  const int n_tiles = A.n_tiles;
 
-  for (int i = tid; i < (kAB + kBB) / 16; i += kWThreads) reinterpret_cast<uint4*>(sa)[i] = make_uint4(0u, 0u, 0u, 0u);
-  __syncthreads();
-  for (int j = tid; j < 8; j += kWThreads)  // the row of ones
-    *reinterpret_cast<uint4*>(sa + j * kLboA + ONES * 16) = make_uint4(0x3F803F80u, 0x3F803F80u, 0x3F803F80u, 0x3F803F80u);
   if (tid == 0) {
     s_abort = 0;
-    asm volatile("mbarrier.init.shared::cta.b64 [%0], 1;" ::"r"(c_su32(bar)));
+    for (int k = 0; k < S::kStages; ++k) {
+      asm volatile("mbarrier.init.shared::cta.b64 [%0], 1;" ::"r"(c_su32(full + k)));
+      asm volatile("mbarrier.init.shared::cta.b64 [%0], 2;" ::"r"(c_su32(ready + k)));
+      asm volatile("mbarrier.init.shared::cta.b64 [%0], 3;" ::"r"(c_su32(empty + k)));
+    }
+    asm volatile("mbarrier.init.shared::cta.b64 [%0], 1;" ::"r"(c_su32(done)));
     asm volatile("fence.mbarrier_init.release.cluster;" ::: "memory");
   }
   if (warp == 0) {
@@ -570,194 +609,158 @@ __global__ void __launch_bounds__(kWThreads) wgrad_tc_kernel(RefineWgradArgs A) 
   __syncthreads();
   asm volatile("tcgen05.fence::after_thread_sync;" ::: "memory");
   const uint32_t tmem = *tslot;
+  const int n_own = (int)blockIdx.x < n_tiles ? (n_tiles - blockIdx.x + gridDim.x - 1) / gridDim.x : 0;
 
-  const int cx = (W + 31) / 32, cy = (H + 1) / 2, n_chunks = cx * cy * A.n;
-  // A chunk's g (its 64 pixels) and input halo, zeros outside the image, travel
-  // through registers: chunk k + 1 is loaded while chunk k's MMAs run, and
-  // stored into the staging buffers once chunk k's transposes have read them.
-  constexpr int GI = MODE == 3 ? 1 : 2;  // g items (16 bytes) per thread
-  constexpr int HI = MODE == 1 ? 2 : 5;  // halo items per thread
-  uint4 gr[GI], hr[HI];
-  auto load = [&](int chunk) {
-    const int img = chunk / (cx * cy), rem = chunk - img * cx * cy;
-    const int y0 = (rem / cx) * 2, x0 = (rem % cx) * 32;  // output origin; halo at (y0-1, x0-1)
-#pragma unroll
-    for (int k = 0; k < GI; ++k) {
-      const int i = tid + k * kWThreads;
-      gr[k] = make_uint4(0u, 0u, 0u, 0u);
-      if (MODE == 3) {
-        const int gy = y0 + (i >> 5), gx = x0 + (i & 31);
-        if (i < kWPx && gy < H && gx < W)
-          gr[k] = reinterpret_cast<const uint4*>(A.g_f)[((size_t)img * H + gy) * W + gx];
-      } else {
-        const int p = i >> 2, q = i & 3, gy = y0 + (p >> 5), gx = x0 + (p & 31);
-        if (gy < H && gx < W) gr[k] = reinterpret_cast<const uint4*>(A.g_h + (((size_t)img * H + gy) * W + gx) * 32)[q];
-      }
-    }
-#pragma unroll
-    for (int k = 0; k < HI; ++k) {
-      const int i = tid + k * kWThreads;
-      hr[k] = make_uint4(0u, 0u, 0u, 0u);
-      if (MODE == 1) {
-        const int gy = y0 - 1 + i / kWHW, gx = x0 - 1 + i % kWHW;
-        if (i < kWHW * kWHH && gy >= 0 && gy < H && gx >= 0 && gx < W)
-          hr[k] = reinterpret_cast<const uint4*>(A.x)[((size_t)img * H + gy) * W + gx];
-      } else {
-        const int P = i >> 2, q = i & 3, gy = y0 - 1 + P / kWHW, gx = x0 - 1 + P % kWHW;
-        if (P < kWHW * kWHH && gy >= 0 && gy < H && gx >= 0 && gx < W)
-          hr[k] = reinterpret_cast<const uint4*>(A.a_h + (((size_t)img * H + gy) * W + gx) * 32)[q];
-      }
-    }
+  // A wait for use j of stage j % kStages; on give-up sets the error bit and the CTA's abort flag.
+  auto wait_use = [&](uint64_t* bar, int j, int err) -> bool {
+    if (s_abort) return false;
+    if (c_wait(bar + j % S::kStages, (uint32_t)(j / S::kStages) & 1u, A.wait_ns) == 0) return true;
+    atomicOr(A.error, err);
+    s_abort = 1;
+    return false;
   };
-  auto store = [&]() {
-#pragma unroll
-    for (int k = 0; k < GI; ++k) {
-      const int i = tid + k * kWThreads;
-      if (MODE == 3) {
-        if (i < kWPx) reinterpret_cast<uint4*>(sg)[i] = gr[k];
-      } else {
-        *reinterpret_cast<uint4*>(sg + (i >> 2) * kWRowB + (i & 3) * 16) = gr[k];
-      }
-    }
-#pragma unroll
-    for (int k = 0; k < HI; ++k) {
-      const int i = tid + k * kWThreads;
-      if (MODE == 1) {
-        if (i < kWHW * kWHH) reinterpret_cast<uint4*>(sh)[i] = hr[k];
-      } else if ((i >> 2) < kWHW * kWHH) {
-        *reinterpret_cast<uint4*>(sh + (i >> 2) * kWRowB + (i & 3) * 16) = hr[k];
-      }
-    }
-  };
-  uint32_t phase = 0;
-  bool issued = false, any = false;
-  if (blockIdx.x < n_chunks) {
-    load(blockIdx.x);
-    store();
-    if (blockIdx.x + gridDim.x < n_chunks) load(blockIdx.x + gridDim.x);
-  }
-  for (int chunk = blockIdx.x; chunk < n_chunks; chunk += gridDim.x) {
-    __syncthreads();  // this chunk's staged g and halo are visible; the previous chunk's MMAs completed
 
-    // ---- A rows (tap, c) and B rows o, K group j = pixels 8j .. 8j + 7 (py = j / 4, px = 8 (j % 4) ..)
-    if (MODE == 1) {  // rows tap * 3 + c from the FP32 halo
-      for (int i = tid; i < 27 * 8; i += kWThreads) {
-        const int row = i >> 3, j = i & 7, tap = row / 3, c = row % 3;
-        const int base = (j / 4 + tap / 3) * kWHW + (j % 4) * 8 + tap % 3;
-        const float* hf = reinterpret_cast<const float*>(sh);
-        uint32_t w[4];
+  if (warp == 0) {
+    // ---------------------------------------------------------------- copies
+    if (lane == 0) {
+      int issued = 0;
+      for (int j = 0; j < n_own; ++j) {
+        if (j >= S::kStages && !wait_use(empty, j - S::kStages, 256)) break;
+        const int tile = blockIdx.x + j * gridDim.x, img = tile / (A.tiles_x * A.tiles_y);
+        const int rem = tile - img * A.tiles_x * A.tiles_y;
+        const int y0 = rem / A.tiles_x * kGTH, x0 = rem % A.tiles_x * kGTW;
+        const uint32_t st = c_su32(sm) + (j % S::kStages) * S::kStageB, sg = st + S::kAB, sf = sg + S::kGB;
+        uint64_t* bar = full + j % S::kStages;
+        asm volatile("mbarrier.arrive.expect_tx.shared::cta.b64 _, [%0], %1;" ::"r"(c_su32(bar)), "r"(S::kTx) : "memory");
+        g_tma4(&amap, MODE == 1 ? sf : st, bar, 0, x0, y0 - 1, img);
+        if (MODE == 3) {
+          g_tma4(&gmap, sf, bar, 0, x0 - 1, y0, img);
+        } else {
 #pragma unroll
-        for (int e = 0; e < 4; ++e) w[e] = c_pack(hf[(base + 2 * e) * 4 + c], hf[(base + 2 * e + 1) * 4 + c]);
-        *reinterpret_cast<uint4*>(sa + j * kLboA + row * 16) = make_uint4(w[0], w[1], w[2], w[3]);
+          for (int kx = 0; kx < 3; ++kx) g_tma4(&gmap, sg + kx * S::kGCopy, bar, 0, x0 + 1 - kx, y0, img);
+        }
+        issued = j + 1;
       }
-    } else {  // 9 taps x 4 channel groups x 8 K groups of 8x8 blocks, four per ldmatrix
-      for (int i = warp; i < 9 * 4 * 8 / 4; i += kWThreads / 32) {
-        const int mat = lane >> 3, r = lane & 7, b = 4 * i + mat;
-        const int tap = b >> 5, cg = (b >> 3) & 3, j = b & 7;
-        const int P = (j / 4 + tap / 3) * kWHW + (j % 4) * 8 + tap % 3 + r;
-        uint32_t v[4];
-        c_ldsm_x4_t(c_su32(sh + P * kWRowB + cg * 16), v);
+      // the last copies land before the CTA can leave (earlier ones have been waited for by their readers or are
+      // waited for here, after an abort)
+      for (int j = issued > S::kStages ? issued - S::kStages : 0; j < issued; ++j)
+        if (c_wait(full + j % S::kStages, (uint32_t)(j / S::kStages) & 1u, kCDrainNs) != 0) atomicOr(A.error, 2048);
+    }
+  } else if (warp == 1) {
+    // ---------------------------------------------------------------- MMAs
+    if (lane == 0) {
+      constexpr uint32_t id = g_idesc(128, S::N);
+      for (int j = 0; j < n_own; ++j) {
+        if (!wait_use(full, j, 256)) break;
+        if (MODE != 2 && !wait_use(ready, j, 256)) break;
+        asm volatile("tcgen05.fence::after_thread_sync;" ::: "memory");
+        const uint32_t st = c_su32(sm) + (j % S::kStages) * S::kStageB;
+        constexpr int kAK = MODE == 1 ? 256 : 1024, kGK = MODE == 3 ? 256 : 1024;  // 16 positions
+        const uint64_t ad = MODE == 1 ? g_desc8(st, kG8Row) : g_desc32(st, kG32Row);
+        const uint64_t bd = MODE == 3 ? g_desc8(st + S::kAB, S::kGCopy) : g_desc32(st + S::kAB, S::kGCopy);
+        for (int r = 0; r < kGTH; ++r)
 #pragma unroll
-        for (int k = 0; k < 4; ++k) {
-          const int bk = 4 * i + k, tk = bk >> 5, ck = (bk >> 3) & 3, jk = bk & 7;
-          *reinterpret_cast<uint32_t*>(sa + jk * kLboA + (tk * 32 + ck * 8 + (lane >> 2)) * 16 + (lane & 3) * 4) = v[k];
+          for (int k = 0; k < 2; ++k)
+            c_mma(tmem, ad + (uint64_t)((r * S::kARow + k * kAK) / 16), bd + (uint64_t)((r * S::kGRow + k * kGK) / 16), id,
+                  j > 0 || r > 0 || k > 0);
+        c_commit(empty + j % S::kStages);
+      }
+      // completes once every MMA issued has: also after an abort, so the tensor memory is never freed under one
+      c_commit(done);
+      if (c_wait(done, 0u, A.wait_ns > kCDrainNs ? A.wait_ns : kCDrainNs) != 0) atomicOr(A.error, 512);
+    }
+  } else {
+    // ---------------------------------------------------------------- rounding of FP32 maps, bias sums
+    const int t = tid - 64;  // 0 .. 63
+    float acc[8];
+#pragma unroll
+    for (int k = 0; k < 8; ++k) acc[k] = 0.f;
+    for (int j = 0; j < n_own; ++j) {
+      int ok = 1;
+      if (lane == 0) ok = wait_use(full, j, 1024);
+      if (!__shfl_sync(0xffffffffu, ok, 0)) break;
+      // (a lane that did not poll sees the copies through the shuffle's warp: every lane tests the phase once)
+      if (c_wait(full + j % S::kStages, (uint32_t)(j / S::kStages) & 1u, kCDrainNs) != 0) break;
+      unsigned char* st = sm + (j % S::kStages) * S::kStageB;
+      unsigned char* sg = st + S::kAB;
+      if (MODE != 2) {
+        const float4* f = reinterpret_cast<const float4*>(sg + S::kGB);
+        for (int i = t; i < S::FW * S::FH; i += 64) {
+          const float4 v = f[i];
+          const uint4 w = make_uint4(c_pack(v.x, v.y), c_pack(v.z, 0.f), 0u, 0u);
+          if (MODE == 1) {
+            reinterpret_cast<uint4*>(st)[i] = w;  // [row][position]
+          } else {
+            const int r = i / S::FW, x = i - r * S::FW;  // image column x0 - 1 + x
+#pragma unroll
+            for (int kx = 0; kx < 3; ++kx) {  // copy kx holds column x0 + 1 - kx first
+              const int q = x - 2 + kx;
+              if (q >= 0 && q < kGTW) *reinterpret_cast<uint4*>(sg + kx * S::kGCopy + r * kG8Row + q * 16) = w;
+            }
+            if (x >= 1 && x <= kGTW) {  // the tile's own pixels, as rounded for the MMAs
+              acc[0] += __uint_as_float(w.x << 16);
+              acc[1] += __uint_as_float(w.x & 0xffff0000u);
+              acc[2] += __uint_as_float(w.y << 16);
+            }
+          }
+        }
+        asm volatile("fence.proxy.async.shared::cta;" ::: "memory");  // visible to the tensor core
+        __syncwarp();
+        if (lane == 0) g_arrive(ready + j % S::kStages);
+      }
+      if (MODE != 3) {  // thread t: channels 8 (t & 3) .., positions t / 4 and t / 4 + 16 of the unshifted copy
+        for (int r = 0; r < kGTH; ++r) {
+#pragma unroll
+          for (int h = 0; h < 2; ++h) {
+            const int q = (t >> 2) + 16 * h;  // the swizzle moves a 16-byte chunk by the position's bits 1 and 2
+            const uint4 v = *reinterpret_cast<const uint4*>(sg + S::kGCopy + r * kG32Row + q * 64 + (((t & 3) ^ ((q >> 1) & 3)) << 4));
+            const uint32_t w[4] = {v.x, v.y, v.z, v.w};
+#pragma unroll
+            for (int k = 0; k < 4; ++k) {
+              acc[2 * k] += __uint_as_float(w[k] << 16);
+              acc[2 * k + 1] += __uint_as_float(w[k] & 0xffff0000u);
+            }
+          }
         }
       }
+      __syncwarp();
+      if (lane == 0) g_arrive(empty + j % S::kStages);
     }
-    if (MODE == 3) {  // rows o < 3 from the FP32 g
-      for (int i = tid; i < 3 * 8; i += kWThreads) {
-        const int o = i >> 3, j = i & 7;
-        const float* gf = reinterpret_cast<const float*>(sg);
-        uint32_t w[4];
 #pragma unroll
-        for (int e = 0; e < 4; ++e) w[e] = c_pack(gf[(8 * j + 2 * e) * 4 + o], gf[(8 * j + 2 * e + 1) * 4 + o]);
-        *reinterpret_cast<uint4*>(sb + j * kLboB + o * 16) = make_uint4(w[0], w[1], w[2], w[3]);
-      }
-    } else {  // 4 channel groups x 8 K groups of 8x8 blocks
-      for (int i = warp; i < 4 * 8 / 4; i += kWThreads / 32) {
-        const int mat = lane >> 3, r = lane & 7, b = 4 * i + mat;
-        const int cg = b >> 3, j = b & 7;
-        uint32_t v[4];
-        c_ldsm_x4_t(c_su32(sg + (8 * j + r) * kWRowB + cg * 16), v);
-#pragma unroll
-        for (int k = 0; k < 4; ++k) {
-          const int bk = 4 * i + k, ck = bk >> 3, jk = bk & 7;
-          *reinterpret_cast<uint32_t*>(sb + jk * kLboB + (ck * 8 + (lane >> 2)) * 16 + (lane & 3) * 4) = v[k];
-        }
-      }
-    }
-    asm volatile("fence.proxy.async.shared::cta;" ::: "memory");  // visible to the tensor core
-    asm volatile("tcgen05.fence::before_thread_sync;" ::: "memory");
-    __syncthreads();
-    asm volatile("tcgen05.fence::after_thread_sync;" ::: "memory");
-
-    // ---- D[m-tile][o] += A[rows][64 px] B[o][64 px]
-    if (tid == 0) {
-      const uint64_t ad = c_desc(c_su32(sa), kLboA, 128), bd = c_desc(c_su32(sb), kLboB, 128);
-      constexpr uint32_t id = c_idesc(128, N);
-      for (int m = 0; m < MT; ++m) {
-#pragma unroll
-        for (int kk = 0; kk < 4; ++kk)  // K = 16: two 8-pixel groups
-          c_mma(tmem + (uint32_t)(m * N), ad + (uint64_t)(m * 128 * 16 / 16) + (uint64_t)(kk * 2 * kLboA / 16),
-                bd + (uint64_t)(kk * 2 * kLboB / 16), id, (any || kk > 0) ? 1u : 0u);
-      }
-      c_commit(bar);
-    }
-    issued = true;
-    any = true;
-    // the staging buffers are free (the transposes read them before the barrier above):
-    // the next chunk moves in while this one's MMAs run, and the one after starts loading
-    if (chunk + gridDim.x < n_chunks) {
-      store();
-      if (chunk + 2 * gridDim.x < n_chunks) load(chunk + 2 * gridDim.x);
-    }
-    if (lane == 0 && c_wait(bar, phase, A.wait_ns) != 0) {
-      atomicOr(A.error, 256);
-      s_abort = 1;
-    }
-    __syncthreads();  // the whole CTA takes the same decision
-    asm volatile("tcgen05.fence::after_thread_sync;" ::: "memory");
-    if (s_abort) break;
-    issued = false;
-    phase ^= 1u;
+    for (int k = 0; k < 8; ++k) s_bias[t][k] = acc[k];
   }
-
-  // ---- this CTA's partial row: warp w reads lanes 32w.. (rows) of each M-tile, N columns (o)
-  float* out = A.partial + (size_t)blockIdx.x * SEG;
-  if (!s_abort) {
-    for (int m = 0; m < MT; ++m) {
-      const int row = m * 128 + 32 * warp + lane;
-      float v[32];
-      if (any) {
-        const uint32_t t = tmem + ((uint32_t)(32 * warp) << 16) + (uint32_t)(m * N);
-        float v0[16];
-        c_tmem_ld16(t, v0);
-#pragma unroll
-        for (int k = 0; k < 16; ++k) v[k] = v0[k];
-        if (N == 32) {
-          c_tmem_ld16(t + 16, v0);
-#pragma unroll
-          for (int k = 0; k < 16; ++k) v[16 + k] = v0[k];
-        }
-        asm volatile("tcgen05.wait::ld.sync.aligned;" ::: "memory");
-      } else {
-#pragma unroll
-        for (int k = 0; k < 32; ++k) v[k] = 0.f;
-      }
-      if (row == ONES) {
-        for (int o = 0; o < COUT; ++o) out[SEG - COUT + o] = v[o];
-      } else if (MODE == 1 && row < 27) {  // row = tap * 3 + c -> W1[o][c][tap]
-        for (int o = 0; o < COUT; ++o) out[o * 27 + (row % 3) * 9 + row / 3] = v[o];
-      } else if (MODE != 1 && row < 288) {  // row = tap * 32 + c -> W[o][c][tap]
-        for (int o = 0; o < COUT; ++o) out[(o * 32 + (row & 31)) * 9 + (row >> 5)] = v[o];
-      }
-    }
-  }
-
-  // A wait that gave up may leave MMAs running: wait for them before the tensor memory is freed.
   asm volatile("tcgen05.fence::before_thread_sync;" ::: "memory");
-  __syncthreads();
-  if (tid == 0 && issued && s_abort && c_wait(bar, phase, kCDrainNs) != 0) atomicOr(A.error, 512);
+  __syncthreads();  // the MMAs are complete (the issuing thread has waited for them)
+  asm volatile("tcgen05.fence::after_thread_sync;" ::: "memory");
+
+  // ---- this CTA's partial row, [ky][kx][o][c] then the biases: warp w reads accumulator rows 32w ..
+  float* out = A.partial + (size_t)blockIdx.x * A.seg;
+  if (!s_abort && n_own > 0) {
+    if (warp < (MODE == 1 ? 1 : 3)) {
+      const int ky = MODE == 1 ? lane >> 3 : warp, c = MODE == 1 ? lane & 7 : lane;
+      const bool keep = c < S::CIN && ky < 3;
+#pragma unroll
+      for (int h = 0; h < S::N / 16; ++h) {
+        float v[16];
+        c_tmem_ld16(tmem + ((uint32_t)(32 * warp) << 16) + 16 * h, v);
+        asm volatile("tcgen05.wait::ld.sync.aligned;" ::: "memory");
+        if (keep) {
+#pragma unroll
+          for (int k = 0; k < 16; ++k) {
+            const int col = 16 * h + k, kx = col / S::OC, o = col % S::OC;
+            if (kx < 3 && o < S::COUT) out[((ky * 3 + kx) * S::COUT + o) * S::CIN + c] = v[k];
+          }
+        }
+      }
+    }
+    if (tid < S::COUT) {  // bias gradient: the threads' sums in a fixed order
+      float b = 0.f;
+      if (MODE == 3) for (int k = 0; k < 64; ++k) b += s_bias[k][tid];
+      else for (int k = 0; k < 16; ++k) b += s_bias[4 * k + (tid >> 3)][tid & 7];
+      out[9 * S::COUT * S::CIN + tid] = b;
+    }
+  }
+  asm volatile("tcgen05.fence::before_thread_sync;" ::: "memory");
   __syncthreads();
   if (warp == 0) {
     asm volatile("tcgen05.fence::after_thread_sync;" ::: "memory");
@@ -767,14 +770,41 @@ __global__ void __launch_bounds__(kWThreads) wgrad_tc_kernel(RefineWgradArgs A) 
 
 namespace {
 
+// Tensor maps over an NHWC map: 32 BF16 channels as {32, W, H, n} under the 64-byte swizzle, or FP32 RGBA as
+// {4, W, H, n}.  (As {8, W, 4 groups, H, n}, 16 bytes at a time, the copies bounded the kernel: 75 us instead of 33 for 32 channels against 32.)
+bool encode_map32(EncodeTiled enc, CUtensorMap* m, const void* p, int n, int H, int W, int box_w, int box_h) {
+  const cuuint64_t dims[4] = {32, (cuuint64_t)W, (cuuint64_t)H, (cuuint64_t)n};
+  const cuuint64_t strides[3] = {64, (cuuint64_t)W * 64, (cuuint64_t)W * H * 64};
+  const cuuint32_t box[4] = {32, (cuuint32_t)box_w, (cuuint32_t)box_h, 1}, step[4] = {1, 1, 1, 1};
+  return enc(m, CU_TENSOR_MAP_DATA_TYPE_BFLOAT16, 4, const_cast<void*>(p), dims, strides, box, step,
+             CU_TENSOR_MAP_INTERLEAVE_NONE, CU_TENSOR_MAP_SWIZZLE_64B, CU_TENSOR_MAP_L2_PROMOTION_L2_128B,
+             CU_TENSOR_MAP_FLOAT_OOB_FILL_NONE) == CUDA_SUCCESS;
+}
+bool encode_rgba(EncodeTiled enc, CUtensorMap* m, const void* p, int n, int H, int W, int box_w, int box_h) {
+  const cuuint64_t dims[4] = {4, (cuuint64_t)W, (cuuint64_t)H, (cuuint64_t)n};
+  const cuuint64_t strides[3] = {16, (cuuint64_t)W * 16, (cuuint64_t)W * H * 16};
+  const cuuint32_t box[4] = {4, (cuuint32_t)box_w, (cuuint32_t)box_h, 1}, step[4] = {1, 1, 1, 1};
+  return enc(m, CU_TENSOR_MAP_DATA_TYPE_FLOAT32, 4, const_cast<void*>(p), dims, strides, box, step,
+             CU_TENSOR_MAP_INTERLEAVE_NONE, CU_TENSOR_MAP_SWIZZLE_NONE, CU_TENSOR_MAP_L2_PROMOTION_L2_128B,
+             CU_TENSOR_MAP_FLOAT_OOB_FILL_NONE) == CUDA_SUCCESS;
+}
+
 template <int MODE>
 cudaError_t launch_wgrad_tc_t(const RefineWgradArgs& a, cudaStream_t s) {
-  constexpr int MR = MODE == 1 ? 128 : 384, N = MODE == 3 ? 16 : 32;
-  constexpr int used = 8 * MR * 16 + 8 * N * 16 + kWHW * kWHH * kWRowB + kWPx * kWRowB + 16;
-  constexpr int smem = used < 54 * 1024 ? 54 * 1024 : used;  // at most four CTAs (their TMEM) per SM
-  cudaError_t e = ensure_dynamic_smem(reinterpret_cast<const void*>(wgrad_tc_kernel<MODE>), smem);
+  using S = WgradShape<MODE>;
+  cudaError_t e = ensure_dynamic_smem(reinterpret_cast<const void*>(wgrad_tc_kernel<MODE>), S::kSmem);
   if (e != cudaSuccess) return e;
-  wgrad_tc_kernel<MODE><<<a.n_ctas, kWThreads, smem, s>>>(a);
+  const EncodeTiled enc = encode_tiled();
+  if (!enc) return cudaErrorNotSupported;
+  CUtensorMap am, gm;
+  std::memset(&am, 0, sizeof(am));
+  std::memset(&gm, 0, sizeof(gm));
+  const bool ok = (MODE == 1 ? encode_rgba(enc, &am, a.x, a.n, a.H, a.W, S::FW, S::FH)
+                             : encode_map32(enc, &am, a.a_h, a.n, a.H, a.W, kGTW, kGTH + 2)) &&
+                  (MODE == 3 ? encode_rgba(enc, &gm, a.g_f, a.n, a.H, a.W, S::FW, S::FH)
+                             : encode_map32(enc, &gm, a.g_h, a.n, a.H, a.W, kGTW, kGTH));
+  if (!ok) return cudaErrorInvalidValue;
+  wgrad_tc_kernel<MODE><<<a.n_ctas, kGThreads, S::kSmem, s>>>(a, am, gm);
   return cudaGetLastError();
 }
 
@@ -785,6 +815,12 @@ cudaError_t launch_refine_wgrad(int mode, const RefineWgradArgs& a, cudaStream_t
   if (mode == 2) return launch_wgrad_tc_t<2>(a, s);
   if (mode == 3) return launch_wgrad_tc_t<3>(a, s);
   return cudaErrorInvalidValue;
+}
+
+int refine_wgrad_tiles(int n, int H, int W, int* tiles_x, int* tiles_y) {
+  *tiles_x = (W + kGTW - 1) / kGTW;
+  *tiles_y = (H + kGTH - 1) / kGTH;
+  return *tiles_x * *tiles_y * n;
 }
 
 }  // namespace lfk
