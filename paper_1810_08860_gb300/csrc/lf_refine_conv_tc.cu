@@ -26,18 +26,18 @@
 // the tile's MMAs and commits to an mbarrier, every warp waits (bounded by
 // wait_ns, an error word on give-up), reads its lane quadrant of each M-tile's
 // accumulators with tcgen05.ld and runs the epilogue.  Halos arrive by TMA: a
-// 32-channel BF16 halo by one tiled copy per group of 8 channels straight into
-// the MMA operand layout, the next tile's copy issued as soon as the current
+// 32-channel BF16 halo by one tiled copy straight into the MMA operand layout, the next tile's copy issued as soon as the current
 // tile's MMAs have read the buffer (it lands during the epilogue); a 3-channel
 // FP32 RGBA halo into a staging buffer that the four warps convert to BF16
 // pairs, the next tile's copy issued as soon as they have read it (it lands
 // during the MMAs and the epilogue).  Four CTAs share an SM, so one CTA's MMAs
 // overlap another's staging and epilogue.
 //
-// Shared-memory operands use the K-major layout without swizzling: a position
-// (row) holds 8 channels in 16 contiguous bytes, rows follow every 16 bytes
-// (8-row core matrices 128 bytes apart), and each further group of 8 channels
-// starts kCGroupB bytes later.  The weights arrive in the packed layouts of
+// A 32-channel halo lies K-major under the 64-byte swizzle, a position's 32 channels
+// in 64 bytes; pair-packed rows and the weights use the layout without swizzling:
+// a row holds 8 channels in 16 contiguous bytes, rows follow every 16 bytes (8-row
+// core matrices 128 bytes apart).  (As four groups of 8 channels, 16 bytes at a time,
+// the halo copies alone took half as long as the MMAs.)  The weights arrive in the packed layouts of
 // pack_weights_kernel (rows of 32 K values per output) and are rearranged into
 // core-matrix blocks when a CTA loads them.
 #include <cuda_bf16.h>
@@ -58,9 +58,9 @@ constexpr int kCHW = 32, kCHH = kCTH + 2;         // halo: 32 positions x 18 row
 constexpr int kCMT = kCTH / 4;                    // M-tiles of 128 positions per tile
 constexpr int kCPos = kCHH * kCHW;                // 576 positions
 constexpr int kCGuard = 2;                        // positions before and after (reads reach one beyond)
-constexpr int kCGroupB = ((kCPos + 2 * kCGuard) * 16 + 127) / 128 * 128;  // bytes per group of 8 channels
-constexpr int kCXOff = 128 - kCGuard * 16;        // halo position 0 of each group starts 128-byte aligned
-constexpr int kCHaloTx = 4 * kCPos * 16;          // bytes of a tile's four TMA copies (32-channel halo)
+constexpr int kCPairB = (kCPos + 2 * kCGuard) * 16;  // 3-channel input: the pair-packed halo
+constexpr int kCXOff = 128 - kCGuard * 16;        // its position 0 starts 128-byte aligned
+constexpr int kCHaloTx = kCPos * 64;              // 32-channel input: a tile's halo, one TMA copy
 constexpr int kCXsB = kCPos * 16;                 // a tile's FP32 RGBA halo (3-channel input), one TMA copy
 constexpr int kCThreads = 128;
 constexpr int kCPerSM = 4;                        // CTAs per SM: 4 x 128 TMEM columns
@@ -123,20 +123,16 @@ __device__ __forceinline__ void c_tmem_ld16(uint32_t addr, float (&v)[16]) {
   for (int i = 0; i < 16; ++i) v[i] = __uint_as_float(r[i]);
 }
 
-// Tile `tile`'s 32-channel BF16 halo by TMA: one tiled copy per group g of 8
-// channels (a box of 8 channels x 32 positions x 18 rows of the 5-D tensor map
-// {8, 4, W, H, n} over the map; zeros where the box leaves the image) into the
-// group's operand rows, completing on `bar` with the copies' byte count.
+// Tile `tile`'s 32-channel BF16 halo by TMA: one tiled copy (32 channels x 32
+// positions x 18 rows of the 4-D tensor map {32, W, H, n}; zeros where the box
+// leaves the image) under the 64-byte swizzle, completing on `bar`.
 __device__ __forceinline__ void c_load_halo(const CUtensorMap* tmap, uint32_t sx0, uint64_t* bar, int img, int x0,
                                             int y0) {
   asm volatile("mbarrier.arrive.expect_tx.shared::cta.b64 _, [%0], %1;" ::"r"(c_su32(bar)), "r"(kCHaloTx) : "memory");
-#pragma unroll
-  for (int g = 0; g < 4; ++g)
-    asm volatile(
-        "cp.async.bulk.tensor.5d.shared::cluster.global.mbarrier::complete_tx::bytes [%0], [%1, {%2, %3, %4, %5, %6}], "
-        "[%7];" ::"r"(sx0 + g * kCGroupB),
-        "l"(reinterpret_cast<uint64_t>(tmap)), "r"(0), "r"(g), "r"(x0 - 1), "r"(y0 - 1), "r"(img), "r"(c_su32(bar))
-        : "memory");
+  asm volatile(
+      "cp.async.bulk.tensor.4d.shared::cluster.global.mbarrier::complete_tx::bytes [%0], [%1, {%2, %3, %4, %5}], [%6];" ::
+          "r"(sx0), "l"(reinterpret_cast<uint64_t>(tmap)), "r"(0), "r"(x0 - 1), "r"(y0 - 1), "r"(img), "r"(c_su32(bar))
+      : "memory");
 }
 
 // Tile `tile`'s FP32 RGBA halo by TMA: one tiled copy (4 channels x 32
@@ -160,22 +156,72 @@ __device__ __forceinline__ uint32_t c_pack(float lo, float hi) {
   return *reinterpret_cast<uint32_t*>(&v);
 }
 
+// 32-channel inputs: one MMA per kernel row and 16 channels, the three kernel columns
+// stacked along N (32 outputs: N = 96, one M-tile of accumulators at a time; 3
+// outputs: N = 16, four columns each).  An MMA of N = 32 or less costs about 45
+// cycles, of N = 96 about 62, so six take 372 cycles an M-tile where eighteen took
+// 810; the epilogue adds two shuffles per output.  16 x 256^2 pixels: 32 -> 32 with
+// the ReLU mask 53 -> 47 us, 32 -> 3 with the loss 44 -> 29 us; a 517 x 731 image's
+// last layer 14.7 -> 9.3 us.  Bound by memory from here (20 to 30 us of it).
+template <int IN, int COUT>
+struct ConvShape {
+  static constexpr bool kStacked = IN == kConvInBF16;
+  static constexpr int kOutStep = COUT == 8 ? 4 : 32;                    // rows of a kernel column along N
+  static constexpr int N = kStacked ? (COUT == 8 ? 16 : 96) : 32;
+  static constexpr int NB = kStacked ? 6 : 3;                            // B blocks: (kernel row, half), or kernel row
+  static constexpr int kMB = N == 96 ? 1 : kCMT;                         // M-tiles per batch of MMAs (128 TMEM columns)
+  static constexpr int kBlkB = 2 * N * 16, kWBytes = NB * kBlkB;
+};
+
+// Four lanes (4 i .. 4 i + 3) hold a pixel each, as four 16-byte pieces; afterwards
+// lane 4 i + r holds piece r of the four pixels, so that a warp's store writes whole
+// pixels (64 contiguous bytes).  Stored a pixel per lane, 16 bytes at a 64-byte
+// stride, every 32-byte sector was written in two halves: on 16 x 256^2 pixels the
+// 3 -> 32 layer took 29 us instead of 22, the 32 -> 32 one 52 instead of 45.
+__device__ __forceinline__ void c_transpose4(uint4 (&c)[4]) {
+  const int lane = threadIdx.x & 31;
+#pragma unroll
+  for (int b = 1; b <= 2; b <<= 1) {
+    const bool up = (lane & b) != 0;
+#pragma unroll
+    for (int i = 0; i < 2; ++i) {
+      const int k = b == 1 ? 2 * i : i, k2 = k + b;
+      const uint4 give = up ? c[k] : c[k2];
+      uint4 got;
+      got.x = __shfl_xor_sync(0xffffffffu, give.x, b);
+      got.y = __shfl_xor_sync(0xffffffffu, give.y, b);
+      got.z = __shfl_xor_sync(0xffffffffu, give.z, b);
+      got.w = __shfl_xor_sync(0xffffffffu, give.w, b);
+      if (up) c[k] = got;
+      else c[k2] = got;
+    }
+  }
+}
+
+// A word of two BF16 values where the same half of `gate` is > 0, else 0.
+__device__ __forceinline__ uint32_t c_gate(uint32_t v, uint32_t gate) {
+  const uint32_t lo = (int32_t)(gate << 16) > 0 ? 0x0000ffffu : 0u, hi = (int32_t)(gate & 0xffff0000u) > 0 ? 0xffff0000u : 0u;
+  return v & (lo | hi);
+}
+
 }  // namespace
 
 template <int IN, int COUT, int EPI>
 __global__ void __launch_bounds__(kCThreads, kCPerSM)
     conv_tc_kernel(RefineConvArgs A, const __grid_constant__ CUtensorMap tmap) {
-  constexpr int N = COUT < 16 ? 16 : COUT;                 // MMA N (the 3-output layer pads to 16)
-  constexpr int NB = IN == kConvInBF16 ? 18 : 3;           // B blocks: (tap, half) or kernel row
-  constexpr int kBlkB = 2 * N * 16;
-  constexpr int kWBytes = NB * kBlkB;
-  constexpr int G = IN == kConvInBF16 ? 4 : 1;             // channel groups in the halo
-  extern __shared__ __align__(128) unsigned char sm[];
+  using S = ConvShape<IN, COUT>;
+  constexpr int N = S::N, NB = S::NB, kBlkB = S::kBlkB, kWBytes = S::kWBytes;
+  constexpr bool kStacked = S::kStacked;
+  extern __shared__ __align__(128) unsigned char sm_raw[];
+  unsigned char* sm = sm_raw + ((1024u - (c_su32(sm_raw) & 1023u)) & 1023u);  // the 32-channel halo starts on a swizzle atom
   unsigned char* sw = sm;
-  unsigned char* sx = sm + kWBytes + kCXOff;  // group g, position p: sx + g * kCGroupB + (p + kCGuard) * 16
-  constexpr int kXsOff = (kWBytes + kCXOff + G * kCGroupB + 127) / 128 * 128;
+  static_assert(IN != kConvInBF16 || kWBytes % 512 == 0, "a swizzle atom is 512 bytes");
+  // 32 channels: position p in the 64 bytes at sx + 64 p (swizzled); windows reach one position before, into the
+  // weights, and one after (output columns that are never used).  3 channels: pairs, 16 bytes at sx + (p + kCGuard) * 16.
+  unsigned char* sx = sm + kWBytes + (IN == kConvInBF16 ? 0 : kCXOff);
+  constexpr int kXsOff = (kWBytes + kCXOff + kCPairB + 127) / 128 * 128;
   unsigned char* xs = sm + kXsOff;             // 3-channel input: the FP32 RGBA halo as it landed
-  constexpr int kBarOff = IN == kConvInBF16 ? kWBytes + kCXOff + G * kCGroupB : kXsOff + kCXsB;
+  constexpr int kBarOff = IN == kConvInBF16 ? kWBytes + kCHaloTx + 128 : kXsOff + kCXsB;
   uint64_t* bar = reinterpret_cast<uint64_t*>(sm + kBarOff);     // the tile's MMAs completed
   uint64_t* xbar = bar + 1;                                         // the tile's TMA halo landed
   uint32_t* tslot = reinterpret_cast<uint32_t*>(bar + 2);
@@ -188,30 +234,32 @@ __global__ void __launch_bounds__(kCThreads, kCPerSM)
   for (int i = tid; i < NB * 2 * N; i += kCThreads) {
     const int b = i / (2 * N), g = (i / N) & 1, n = i % N;
     uint4 v = make_uint4(0u, 0u, 0u, 0u);
-    if (n < COUT) {
-      if (IN == kConvInBF16) {  // packed [tap][n][32]: block b = 2 tap + half
-        v = *reinterpret_cast<const uint4*>(A.wt + ((size_t)(b >> 1) * COUT + n) * 32 + 16 * (b & 1) + 8 * g);
-      } else {  // packed [n][32], k = tap * 3 + c; block b = ky, element e: kx = 2g + e / 4, c = e % 4
-        uint32_t w[4];
+    if (IN == kConvInBF16) {  // packed [tap][o][32]: block b = 2 ky + half, row n = kx * S::kOutStep + o
+      const int kx = n / S::kOutStep, o = n % S::kOutStep;
+      if (kx < 3) v = *reinterpret_cast<const uint4*>(A.wt + ((size_t)(3 * (b >> 1) + kx) * COUT + o) * 32 + 16 * (b & 1) + 8 * g);
+    } else {  // packed [n][32], k = tap * 3 + c; block b = ky, element e: kx = 2g + e / 4, c = e % 4
+      uint32_t w[4];
 #pragma unroll
-        for (int j = 0; j < 4; ++j) {
-          uint32_t half2 = 0;
+      for (int j = 0; j < 4; ++j) {
+        uint32_t half2 = 0;
 #pragma unroll
-          for (int h = 0; h < 2; ++h) {
-            const int e = 2 * j + h, kx = 2 * g + (e >> 2), c = e & 3;
-            uint32_t bits = 0;
-            if (kx < 3 && c < 3) bits = *reinterpret_cast<const uint16_t*>(A.wt + n * 32 + (b * 3 + kx) * 3 + c);
-            half2 |= bits << (16 * h);
-          }
-          w[j] = half2;
+        for (int h = 0; h < 2; ++h) {
+          const int e = 2 * j + h, kx = 2 * g + (e >> 2), c = e & 3;
+          uint32_t bits = 0;
+          if (kx < 3 && c < 3) bits = *reinterpret_cast<const uint16_t*>(A.wt + n * 32 + (b * 3 + kx) * 3 + c);
+          half2 |= bits << (16 * h);
         }
-        v = make_uint4(w[0], w[1], w[2], w[3]);
+        w[j] = half2;
       }
+      v = make_uint4(w[0], w[1], w[2], w[3]);
     }
     *reinterpret_cast<uint4*>(sw + b * kBlkB + (g * N + n) * 16) = v;
   }
-  for (int i = tid; i < G * kCGroupB / 16; i += kCThreads)  // the guard rows stay zero
-    reinterpret_cast<uint4*>(sx)[i] = make_uint4(0u, 0u, 0u, 0u);
+  if (IN == kConvInRGBA)
+    for (int i = tid; i < kCPairB / 16; i += kCThreads)  // the guard rows stay zero
+      reinterpret_cast<uint4*>(sx)[i] = make_uint4(0u, 0u, 0u, 0u);
+  else if (tid < 8)
+    reinterpret_cast<uint4*>(sx + kCHaloTx)[tid] = make_uint4(0u, 0u, 0u, 0u);
   asm volatile("fence.proxy.async.shared::cta;" ::: "memory");  // the zeros, to the tensor core and TMA
   if (tid < 32) s_bias[tid] = (EPI == kEpiRelu || (EPI != kEpiMask && tid < 3)) ? A.bias[tid] : 0.f;
   if (tid == 0) {
@@ -244,7 +292,7 @@ __global__ void __launch_bounds__(kCThreads, kCPerSM)
     y0 = (rem / tiles_x) * kCTH;
     x0 = (rem % tiles_x) * kCTW;
   };
-  const uint32_t sx0 = c_su32(sx) + kCGuard * 16;  // halo position 0 of group 0 (128-byte aligned)
+  const uint32_t sx0 = c_su32(sx);  // 32 channels: halo position 0
   uint32_t phase = 0, xphase = 0;
   bool issued = false;        // an MMA commit of this CTA may still be outstanding
   bool halo_pending = false;  // thread 0: a TMA halo copy may still be landing
@@ -301,114 +349,162 @@ __global__ void __launch_bounds__(kCThreads, kCPerSM)
       halo_pending = true;
     }
 
-    // ---- the tile's MMAs: M-tile m holds output positions 32 (4m + 1) + r, r < 128
-    if (tid == 0) {
-      const uint32_t sxa = c_su32(sx) + kCGuard * 16;  // position 0
-      const uint64_t ad = c_desc(sxa, IN == kConvInBF16 ? kCGroupB : 32, 128);
+    // ---- the tile's MMAs, a batch of kMB M-tiles at a time: M-tile m holds output positions 32 (4m + 1) + r, r < 128
+    // (one thread issues them)
+    auto issue = [&](int m0) {
+      // A, 32 channels: positions (rows) of 64 bytes under the 64-byte swizzle, 8 of them 512 bytes on; the swizzle
+      // goes by address, so a window's shift by whole positions and the second 16 channels only move the start.
+      const uint64_t ad = IN == kConvInBF16 ? c_desc(sx0, 16, 512) | (4ull << 61)
+                                            : c_desc(c_su32(sx) + kCGuard * 16, 32, 128);
       const uint64_t bd = c_desc(c_su32(sw), N * 16, 128);
       constexpr uint32_t id = c_idesc(128, N);
-      for (int m = 0; m < kCMT; ++m) {
-        const uint32_t d = tmem + (uint32_t)(m * N);
-        if (IN == kConvInBF16) {
+#pragma unroll 1
+      for (int m = m0; m < m0 + S::kMB; ++m) {
+        const uint32_t d = tmem + (uint32_t)((m - m0) * N);
 #pragma unroll
-          for (int t = 0; t < 9; ++t) {  // tap t = 3 ky + kx starts at 32 (4m + ky) + kx - 1
+        for (int ky = 0; ky < 3; ++ky) {
+          if (IN == kConvInBF16) {  // kernel row ky reads positions 32 (4m + ky) + r, its columns lie along N
 #pragma unroll
             for (int h = 0; h < 2; ++h)
-              c_mma(d, ad + (uint64_t)(int64_t)(32 * (4 * m + t / 3) + t % 3 - 1) + (uint64_t)(h * (2 * kCGroupB / 16)),
-                    bd + (uint64_t)((2 * t + h) * (kBlkB / 16)), id, t > 0 || h > 0);
-          }
-        } else {
-#pragma unroll
-          for (int ky = 0; ky < 3; ++ky)  // kernel row ky: pairs from 32 (4m + ky) - 1
+              c_mma(d, ad + (uint64_t)(4 * 32 * (4 * m + ky) + 2 * h), bd + (uint64_t)((2 * ky + h) * (kBlkB / 16)), id,
+                    ky > 0 || h > 0);
+          } else {  // pairs from 32 (4m + ky) - 1
             c_mma(d, ad + (uint64_t)(int64_t)(32 * (4 * m + ky) - 1), bd + (uint64_t)(ky * (kBlkB / 16)), id, ky > 0);
+          }
         }
       }
       c_commit(bar);
-    }
+    };
+    // every warp waits for the batch; false when a wait of the CTA gave up (the same for the whole CTA)
+    auto landed = [&]() -> bool {
+      if (lane == 0 && c_wait(bar, phase, A.wait_ns) != 0) {
+        atomicOr(A.error, 64);
+        s_abort = 1;
+      }
+      __syncthreads();
+      asm volatile("tcgen05.fence::after_thread_sync;" ::: "memory");
+      if (s_abort) return false;
+      issued = false;
+      phase ^= 1u;
+      return true;
+    };
+    // the accumulators of M-tile m are in registers in every warp: the next batch may overwrite them
+    auto next_batch = [&](int m) {
+      if (S::kMB == kCMT || m + 1 == kCMT) return;
+      asm volatile("tcgen05.fence::before_thread_sync;" ::: "memory");
+      __syncthreads();
+      asm volatile("tcgen05.fence::after_thread_sync;" ::: "memory");
+      if (tid == 0) issue(m + 1);
+      issued = true;
+    };
+    if (tid == 0) issue(0);
     issued = true;
-    if (lane == 0 && c_wait(bar, phase, A.wait_ns) != 0) {
-      atomicOr(A.error, 64);
-      s_abort = 1;
-    }
-    __syncthreads();  // every warp has waited: the abort decision is the same for the whole CTA
-    asm volatile("tcgen05.fence::after_thread_sync;" ::: "memory");
-    if (s_abort) break;
-    issued = false;
-    phase ^= 1u;
-    // the MMAs have read the halo: the next tile's copy lands during this epilogue
-    if (IN == kConvInBF16 && tid == 0 && tile + (int)gridDim.x < n_tiles) {
-      int nimg, nx0, ny0;
-      origin(tile + gridDim.x, nimg, nx0, ny0);
-      c_load_halo(&tmap, sx0, xbar, nimg, nx0, ny0);
-      halo_pending = true;
-    }
 
-    // ---- epilogue: warp w reads lanes 32w.. (halo row 4m + 1 + w, column lane) of each M-tile
+    // ---- epilogue: warp w reads lanes 32w.. (halo row 4m + 1 + w, column lane) of each M-tile.  With the kernel
+    // columns along N an output is D[q-1][kx = 0] + D[q][1] + D[q+1][2]; the neighbours' parts come from the
+    // neighbouring lanes (columns 0 and 31 get a wrong one and are never used).
     const uint32_t lane_base = (uint32_t)(32 * warp) << 16;
     const int gx = x0 + lane - 1;
     float lsum = 0.f;
+    bool ok = true;
+#pragma unroll 1
     for (int m = 0; m < kCMT; ++m) {
+      if (m % S::kMB == 0 && !landed()) {
+        ok = false;
+        break;
+      }
+      // the MMAs have read the halo: the next tile's copy lands during this epilogue
+      if (IN == kConvInBF16 && tid == 0 && m == kCMT - S::kMB && tile + (int)gridDim.x < n_tiles) {
+        int nimg, nx0, ny0;
+        origin(tile + gridDim.x, nimg, nx0, ny0);
+        c_load_halo(&tmap, sx0, xbar, nimg, nx0, ny0);
+        halo_pending = true;
+      }
       const int gy = y0 + 4 * m + warp;
       const bool store = lane >= 1 && lane <= kCTW && gy < H && gx < W;
-      const size_t pix = ((size_t)img * H + (store ? gy : 0)) * W + (store ? gx : 0);
-      const uint32_t t = tmem + lane_base + (uint32_t)(m * N);
+      const uint32_t t = tmem + lane_base + (uint32_t)((m % S::kMB) * N);
       if (EPI == kEpiRelu || EPI == kEpiMask) {
-        float v0[16], v1[16];
-        c_tmem_ld16(t, v0);
-        c_tmem_ld16(t + 16, v1);
-        asm volatile("tcgen05.wait::ld.sync.aligned;" ::: "memory");
-        if (!store) continue;
-        float v[32];
+        // after the transpose this lane holds piece lane % 4 of the pixels in columns (lane & ~3) + j
+        const int col0 = lane & ~3;
+        const size_t at0 = (((size_t)img * H + gy) * W + x0 + col0 - 1) * 32 + 8 * (lane & 3);
+        bool keep[4];
+        uint4 gate[4];
 #pragma unroll
-        for (int k = 0; k < 16; ++k) {
-          v[k] = v0[k];
-          v[16 + k] = v1[k];
+        for (int j = 0; j < 4; ++j) {
+          keep[j] = col0 + j >= 1 && col0 + j <= kCTW && gy < H && x0 + col0 + j - 1 < W;
+          gate[j] = make_uint4(0u, 0u, 0u, 0u);
+          if (EPI == kEpiMask && keep[j]) gate[j] = *reinterpret_cast<const uint4*>(A.mask + at0 + 32 * j);
         }
-        uint32_t w[16];
-        if (EPI == kEpiRelu) {
+        uint4 w[4];
 #pragma unroll
-          for (int j = 0; j < 16; ++j)
-            w[j] = c_pack(fmaxf(v[2 * j] + s_bias[2 * j], 0.f), fmaxf(v[2 * j + 1] + s_bias[2 * j + 1], 0.f));
-        } else {
-          const uint4* mk = reinterpret_cast<const uint4*>(A.mask + pix * 32);
+        for (int h = 0; h < 2; ++h) {  // output channels 16 h .. 16 h + 15
+          float v[16];
+          if (kStacked) {
+            float d0[16], d2[16];
+            c_tmem_ld16(t + 16 * h, d0);
+            c_tmem_ld16(t + 32 + 16 * h, v);
+            c_tmem_ld16(t + 64 + 16 * h, d2);
+            asm volatile("tcgen05.wait::ld.sync.aligned;" ::: "memory");
+            if (h == 1) next_batch(m);
 #pragma unroll
-          for (int q = 0; q < 4; ++q) {
-            const uint4 mq = mk[q];
-            const uint32_t mw[4] = {mq.x, mq.y, mq.z, mq.w};
-#pragma unroll
-            for (int j = 0; j < 4; ++j) {
-              const __nv_bfloat162 mm = *reinterpret_cast<const __nv_bfloat162*>(&mw[j]);
-              const int k = 8 * q + 2 * j;
-              w[4 * q + j] = c_pack(__bfloat162float(mm.x) > 0.f ? v[k] : 0.f, __bfloat162float(mm.y) > 0.f ? v[k + 1] : 0.f);
-            }
+            for (int k = 0; k < 16; ++k)
+              v[k] += __shfl_up_sync(0xffffffffu, d0[k], 1) + __shfl_down_sync(0xffffffffu, d2[k], 1);
+          } else {
+            c_tmem_ld16(t + 16 * h, v);
+            asm volatile("tcgen05.wait::ld.sync.aligned;" ::: "memory");
           }
-        }
-        uint4* dst = reinterpret_cast<uint4*>(A.out_h + pix * 32);
+          uint32_t p[8];
 #pragma unroll
-        for (int q = 0; q < 4; ++q) dst[q] = make_uint4(w[4 * q], w[4 * q + 1], w[4 * q + 2], w[4 * q + 3]);
-      } else {  // kEpiResid / kEpiLoss: outputs 0..2
-        float v[16];
+          for (int j = 0; j < 8; ++j) {
+            float lo = v[2 * j], hi = v[2 * j + 1];
+            if (EPI == kEpiRelu) {
+              lo = fmaxf(lo + s_bias[16 * h + 2 * j], 0.f);
+              hi = fmaxf(hi + s_bias[16 * h + 2 * j + 1], 0.f);
+            }
+            p[j] = c_pack(lo, hi);
+          }
+          w[2 * h] = make_uint4(p[0], p[1], p[2], p[3]);
+          w[2 * h + 1] = make_uint4(p[4], p[5], p[6], p[7]);
+        }
+        c_transpose4(w);
+#pragma unroll
+        for (int j = 0; j < 4; ++j) {
+          if (!keep[j]) continue;
+          if (EPI == kEpiMask)
+            w[j] = make_uint4(c_gate(w[j].x, gate[j].x), c_gate(w[j].y, gate[j].y), c_gate(w[j].z, gate[j].z),
+                              c_gate(w[j].w, gate[j].w));
+          *reinterpret_cast<uint4*>(A.out_h + at0 + 32 * j) = w[j];
+        }
+      } else {  // kEpiResid / kEpiLoss: outputs 0..2, column kx in 4 kx ..
+        const size_t pix = ((size_t)img * H + (store ? gy : 0)) * W + (store ? gx : 0);
+        float4 x = make_float4(0.f, 0.f, 0.f, 0.f), tg = x;
+        if (store) {
+          x = reinterpret_cast<const float4*>(A.x)[pix];
+          if (EPI == kEpiLoss) tg = reinterpret_cast<const float4*>(A.target)[pix];
+        }
+        float v[16], r[3];
         c_tmem_ld16(t, v);
         asm volatile("tcgen05.wait::ld.sync.aligned;" ::: "memory");
+#pragma unroll
+        for (int o = 0; o < 3; ++o)
+          r[o] = __shfl_up_sync(0xffffffffu, v[o], 1) + v[4 + o] + __shfl_down_sync(0xffffffffu, v[8 + o], 1) + s_bias[o];
         if (!store) continue;
-        const float4 x = reinterpret_cast<const float4*>(A.x)[pix];
-        const float r0 = v[0] + s_bias[0], r1 = v[1] + s_bias[1], r2 = v[2] + s_bias[2];
         if (EPI == kEpiResid) {
           const bool valid = x.w > 0.f;
           reinterpret_cast<float4*>(A.out_f)[pix] =
-              valid ? make_float4(x.x + r0, x.y + r1, x.z + r2, 1.f) : make_float4(0.f, 0.f, 0.f, 0.f);
+              valid ? make_float4(x.x + r[0], x.y + r[1], x.z + r[2], 1.f) : make_float4(0.f, 0.f, 0.f, 0.f);
         } else {
-          const float4 tg = reinterpret_cast<const float4*>(A.target)[pix];
           const bool valid = x.w > 0.f && tg.w > 0.f;
-          const float d0 = valid ? (x.x + r0) - tg.x : 0.f;
-          const float d1 = valid ? (x.y + r1) - tg.y : 0.f;
-          const float d2 = valid ? (x.z + r2) - tg.z : 0.f;
+          const float d0 = valid ? (x.x + r[0]) - tg.x : 0.f;
+          const float d1 = valid ? (x.y + r[1]) - tg.y : 0.f;
+          const float d2 = valid ? (x.z + r[2]) - tg.z : 0.f;
           lsum += d0 * d0 + d1 * d1 + d2 * d2;
           reinterpret_cast<float4*>(A.out_f)[pix] =
               make_float4(2.f * loss_scale * d0, 2.f * loss_scale * d1, 2.f * loss_scale * d2, 0.f);
         }
       }
     }
+    if (!ok) break;
     if (EPI == kEpiLoss) {
 #pragma unroll
       for (int o = 16; o > 0; o >>= 1) lsum += __shfl_xor_sync(0xffffffffu, lsum, o);
@@ -435,12 +531,30 @@ __global__ void __launch_bounds__(kCThreads, kCPerSM)
 
 namespace {
 
+// Tensor maps over an NHWC map: 32 BF16 channels as {32, W, H, n} under the 64-byte swizzle, or FP32 RGBA as
+// {4, W, H, n}.
+bool encode_map32(EncodeTiled enc, CUtensorMap* m, const void* p, int n, int H, int W, int box_w, int box_h) {
+  const cuuint64_t dims[4] = {32, (cuuint64_t)W, (cuuint64_t)H, (cuuint64_t)n};
+  const cuuint64_t strides[3] = {64, (cuuint64_t)W * 64, (cuuint64_t)W * H * 64};
+  const cuuint32_t box[4] = {32, (cuuint32_t)box_w, (cuuint32_t)box_h, 1}, step[4] = {1, 1, 1, 1};
+  return enc(m, CU_TENSOR_MAP_DATA_TYPE_BFLOAT16, 4, const_cast<void*>(p), dims, strides, box, step,
+             CU_TENSOR_MAP_INTERLEAVE_NONE, CU_TENSOR_MAP_SWIZZLE_64B, CU_TENSOR_MAP_L2_PROMOTION_L2_128B,
+             CU_TENSOR_MAP_FLOAT_OOB_FILL_NONE) == CUDA_SUCCESS;
+}
+bool encode_rgba(EncodeTiled enc, CUtensorMap* m, const void* p, int n, int H, int W, int box_w, int box_h) {
+  const cuuint64_t dims[4] = {4, (cuuint64_t)W, (cuuint64_t)H, (cuuint64_t)n};
+  const cuuint64_t strides[3] = {16, (cuuint64_t)W * 16, (cuuint64_t)W * H * 16};
+  const cuuint32_t box[4] = {4, (cuuint32_t)box_w, (cuuint32_t)box_h, 1}, step[4] = {1, 1, 1, 1};
+  return enc(m, CU_TENSOR_MAP_DATA_TYPE_FLOAT32, 4, const_cast<void*>(p), dims, strides, box, step,
+             CU_TENSOR_MAP_INTERLEAVE_NONE, CU_TENSOR_MAP_SWIZZLE_NONE, CU_TENSOR_MAP_L2_PROMOTION_L2_128B,
+             CU_TENSOR_MAP_FLOAT_OOB_FILL_NONE) == CUDA_SUCCESS;
+}
+
 template <int IN, int COUT, int EPI>
 cudaError_t launch_conv_tc_t(const RefineConvArgs& a, cudaStream_t s) {
-  constexpr int N = COUT < 16 ? 16 : COUT;
-  constexpr int kW = (IN == kConvInBF16 ? 18 : 3) * 2 * N * 16;
-  constexpr int used = IN == kConvInBF16 ? kW + kCXOff + 4 * kCGroupB + 24
-                                         : (kW + kCXOff + kCGroupB + 127) / 128 * 128 + kCXsB + 24;
+  constexpr int kW = ConvShape<IN, COUT>::kWBytes;
+  constexpr int used = 1024 + (IN == kConvInBF16 ? kW + kCHaloTx + 128 + 24
+                                                 : (kW + kCXOff + kCPairB + 127) / 128 * 128 + kCXsB + 24);
   // At least 54 KB: no more than kCPerSM CTAs share an SM, so their tensor memory (128 columns each)
   // always fits and no CTA waits in tcgen05.alloc for another persistent CTA to finish.
   constexpr int smem = used < 54 * 1024 ? 54 * 1024 : used;
@@ -451,35 +565,16 @@ cudaError_t launch_conv_tc_t(const RefineConvArgs& a, cudaStream_t s) {
   int dev = 0, sms = 0;
   if ((e = cudaGetDevice(&dev)) != cudaSuccess) return e;
   if ((e = cudaDeviceGetAttribute(&sms, cudaDevAttrMultiProcessorCount, dev)) != cudaSuccess) return e;
-  // The halo copies' tensor map, over a 16-byte aligned base.  32-channel input: a 5-D tensor
-  // {8 channels, 4 groups, W, H, n} of BF16, with group, position, row and image strides of 16,
-  // 64, W * 64 and W * H * 64 bytes.  3-channel input: a 4-D tensor {4 channels, W, H, n} of FP32
-  // RGBA, strides 16, W * 16 and W * H * 16 bytes.
+  // the halo copies' tensor map, over a 16-byte aligned base
   CUtensorMap tmap;
   std::memset(&tmap, 0, sizeof(tmap));
   const EncodeTiled enc = encode_tiled();
   if (!enc) return cudaErrorNotSupported;
-  if (IN == kConvInBF16) {
-    if ((reinterpret_cast<uintptr_t>(a.src_h) & 15u) != 0) return cudaErrorInvalidValue;
-    const cuuint64_t dims[5] = {8, 4, (cuuint64_t)a.W, (cuuint64_t)a.H, (cuuint64_t)a.n};
-    const cuuint64_t strides[4] = {16, 64, (cuuint64_t)a.W * 64, (cuuint64_t)a.W * a.H * 64};
-    const cuuint32_t box[5] = {8, 1, (cuuint32_t)kCHW, (cuuint32_t)kCHH, 1};
-    const cuuint32_t step[5] = {1, 1, 1, 1, 1};
-    if (enc(&tmap, CU_TENSOR_MAP_DATA_TYPE_BFLOAT16, 5, const_cast<__nv_bfloat16*>(a.src_h), dims, strides, box,
-            step, CU_TENSOR_MAP_INTERLEAVE_NONE, CU_TENSOR_MAP_SWIZZLE_NONE, CU_TENSOR_MAP_L2_PROMOTION_L2_128B,
-            CU_TENSOR_MAP_FLOAT_OOB_FILL_NONE) != CUDA_SUCCESS)
-      return cudaErrorInvalidValue;
-  } else {
-    if ((reinterpret_cast<uintptr_t>(a.src_f) & 15u) != 0) return cudaErrorInvalidValue;
-    const cuuint64_t dims[4] = {4, (cuuint64_t)a.W, (cuuint64_t)a.H, (cuuint64_t)a.n};
-    const cuuint64_t strides[3] = {16, (cuuint64_t)a.W * 16, (cuuint64_t)a.W * a.H * 16};
-    const cuuint32_t box[4] = {4, (cuuint32_t)kCHW, (cuuint32_t)kCHH, 1};
-    const cuuint32_t step[4] = {1, 1, 1, 1};
-    if (enc(&tmap, CU_TENSOR_MAP_DATA_TYPE_FLOAT32, 4, const_cast<float*>(a.src_f), dims, strides, box, step,
-            CU_TENSOR_MAP_INTERLEAVE_NONE, CU_TENSOR_MAP_SWIZZLE_NONE, CU_TENSOR_MAP_L2_PROMOTION_L2_128B,
-            CU_TENSOR_MAP_FLOAT_OOB_FILL_NONE) != CUDA_SUCCESS)
-      return cudaErrorInvalidValue;
-  }
+  const void* src = IN == kConvInBF16 ? static_cast<const void*>(a.src_h) : a.src_f;
+  if ((reinterpret_cast<uintptr_t>(src) & 15u) != 0) return cudaErrorInvalidValue;
+  if (!(IN == kConvInBF16 ? encode_map32(enc, &tmap, src, a.n, a.H, a.W, kCHW, kCHH)
+                          : encode_rgba(enc, &tmap, src, a.n, a.H, a.W, kCHW, kCHH)))
+    return cudaErrorInvalidValue;
   const int grid = n_tiles < sms * kCPerSM ? n_tiles : sms * kCPerSM;
   conv_tc_kernel<IN, COUT, EPI><<<grid, kCThreads, smem, s>>>(a, tmap);
   return cudaGetLastError();
@@ -506,49 +601,49 @@ cudaError_t launch_refine_conv(int in_mode, int cout, int epi, const RefineConvA
 // positions of a; per image row r of g
 //   D[(i, c)][(kx, o)] += sum_x a[r - 1 + i][x][c] g[r][x + 1 - kx][o]
 // with M = 128: four consecutive rows i of a (ky = i; the fourth is not used) of
-// 32 channels, and N = 96: three copies of g, each loaded by TMA with its own shift
-// (zeros outside the image).  A 32-channel map lies as [row][position][32 channels]
-// under the 64-byte swizzle, so M steps from row to row of a and N from copy to copy
-// of g.  The 3-channel maps (the network input, dL/dr) land as FP32 RGBA and two
-// warps round them to BF16 rows of 8 channels, the last five zero, without swizzle:
-// M then covers sixteen rows (three used), N = 32 four copies (three used).  The
-// same two warps sum g for the bias gradient.
+// 32 channels, and N = 96: g's row (34 positions, zeros outside the image) at three
+// starts one position apart, which the operand's N stride of one position gives
+// without a copy.  A 32-channel map lies as [row][position][32 channels] under the
+// 64-byte swizzle, which goes by address, so shifted starts read it correctly.  The
+// 3-channel maps (the network input, dL/dr) land as FP32 RGBA and four warps round
+// them to BF16 rows of 8 channels, the last five zero, without swizzle: M then covers
+// sixteen rows (three used), N = 32 four starts (three used).  The same warps
+// sum g for the bias gradient.
 //   MODE 1: g = dL/dz1 (BF16, 32), a = the network input (FP32 RGBA, 3).  W1, b1.
 //   MODE 2: g = dL/dz2 (BF16, 32), a = a1 (BF16, 32).                        W2, b2.
 //   MODE 3: g = dL/dr  (FP32 RGBA, 3), a = a2 (BF16, 32).                    W3, b3.
 //
-// One CTA per SM, a ring of stages between a TMA warp, an MMA warp and the two
-// warps above; the accumulators stay in TMEM over all tiles of a CTA, which then
+// One CTA per SM, a ring of stages between a TMA warp, an MMA warp and the
+// four warps above; the accumulators stay in TMEM over all tiles of a CTA, which then
 // writes one partial row; the rows are summed in a fixed order afterwards
-// (deterministic).  Bound by the operands' way through shared memory (an MMA reads
-// 4 KB of A and 3 KB of B, 62 cycles against the 53 of its arithmetic) and by the
-// three copies of g from L2.  Against kernels that transposed chunks of 64 pixels
-// with ldmatrix and wrote every input nine times for its taps, 16 crops of 256^2:
-// 109, 67 and 93 us for W2, W1 and W3 -> 33, 32 and 23 us (training step 564 -> 370).
+// (deterministic).  Bound by reading the maps (134 and 84 MB at 16 x 256^2: 20 and 12
+// us) and a start and an end of some 8 us; halving the MMAs changes nothing.  Against
+// kernels that transposed chunks of 64 pixels with ldmatrix and wrote every input nine
+// times for its taps, 16 crops of 256^2: 109, 67 and 93 us for W2, W1 and W3 -> 31, 25
+// and 23 us.  With three shifted copies of g loaded instead of one, W2 took 33 us, and
+// 75 when the copies came as {8 channels, W, group} boxes, 16 bytes at a time.
 
 namespace {
 
 constexpr int kGTW = 32, kGTH = 8;               // tile: 32 x 8 positions
-constexpr int kG32Row = kGTW * 64;               // a row of 32 channels
-constexpr int kG8Row = kGTW * 16;                // a row of 8 channels
-constexpr int kGThreads = 128;
+constexpr int kGHelpers = 4;                     // warps that round FP32 maps and sum g
+constexpr int kGThreads = 64 + 32 * kGHelpers;
 
 template <int MODE>
 struct WgradShape {
   static constexpr int OC = MODE == 3 ? 8 : 32;          // channels of g as held
-  static constexpr int KX = MODE == 3 ? 4 : 3;           // copies of g held (three loaded)
-  static constexpr int N = KX * OC;
+  static constexpr int N = MODE == 3 ? 32 : 96;          // starts x channels
   static constexpr int COUT = MODE == 3 ? 3 : 32, CIN = MODE == 1 ? 3 : 32;
-  static constexpr int kARow = MODE == 1 ? kG8Row : kG32Row, kAB = (kGTH + 2) * kARow;
-  static constexpr int kGRow = MODE == 3 ? kG8Row : kG32Row, kGCopy = kGTH * kGRow, kGB = KX * kGCopy;
-  static constexpr int FW = MODE == 1 ? kGTW : kGTW + 2, FH = MODE == 1 ? kGTH + 2 : kGTH;  // FP32 RGBA positions
-  static constexpr int kFB = MODE == 2 ? 0 : (FW * FH * 16 + 511) / 512 * 512;
-  static constexpr int kStageB = kAB + kGB + kFB;
-  static constexpr int kTx = MODE == 1 ? kGB + FW * FH * 16 : MODE == 2 ? kAB + kGB : kAB + FW * FH * 16;
-  static constexpr int kStages = MODE == 3 ? 5 : 3;
+  static constexpr int kARow = kGTW * (MODE == 1 ? 16 : 64), kAB = (kGTH + 2) * kARow;  // rows of 32 positions
+  static constexpr int GW = kGTW + 2, kGPos = 2 * OC, kGRow = GW * kGPos, kGB = kGTH * kGRow + 512;  // rows of 34
+  static constexpr int FW = MODE == 1 ? kGTW : GW, FH = MODE == 1 ? kGTH + 2 : kGTH;    // FP32 RGBA positions
+  static constexpr int kFB = MODE == 2 ? 0 : FW * FH * 16;
+  static constexpr int kStageB = (kAB + kGB + kFB + 511) / 512 * 512;
+  static constexpr int kTx = (MODE == 1 ? 0 : kAB) + (MODE == 3 ? 0 : kGTH * kGRow) + FW * FH * (MODE == 2 ? 0 : 16);
+  static constexpr int kStages = 5;
   // The unused accumulator rows take what lies behind a tile's rows of a: the stage's g
   static_assert((kGTH - 1) * kARow + (MODE == 1 ? 16 : 4) * kARow <= kStageB, "MMAs read within the stage");
-  static_assert(kStageB % 512 == 0, "stages start on a swizzle atom");
+  static_assert(kAB % 512 == 0, "g starts on a swizzle atom");
   static constexpr int kBarOff = kStages * kStageB;
   static constexpr int kSmem = 1024 + kBarOff + (3 * kStages + 1) * 8 + 16;  // 1024: the base is rounded up
   static_assert(kSmem <= 224 * 1024, "fits one CTA's shared memory");
@@ -586,7 +681,7 @@ __global__ void __launch_bounds__(kGThreads) wgrad_tc_kernel(RefineWgradArgs A, 
   uint64_t* done = empty + S::kStages;                             // all MMAs of the CTA are complete
   uint32_t* tslot = reinterpret_cast<uint32_t*>(done + 1);
   __shared__ volatile int s_abort;
-  __shared__ float s_bias[64][8];
+  __shared__ float s_bias[32 * kGHelpers][8];
   const int tid = threadIdx.x, warp = tid >> 5, lane = tid & 31;
   const int n_tiles = A.n_tiles;
 
@@ -594,8 +689,8 @@ __global__ void __launch_bounds__(kGThreads) wgrad_tc_kernel(RefineWgradArgs A, 
     s_abort = 0;
     for (int k = 0; k < S::kStages; ++k) {
       asm volatile("mbarrier.init.shared::cta.b64 [%0], 1;" ::"r"(c_su32(full + k)));
-      asm volatile("mbarrier.init.shared::cta.b64 [%0], 2;" ::"r"(c_su32(ready + k)));
-      asm volatile("mbarrier.init.shared::cta.b64 [%0], 3;" ::"r"(c_su32(empty + k)));
+      asm volatile("mbarrier.init.shared::cta.b64 [%0], %1;" ::"r"(c_su32(ready + k)), "r"(kGHelpers));
+      asm volatile("mbarrier.init.shared::cta.b64 [%0], %1;" ::"r"(c_su32(empty + k)), "r"(1 + kGHelpers));
     }
     asm volatile("mbarrier.init.shared::cta.b64 [%0], 1;" ::"r"(c_su32(done)));
     asm volatile("fence.mbarrier_init.release.cluster;" ::: "memory");
@@ -633,12 +728,7 @@ __global__ void __launch_bounds__(kGThreads) wgrad_tc_kernel(RefineWgradArgs A, 
         uint64_t* bar = full + j % S::kStages;
         asm volatile("mbarrier.arrive.expect_tx.shared::cta.b64 _, [%0], %1;" ::"r"(c_su32(bar)), "r"(S::kTx) : "memory");
         g_tma4(&amap, MODE == 1 ? sf : st, bar, 0, x0, y0 - 1, img);
-        if (MODE == 3) {
-          g_tma4(&gmap, sf, bar, 0, x0 - 1, y0, img);
-        } else {
-#pragma unroll
-          for (int kx = 0; kx < 3; ++kx) g_tma4(&gmap, sg + kx * S::kGCopy, bar, 0, x0 + 1 - kx, y0, img);
-        }
+        g_tma4(&gmap, MODE == 3 ? sf : sg, bar, 0, x0 - 1, y0, img);
         issued = j + 1;
       }
       // the last copies land before the CTA can leave (earlier ones have been waited for by their readers or are
@@ -656,8 +746,8 @@ __global__ void __launch_bounds__(kGThreads) wgrad_tc_kernel(RefineWgradArgs A, 
         asm volatile("tcgen05.fence::after_thread_sync;" ::: "memory");
         const uint32_t st = c_su32(sm) + (j % S::kStages) * S::kStageB;
         constexpr int kAK = MODE == 1 ? 256 : 1024, kGK = MODE == 3 ? 256 : 1024;  // 16 positions
-        const uint64_t ad = MODE == 1 ? g_desc8(st, kG8Row) : g_desc32(st, kG32Row);
-        const uint64_t bd = MODE == 3 ? g_desc8(st + S::kAB, S::kGCopy) : g_desc32(st + S::kAB, S::kGCopy);
+        const uint64_t ad = MODE == 1 ? g_desc8(st, S::kARow) : g_desc32(st, S::kARow);
+        const uint64_t bd = MODE == 3 ? g_desc8(st + S::kAB, S::kGPos) : g_desc32(st + S::kAB, S::kGPos);
         for (int r = 0; r < kGTH; ++r)
 #pragma unroll
           for (int k = 0; k < 2; ++k)
@@ -671,7 +761,7 @@ __global__ void __launch_bounds__(kGThreads) wgrad_tc_kernel(RefineWgradArgs A, 
     }
   } else {
     // ---------------------------------------------------------------- rounding of FP32 maps, bias sums
-    const int t = tid - 64;  // 0 .. 63
+    const int t = tid - 64;
     float acc[8];
 #pragma unroll
     for (int k = 0; k < 8; ++k) acc[k] = 0.f;
@@ -685,18 +775,14 @@ __global__ void __launch_bounds__(kGThreads) wgrad_tc_kernel(RefineWgradArgs A, 
       unsigned char* sg = st + S::kAB;
       if (MODE != 2) {
         const float4* f = reinterpret_cast<const float4*>(sg + S::kGB);
-        for (int i = t; i < S::FW * S::FH; i += 64) {
+        for (int i = t; i < S::FW * S::FH; i += 32 * kGHelpers) {
           const float4 v = f[i];
           const uint4 w = make_uint4(c_pack(v.x, v.y), c_pack(v.z, 0.f), 0u, 0u);
           if (MODE == 1) {
             reinterpret_cast<uint4*>(st)[i] = w;  // [row][position]
           } else {
-            const int r = i / S::FW, x = i - r * S::FW;  // image column x0 - 1 + x
-#pragma unroll
-            for (int kx = 0; kx < 3; ++kx) {  // copy kx holds column x0 + 1 - kx first
-              const int q = x - 2 + kx;
-              if (q >= 0 && q < kGTW) *reinterpret_cast<uint4*>(sg + kx * S::kGCopy + r * kG8Row + q * 16) = w;
-            }
+            const int x = i % S::FW;  // image column x0 - 1 + x
+            reinterpret_cast<uint4*>(sg)[i] = w;  // [row][position]
             if (x >= 1 && x <= kGTW) {  // the tile's own pixels, as rounded for the MMAs
               acc[0] += __uint_as_float(w.x << 16);
               acc[1] += __uint_as_float(w.x & 0xffff0000u);
@@ -708,18 +794,17 @@ __global__ void __launch_bounds__(kGThreads) wgrad_tc_kernel(RefineWgradArgs A, 
         __syncwarp();
         if (lane == 0) g_arrive(ready + j % S::kStages);
       }
-      if (MODE != 3) {  // thread t: channels 8 (t & 3) .., positions t / 4 and t / 4 + 16 of the unshifted copy
+      if (MODE != 3) {  // thread t: channels 8 (t & 3) .. of the tile's column t / 4
+        static_assert(kGHelpers * 32 == kGTW * 4, "a thread per column and 8 channels");
+#pragma unroll
         for (int r = 0; r < kGTH; ++r) {
+          const int at = r * S::kGRow + ((t >> 2) + 1) * 64;  // the swizzle moves a 16-byte piece by bits 7 and 8
+          const uint4 v = *reinterpret_cast<const uint4*>(sg + at + (((t & 3) ^ ((at >> 7) & 3)) << 4));
+          const uint32_t w[4] = {v.x, v.y, v.z, v.w};
 #pragma unroll
-          for (int h = 0; h < 2; ++h) {
-            const int q = (t >> 2) + 16 * h;  // the swizzle moves a 16-byte chunk by the position's bits 1 and 2
-            const uint4 v = *reinterpret_cast<const uint4*>(sg + S::kGCopy + r * kG32Row + q * 64 + (((t & 3) ^ ((q >> 1) & 3)) << 4));
-            const uint32_t w[4] = {v.x, v.y, v.z, v.w};
-#pragma unroll
-            for (int k = 0; k < 4; ++k) {
-              acc[2 * k] += __uint_as_float(w[k] << 16);
-              acc[2 * k + 1] += __uint_as_float(w[k] & 0xffff0000u);
-            }
+          for (int k = 0; k < 4; ++k) {
+            acc[2 * k] += __uint_as_float(w[k] << 16);
+            acc[2 * k + 1] += __uint_as_float(w[k] & 0xffff0000u);
           }
         }
       }
@@ -747,16 +832,16 @@ __global__ void __launch_bounds__(kGThreads) wgrad_tc_kernel(RefineWgradArgs A, 
         if (keep) {
 #pragma unroll
           for (int k = 0; k < 16; ++k) {
-            const int col = 16 * h + k, kx = col / S::OC, o = col % S::OC;
-            if (kx < 3 && o < S::COUT) out[((ky * 3 + kx) * S::COUT + o) * S::CIN + c] = v[k];
+            const int col = 16 * h + k, kx = 2 - col / S::OC, o = col % S::OC;  // start i holds g[x - 1 + i]
+            if (kx >= 0 && o < S::COUT) out[((ky * 3 + kx) * S::COUT + o) * S::CIN + c] = v[k];
           }
         }
       }
     }
     if (tid < S::COUT) {  // bias gradient: the threads' sums in a fixed order
       float b = 0.f;
-      if (MODE == 3) for (int k = 0; k < 64; ++k) b += s_bias[k][tid];
-      else for (int k = 0; k < 16; ++k) b += s_bias[4 * k + (tid >> 3)][tid & 7];
+      if (MODE == 3) for (int k = 0; k < 32 * kGHelpers; ++k) b += s_bias[k][tid];
+      else for (int k = 0; k < 8 * kGHelpers; ++k) b += s_bias[4 * k + (tid >> 3)][tid & 7];
       out[9 * S::COUT * S::CIN + tid] = b;
     }
   }
@@ -769,25 +854,6 @@ __global__ void __launch_bounds__(kGThreads) wgrad_tc_kernel(RefineWgradArgs A, 
 }
 
 namespace {
-
-// Tensor maps over an NHWC map: 32 BF16 channels as {32, W, H, n} under the 64-byte swizzle, or FP32 RGBA as
-// {4, W, H, n}.  (As {8, W, 4 groups, H, n}, 16 bytes at a time, the copies bounded the kernel: 75 us instead of 33 for 32 channels against 32.)
-bool encode_map32(EncodeTiled enc, CUtensorMap* m, const void* p, int n, int H, int W, int box_w, int box_h) {
-  const cuuint64_t dims[4] = {32, (cuuint64_t)W, (cuuint64_t)H, (cuuint64_t)n};
-  const cuuint64_t strides[3] = {64, (cuuint64_t)W * 64, (cuuint64_t)W * H * 64};
-  const cuuint32_t box[4] = {32, (cuuint32_t)box_w, (cuuint32_t)box_h, 1}, step[4] = {1, 1, 1, 1};
-  return enc(m, CU_TENSOR_MAP_DATA_TYPE_BFLOAT16, 4, const_cast<void*>(p), dims, strides, box, step,
-             CU_TENSOR_MAP_INTERLEAVE_NONE, CU_TENSOR_MAP_SWIZZLE_64B, CU_TENSOR_MAP_L2_PROMOTION_L2_128B,
-             CU_TENSOR_MAP_FLOAT_OOB_FILL_NONE) == CUDA_SUCCESS;
-}
-bool encode_rgba(EncodeTiled enc, CUtensorMap* m, const void* p, int n, int H, int W, int box_w, int box_h) {
-  const cuuint64_t dims[4] = {4, (cuuint64_t)W, (cuuint64_t)H, (cuuint64_t)n};
-  const cuuint64_t strides[3] = {16, (cuuint64_t)W * 16, (cuuint64_t)W * H * 16};
-  const cuuint32_t box[4] = {4, (cuuint32_t)box_w, (cuuint32_t)box_h, 1}, step[4] = {1, 1, 1, 1};
-  return enc(m, CU_TENSOR_MAP_DATA_TYPE_FLOAT32, 4, const_cast<void*>(p), dims, strides, box, step,
-             CU_TENSOR_MAP_INTERLEAVE_NONE, CU_TENSOR_MAP_SWIZZLE_NONE, CU_TENSOR_MAP_L2_PROMOTION_L2_128B,
-             CU_TENSOR_MAP_FLOAT_OOB_FILL_NONE) == CUDA_SUCCESS;
-}
 
 template <int MODE>
 cudaError_t launch_wgrad_tc_t(const RefineWgradArgs& a, cudaStream_t s) {
@@ -802,7 +868,7 @@ cudaError_t launch_wgrad_tc_t(const RefineWgradArgs& a, cudaStream_t s) {
   const bool ok = (MODE == 1 ? encode_rgba(enc, &am, a.x, a.n, a.H, a.W, S::FW, S::FH)
                              : encode_map32(enc, &am, a.a_h, a.n, a.H, a.W, kGTW, kGTH + 2)) &&
                   (MODE == 3 ? encode_rgba(enc, &gm, a.g_f, a.n, a.H, a.W, S::FW, S::FH)
-                             : encode_map32(enc, &gm, a.g_h, a.n, a.H, a.W, kGTW, kGTH));
+                             : encode_map32(enc, &gm, a.g_h, a.n, a.H, a.W, S::GW, kGTH));
   if (!ok) return cudaErrorInvalidValue;
   wgrad_tc_kernel<MODE><<<a.n_ctas, kGThreads, S::kSmem, s>>>(a, am, gm);
   return cudaGetLastError();
