@@ -1171,27 +1171,28 @@ RefineConvArgs conv_args(lf_ctx* c, int32_t n, int32_t w, int32_t h) {
 }
 
 // The three layer launches of the per-layer path (inference).
-lf_status refine_layers(lf_ctx* c, int32_t n, int32_t w, int32_t h, const float* in, float* out, cudaStream_t s) {
+lf_status refine_layers(lf_ctx* c, int32_t n, int32_t w, int32_t h, const float* in, float* out, cudaStream_t s,
+                        bool pdl) {
   const float* prm = rf_params(c);
   RefineConvArgs a = conv_args(c, n, w, h);
   a.src_f = in;
   a.wt = rf_w(c, kPackW1f);
   a.bias = prm + kRefineOffB1;
   a.out_h = static_cast<__nv_bfloat16*>(c->rf.a1.p);
-  LF_CUDA(c, launch_refine_conv(kConvInRGBA, 32, kEpiRelu, a, s));
+  LF_CUDA(c, launch_refine_conv(kConvInRGBA, 32, kEpiRelu, a, s, pdl));
   a = conv_args(c, n, w, h);
   a.src_h = static_cast<const __nv_bfloat16*>(c->rf.a1.p);
   a.wt = rf_w(c, kPackW2f);
   a.bias = prm + kRefineOffB2;
   a.out_h = static_cast<__nv_bfloat16*>(c->rf.a2.p);
-  LF_CUDA(c, launch_refine_conv(kConvInBF16, 32, kEpiRelu, a, s));
+  LF_CUDA(c, launch_refine_conv(kConvInBF16, 32, kEpiRelu, a, s, true));
   a = conv_args(c, n, w, h);
   a.src_h = static_cast<const __nv_bfloat16*>(c->rf.a2.p);
   a.wt = rf_w(c, kPackW3f);
   a.bias = prm + kRefineOffB3;
   a.x = in;
   a.out_f = out;
-  LF_CUDA(c, launch_refine_conv(kConvInBF16, 8, kEpiResid, a, s));
+  LF_CUDA(c, launch_refine_conv(kConvInBF16, 8, kEpiResid, a, s, true));
   return LF_OK;
 }
 
@@ -1209,7 +1210,7 @@ lf_status refine_apply(lf_ctx* c, int32_t n, int32_t w, int32_t h, const float* 
   }
   lf_status st = refine_hidden(c, (int64_t)n * w * h, false);
   if (st != LF_OK) return st;
-  return refine_layers(c, n, w, h, in, out, s);
+  return refine_layers(c, n, w, h, in, out, s, pdl);
 }
 
 // The refinement of a rendered frame: eye e's image in[e] (FP32 RGBA) into
@@ -1242,8 +1243,10 @@ lf_status refine_backward(lf_ctx* c, int32_t n, int32_t w, int32_t h, const floa
   float* loss = static_cast<float*>(c->rf.scal.p);
   int32_t* count = reinterpret_cast<int32_t*>(loss + 1);
   LF_CUDA(c, cudaMemsetAsync(c->rf.scal.p, 0, 8, s));
-  LF_CUDA(c, cudaMemsetAsync(rf_grad(c), 0, sizeof(float) * kRefineParams, s));
-  if (n_pix == 0) return LF_OK;
+  if (n_pix == 0) {
+    LF_CUDA(c, cudaMemsetAsync(rf_grad(c), 0, sizeof(float) * kRefineParams, s));
+    return LF_OK;
+  }
   LF_CUDA(c, launch_refine_count(in, tgt, n_pix, count, s));
   const float* prm = rf_params(c);
   auto* a1 = static_cast<__nv_bfloat16*>(c->rf.a1.p);
@@ -1252,14 +1255,14 @@ lf_status refine_backward(lf_ctx* c, int32_t n, int32_t w, int32_t h, const floa
   float* gr = static_cast<float*>(c->rf.gr.p);
   RefineConvArgs a = conv_args(c, n, w, h);
   a.src_f = in; a.wt = rf_w(c, kPackW1f); a.bias = prm + kRefineOffB1; a.out_h = a1;
-  LF_CUDA(c, launch_refine_conv(kConvInRGBA, 32, kEpiRelu, a, s));
+  LF_CUDA(c, launch_refine_conv(kConvInRGBA, 32, kEpiRelu, a, s, true));
   a = conv_args(c, n, w, h);
   a.src_h = a1; a.wt = rf_w(c, kPackW2f); a.bias = prm + kRefineOffB2; a.out_h = a2;
-  LF_CUDA(c, launch_refine_conv(kConvInBF16, 32, kEpiRelu, a, s));
+  LF_CUDA(c, launch_refine_conv(kConvInBF16, 32, kEpiRelu, a, s, true));
   a = conv_args(c, n, w, h);
   a.src_h = a2; a.wt = rf_w(c, kPackW3f); a.bias = prm + kRefineOffB3; a.x = in; a.target = tgt; a.out_f = gr;
   a.loss = loss; a.count = count;
-  LF_CUDA(c, launch_refine_conv(kConvInBF16, 8, kEpiLoss, a, s));
+  LF_CUDA(c, launch_refine_conv(kConvInBF16, 8, kEpiLoss, a, s, true));
 
   RefineWgradArgs g;
   std::memset(&g, 0, sizeof(g));
@@ -1275,11 +1278,11 @@ lf_status refine_backward(lf_ctx* c, int32_t n, int32_t w, int32_t h, const floa
   LF_CUDA(c, launch_refine_wgrad(3, g, s));
   a = conv_args(c, n, w, h);
   a.src_f = gr; a.wt = rf_w(c, kPackW3b); a.mask = a2; a.out_h = gz2;
-  LF_CUDA(c, launch_refine_conv(kConvInRGBA, 32, kEpiMask, a, s));
+  LF_CUDA(c, launch_refine_conv(kConvInRGBA, 32, kEpiMask, a, s, true));
   // dL/dz1 through layer 2's input (into a2's buffer, no longer needed)
   a = conv_args(c, n, w, h);
   a.src_h = gz2; a.wt = rf_w(c, kPackW2b); a.mask = a1; a.out_h = a2;
-  LF_CUDA(c, launch_refine_conv(kConvInBF16, 32, kEpiMask, a, s));
+  LF_CUDA(c, launch_refine_conv(kConvInBF16, 32, kEpiMask, a, s, true));
   g.g_f = nullptr; g.g_h = gz2; g.a_h = a1; g.partial = part2; g.seg = kRefineSegs[1];
   LF_CUDA(c, launch_refine_wgrad(2, g, s));
   g.g_h = a2; g.a_h = nullptr; g.x = in; g.partial = part1; g.seg = kRefineSegs[0];
@@ -1307,7 +1310,7 @@ lf_status lf_load_refiner(lf_ctx* c, const float* params) {
   LF_CUDA(c, cudaMemsetAsync(c->rf.state.p, 0, sizeof(float) * 4 * kRefineParams, s));
   LF_CUDA(c, cudaMemcpyAsync(c->rf.state.p, params, sizeof(float) * kRefineParams, cudaMemcpyHostToDevice, s));
   LF_CUDA(c, cudaMemsetAsync(c->rf.scal.p, 0, 64, s));
-  LF_CUDA(c, launch_refine_pack(rf_params(c), static_cast<__nv_bfloat16*>(c->rf.packed.p), s));
+  LF_CUDA(c, launch_refine_pack(rf_params(c), static_cast<__nv_bfloat16*>(c->rf.packed.p), s, false));
   LF_CUDA(c, cudaStreamSynchronize(s));
   c->rf.loaded = true;
   c->rf.step = 0;
@@ -1372,7 +1375,7 @@ lf_status lf_refine_train_step(lf_ctx* c, int32_t n_images, int32_t width, int32
   const float c1 = (float)(1.0 / (1.0 - std::pow(beta1, t))), c2 = (float)(1.0 / (1.0 - std::pow(beta2, t)));
   LF_CUDA(c, launch_refine_adam(rf_params(c), rf_m(c), rf_v(c), rf_grad(c), kRefineParams, lr, beta1, beta2, 1e-8f,
                                 c1, c2, s));
-  LF_CUDA(c, launch_refine_pack(rf_params(c), static_cast<__nv_bfloat16*>(c->rf.packed.p), s));
+  LF_CUDA(c, launch_refine_pack(rf_params(c), static_cast<__nv_bfloat16*>(c->rf.packed.p), s, true));
   c->rf.step = t;
   return LF_OK;
 }

@@ -259,7 +259,9 @@ struct RefineWgradArgs {
   uint64_t wait_ns;            // bound on each wait
 };
 
-cudaError_t launch_refine_conv(int in_mode, int cout, int epi, const RefineConvArgs& a, cudaStream_t s);
+// (the training and per-layer kernels wait for the kernel before them themselves: launched as its programmatic
+// dependents, always or with pdl)
+cudaError_t launch_refine_conv(int in_mode, int cout, int epi, const RefineConvArgs& a, cudaStream_t s, bool pdl);
 cudaError_t launch_refine_wgrad(int mode, const RefineWgradArgs& a, cudaStream_t s);
 // The weight-gradient kernels' tiles of n H x W images: their number, and per row and column.
 int refine_wgrad_tiles(int n, int H, int W, int* tiles_x, int* tiles_y);
@@ -268,7 +270,7 @@ cudaError_t launch_refine_reduce(const float* const partial[3], int n_rows, floa
 cudaError_t launch_refine_count(const float* x, const float* t, int64_t n_pix, int32_t* count, cudaStream_t s);
 cudaError_t launch_refine_adam(float* p, float* m, float* v, const float* g, int n, float lr, double beta1,
                                double beta2, float eps, float c1, float c2, cudaStream_t s);
-cudaError_t launch_refine_pack(const float* params, __nv_bfloat16* w, cudaStream_t s);
+cudaError_t launch_refine_pack(const float* params, __nv_bfloat16* w, cudaStream_t s, bool pdl);
 // Fused inference (lf_refine_tc.cu): all three layers per tile, tcgen05 MMAs.
 // Image i goes to out + i*h*w*4, except image 1 to out1 when out1 is set; with
 // pdl the launch is a programmatic dependent of the kernel before it.

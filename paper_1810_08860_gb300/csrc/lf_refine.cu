@@ -40,9 +40,12 @@ __global__ void reduce_partials_kernel(ReduceArgs A) {
   const int lane = threadIdx.x & 31, k = threadIdx.x >> 5, layer = blockIdx.y;
   const int cin = kCin[layer], cout = kCout[layer], nw = 9 * cin * cout, seg = nw + cout;
   const int i = blockIdx.x * 32 + lane;
+  griddep_release();
+  griddep_wait();
   if (blockIdx.x * 32 >= seg) return;
   float s = 0.f;
   if (i < seg)
+#pragma unroll 8
     for (int b = k; b < A.n_rows; b += 8) s += A.partial[layer][(size_t)b * seg + i];
   part[k][lane] = s;
   __syncthreads();
@@ -58,8 +61,19 @@ __global__ void reduce_partials_kernel(ReduceArgs A) {
 __global__ void count_valid_kernel(const float4* __restrict__ x, const float4* __restrict__ t, int64_t n,
                                    int* __restrict__ count) {
   int c = 0;
-  for (int64_t i = blockIdx.x * (int64_t)blockDim.x + threadIdx.x; i < n; i += (int64_t)gridDim.x * blockDim.x)
-    c += (x[i].w > 0.f && t[i].w > 0.f) ? 1 : 0;
+  griddep_release();
+  const int64_t step = (int64_t)gridDim.x * blockDim.x;
+  for (int64_t i = blockIdx.x * (int64_t)blockDim.x + threadIdx.x; i < n; i += 4 * step) {
+    float a[4], b[4];
+#pragma unroll
+    for (int u = 0; u < 4; ++u) {  // eight loads in flight
+      const bool in = i + u * step < n;
+      a[u] = in ? x[i + u * step].w : 0.f;
+      b[u] = in ? t[i + u * step].w : 0.f;
+    }
+#pragma unroll
+    for (int u = 0; u < 4; ++u) c += a[u] > 0.f && b[u] > 0.f ? 1 : 0;
+  }
 #pragma unroll
   for (int o = 16; o > 0; o >>= 1) c += __shfl_xor_sync(0xffffffffu, c, o);
   if ((threadIdx.x & 31) == 0 && c) atomicAdd(count, c);
@@ -71,6 +85,8 @@ __global__ void adam_kernel(float* __restrict__ p, float* __restrict__ m, float*
                             const float* __restrict__ g, int n, float lr, float beta1, float beta2, float omb1,
                             float omb2, float eps, float c1, float c2) {
   const int i = blockIdx.x * blockDim.x + threadIdx.x;
+  griddep_release();
+  griddep_wait();
   if (i >= n) return;
   const float gi = g[i];
   const float mi = __fadd_rn(__fmul_rn(beta1, m[i]), __fmul_rn(omb1, gi));
@@ -97,6 +113,8 @@ __global__ void pack_weights_kernel(const float* __restrict__ prm, __nv_bfloat16
   constexpr int n1 = 32 * 32, n2 = 9 * 32 * 32, n3 = 9 * 8 * 32, n3b = 32 * 32, n2b = 9 * 32 * 32;
   const int i = blockIdx.x * blockDim.x + threadIdx.x;
   float v = 0.f;
+  griddep_release();
+  griddep_wait();
   if (i < n1) {
     const int o = i >> 5, k = i & 31;
     if (k < 27) v = prm[kRefineOffW1 + o * 27 + (k % 3) * 9 + k / 3];
@@ -135,8 +153,7 @@ __global__ void pack_weights_kernel(const float* __restrict__ prm, __nv_bfloat16
 
 cudaError_t launch_refine_reduce(const float* const partial[3], int n_rows, float* grad, cudaStream_t s) {
   const ReduceArgs a = {{partial[0], partial[1], partial[2]}, grad, n_rows};
-  reduce_partials_kernel<<<dim3((9 * 32 * 32 + 32 + 31) / 32, 3), 256, 0, s>>>(a);
-  return cudaGetLastError();
+  return launch_kernel(reduce_partials_kernel, dim3((9 * 32 * 32 + 32 + 31) / 32, 3), dim3(256), 0, s, true, a);
 }
 
 cudaError_t launch_refine_count(const float* x, const float* t, int64_t n_pix, int* count, cudaStream_t s) {
@@ -148,14 +165,12 @@ cudaError_t launch_refine_count(const float* x, const float* t, int64_t n_pix, i
 
 cudaError_t launch_refine_adam(float* p, float* m, float* v, const float* g, int n, float lr, double beta1,
                                double beta2, float eps, float c1, float c2, cudaStream_t s) {
-  adam_kernel<<<(n + 255) / 256, 256, 0, s>>>(p, m, v, g, n, lr, (float)beta1, (float)beta2, (float)(1.0 - beta1),
-                                              (float)(1.0 - beta2), eps, c1, c2);
-  return cudaGetLastError();
+  return launch_kernel(adam_kernel, dim3((n + 255) / 256), dim3(256), 0, s, true, p, m, v, g, n, lr, (float)beta1,
+                       (float)beta2, (float)(1.0 - beta1), (float)(1.0 - beta2), eps, c1, c2);
 }
 
-cudaError_t launch_refine_pack(const float* params, __nv_bfloat16* w, cudaStream_t s) {
-  pack_weights_kernel<<<(kRefinePackedElems + 255) / 256, 256, 0, s>>>(params, w);
-  return cudaGetLastError();
+cudaError_t launch_refine_pack(const float* params, __nv_bfloat16* w, cudaStream_t s, bool pdl) {
+  return launch_kernel(pack_weights_kernel, dim3((kRefinePackedElems + 255) / 256), dim3(256), 0, s, pdl, params, w);
 }
 
 }  // namespace lfk

@@ -230,6 +230,31 @@ __global__ void __launch_bounds__(kCThreads, kCPerSM)
   const int tid = threadIdx.x, warp = tid >> 5, lane = tid & 31;
   const int H = A.H, W = A.W;
 
+  if (IN == kConvInRGBA)
+    for (int i = tid; i < kCPairB / 16; i += kCThreads)  // the guard rows stay zero
+      reinterpret_cast<uint4*>(sx)[i] = make_uint4(0u, 0u, 0u, 0u);
+  else if (tid < 8)
+    reinterpret_cast<uint4*>(sx + kCHaloTx)[tid] = make_uint4(0u, 0u, 0u, 0u);
+  if (tid == 0) {
+    s_abort = 0;
+    asm volatile("mbarrier.init.shared::cta.b64 [%0], 1;" ::"r"(c_su32(bar)));
+    asm volatile("mbarrier.init.shared::cta.b64 [%0], 1;" ::"r"(c_su32(xbar)));
+    asm volatile("fence.mbarrier_init.release.cluster;" ::: "memory");
+  }
+  if (warp == 0) {
+    asm volatile("tcgen05.alloc.cta_group::1.sync.aligned.shared::cta.b32 [%0], %1;" ::"r"(c_su32(tslot)),
+                 "r"(kCTmemCols));
+    asm volatile("tcgen05.relinquish_alloc_permit.cta_group::1.sync.aligned;");
+  }
+  asm volatile("tcgen05.fence::before_thread_sync;" ::: "memory");
+  __syncthreads();
+  asm volatile("tcgen05.fence::after_thread_sync;" ::: "memory");
+  const uint32_t tmem = *tslot;
+  // Launched as a programmatic dependent, what is above overlaps the end of the kernel before; everything read below
+  // is written by it or by earlier ones.  The next kernel may launch once every CTA of this one holds its tensor
+  // memory (it would otherwise take columns that a CTA of this grid still waits for).
+  griddep_release();
+  griddep_wait();
   // Weights into core-matrix blocks: block b, K group g, row n at sw + b * kBlkB + (g * N + n) * 16.
   for (int i = tid; i < NB * 2 * N; i += kCThreads) {
     const int b = i / (2 * N), g = (i / N) & 1, n = i % N;
@@ -255,28 +280,9 @@ __global__ void __launch_bounds__(kCThreads, kCPerSM)
     }
     *reinterpret_cast<uint4*>(sw + b * kBlkB + (g * N + n) * 16) = v;
   }
-  if (IN == kConvInRGBA)
-    for (int i = tid; i < kCPairB / 16; i += kCThreads)  // the guard rows stay zero
-      reinterpret_cast<uint4*>(sx)[i] = make_uint4(0u, 0u, 0u, 0u);
-  else if (tid < 8)
-    reinterpret_cast<uint4*>(sx + kCHaloTx)[tid] = make_uint4(0u, 0u, 0u, 0u);
-  asm volatile("fence.proxy.async.shared::cta;" ::: "memory");  // the zeros, to the tensor core and TMA
   if (tid < 32) s_bias[tid] = (EPI == kEpiRelu || (EPI != kEpiMask && tid < 3)) ? A.bias[tid] : 0.f;
-  if (tid == 0) {
-    s_abort = 0;
-    asm volatile("mbarrier.init.shared::cta.b64 [%0], 1;" ::"r"(c_su32(bar)));
-    asm volatile("mbarrier.init.shared::cta.b64 [%0], 1;" ::"r"(c_su32(xbar)));
-    asm volatile("fence.mbarrier_init.release.cluster;" ::: "memory");
-  }
-  if (warp == 0) {
-    asm volatile("tcgen05.alloc.cta_group::1.sync.aligned.shared::cta.b32 [%0], %1;" ::"r"(c_su32(tslot)),
-                 "r"(kCTmemCols));
-    asm volatile("tcgen05.relinquish_alloc_permit.cta_group::1.sync.aligned;");
-  }
-  asm volatile("tcgen05.fence::before_thread_sync;" ::: "memory");
+  asm volatile("fence.proxy.async.shared::cta;" ::: "memory");  // weights and zeros, to the tensor core and TMA
   __syncthreads();
-  asm volatile("tcgen05.fence::after_thread_sync;" ::: "memory");
-  const uint32_t tmem = *tslot;
 
   float loss_scale = 0.f;
   if (EPI == kEpiLoss) {
@@ -358,7 +364,7 @@ __global__ void __launch_bounds__(kCThreads, kCPerSM)
                                             : c_desc(c_su32(sx) + kCGuard * 16, 32, 128);
       const uint64_t bd = c_desc(c_su32(sw), N * 16, 128);
       constexpr uint32_t id = c_idesc(128, N);
-#pragma unroll 1
+#pragma unroll (S::kMB == kCMT ? kCMT : 1)
       for (int m = m0; m < m0 + S::kMB; ++m) {
         const uint32_t d = tmem + (uint32_t)((m - m0) * N);
 #pragma unroll
@@ -407,7 +413,7 @@ __global__ void __launch_bounds__(kCThreads, kCPerSM)
     const int gx = x0 + lane - 1;
     float lsum = 0.f;
     bool ok = true;
-#pragma unroll 1
+#pragma unroll (S::kMB == kCMT ? kCMT : 1)
     for (int m = 0; m < kCMT; ++m) {
       if (m % S::kMB == 0 && !landed()) {
         ok = false;
@@ -551,7 +557,7 @@ bool encode_rgba(EncodeTiled enc, CUtensorMap* m, const void* p, int n, int H, i
 }
 
 template <int IN, int COUT, int EPI>
-cudaError_t launch_conv_tc_t(const RefineConvArgs& a, cudaStream_t s) {
+cudaError_t launch_conv_tc_t(const RefineConvArgs& a, cudaStream_t s, bool pdl) {
   constexpr int kW = ConvShape<IN, COUT>::kWBytes;
   constexpr int used = 1024 + (IN == kConvInBF16 ? kW + kCHaloTx + 128 + 24
                                                  : (kW + kCXOff + kCPairB + 127) / 128 * 128 + kCXsB + 24);
@@ -576,19 +582,18 @@ cudaError_t launch_conv_tc_t(const RefineConvArgs& a, cudaStream_t s) {
                           : encode_rgba(enc, &tmap, src, a.n, a.H, a.W, kCHW, kCHH)))
     return cudaErrorInvalidValue;
   const int grid = n_tiles < sms * kCPerSM ? n_tiles : sms * kCPerSM;
-  conv_tc_kernel<IN, COUT, EPI><<<grid, kCThreads, smem, s>>>(a, tmap);
-  return cudaGetLastError();
+  return launch_kernel(conv_tc_kernel<IN, COUT, EPI>, dim3(grid), dim3(kCThreads), smem, s, pdl, a, tmap);
 }
 
 }  // namespace
 
-cudaError_t launch_refine_conv(int in_mode, int cout, int epi, const RefineConvArgs& a, cudaStream_t s) {
-  if (in_mode == kConvInRGBA && cout == 32 && epi == kEpiRelu) return launch_conv_tc_t<kConvInRGBA, 32, kEpiRelu>(a, s);
-  if (in_mode == kConvInRGBA && cout == 32 && epi == kEpiMask) return launch_conv_tc_t<kConvInRGBA, 32, kEpiMask>(a, s);
-  if (in_mode == kConvInBF16 && cout == 32 && epi == kEpiRelu) return launch_conv_tc_t<kConvInBF16, 32, kEpiRelu>(a, s);
-  if (in_mode == kConvInBF16 && cout == 32 && epi == kEpiMask) return launch_conv_tc_t<kConvInBF16, 32, kEpiMask>(a, s);
-  if (in_mode == kConvInBF16 && cout == 8 && epi == kEpiResid) return launch_conv_tc_t<kConvInBF16, 8, kEpiResid>(a, s);
-  if (in_mode == kConvInBF16 && cout == 8 && epi == kEpiLoss) return launch_conv_tc_t<kConvInBF16, 8, kEpiLoss>(a, s);
+cudaError_t launch_refine_conv(int in_mode, int cout, int epi, const RefineConvArgs& a, cudaStream_t s, bool pdl) {
+  if (in_mode == kConvInRGBA && cout == 32 && epi == kEpiRelu) return launch_conv_tc_t<kConvInRGBA, 32, kEpiRelu>(a, s, pdl);
+  if (in_mode == kConvInRGBA && cout == 32 && epi == kEpiMask) return launch_conv_tc_t<kConvInRGBA, 32, kEpiMask>(a, s, pdl);
+  if (in_mode == kConvInBF16 && cout == 32 && epi == kEpiRelu) return launch_conv_tc_t<kConvInBF16, 32, kEpiRelu>(a, s, pdl);
+  if (in_mode == kConvInBF16 && cout == 32 && epi == kEpiMask) return launch_conv_tc_t<kConvInBF16, 32, kEpiMask>(a, s, pdl);
+  if (in_mode == kConvInBF16 && cout == 8 && epi == kEpiResid) return launch_conv_tc_t<kConvInBF16, 8, kEpiResid>(a, s, pdl);
+  if (in_mode == kConvInBF16 && cout == 8 && epi == kEpiLoss) return launch_conv_tc_t<kConvInBF16, 8, kEpiLoss>(a, s, pdl);
   return cudaErrorInvalidValue;
 }
 
@@ -704,6 +709,8 @@ __global__ void __launch_bounds__(kGThreads) wgrad_tc_kernel(RefineWgradArgs A, 
   __syncthreads();
   asm volatile("tcgen05.fence::after_thread_sync;" ::: "memory");
   const uint32_t tmem = *tslot;
+  griddep_release();  // every CTA holds its tensor memory (see conv_tc_kernel)
+  griddep_wait();     // the maps are written by the kernels before
   const int n_own = (int)blockIdx.x < n_tiles ? (n_tiles - blockIdx.x + gridDim.x - 1) / gridDim.x : 0;
 
   // A wait for use j of stage j % kStages; on give-up sets the error bit and the CTA's abort flag.
@@ -870,8 +877,7 @@ cudaError_t launch_wgrad_tc_t(const RefineWgradArgs& a, cudaStream_t s) {
                   (MODE == 3 ? encode_rgba(enc, &gm, a.g_f, a.n, a.H, a.W, S::FW, S::FH)
                              : encode_map32(enc, &gm, a.g_h, a.n, a.H, a.W, S::GW, kGTH));
   if (!ok) return cudaErrorInvalidValue;
-  wgrad_tc_kernel<MODE><<<a.n_ctas, kGThreads, S::kSmem, s>>>(a, am, gm);
-  return cudaGetLastError();
+  return launch_kernel(wgrad_tc_kernel<MODE>, dim3(a.n_ctas), dim3(kGThreads), S::kSmem, s, true, a, am, gm);
 }
 
 }  // namespace
