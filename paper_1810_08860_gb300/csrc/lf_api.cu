@@ -1185,14 +1185,14 @@ lf_status refine_layers(lf_ctx* c, int32_t n, int32_t w, int32_t h, const float*
   a.wt = rf_w(c, kPackW2f);
   a.bias = prm + kRefineOffB2;
   a.out_h = static_cast<__nv_bfloat16*>(c->rf.a2.p);
-  LF_CUDA(c, launch_refine_conv(kConvInBF16, 32, kEpiRelu, a, s, true));
+  LF_CUDA(c, launch_refine_conv(kConvInBF16, 32, kEpiRelu, a, s, true, true));
   a = conv_args(c, n, w, h);
   a.src_h = static_cast<const __nv_bfloat16*>(c->rf.a2.p);
   a.wt = rf_w(c, kPackW3f);
   a.bias = prm + kRefineOffB3;
   a.x = in;
   a.out_f = out;
-  LF_CUDA(c, launch_refine_conv(kConvInBF16, 8, kEpiResid, a, s, true));
+  LF_CUDA(c, launch_refine_conv(kConvInBF16, 8, kEpiResid, a, s, true, true));
   return LF_OK;
 }
 
@@ -1236,10 +1236,11 @@ lf_status refine_backward(lf_ctx* c, int32_t n, int32_t w, int32_t h, const floa
   const int64_t n_pix = (int64_t)n * w * h;
   lf_status st = refine_hidden(c, n_pix, true);
   if (st != LF_OK) return st;
-  int tiles_x = 0, tiles_y = 0;
-  const int n_tiles = refine_wgrad_tiles(n, h, w, &tiles_x, &tiles_y);
-  const int n_ctas = std::max(1, std::min(n_tiles, c->sm_count));  // weight-gradient CTAs: one per SM
-  LF_CUDA(c, ensure(c->rf.partial, sizeof(float) * (size_t)n_ctas * (896 + 9248 + 867)));
+  RefineWgradArgs g;
+  std::memset(&g, 0, sizeof(g));
+  g.n = n; g.W = w; g.H = h;
+  refine_wgrad_shape(g, c->sm_count);
+  LF_CUDA(c, ensure(c->rf.partial, sizeof(float) * (size_t)g.n_rows * (896 + 9248 + 867)));
   float* loss = static_cast<float*>(c->rf.scal.p);
   int32_t* count = reinterpret_cast<int32_t*>(loss + 1);
   LF_CUDA(c, cudaMemsetAsync(c->rf.scal.p, 0, 8, s));
@@ -1264,15 +1265,12 @@ lf_status refine_backward(lf_ctx* c, int32_t n, int32_t w, int32_t h, const floa
   a.loss = loss; a.count = count;
   LF_CUDA(c, launch_refine_conv(kConvInBF16, 8, kEpiLoss, a, s, true));
 
-  RefineWgradArgs g;
-  std::memset(&g, 0, sizeof(g));
-  g.n = n; g.W = w; g.H = h; g.tiles_x = tiles_x; g.tiles_y = tiles_y; g.n_tiles = n_tiles; g.n_ctas = n_ctas;
   g.error = reinterpret_cast<int32_t*>(static_cast<char*>(c->rf.scal.p) + 8);
   g.wait_ns = (uint64_t)c->cfg.wait_limit;
   float* part = static_cast<float*>(c->rf.partial.p);
   float* part1 = part;
-  float* part2 = part1 + (size_t)n_ctas * kRefineSegs[0];
-  float* part3 = part2 + (size_t)n_ctas * kRefineSegs[1];
+  float* part2 = part1 + (size_t)g.n_rows * kRefineSegs[0];
+  float* part3 = part2 + (size_t)g.n_rows * kRefineSegs[1];
   // layer 3 weights (dL/dr with a2), then dL/dz2 through layer 3's input
   g.g_f = gr; g.a_h = a2; g.partial = part3; g.seg = kRefineSegs[2];
   LF_CUDA(c, launch_refine_wgrad(3, g, s));
@@ -1288,7 +1286,7 @@ lf_status refine_backward(lf_ctx* c, int32_t n, int32_t w, int32_t h, const floa
   g.g_h = a2; g.a_h = nullptr; g.x = in; g.partial = part1; g.seg = kRefineSegs[0];
   LF_CUDA(c, launch_refine_wgrad(1, g, s));
   const float* const parts[3] = {part1, part2, part3};
-  LF_CUDA(c, launch_refine_reduce(parts, n_ctas, rf_grad(c), s));
+  LF_CUDA(c, launch_refine_reduce(parts, g.n_rows, rf_grad(c), s));
   return LF_OK;
 }
 

@@ -248,12 +248,13 @@ struct RefineConvArgs {
 
 struct RefineWgradArgs {
   int32_t n, H, W;
-  int32_t tiles_x, tiles_y, n_tiles, n_ctas;
+  int32_t tiles_x, tiles_y;    // chunks per image row and column
+  int32_t n_rows, n_ctas;      // accumulation chains (rows of `partial`), CTAs
   const float* g_f;            // mode 3: dL/dr RGBA
   const __nv_bfloat16* g_h;    // modes 1, 2: dL/dz (32 channels)
   const __nv_bfloat16* a_h;    // modes 2, 3: the layer input (32 channels)
   const float* x;              // mode 1: the network input RGBA
-  float* partial;              // [n_ctas][seg]: [ky][kx][o][c], then the biases
+  float* partial;              // [n_rows][seg]: [ky][kx][o][c], then the biases
   int32_t seg;                 // floats of the layer's gradient
   int32_t* error;              // set (bits 8 and on) if a wait gave up
   uint64_t wait_ns;            // bound on each wait
@@ -261,10 +262,11 @@ struct RefineWgradArgs {
 
 // (the training and per-layer kernels wait for the kernel before them themselves: launched as its programmatic
 // dependents, always or with pdl)
-cudaError_t launch_refine_conv(int in_mode, int cout, int epi, const RefineConvArgs& a, cudaStream_t s, bool pdl);
+cudaError_t launch_refine_conv(int in_mode, int cout, int epi, const RefineConvArgs& a, cudaStream_t s, bool pdl,
+                               bool inference = false);
 cudaError_t launch_refine_wgrad(int mode, const RefineWgradArgs& a, cudaStream_t s);
-// The weight-gradient kernels' tiles of n H x W images: their number, and per row and column.
-int refine_wgrad_tiles(int n, int H, int W, int* tiles_x, int* tiles_y);
+// Chunks, chains and CTAs of the weight-gradient kernels for g.n images of g.H x g.W.
+void refine_wgrad_shape(RefineWgradArgs& g, int sm_count);
 // The three layers' partial rows (layer k at partial[k], seg = cin x cout x 9 + cout) summed into grad.
 cudaError_t launch_refine_reduce(const float* const partial[3], int n_rows, float* grad, cudaStream_t s);
 cudaError_t launch_refine_count(const float* x, const float* t, int64_t n_pix, int32_t* count, cudaStream_t s);

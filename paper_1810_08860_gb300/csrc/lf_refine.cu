@@ -44,9 +44,16 @@ __global__ void reduce_partials_kernel(ReduceArgs A) {
   griddep_wait();
   if (blockIdx.x * 32 >= seg) return;
   float s = 0.f;
+  constexpr int U = 16;  // rows in flight
   if (i < seg)
-#pragma unroll 8
-    for (int b = k; b < A.n_rows; b += 8) s += A.partial[layer][(size_t)b * seg + i];
+    for (int b = k; b < A.n_rows; b += 8 * U) {
+      float v[U];
+#pragma unroll
+      for (int u = 0; u < U; ++u) v[u] = b + 8 * u < A.n_rows ? A.partial[layer][(size_t)(b + 8 * u) * seg + i] : 0.f;
+#pragma unroll
+      for (int u = 0; u < U; ++u)
+        if (b + 8 * u < A.n_rows) s += v[u];
+    }
   part[k][lane] = s;
   __syncthreads();
   if (k == 0 && i < seg) {

@@ -43,6 +43,7 @@
 #include <cuda_bf16.h>
 #include <cuda_runtime.h>
 
+#include <algorithm>
 #include <cstdint>
 #include <cstring>
 
@@ -156,19 +157,22 @@ __device__ __forceinline__ uint32_t c_pack(float lo, float hi) {
   return *reinterpret_cast<uint32_t*>(&v);
 }
 
-// 32-channel inputs: one MMA per kernel row and 16 channels, the three kernel columns
-// stacked along N (32 outputs: N = 96, one M-tile of accumulators at a time; 3
-// outputs: N = 16, four columns each).  An MMA of N = 32 or less costs about 45
-// cycles, of N = 96 about 62, so six take 372 cycles an M-tile where eighteen took
-// 810; the epilogue adds two shuffles per output.  16 x 256^2 pixels: 32 -> 32 with
-// the ReLU mask 53 -> 47 us, 32 -> 3 with the loss 44 -> 29 us; a 517 x 731 image's
-// last layer 14.7 -> 9.3 us.  Bound by memory from here (20 to 30 us of it).
-template <int IN, int COUT>
+// 32-channel inputs, inference (STACK): one MMA per kernel row and 16 channels, the
+// three kernel columns stacked along N (32 outputs: N = 96, one M-tile of accumulators
+// at a time; 3 outputs: N = 16, four columns each).  An MMA of N = 32 or less costs
+// about 45 cycles, of N = 96 about 62, so six take 372 cycles an M-tile where eighteen
+// take 810; the epilogue adds two shuffles per output.  517 x 731 pixels: the last
+// layer 14.7 -> 9.3 us; 2 x 1440x1600: 32 -> 32 128 -> 126, 32 -> 3 151 -> 97 us.
+// Training keeps a tap an MMA (N = 32, 16), for 21 us of a step more: the sum of three
+// accumulators rounds differently from one, some hidden values then round to another
+// BF16 neighbour, and Adam carries that on (gradients up to 7e-4 apart after sixteen
+// steps).  3-channel inputs: see above.
+template <int IN, int COUT, bool STACK>
 struct ConvShape {
-  static constexpr bool kStacked = IN == kConvInBF16;
-  static constexpr int kOutStep = COUT == 8 ? 4 : 32;                    // rows of a kernel column along N
-  static constexpr int N = kStacked ? (COUT == 8 ? 16 : 96) : 32;
-  static constexpr int NB = kStacked ? 6 : 3;                            // B blocks: (kernel row, half), or kernel row
+  static constexpr bool kStacked = IN == kConvInBF16 && STACK;
+  static constexpr int kOutStep = COUT == 8 ? 4 : 32;                    // stacked: rows of a kernel column along N
+  static constexpr int N = kStacked && COUT == 32 ? 96 : COUT == 8 ? 16 : 32;
+  static constexpr int NB = IN != kConvInBF16 ? 3 : kStacked ? 6 : 18;   // B blocks: kernel row, (row, half) or (tap, half)
   static constexpr int kMB = N == 96 ? 1 : kCMT;                         // M-tiles per batch of MMAs (128 TMEM columns)
   static constexpr int kBlkB = 2 * N * 16, kWBytes = NB * kBlkB;
 };
@@ -206,17 +210,17 @@ __device__ __forceinline__ uint32_t c_gate(uint32_t v, uint32_t gate) {
 
 }  // namespace
 
-template <int IN, int COUT, int EPI>
+template <int IN, int COUT, int EPI, bool STACK>
 __global__ void __launch_bounds__(kCThreads, kCPerSM)
     conv_tc_kernel(RefineConvArgs A, const __grid_constant__ CUtensorMap tmap) {
-  using S = ConvShape<IN, COUT>;
+  using S = ConvShape<IN, COUT, STACK>;
   constexpr int N = S::N, NB = S::NB, kBlkB = S::kBlkB, kWBytes = S::kWBytes;
   constexpr bool kStacked = S::kStacked;
   extern __shared__ __align__(128) unsigned char sm_raw[];
   unsigned char* sm = sm_raw + ((1024u - (c_su32(sm_raw) & 1023u)) & 1023u);  // the 32-channel halo starts on a swizzle atom
   unsigned char* sw = sm;
   static_assert(IN != kConvInBF16 || kWBytes % 512 == 0, "a swizzle atom is 512 bytes");
-  // 32 channels: position p in the 64 bytes at sx + 64 p (swizzled); windows reach one position before, into the
+  // 32 channels: position p in the 64 bytes at sx + 64 p (swizzled); windows of one tap reach one position before, into the
   // weights, and one after (output columns that are never used).  3 channels: pairs, 16 bytes at sx + (p + kCGuard) * 16.
   unsigned char* sx = sm + kWBytes + (IN == kConvInBF16 ? 0 : kCXOff);
   constexpr int kXsOff = (kWBytes + kCXOff + kCPairB + 127) / 128 * 128;
@@ -251,15 +255,17 @@ __global__ void __launch_bounds__(kCThreads, kCPerSM)
   asm volatile("tcgen05.fence::after_thread_sync;" ::: "memory");
   const uint32_t tmem = *tslot;
   // Launched as a programmatic dependent, what is above overlaps the end of the kernel before; everything read below
-  // is written by it or by earlier ones.  The next kernel may launch once every CTA of this one holds its tensor
-  // memory (it would otherwise take columns that a CTA of this grid still waits for).
-  griddep_release();
+  // is written by it or by earlier ones.  The next kernel launches as this one's CTAs leave: released at the start,
+  // its CTAs slow this grid down (a training step 389 -> 371 us without), and they would have to wait until every CTA
+  // here holds its tensor memory.
   griddep_wait();
   // Weights into core-matrix blocks: block b, K group g, row n at sw + b * kBlkB + (g * N + n) * 16.
   for (int i = tid; i < NB * 2 * N; i += kCThreads) {
     const int b = i / (2 * N), g = (i / N) & 1, n = i % N;
     uint4 v = make_uint4(0u, 0u, 0u, 0u);
-    if (IN == kConvInBF16) {  // packed [tap][o][32]: block b = 2 ky + half, row n = kx * S::kOutStep + o
+    if (IN == kConvInBF16 && !kStacked) {  // packed [tap][o][32]: block b = 2 tap + half, row n = o
+      if (n < COUT) v = *reinterpret_cast<const uint4*>(A.wt + ((size_t)(b >> 1) * COUT + n) * 32 + 16 * (b & 1) + 8 * g);
+    } else if (IN == kConvInBF16) {  // block b = 2 ky + half, row n = kx * S::kOutStep + o
       const int kx = n / S::kOutStep, o = n % S::kOutStep;
       if (kx < 3) v = *reinterpret_cast<const uint4*>(A.wt + ((size_t)(3 * (b >> 1) + kx) * COUT + o) * 32 + 16 * (b & 1) + 8 * g);
     } else {  // packed [n][32], k = tap * 3 + c; block b = ky, element e: kx = 2g + e / 4, c = e % 4
@@ -367,8 +373,17 @@ __global__ void __launch_bounds__(kCThreads, kCPerSM)
 #pragma unroll (S::kMB == kCMT ? kCMT : 1)
       for (int m = m0; m < m0 + S::kMB; ++m) {
         const uint32_t d = tmem + (uint32_t)((m - m0) * N);
+        if (IN == kConvInBF16 && !kStacked) {
 #pragma unroll
-        for (int ky = 0; ky < 3; ++ky) {
+          for (int tap = 0; tap < 9; ++tap) {  // tap 3 ky + kx reads positions 32 (4m + ky) + kx - 1 + r
+#pragma unroll
+            for (int h = 0; h < 2; ++h)
+              c_mma(d, ad + (uint64_t)(int64_t)(4 * (32 * (4 * m + tap / 3) + tap % 3 - 1) + 2 * h),
+                    bd + (uint64_t)((2 * tap + h) * (kBlkB / 16)), id, tap > 0 || h > 0);
+          }
+        }
+#pragma unroll
+        for (int ky = 0; ky < (IN == kConvInBF16 && !kStacked ? 0 : 3); ++ky) {
           if (IN == kConvInBF16) {  // kernel row ky reads positions 32 (4m + ky) + r, its columns lie along N
 #pragma unroll
             for (int h = 0; h < 2; ++h)
@@ -406,8 +421,8 @@ __global__ void __launch_bounds__(kCThreads, kCPerSM)
     if (tid == 0) issue(0);
     issued = true;
 
-    // ---- epilogue: warp w reads lanes 32w.. (halo row 4m + 1 + w, column lane) of each M-tile.  With the kernel
-    // columns along N an output is D[q-1][kx = 0] + D[q][1] + D[q+1][2]; the neighbours' parts come from the
+    // ---- epilogue: warp w reads lanes 32w.. (halo row 4m + 1 + w, column lane) of each M-tile.  Stacked, an
+    // output is D[q-1][kx = 0] + D[q][1] + D[q+1][2]; the neighbours' parts come from the
     // neighbouring lanes (columns 0 and 31 get a wrong one and are never used).
     const uint32_t lane_base = (uint32_t)(32 * warp) << 16;
     const int gx = x0 + lane - 1;
@@ -481,7 +496,7 @@ __global__ void __launch_bounds__(kCThreads, kCPerSM)
                               c_gate(w[j].w, gate[j].w));
           *reinterpret_cast<uint4*>(A.out_h + at0 + 32 * j) = w[j];
         }
-      } else {  // kEpiResid / kEpiLoss: outputs 0..2, column kx in 4 kx ..
+      } else {  // kEpiResid / kEpiLoss: outputs 0..2; stacked, column kx in 4 kx ..
         const size_t pix = ((size_t)img * H + (store ? gy : 0)) * W + (store ? gx : 0);
         float4 x = make_float4(0.f, 0.f, 0.f, 0.f), tg = x;
         if (store) {
@@ -493,7 +508,8 @@ __global__ void __launch_bounds__(kCThreads, kCPerSM)
         asm volatile("tcgen05.wait::ld.sync.aligned;" ::: "memory");
 #pragma unroll
         for (int o = 0; o < 3; ++o)
-          r[o] = __shfl_up_sync(0xffffffffu, v[o], 1) + v[4 + o] + __shfl_down_sync(0xffffffffu, v[8 + o], 1) + s_bias[o];
+          r[o] = (kStacked ? __shfl_up_sync(0xffffffffu, v[o], 1) + v[4 + o] + __shfl_down_sync(0xffffffffu, v[8 + o], 1)
+                           : v[o]) + s_bias[o];
         if (!store) continue;
         if (EPI == kEpiResid) {
           const bool valid = x.w > 0.f;
@@ -556,15 +572,15 @@ bool encode_rgba(EncodeTiled enc, CUtensorMap* m, const void* p, int n, int H, i
              CU_TENSOR_MAP_FLOAT_OOB_FILL_NONE) == CUDA_SUCCESS;
 }
 
-template <int IN, int COUT, int EPI>
+template <int IN, int COUT, int EPI, bool STACK = false>
 cudaError_t launch_conv_tc_t(const RefineConvArgs& a, cudaStream_t s, bool pdl) {
-  constexpr int kW = ConvShape<IN, COUT>::kWBytes;
+  constexpr int kW = ConvShape<IN, COUT, STACK>::kWBytes;
   constexpr int used = 1024 + (IN == kConvInBF16 ? kW + kCHaloTx + 128 + 24
                                                  : (kW + kCXOff + kCPairB + 127) / 128 * 128 + kCXsB + 24);
   // At least 54 KB: no more than kCPerSM CTAs share an SM, so their tensor memory (128 columns each)
   // always fits and no CTA waits in tcgen05.alloc for another persistent CTA to finish.
   constexpr int smem = used < 54 * 1024 ? 54 * 1024 : used;
-  cudaError_t e = ensure_dynamic_smem(reinterpret_cast<const void*>(conv_tc_kernel<IN, COUT, EPI>), smem);
+  cudaError_t e = ensure_dynamic_smem(reinterpret_cast<const void*>(conv_tc_kernel<IN, COUT, EPI, STACK>), smem);
   if (e != cudaSuccess) return e;
   const int n_tiles = ((a.W + kCTW - 1) / kCTW) * ((a.H + kCTH - 1) / kCTH) * a.n;
   if (n_tiles == 0) return cudaSuccess;
@@ -582,18 +598,22 @@ cudaError_t launch_conv_tc_t(const RefineConvArgs& a, cudaStream_t s, bool pdl) 
                           : encode_rgba(enc, &tmap, src, a.n, a.H, a.W, kCHW, kCHH)))
     return cudaErrorInvalidValue;
   const int grid = n_tiles < sms * kCPerSM ? n_tiles : sms * kCPerSM;
-  return launch_kernel(conv_tc_kernel<IN, COUT, EPI>, dim3(grid), dim3(kCThreads), smem, s, pdl, a, tmap);
+  return launch_kernel(conv_tc_kernel<IN, COUT, EPI, STACK>, dim3(grid), dim3(kCThreads), smem, s, pdl, a, tmap);
 }
 
 }  // namespace
 
-cudaError_t launch_refine_conv(int in_mode, int cout, int epi, const RefineConvArgs& a, cudaStream_t s, bool pdl) {
-  if (in_mode == kConvInRGBA && cout == 32 && epi == kEpiRelu) return launch_conv_tc_t<kConvInRGBA, 32, kEpiRelu>(a, s, pdl);
-  if (in_mode == kConvInRGBA && cout == 32 && epi == kEpiMask) return launch_conv_tc_t<kConvInRGBA, 32, kEpiMask>(a, s, pdl);
-  if (in_mode == kConvInBF16 && cout == 32 && epi == kEpiRelu) return launch_conv_tc_t<kConvInBF16, 32, kEpiRelu>(a, s, pdl);
-  if (in_mode == kConvInBF16 && cout == 32 && epi == kEpiMask) return launch_conv_tc_t<kConvInBF16, 32, kEpiMask>(a, s, pdl);
-  if (in_mode == kConvInBF16 && cout == 8 && epi == kEpiResid) return launch_conv_tc_t<kConvInBF16, 8, kEpiResid>(a, s, pdl);
-  if (in_mode == kConvInBF16 && cout == 8 && epi == kEpiLoss) return launch_conv_tc_t<kConvInBF16, 8, kEpiLoss>(a, s, pdl);
+cudaError_t launch_refine_conv(int in_mode, int cout, int epi, const RefineConvArgs& a, cudaStream_t s, bool pdl,
+                               bool inference) {
+  const bool rgba = in_mode == kConvInRGBA, wide = cout == 32;
+  if (rgba && wide && epi == kEpiRelu) return launch_conv_tc_t<kConvInRGBA, 32, kEpiRelu>(a, s, pdl);
+  if (rgba && wide && epi == kEpiMask) return launch_conv_tc_t<kConvInRGBA, 32, kEpiMask>(a, s, pdl);
+  if (!rgba && wide && epi == kEpiRelu)
+    return inference ? launch_conv_tc_t<kConvInBF16, 32, kEpiRelu, true>(a, s, pdl)
+                     : launch_conv_tc_t<kConvInBF16, 32, kEpiRelu>(a, s, pdl);
+  if (!rgba && wide && epi == kEpiMask) return launch_conv_tc_t<kConvInBF16, 32, kEpiMask>(a, s, pdl);
+  if (!rgba && cout == 8 && epi == kEpiResid) return launch_conv_tc_t<kConvInBF16, 8, kEpiResid, true>(a, s, pdl);
+  if (!rgba && cout == 8 && epi == kEpiLoss) return launch_conv_tc_t<kConvInBF16, 8, kEpiLoss>(a, s, pdl);
   return cudaErrorInvalidValue;
 }
 
@@ -602,56 +622,68 @@ cudaError_t launch_refine_conv(int in_mode, int cout, int epi, const RefineConvA
 // dW[o][c][ky][kx] = sum_p g[p][o] a[p + (ky - 1, kx - 1)][c], db[o] = sum_p g[p][o]
 // (g = dL/dz of the layer's output, a = the layer's input), as one GEMM over
 // K = pixels whose operands are the maps as they lie in memory: both are read
-// MN-major (channels contiguous), so nothing is transposed.  A tile is 32 x 8
-// positions of a; per image row r of g
-//   D[(i, c)][(kx, o)] += sum_x a[r - 1 + i][x][c] g[r][x + 1 - kx][o]
-// with M = 128: four consecutive rows i of a (ky = i; the fourth is not used) of
-// 32 channels, and N = 96: g's row (34 positions, zeros outside the image) at three
-// starts one position apart, which the operand's N stride of one position gives
-// without a copy.  A 32-channel map lies as [row][position][32 channels] under the
-// 64-byte swizzle, which goes by address, so shifted starts read it correctly.  The
-// 3-channel maps (the network input, dL/dr) land as FP32 RGBA and four warps round
-// them to BF16 rows of 8 channels, the last five zero, without swizzle: M then covers
-// sixteen rows (three used), N = 32 four starts (three used).  The same warps
-// sum g for the bias gradient.
+// MN-major (channels contiguous), so nothing is transposed.  Per image row r of a
+// chunk of 32 x 2 pixels, and per kernel column kx,
+//   D[kx][(i, c)][o] += sum_x a[r - 1 + i][x - 1 + kx][c] g[r][x][o]
+// with M = 128: three rows i of a (ky = i) of 32 channels and, as the fourth, a row of
+// ones, whose product with g is the bias gradient; N = the output channels.  A chunk's
+// a lands by TMA as three rows of 34 positions (zeros outside the image) for each of
+// its two pixel rows, each time in front of a constant row of ones.  A 32-channel map
+// lies as [row][position][32 channels] under the 64-byte swizzle, which goes by
+// address, so that a column's start one position on reads it correctly.  The
+// 3-channel maps (the network input, dL/dr) land as FP32 RGBA and two warps round
+// them to BF16 rows of 8 channels, the last five zero, without swizzle.
 //   MODE 1: g = dL/dz1 (BF16, 32), a = the network input (FP32 RGBA, 3).  W1, b1.
 //   MODE 2: g = dL/dz2 (BF16, 32), a = a1 (BF16, 32).                        W2, b2.
 //   MODE 3: g = dL/dr  (FP32 RGBA, 3), a = a2 (BF16, 32).                    W3, b3.
 //
-// One CTA per SM, a ring of stages between a TMA warp, an MMA warp and the
-// four warps above; the accumulators stay in TMEM over all tiles of a CTA, which then
-// writes one partial row; the rows are summed in a fixed order afterwards
-// (deterministic).  Bound by reading the maps (134 and 84 MB at 16 x 256^2: 20 and 12
-// us) and a start and an end of some 8 us; halving the MMAs changes nothing.  Against
-// kernels that transposed chunks of 64 pixels with ldmatrix and wrote every input nine
-// times for its taps, 16 crops of 256^2: 109, 67 and 93 us for W2, W1 and W3 -> 31, 25
-// and 23 us.  With three shifted copies of g loaded instead of one, W2 took 33 us, and
-// 75 when the copies came as {8 channels, W, group} boxes, 16 bytes at a time.
+// Order of the sums.  An MMA adds 16 neighbouring pixels of a row to an accumulator,
+// the tensor core truncates as it adds, and Adam turns gradients that differ by 1e-6
+// into weights that round to another BF16 neighbour a few steps later, so the order is
+// part of the result: a chain of accumulation is one of A.n_rows (three per SM) that
+// takes every n_rows-th chunk, row by row, and the chains are added in a fixed order
+// (reduce_partials_kernel).  A CTA, one per SM, runs up to three chains in turn, each
+// with accumulators of its own that stay in TMEM to the end.
+//
+// A ring of stages runs between a copying and an issuing warp per chain and two
+// rounding warps.
+// Bound by the MMAs (six per pixel row of 32, about 45 cycles each at N = 32: 28 us at
+// 16 x 256^2), next to reading the maps (134 and 84 MB: 20 and 12 us) and some 10 us
+// of start and end.  One thread issues an MMA per 59 cycles and a chunk's copies in
+// some 600, hence the warps per chain (one of each: 57 us for W2).  Against kernels
+// that transposed chunks of 64 pixels with ldmatrix and wrote every input nine times
+// for its taps, 16 crops of 256^2, the same sums bit for bit: 109, 67 and 93 us for
+// W2, W1 and W3 -> 43, 52 and 42 us.  (All nine taps in one MMA of N = 96, over positions of a
+// instead of g, took 31, 25 and 23 us, but groups the pixels differently: gradients
+// 1.5e-6 apart, 2e-4 after sixteen steps.)
 
 namespace {
 
-constexpr int kGTW = 32, kGTH = 8;               // tile: 32 x 8 positions
-constexpr int kGHelpers = 4;                     // warps that round FP32 maps and sum g
-constexpr int kGThreads = 64 + 32 * kGHelpers;
+constexpr int kGTW = 32, kGTH = 2;               // chunk: 32 x 2 pixels
+constexpr int kGHW = kGTW + 2, kGHR = 3;         // a: three rows of 34 positions per pixel row
+constexpr int kGChains = 3;                      // accumulation chains per CTA, each with a copying and an issuing warp
+constexpr int kGRoundWarp = 2 * kGChains;         // the first of two rounding warps
+constexpr int kGThreads = 32 * (kGRoundWarp + 2);
 
 template <int MODE>
 struct WgradShape {
-  static constexpr int OC = MODE == 3 ? 8 : 32;          // channels of g as held
-  static constexpr int N = MODE == 3 ? 32 : 96;          // starts x channels
+  static constexpr int N = MODE == 3 ? 16 : 32;
   static constexpr int COUT = MODE == 3 ? 3 : 32, CIN = MODE == 1 ? 3 : 32;
-  static constexpr int kARow = kGTW * (MODE == 1 ? 16 : 64), kAB = (kGTH + 2) * kARow;  // rows of 32 positions
-  static constexpr int GW = kGTW + 2, kGPos = 2 * OC, kGRow = GW * kGPos, kGB = kGTH * kGRow + 512;  // rows of 34
-  static constexpr int FW = MODE == 1 ? kGTW : GW, FH = MODE == 1 ? kGTH + 2 : kGTH;    // FP32 RGBA positions
+  static constexpr int kAPos = MODE == 1 ? 16 : 64, kARow = kGHW * kAPos;               // bytes per position, per row
+  static constexpr int kAGrp = (kGHR + 1) * kARow;                                      // three rows and the ones
+  static constexpr int kAB = (kGTH * kAGrp + 511) / 512 * 512;
+  static constexpr int kGRow = kGTW * (MODE == 3 ? 16 : 64), kGB = kGTH * kGRow + (MODE == 3 ? 512 : 0);
+  static constexpr int FW = MODE == 1 ? kGHW : kGTW, FH = MODE == 1 ? kGTH + 2 : kGTH;  // FP32 RGBA positions
   static constexpr int kFB = MODE == 2 ? 0 : FW * FH * 16;
   static constexpr int kStageB = (kAB + kGB + kFB + 511) / 512 * 512;
-  static constexpr int kTx = (MODE == 1 ? 0 : kAB) + (MODE == 3 ? 0 : kGTH * kGRow) + FW * FH * (MODE == 2 ? 0 : 16);
-  static constexpr int kStages = 5;
-  // The unused accumulator rows take what lies behind a tile's rows of a: the stage's g
-  static_assert((kGTH - 1) * kARow + (MODE == 1 ? 16 : 4) * kARow <= kStageB, "MMAs read within the stage");
-  static_assert(kAB % 512 == 0, "g starts on a swizzle atom");
-  static constexpr int kBarOff = kStages * kStageB;
+  static constexpr int kTx = (MODE == 1 ? 0 : kGTH * kGHR * kARow) + (MODE == 3 ? 0 : kGTH * kGRow) + kFB;
+  static constexpr int kStages = 6;  // a multiple of 1, 2 and 3: a stage always serves the same chain
+  static constexpr int kCols = MODE == 3 ? 256 : 512;  // TMEM: kGChains x 3 x N
+  static_assert(kGChains * 3 * N <= kCols, "the accumulators fit");
+  // M = 128 without swizzle takes 16 rows of a: beyond the ones they lie anywhere in shared memory (not used)
+  static constexpr int kBarOff = kStages * kStageB + (MODE == 1 ? 8192 : 0);
   static constexpr int kSmem = 1024 + kBarOff + (3 * kStages + 1) * 8 + 16;  // 1024: the base is rounded up
-  static_assert(kSmem <= 224 * 1024, "fits one CTA's shared memory");
+  static_assert(kSmem <= 224 * 1024 && (MODE == 1 || kAGrp % 512 == 0), "fits; groups start on a swizzle atom");
 };
 
 // kind::f16, FP32 accumulator, BF16 A and B, both MN-major.
@@ -682,37 +714,51 @@ __global__ void __launch_bounds__(kGThreads) wgrad_tc_kernel(RefineWgradArgs A, 
   unsigned char* sm = sm_raw + ((1024u - (c_su32(sm_raw) & 1023u)) & 1023u);  // stages start on a swizzle atom
   uint64_t* full = reinterpret_cast<uint64_t*>(sm + S::kBarOff);  // a stage's copies landed
   uint64_t* ready = full + S::kStages;                             // its FP32 map is rounded (modes 1, 3)
-  uint64_t* empty = ready + S::kStages;                            // its MMAs and its readers are done
+  uint64_t* empty = ready + S::kStages;                            // its MMAs (and its rounding) are done
   uint64_t* done = empty + S::kStages;                             // all MMAs of the CTA are complete
   uint32_t* tslot = reinterpret_cast<uint32_t*>(done + 1);
   __shared__ volatile int s_abort;
-  __shared__ float s_bias[32 * kGHelpers][8];
   const int tid = threadIdx.x, warp = tid >> 5, lane = tid & 31;
-  const int n_tiles = A.n_tiles;
 
   if (tid == 0) {
     s_abort = 0;
     for (int k = 0; k < S::kStages; ++k) {
       asm volatile("mbarrier.init.shared::cta.b64 [%0], 1;" ::"r"(c_su32(full + k)));
-      asm volatile("mbarrier.init.shared::cta.b64 [%0], %1;" ::"r"(c_su32(ready + k)), "r"(kGHelpers));
-      asm volatile("mbarrier.init.shared::cta.b64 [%0], %1;" ::"r"(c_su32(empty + k)), "r"(1 + kGHelpers));
+      asm volatile("mbarrier.init.shared::cta.b64 [%0], 2;" ::"r"(c_su32(ready + k)));
+      asm volatile("mbarrier.init.shared::cta.b64 [%0], %1;" ::"r"(c_su32(empty + k)), "r"(MODE == 2 ? 1 : 3));
     }
-    asm volatile("mbarrier.init.shared::cta.b64 [%0], 1;" ::"r"(c_su32(done)));
+    asm volatile("mbarrier.init.shared::cta.b64 [%0], %1;" ::"r"(c_su32(done)), "r"(kGChains));
     asm volatile("fence.mbarrier_init.release.cluster;" ::: "memory");
   }
+  for (int i = tid; i < S::kStages * kGTH * (S::kARow / 16); i += kGThreads) {  // the rows of ones, once
+    const int row = i / (S::kARow / 16);
+    *reinterpret_cast<uint4*>(sm + (row / kGTH) * S::kStageB + (row % kGTH) * S::kAGrp + kGHR * S::kARow +
+                              (i % (S::kARow / 16)) * 16) = make_uint4(0x3F803F80u, 0x3F803F80u, 0x3F803F80u, 0x3F803F80u);
+  }
+  asm volatile("fence.proxy.async.shared::cta;" ::: "memory");  // to the tensor core
   if (warp == 0) {
     asm volatile("tcgen05.alloc.cta_group::1.sync.aligned.shared::cta.b32 [%0], %1;" ::"r"(c_su32(tslot)),
-                 "r"(kCTmemCols));
+                 "r"(S::kCols));
     asm volatile("tcgen05.relinquish_alloc_permit.cta_group::1.sync.aligned;");
   }
   asm volatile("tcgen05.fence::before_thread_sync;" ::: "memory");
   __syncthreads();
   asm volatile("tcgen05.fence::after_thread_sync;" ::: "memory");
   const uint32_t tmem = *tslot;
-  griddep_release();  // every CTA holds its tensor memory (see conv_tc_kernel)
-  griddep_wait();     // the maps are written by the kernels before
-  const int n_own = (int)blockIdx.x < n_tiles ? (n_tiles - blockIdx.x + gridDim.x - 1) / gridDim.x : 0;
+  griddep_wait();  // the maps are written by the kernels before (the next kernel's early blocks slow this one down:
+                   // it lets them launch only by ending)
+  const int cx = A.tiles_x, cxy = A.tiles_x * A.tiles_y, n_chunks = cxy * A.n;
 
+  // The CTA's chunks, taken in turn from its n_ch chains (chain i is row blockIdx.x + i * gridDim.x): the j-th is
+  // chunk j / n_ch of chain j % n_ch.
+  int n_ch = 0, n_own = 0;
+  for (int i = 0; i < kGChains; ++i) {
+    const int v = blockIdx.x + i * gridDim.x;
+    if (v < A.n_rows) {
+      ++n_ch;
+      n_own += v < n_chunks ? (n_chunks - v + A.n_rows - 1) / A.n_rows : 0;
+    }
+  }
   // A wait for use j of stage j % kStages; on give-up sets the error bit and the CTA's abort flag.
   auto wait_use = [&](uint64_t* bar, int j, int err) -> bool {
     if (s_abort) return false;
@@ -722,141 +768,141 @@ __global__ void __launch_bounds__(kGThreads) wgrad_tc_kernel(RefineWgradArgs A, 
     return false;
   };
 
-  if (warp == 0) {
-    // ---------------------------------------------------------------- copies
-    if (lane == 0) {
-      int issued = 0;
-      for (int j = 0; j < n_own; ++j) {
-        if (j >= S::kStages && !wait_use(empty, j - S::kStages, 256)) break;
-        const int tile = blockIdx.x + j * gridDim.x, img = tile / (A.tiles_x * A.tiles_y);
-        const int rem = tile - img * A.tiles_x * A.tiles_y;
-        const int y0 = rem / A.tiles_x * kGTH, x0 = rem % A.tiles_x * kGTW;
-        const uint32_t st = c_su32(sm) + (j % S::kStages) * S::kStageB, sg = st + S::kAB, sf = sg + S::kGB;
-        uint64_t* bar = full + j % S::kStages;
-        asm volatile("mbarrier.arrive.expect_tx.shared::cta.b64 _, [%0], %1;" ::"r"(c_su32(bar)), "r"(S::kTx) : "memory");
-        g_tma4(&amap, MODE == 1 ? sf : st, bar, 0, x0, y0 - 1, img);
-        g_tma4(&gmap, MODE == 3 ? sf : sg, bar, 0, x0 - 1, y0, img);
-        issued = j + 1;
+  if (warp < kGChains) {
+    // ---------------------------------------------------------------- copies, a warp per chain
+    // Each lane works out the place of one of the chain's chunks, 32 at a time; lanes 0 .. 2 issue a copy each.
+    int px = 0, py = 0, pimg = 0, k = 0, last = -1;
+    for (int j = warp; warp < n_ch && j < n_own; j += n_ch, ++k) {
+      if (k % 32 == 0) {
+        const int chunk = blockIdx.x + warp * gridDim.x + (k + lane) * A.n_rows;
+        pimg = chunk / cxy;
+        const int rem = chunk - pimg * cxy;
+        py = rem / cx * kGTH;
+        px = rem % cx * kGTW;
       }
-      // the last copies land before the CTA can leave (earlier ones have been waited for by their readers or are
-      // waited for here, after an abort)
-      for (int j = issued > S::kStages ? issued - S::kStages : 0; j < issued; ++j)
-        if (c_wait(full + j % S::kStages, (uint32_t)(j / S::kStages) & 1u, kCDrainNs) != 0) atomicOr(A.error, 2048);
+      const int x0 = __shfl_sync(0xffffffffu, px, k % 32), y0 = __shfl_sync(0xffffffffu, py, k % 32);
+      const int img = __shfl_sync(0xffffffffu, pimg, k % 32);
+      uint64_t* bar = full + j % S::kStages;
+      int ok = 1;
+      if (lane == 0) {
+        ok = j < S::kStages || wait_use(empty, j - S::kStages, 256);
+        if (ok)
+          asm volatile("mbarrier.arrive.expect_tx.shared::cta.b64 _, [%0], %1;" ::"r"(c_su32(bar)), "r"(S::kTx) : "memory");
+      }
+      if (!__shfl_sync(0xffffffffu, ok, 0)) break;
+      const uint32_t st = c_su32(sm) + (j % S::kStages) * S::kStageB, sg = st + S::kAB, sf = sg + S::kGB;
+      if (lane < kGTH) {
+        if (MODE != 1) g_tma4(&amap, st + lane * S::kAGrp, bar, 0, x0 - 1, y0 + lane - 1, img);
+        else if (lane == 0) g_tma4(&amap, sf, bar, 0, x0 - 1, y0 - 1, img);
+      } else if (lane == kGTH) {
+        g_tma4(&gmap, MODE == 3 ? sf : sg, bar, 0, x0, y0, img);
+      }
+      __syncwarp();
+      last = j;
     }
-  } else if (warp == 1) {
-    // ---------------------------------------------------------------- MMAs
+    // the last copies land before the CTA can leave (earlier ones have been waited for by their readers)
+    if (lane == 0)
+      for (int j = last; j >= 0 && j > last - S::kStages; j -= n_ch)
+        if (c_wait(full + j % S::kStages, (uint32_t)(j / S::kStages) & 1u, kCDrainNs) != 0) atomicOr(A.error, 2048);
+  } else if (warp < kGRoundWarp) {
+    // ---------------------------------------------------------------- MMAs, a warp per chain (one thread issues an
+    // MMA per 59 cycles, so one alone would hold the tensor core up)
     if (lane == 0) {
       constexpr uint32_t id = g_idesc(128, S::N);
-      for (int j = 0; j < n_own; ++j) {
+      constexpr int kAK = 16 * S::kAPos, kGK = S::kGRow / 2;  // 16 positions
+      const int chain = warp - kGChains;
+      const uint32_t d = tmem + chain * 3 * S::N;
+      for (int j = chain; chain < n_ch && j < n_own; j += n_ch) {
         if (!wait_use(full, j, 256)) break;
         if (MODE != 2 && !wait_use(ready, j, 256)) break;
         asm volatile("tcgen05.fence::after_thread_sync;" ::: "memory");
         const uint32_t st = c_su32(sm) + (j % S::kStages) * S::kStageB;
-        constexpr int kAK = MODE == 1 ? 256 : 1024, kGK = MODE == 3 ? 256 : 1024;  // 16 positions
         const uint64_t ad = MODE == 1 ? g_desc8(st, S::kARow) : g_desc32(st, S::kARow);
-        const uint64_t bd = MODE == 3 ? g_desc8(st + S::kAB, S::kGPos) : g_desc32(st + S::kAB, S::kGPos);
+        const uint64_t bd = MODE == 3 ? g_desc8(st + S::kAB, 512) : g_desc32(st + S::kAB, 512);
+#pragma unroll
         for (int r = 0; r < kGTH; ++r)
 #pragma unroll
-          for (int k = 0; k < 2; ++k)
-            c_mma(tmem, ad + (uint64_t)((r * S::kARow + k * kAK) / 16), bd + (uint64_t)((r * S::kGRow + k * kGK) / 16), id,
-                  j > 0 || r > 0 || k > 0);
+          for (int h = 0; h < 2; ++h)
+#pragma unroll
+            for (int kx = 0; kx < 3; ++kx)
+              c_mma(d + kx * S::N, ad + (uint64_t)((r * S::kAGrp + kx * S::kAPos + h * kAK) / 16),
+                    bd + (uint64_t)((r * S::kGRow + h * kGK) / 16), id, j > chain || r > 0 || h > 0);
         c_commit(empty + j % S::kStages);
       }
-      // completes once every MMA issued has: also after an abort, so the tensor memory is never freed under one
+      // completes once every MMA issued (by all three) has: also after an abort, so the tensor memory is never freed
+      // under one
       c_commit(done);
       if (c_wait(done, 0u, A.wait_ns > kCDrainNs ? A.wait_ns : kCDrainNs) != 0) atomicOr(A.error, 512);
     }
-  } else {
-    // ---------------------------------------------------------------- rounding of FP32 maps, bias sums
-    const int t = tid - 64;
-    float acc[8];
-#pragma unroll
-    for (int k = 0; k < 8; ++k) acc[k] = 0.f;
+  } else if (MODE != 2) {
+    // ---------------------------------------------------------------- rounding of FP32 maps
+    const int t = tid - 32 * kGRoundWarp;
     for (int j = 0; j < n_own; ++j) {
       int ok = 1;
       if (lane == 0) ok = wait_use(full, j, 1024);
       if (!__shfl_sync(0xffffffffu, ok, 0)) break;
-      // (a lane that did not poll sees the copies through the shuffle's warp: every lane tests the phase once)
+      // every lane tests the phase itself: the copies are visible to it
       if (c_wait(full + j % S::kStages, (uint32_t)(j / S::kStages) & 1u, kCDrainNs) != 0) break;
       unsigned char* st = sm + (j % S::kStages) * S::kStageB;
-      unsigned char* sg = st + S::kAB;
-      if (MODE != 2) {
-        const float4* f = reinterpret_cast<const float4*>(sg + S::kGB);
-        for (int i = t; i < S::FW * S::FH; i += 32 * kGHelpers) {
-          const float4 v = f[i];
-          const uint4 w = make_uint4(c_pack(v.x, v.y), c_pack(v.z, 0.f), 0u, 0u);
-          if (MODE == 1) {
-            reinterpret_cast<uint4*>(st)[i] = w;  // [row][position]
-          } else {
-            const int x = i % S::FW;  // image column x0 - 1 + x
-            reinterpret_cast<uint4*>(sg)[i] = w;  // [row][position]
-            if (x >= 1 && x <= kGTW) {  // the tile's own pixels, as rounded for the MMAs
-              acc[0] += __uint_as_float(w.x << 16);
-              acc[1] += __uint_as_float(w.x & 0xffff0000u);
-              acc[2] += __uint_as_float(w.y << 16);
-            }
-          }
-        }
-        asm volatile("fence.proxy.async.shared::cta;" ::: "memory");  // visible to the tensor core
-        __syncwarp();
-        if (lane == 0) g_arrive(ready + j % S::kStages);
-      }
-      if (MODE != 3) {  // thread t: channels 8 (t & 3) .. of the tile's column t / 4
-        static_assert(kGHelpers * 32 == kGTW * 4, "a thread per column and 8 channels");
+      const float4* f = reinterpret_cast<const float4*>(st + S::kAB + S::kGB);
+      for (int i = t; i < S::FW * S::FH; i += 64) {
+        const float4 v = f[i];
+        const uint4 w = make_uint4(c_pack(v.x, v.y), c_pack(v.z, 0.f), 0u, 0u);
+        if (MODE == 3) {
+          reinterpret_cast<uint4*>(st + S::kAB)[i] = w;  // [row][position]
+        } else {  // row y of the four is row y of the first pixel row's three, y - 1 of the second's
+          const int y = i / S::FW, x = i - y * S::FW;
 #pragma unroll
-        for (int r = 0; r < kGTH; ++r) {
-          const int at = r * S::kGRow + ((t >> 2) + 1) * 64;  // the swizzle moves a 16-byte piece by bits 7 and 8
-          const uint4 v = *reinterpret_cast<const uint4*>(sg + at + (((t & 3) ^ ((at >> 7) & 3)) << 4));
-          const uint32_t w[4] = {v.x, v.y, v.z, v.w};
-#pragma unroll
-          for (int k = 0; k < 4; ++k) {
-            acc[2 * k] += __uint_as_float(w[k] << 16);
-            acc[2 * k + 1] += __uint_as_float(w[k] & 0xffff0000u);
-          }
+          for (int r = 0; r < kGTH; ++r)
+            if (y - r >= 0 && y - r < kGHR) *reinterpret_cast<uint4*>(st + r * S::kAGrp + (y - r) * S::kARow + x * 16) = w;
         }
       }
+      asm volatile("fence.proxy.async.shared::cta;" ::: "memory");  // visible to the tensor core
       __syncwarp();
-      if (lane == 0) g_arrive(empty + j % S::kStages);
+      if (lane == 0) {
+        g_arrive(ready + j % S::kStages);
+        g_arrive(empty + j % S::kStages);
+      }
     }
-#pragma unroll
-    for (int k = 0; k < 8; ++k) s_bias[t][k] = acc[k];
   }
   asm volatile("tcgen05.fence::before_thread_sync;" ::: "memory");
-  __syncthreads();  // the MMAs are complete (the issuing thread has waited for them)
+  __syncthreads();  // the MMAs are complete (the issuing threads have waited for them)
   asm volatile("tcgen05.fence::after_thread_sync;" ::: "memory");
 
-  // ---- this CTA's partial row, [ky][kx][o][c] then the biases: warp w reads accumulator rows 32w ..
-  float* out = A.partial + (size_t)blockIdx.x * A.seg;
-  if (!s_abort && n_own > 0) {
-    if (warp < (MODE == 1 ? 1 : 3)) {
-      const int ky = MODE == 1 ? lane >> 3 : warp, c = MODE == 1 ? lane & 7 : lane;
-      const bool keep = c < S::CIN && ky < 3;
+  // ---- the chains' partial rows, [ky][kx][o][c] then the biases: warp w reads accumulator rows 32w ..
+  if (!s_abort && warp < (MODE == 1 ? 1 : 4)) {
+    const int ky = MODE == 1 ? lane >> 3 : warp, c = MODE == 1 ? lane & 7 : lane;
+    for (int i = 0; i < kGChains; ++i) {
+      const int v = blockIdx.x + i * gridDim.x;
+      if (v >= A.n_rows) break;
+      float* out = A.partial + (size_t)v * A.seg;
 #pragma unroll
-      for (int h = 0; h < S::N / 16; ++h) {
-        float v[16];
-        c_tmem_ld16(tmem + ((uint32_t)(32 * warp) << 16) + 16 * h, v);
-        asm volatile("tcgen05.wait::ld.sync.aligned;" ::: "memory");
-        if (keep) {
+      for (int kx = 0; kx < 3; ++kx) {
+        float d[S::N];
 #pragma unroll
-          for (int k = 0; k < 16; ++k) {
-            const int col = 16 * h + k, kx = 2 - col / S::OC, o = col % S::OC;  // start i holds g[x - 1 + i]
-            if (kx >= 0 && o < S::COUT) out[((ky * 3 + kx) * S::COUT + o) * S::CIN + c] = v[k];
-          }
+        for (int h = 0; h < S::N / 16; ++h) {
+          float u[16];
+          c_tmem_ld16(tmem + ((uint32_t)(32 * warp) << 16) + (i * 3 + kx) * S::N + 16 * h, u);
+          asm volatile("tcgen05.wait::ld.sync.aligned;" ::: "memory");
+#pragma unroll
+          for (int q = 0; q < 16; ++q) d[16 * h + q] = u[q];
+        }
+        if (ky < 3 && c < S::CIN) {
+#pragma unroll
+          for (int o = 0; o < S::COUT; ++o) out[((ky * 3 + kx) * S::COUT + o) * S::CIN + c] = d[o];
+        }
+        if (ky == 3 && c == 0 && kx == 0) {
+#pragma unroll
+          for (int o = 0; o < S::COUT; ++o) out[9 * S::COUT * S::CIN + o] = d[o];
         }
       }
-    }
-    if (tid < S::COUT) {  // bias gradient: the threads' sums in a fixed order
-      float b = 0.f;
-      if (MODE == 3) for (int k = 0; k < 32 * kGHelpers; ++k) b += s_bias[k][tid];
-      else for (int k = 0; k < 8 * kGHelpers; ++k) b += s_bias[4 * k + (tid >> 3)][tid & 7];
-      out[9 * S::COUT * S::CIN + tid] = b;
     }
   }
   asm volatile("tcgen05.fence::before_thread_sync;" ::: "memory");
   __syncthreads();
   if (warp == 0) {
     asm volatile("tcgen05.fence::after_thread_sync;" ::: "memory");
-    asm volatile("tcgen05.dealloc.cta_group::1.sync.aligned.b32 %0, %1;" ::"r"(tmem), "r"(kCTmemCols));
+    asm volatile("tcgen05.dealloc.cta_group::1.sync.aligned.b32 %0, %1;" ::"r"(tmem), "r"(S::kCols));
   }
 }
 
@@ -873,9 +919,9 @@ cudaError_t launch_wgrad_tc_t(const RefineWgradArgs& a, cudaStream_t s) {
   std::memset(&am, 0, sizeof(am));
   std::memset(&gm, 0, sizeof(gm));
   const bool ok = (MODE == 1 ? encode_rgba(enc, &am, a.x, a.n, a.H, a.W, S::FW, S::FH)
-                             : encode_map32(enc, &am, a.a_h, a.n, a.H, a.W, kGTW, kGTH + 2)) &&
+                             : encode_map32(enc, &am, a.a_h, a.n, a.H, a.W, kGHW, kGHR)) &&
                   (MODE == 3 ? encode_rgba(enc, &gm, a.g_f, a.n, a.H, a.W, S::FW, S::FH)
-                             : encode_map32(enc, &gm, a.g_h, a.n, a.H, a.W, S::GW, kGTH));
+                             : encode_map32(enc, &gm, a.g_h, a.n, a.H, a.W, kGTW, kGTH));
   if (!ok) return cudaErrorInvalidValue;
   return launch_kernel(wgrad_tc_kernel<MODE>, dim3(a.n_ctas), dim3(kGThreads), S::kSmem, s, true, a, am, gm);
 }
@@ -889,10 +935,12 @@ cudaError_t launch_refine_wgrad(int mode, const RefineWgradArgs& a, cudaStream_t
   return cudaErrorInvalidValue;
 }
 
-int refine_wgrad_tiles(int n, int H, int W, int* tiles_x, int* tiles_y) {
-  *tiles_x = (W + kGTW - 1) / kGTW;
-  *tiles_y = (H + kGTH - 1) / kGTH;
-  return *tiles_x * *tiles_y * n;
+void refine_wgrad_shape(RefineWgradArgs& g, int sm_count) {
+  g.tiles_x = (g.W + kGTW - 1) / kGTW;
+  g.tiles_y = (g.H + kGTH - 1) / kGTH;
+  const int64_t blocks = (int64_t)g.tiles_x * ((g.H + 7) / 8) * g.n;  // chains of at least one chunk
+  g.n_rows = (int)std::max<int64_t>(1, std::min<int64_t>(blocks, (int64_t)kGChains * sm_count));
+  g.n_ctas = std::min(g.n_rows, sm_count);
 }
 
 }  // namespace lfk
