@@ -160,7 +160,7 @@ def measured_peak():
         return HBM_FALLBACK_GBS, "fallback"
 
 
-RASTER_SOURCES = ("lf_raster.cu", "lf_internal.h")
+RASTER_SOURCES = ("lf_raster_impl.h", "lf_ray.h", "lf_internal.h")
 REFINE_SOURCES = ("lf_refine_tc.cu", "lf_internal.h")
 REFINE_PROFILE = "refine_fused_stereo_2x1440x1600"
 

@@ -244,7 +244,7 @@ LF_API lf_status lf_render_inspect(lf_ctx* ctx, const lf_pose* eye, const lf_int
  * is reserved up front by another allocator, a plug-in that may not allocate.
  * lf_render grows its scratch with cudaMalloc on first use; this entry point
  * instead takes all per-call scratch from one static device array of about
- * 16.8 MB that every GPU loading the library holds until the process exits.
+ * 17.9 MB that every GPU loading the library holds until the process exits.
  *   Limits (else LF_ERR_CAPACITY and a message in lf_last_error): at most 32
  *   loaded views, a mesh grid of at most 33 x 33, at most 8192 screen tiles
  *   (1024 x 512 pixels with 8 x 8 tiles, 1024 x 2048 with 16 x 16).  Within

@@ -75,7 +75,7 @@ struct lf_ctx {
   lf_mesh_format mesh_fmt = LF_MESH_F32_DEPTH;
   Buffer depth, tab_a, tab_b, cluster_z;
   // per-call scratch
-  Buffer eyes, eyes_f, vrecs, masks, pool, pool_owner, bin_offsets, bin_entries, small, active;
+  Buffer eyes, eyes_f, ray_cols, ray_rows, vrecs, masks, pool, pool_owner, bin_offsets, bin_entries, small, active;
   EyeParams* pinned = nullptr;  // kRing slots of max_eyes
   cudaEvent_t ring_ev[kRing] = {};
   int ring_next = 0;
@@ -167,8 +167,12 @@ bool valid_tile(int w, int h) { return (w == 16 && h == 16) || (w == 32 && h == 
 
 struct Layout {
   int32_t total_tiles = 0;
+  int64_t total_lines = 0;  // of the ray tables: per eye room for max(its rows, a quarter of its columns)
   std::vector<EyeParams> eyes;
 };
+
+// Lines that an eye takes in the ray tables.
+inline int64_t ray_lines(const EyeParams& P) { return std::max(P.H, (P.W + 3) / 4); }
 
 // RGBA images are read and written as 16-byte texels.
 inline bool aligned16(const void* p) { return (reinterpret_cast<uintptr_t>(p) & 15u) == 0; }
@@ -196,6 +200,8 @@ lf_status make_layout(lf_ctx* c, int32_t n_eyes, const lf_pose* eyes, const lf_i
     P.tiles_y = (K.height + c->cfg.tile_h - 1) / c->cfg.tile_h;
     P.tile_base = (int32_t)base;
     P.out = out[e];
+    P.line_base = (int32_t)L.total_lines;
+    L.total_lines += ray_lines(P);
     base += (int64_t)P.tiles_x * P.tiles_y;
     if (base > (int64_t)1 << 30) return fail(c, LF_ERR_INVALID_ARG, "too many tiles");
   }
@@ -217,7 +223,10 @@ int64_t bin_entries_capacity(const lf_ctx* c, int64_t total_tiles) {
   return std::max(c->cfg.tri_capacity * 4, 32 * total_tiles);
 }
 
-lf_status ensure_scratch(lf_ctx* c, int32_t n_eyes, int32_t total_tiles) {
+lf_status ensure_scratch(lf_ctx* c, const Layout& L) {
+  const int32_t n_eyes = (int32_t)L.eyes.size(), total_tiles = L.total_tiles;
+  LF_CUDA(c, ensure(c->ray_cols, sizeof(float) * 4 * (size_t)L.total_lines));
+  LF_CUDA(c, ensure(c->ray_rows, sizeof(float4) * (size_t)L.total_lines));
   LF_CUDA(c, ensure(c->eyes, sizeof(EyeParams) * (size_t)c->cfg.max_eyes));
   LF_CUDA(c, ensure(c->eyes_f, sizeof(EyeFloat) * (size_t)c->cfg.max_eyes));
   LF_CUDA(c, ensure(c->vrecs, sizeof(ViewRec) * (size_t)n_eyes * c->n_views));
@@ -295,6 +304,8 @@ FrameArgs frame_args(lf_ctx* c, const Layout& L) {
   a.vrecs = static_cast<ViewRec*>(c->vrecs.p);
   a.tile_masks = static_cast<uint32_t*>(c->masks.p);
   a.eyes_f = static_cast<EyeFloat*>(c->eyes_f.p);
+  a.ray_cols = static_cast<float*>(c->ray_cols.p);
+  a.ray_rows = static_cast<float4*>(c->ray_rows.p);
   a.pool = static_cast<TriRec*>(c->pool.p);
   a.pool_owner = static_cast<int32_t*>(c->pool_owner.p);
   a.pool_capacity = c->cfg.tri_capacity;
@@ -547,7 +558,7 @@ void lf_destroy(lf_ctx* ctx) {
   if (ctx->has_call && ctx->last_stream) cudaStreamSynchronize(ctx->last_stream);
   cudaDeviceSynchronize();
   if (ctx->graph) cudaGraphExecDestroy(ctx->graph);
-  for (Buffer* b : {&ctx->views, &ctx->tex, &ctx->depth, &ctx->tab_a, &ctx->tab_b, &ctx->cluster_z, &ctx->pool_owner, &ctx->eyes, &ctx->eyes_f,
+  for (Buffer* b : {&ctx->views, &ctx->tex, &ctx->depth, &ctx->tab_a, &ctx->tab_b, &ctx->cluster_z, &ctx->pool_owner, &ctx->eyes, &ctx->eyes_f, &ctx->ray_cols, &ctx->ray_rows,
                     &ctx->vrecs, &ctx->masks, &ctx->pool, &ctx->bin_offsets, &ctx->bin_entries, &ctx->small,
                     &ctx->active})
     release(*b);
@@ -734,7 +745,7 @@ lf_status lf_render(lf_ctx* c, int32_t n_eyes, const lf_pose* eyes, const lf_int
   if (st != LF_OK) return st;
   Layout L;
   if ((st = make_layout(c, n_eyes, eyes, intr, out_rgba, L)) != LF_OK) return st;
-  if ((st = ensure_scratch(c, n_eyes, L.total_tiles)) != LF_OK) return st;
+  if ((st = ensure_scratch(c, L)) != LF_OK) return st;
   cudaStream_t s = static_cast<cudaStream_t>(stream);
   if ((st = stage_eyes(c, L, s)) != LF_OK) return st;
   FrameArgs a = frame_args(c, L);
@@ -755,7 +766,7 @@ lf_status lf_render_inspect(lf_ctx* c, const lf_pose* eye, const lf_intrinsics* 
   Layout L;
   float* outs[1] = {out_rgba};
   if ((st = make_layout(c, 1, eye, intr, outs, L)) != LF_OK) return st;
-  if ((st = ensure_scratch(c, 1, L.total_tiles)) != LF_OK) return st;
+  if ((st = ensure_scratch(c, L)) != LF_OK) return st;
   cudaStream_t s = static_cast<cudaStream_t>(stream);
   if ((st = stage_eyes(c, L, s)) != LF_OK) return st;
   FrameArgs a = frame_args(c, L);
@@ -778,11 +789,11 @@ lf_status lf_render_batch(lf_ctx* c, int32_t n_eyes, const lf_pose* eyes, const 
   if (st != LF_OK) return st;
   Layout L;
   if ((st = make_layout(c, n_eyes, eyes, intr, out_rgba, L)) != LF_OK) return st;
-  if ((st = ensure_scratch(c, n_eyes, L.total_tiles)) != LF_OK) return st;
+  if ((st = ensure_scratch(c, L)) != LF_OK) return st;
   if ((st = ensure_persistent_blocks(c)) != LF_OK) return st;
   // The graph depends on the layout and on every scratch address it names.
   std::vector<int64_t> sig = {n_eyes, L.total_tiles, c->n_views, c->G, c->tex_fmt, c->mesh_fmt,
-                              (int64_t)(intptr_t)c->eyes.p, (int64_t)(intptr_t)c->eyes_f.p,
+                              (int64_t)(intptr_t)c->eyes.p, (int64_t)(intptr_t)c->eyes_f.p, (int64_t)(intptr_t)c->ray_cols.p, (int64_t)(intptr_t)c->ray_rows.p,
                               (int64_t)(intptr_t)c->bin_offsets.p, (int64_t)(intptr_t)c->bin_entries.p,
                               (int64_t)(intptr_t)c->vrecs.p, (int64_t)(intptr_t)c->pool_owner.p, (int64_t)(intptr_t)c->cluster_z.p,
                               (int64_t)(intptr_t)c->masks.p, (int64_t)(intptr_t)c->pool.p,
@@ -1023,13 +1034,17 @@ constexpr size_t align256(size_t x) { return (x + 255) & ~(size_t)255; }
 constexpr size_t kOffCounters = 0;
 constexpr size_t kOffEye = align256(kOffCounters + 64);
 constexpr size_t kOffEyeF = align256(kOffEye + sizeof(EyeParams));
-constexpr size_t kOffVrecs = align256(kOffEyeF + sizeof(EyeFloat));
+// ray tables: the widest and the tallest eye of at most 8192 tiles of 32 pixels, or the largest eye
+constexpr size_t kStaticLines = 32768;
+constexpr size_t kOffRayCols = align256(kOffEyeF + sizeof(EyeFloat));
+constexpr size_t kOffRayRows = align256(kOffRayCols + sizeof(float) * 4 * kStaticLines);
+constexpr size_t kOffVrecs = align256(kOffRayRows + sizeof(float4) * kStaticLines);
 constexpr size_t kOffActive = align256(kOffVrecs + sizeof(ViewRec) * kStaticMaxViews);
 constexpr size_t kOffMasks = align256(kOffActive + kStaticMaxViews);
 constexpr size_t kOffBinOffsets = align256(kOffMasks + sizeof(uint32_t) * kStaticMaxTiles * ((kStaticMaxViews + 31) / 32));
 constexpr size_t kOffBinEntries = align256(kOffBinOffsets + sizeof(int32_t) * kStaticBinOffsets);
 constexpr size_t kOffPool = align256(kOffBinEntries + sizeof(int32_t) * kStaticBinEntries);
-constexpr size_t kStaticBytes = align256(kOffPool + sizeof(TriRec) * kStaticTris);  // about 16.8 MB
+constexpr size_t kStaticBytes = align256(kOffPool + sizeof(TriRec) * kStaticTris);  // about 17.9 MB
 
 }  // namespace
 
@@ -1106,6 +1121,8 @@ extern "C" lf_status lf_render_static(lf_ctx* c, const lf_pose* eye, const lf_in
   a.fine_mesh = fine_mesh(c, P);
   a.eyes = reinterpret_cast<const EyeParams*>(base + kOffEye);
   a.eyes_f = reinterpret_cast<EyeFloat*>(base + kOffEyeF);
+  a.ray_cols = reinterpret_cast<float*>(base + kOffRayCols);
+  a.ray_rows = reinterpret_cast<float4*>(base + kOffRayRows);
   a.vrecs = reinterpret_cast<ViewRec*>(base + kOffVrecs);
   a.active = base + kOffActive;
   a.tile_masks = reinterpret_cast<uint32_t*>(base + kOffMasks);
@@ -1457,7 +1474,7 @@ lf_status host_enqueue(lf_ctx* c, int slot, int32_t n_eyes, const lf_pose* eyes,
   lf_status st;
   Layout L;
   if ((st = make_layout(c, n_eyes, eyes, intr, target.data(), L)) != LF_OK) return st;
-  if ((st = ensure_scratch(c, n_eyes, L.total_tiles)) != LF_OK) return st;
+  if ((st = ensure_scratch(c, L)) != LF_OK) return st;
   if ((st = stage_eyes(c, L, s)) != LF_OK) return st;
   FrameArgs a = frame_args(c, L);
   unsigned char* counters = static_cast<unsigned char*>(H.counters.p) + kCounterBlock * slot;

@@ -13,6 +13,7 @@
 //   tile masks                    per eye tile, one bit per view whose disk footprint
 //                                 overlaps the tile (ceil(n_views/32) words)
 //   EyeFloat[n_eyes]              the eye's FP32 constants (rounded once, on the device)
+//   ray columns / ray rows        the eyes' ray slopes by column and ray terms by row
 //   TriRec pool                   set-up (sub-)triangles, in runs of one 4x4-cell cluster
 //   bin offsets / bin entries     per (eye, view): its triangles binned into the screen
 //                                 tiles of its footprint (pool indices), plus a list of
@@ -71,7 +72,7 @@ struct EyeParams {
   int32_t W, H;
   int32_t tiles_x, tiles_y;
   int32_t tile_base;    // first tile index of this eye in the call's flattened tile range
-  int32_t pad;
+  int32_t line_base;    // first row of this eye in the call's ray rows (and first 4 columns in its ray columns)
   float* out;           // H x W float4
 };
 
@@ -81,9 +82,10 @@ struct __align__(16) EyeFloat {
   float R[9];
   float o[3];           // eye centre minus capture-sphere centre
   float fx, fy, cx, cy;
-  float R2;             // capture-sphere radius squared
-  float pad[3];
+  float4 ray;           // R[0], R[3], R[6] and qc = |o|^2 - (sphere radius)^2
+  float4 centre;        // o, 0
 };
+static_assert(sizeof(EyeFloat) == 96 && offsetof(EyeFloat, ray) == 64, "EyeFloat layout");
 
 struct __align__(16) ViewRec {
   // what the raster copies to shared memory per tile, 16 bytes at a time
@@ -154,6 +156,8 @@ struct FrameArgs {
   ViewRec* vrecs;
   uint32_t* tile_masks;
   EyeFloat* eyes_f;
+  float* ray_cols;         // per eye from 4 line_base: each column's ray slope
+  float4* ray_rows;        // per eye from line_base: each row's ray terms (ray_row)
   TriRec* pool;
   int32_t* pool_owner;     // per record its eye * n_views + view (grids set up by several blocks per view)
   int64_t pool_capacity;

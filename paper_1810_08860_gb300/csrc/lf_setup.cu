@@ -27,14 +27,11 @@
 
 #include "lf_internal.h"
 #include "lf_launch.h"
+#include "lf_ray.h"
 
 namespace lfk {
 
 // ------------------------------------------------------------------ small helpers
-
-__device__ __forceinline__ float dot3_rn(float a0, float a1, float a2, float b0, float b1, float b2) {
-  return __fmaf_rn(a0, b0, __fmaf_rn(a1, b1, __fmul_rn(a2, b2)));
-}
 
 __device__ __forceinline__ bool snap_rn(float x, float y, float z, float fx, float fy, float cx, float cy,
                                         int32_t& sx, int32_t& sy) {
@@ -196,6 +193,29 @@ constexpr int kViewsPerSetupBlock = 16;
 constexpr int kViewSetupThreads = 128;
 constexpr int kViewSetupSlices = 8;  // blocks sharing one group of views' (view, tile) cone tests
 
+// Two-level frames, round disks: a first look at which views an eye selects, 64 pixels
+// spread over each view's footprint (the block's slice takes two views).  What it finds
+// is exact; the views it misses are left to select_kernel, which tests every pixel of
+// the tiles that may see them.  With it select_kernel takes 9 us of a 2 x 1440x1600
+// frame of 640 views instead of 85.
+__device__ void mark_visible(const FrameArgs& A, const EyeParams& E, const EyeFloat& F, int e, int v0, const int4* s_bb) {
+  constexpr int kPer = kViewsPerSetupBlock / kViewSetupSlices, kLanes = kViewSetupThreads / kPer;  // 2 views, 64 pixels
+  const int k = blockIdx.z * kPer + threadIdx.x / kLanes, q = threadIdx.x % kLanes, v = v0 + k;
+  if (v >= A.n_views) return;
+  const int4 bb = s_bb[k];
+  if (bb.x > bb.z || bb.y > bb.w) return;
+  const int x = bb.x + (int)((int64_t)(2 * (q & 7) + 1) * (bb.z - bb.x + 1) / 16);
+  const int y = bb.y + (int)((int64_t)(2 * (q >> 3) + 1) * (bb.w - bb.y + 1) / 16);
+  float p[3];
+  sphere_crossing(F.ray, F.centre, ray_slope(x, F.cx, F.fx), ray_row(F, ray_slope(y, F.cy, F.fy)), p);
+  const ViewStatic& V = A.views[v];
+  const float4 cc = make_float4(__double2float_rn(__dsub_rn((double)V.disk_c[0], A.sphere_c[0])),
+                                __double2float_rn(__dsub_rn((double)V.disk_c[1], A.sphere_c[1])),
+                                __double2float_rn(__dsub_rn((double)V.disk_c[2], A.sphere_c[2])),
+                                __fmul_rn(V.disk_r, V.disk_r));
+  if (disk_d2(cc, p) < cc.w) A.visible[(int64_t)e * A.n_views + v] = 1;
+}
+
 // A block takes 16 views of one eye.  Threads 0-15 do the per-view set-up
 // (FP64 composition, FP32 shading map and disk constants, conservative
 // footprint); then all threads test every (view, tile) pair of the block's
@@ -209,6 +229,7 @@ __global__ void __launch_bounds__(kViewSetupThreads) view_setup_kernel(FrameArgs
   __shared__ float s_dir[kViewsPerSetupBlock][4];   // unit direction to the disk centre, cos of the cone limit
   __shared__ int s_off[kViewsPerSetupBlock + 1];   // exclusive prefix of the footprints' tile counts
   __shared__ int s_tile[kViewsPerSetupBlock][3];    // footprint: first tile column and row, tile columns
+  __shared__ int4 s_tile_bb[kViewsPerSetupBlock];   // footprint in pixels
   const int e = blockIdx.y;
   const int v0 = blockIdx.x * kViewsPerSetupBlock;
   const EyeParams& E = A.eyes[e];
@@ -227,15 +248,21 @@ __global__ void __launch_bounds__(kViewSetupThreads) view_setup_kernel(FrameArgs
     *A.bin_offsets_counter = 0ull;
     *A.bin_entries_counter = 0ull;
   }
-  if (writer && blockIdx.x == 0 && threadIdx.x == 0) {
-    // the eye's FP32 decision constants, each rounded once from FP64
-    EyeFloat& F = A.eyes_f[e];
-    for (int k = 0; k < 9; ++k) F.R[k] = __double2float_rn(E.R[k]);
-    for (int k = 0; k < 3; ++k) F.o[k] = __double2float_rn(__dsub_rn(E.t[k], A.sphere_c[k]));
-    F.fx = __double2float_rn(E.fx); F.fy = __double2float_rn(E.fy);
-    F.cx = __double2float_rn(E.cx); F.cy = __double2float_rn(E.cy);
-    F.R2 = __double2float_rn(__dmul_rn(A.sphere_r, A.sphere_r));
-    F.pad[0] = F.pad[1] = F.pad[2] = 0.0f;
+  // the eye's FP32 decision constants, each rounded once from FP64 (every block for itself: its share of the ray tables)
+  __shared__ EyeFloat F;
+  if (threadIdx.x >= 32 && threadIdx.x < 32 + 16) {
+    const int k = threadIdx.x - 32;
+    if (k < 9) F.R[k] = __double2float_rn(E.R[k]);
+    else if (k < 12) F.o[k - 9] = __double2float_rn(__dsub_rn(E.t[k - 9], A.sphere_c[k - 9]));
+    else (&F.fx)[k - 12] = __double2float_rn((&E.fx)[k - 12]);
+    __syncwarp(0xffffu);
+    if (k == 0) {
+      const float R2 = __double2float_rn(__dmul_rn(A.sphere_r, A.sphere_r));
+      F.ray = make_float4(F.R[0], F.R[3], F.R[6],
+                          __fsub_rn(dot3_rn(F.o[0], F.o[1], F.o[2], F.o[0], F.o[1], F.o[2]), R2));
+      F.centre = make_float4(F.o[0], F.o[1], F.o[2], 0.0f);
+      if (writer && blockIdx.x == 0) A.eyes_f[e] = F;
+    }
   }
   int n_tiles = 0;  // tiles of this thread's view's footprint (threads 0-15)
   if (threadIdx.x < kViewsPerSetupBlock) {
@@ -373,6 +400,7 @@ __global__ void __launch_bounds__(kViewSetupThreads) view_setup_kernel(FrameArgs
       }
     }
     for (int k = 0; k < 4; ++k) s_dir[threadIdx.x][k] = dir[k];
+    s_tile_bb[threadIdx.x] = make_int4(bb[0], bb[1], bb[2], bb[3]);
     int tx0 = 0, ty0 = 0, ntx = 1;
     if (bb[0] <= bb[2] && bb[1] <= bb[3]) {
       tx0 = bb[0] / A.tile_w;
@@ -396,6 +424,16 @@ __global__ void __launch_bounds__(kViewSetupThreads) view_setup_kernel(FrameArgs
     if (threadIdx.x == kViewsPerSetupBlock - 1) s_off[kViewsPerSetupBlock] = incl;
   }
   __syncthreads();
+  // the eye's ray tables, shared by all its blocks: the raster reads a column's slope and a row's terms instead of
+  // dividing for every pixel
+  {
+    const int step = gridDim.x * gridDim.z * kViewSetupThreads;
+    for (int i = (blockIdx.z * gridDim.x + blockIdx.x) * kViewSetupThreads + threadIdx.x; i < E.W + E.H; i += step) {
+      if (i < E.W) A.ray_cols[4 * (int64_t)E.line_base + i] = ray_slope(i, F.cx, F.fx);
+      else A.ray_rows[(int64_t)E.line_base + i - E.W] = ray_row(F, ray_slope(i - E.W, F.cy, F.fy));
+    }
+  }
+  if (A.visible && A.disk_mode == 0) mark_visible(A, E, F, e, v0, s_tile_bb);
   const int total = s_off[kViewsPerSetupBlock];
   const float fx = (float)E.fx, fy = (float)E.fy, cx = (float)E.cx, cy = (float)E.cy;
   for (int f = threadIdx.x + blockIdx.z * kViewSetupThreads; f < total; f += kViewSetupThreads * kViewSetupSlices) {

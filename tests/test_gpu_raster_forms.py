@@ -58,6 +58,34 @@ def test_every_form_draws_the_inspection_image(views, size, grid, disk, eye, ova
     r.close()
 
 
+# Four pixels per lane: 256-pixel tiles of the narrow texture formats, in eyes of at least 3648 tiles (whole tiles).
+@pytest.mark.parametrize("fmt", ["u8", "bf16", "fp8"])
+@pytest.mark.parametrize("tile", [(16, 16), (32, 8)])
+@pytest.mark.parametrize("views,grid,disk,oval", [(9, 5, 1.2, True), (40, 17, 6.0, False)])
+def test_wide_lanes_draw_the_inspection_image(fmt, tile, views, grid, disk, oval):
+    torch = pytest.importorskip("torch")
+    import __graft_entry__
+
+    __graft_entry__.build()
+    import paper_1810_08860_gb300 as lfm
+    from paper_1810_08860_gb300 import disks
+
+    side = math.isqrt(views - 1) + 1
+    lf = scene.build_light_field(scene.sphere_scene(3, 8, forward_cone_deg=35.0), scene.cap_grid_directions(side, 40.0)[:views],
+                                 64, 64, 90.0, grid, disk_scale=disk)
+    e = scene.head_pose_eyes(scene.SplitMix64(11), 1100, 901, 90.0, yaw_range=(-0.1, 0.1), pitch_deg=6.0, stereo=False)[0]
+    r = lfm.Renderer(0, tile=tile)
+    r.load_views(lf, tex_format=fmt)
+    r.build_meshes(lf)
+    if oval:
+        r.set_disk_ovals(disks.oval_extents(lf))
+    want = r.render_inspect(e, max_records=views)["rgba"]
+    assert int((want[..., 3] > 0).sum()) > 0
+    assert torch.equal(r.render([e])[0], want)
+    assert torch.equal(r.render_batch([e, e])[1], want)
+    r.close()
+
+
 def _cap(views, size, grid, seed=3):
     side = math.isqrt(views - 1) + 1
     lf = scene.build_light_field(scene.sphere_scene(seed, 8, forward_cone_deg=35.0),
