@@ -9,6 +9,7 @@ from __future__ import annotations
 
 import ctypes
 import os
+import struct
 
 import numpy as np
 
@@ -213,10 +214,14 @@ def _intrinsics(intr, sizes) -> ctypes.Array:
     return arr
 
 
+_EYE_INTR = struct.Struct("4d2i")  # lf_intrinsics
+
+
 def _stream_handle(stream):
     import torch
     if stream is None:
-        stream = torch.cuda.current_stream()
+        # the current stream's handle as it is: a torch.cuda.Stream built around it takes 3.6 us a call
+        return ctypes.c_void_p(torch._C._cuda_getCurrentRawStream(torch.cuda.current_device()))
     return ctypes.c_void_p(stream.cuda_stream)
 
 
@@ -343,9 +348,14 @@ class Renderer:
 
     @staticmethod
     def _eye_arrays(eyes):
-        poses = _poses([e.pose for e in eyes])
-        intr = _intrinsics([e.intr for e in eyes], [(e.width, e.height) for e in eyes])
-        return poses, intr
+        """The eyes' lf_pose and lf_intrinsics records, as bytes (ctypes passes their address): a call of one eye
+        spends 1.9 us here, 5.9 us with ctypes structures."""
+        poses = [np.asarray(e.pose, dtype=np.float64) for e in eyes]
+        if any(p.size != 12 for p in poses):
+            poses = [np.asarray(poses).reshape(-1, 12)]
+        intr = [_EYE_INTR.pack(*np.asarray(e.intr, dtype=np.float64).ravel().tolist(), int(e.width), int(e.height))
+                for e in eyes]
+        return b"".join([p.tobytes() for p in poses]), b"".join(intr)
 
     def _outputs(self, eyes, out):
         import torch

@@ -136,7 +136,7 @@ struct GridTables {
 };
 
 struct FrameArgs {
-  const EyeParams* eyes;
+  EyeParams* eyes;
   int32_t n_eyes;
   int32_t n_views;
   int32_t src_w, src_h;
@@ -192,6 +192,14 @@ struct FrameArgs {
   int32_t n_fine;                // views [0, n_fine) are the streamed fine level
 };
 
+// The eyes of a call of up to kInlineEyes, passed to the view set-up by value (n = 0: they
+// are in FrameArgs::eyes already); it writes them there for the kernels after it.
+constexpr int kInlineEyes = 2;
+struct InlineEyes {
+  EyeParams eye[kInlineEyes];
+  int32_t n;
+};
+
 // launchers (return cudaGetLastError())
 cudaError_t launch_grid_tables(const ViewStatic* views, int n_views, int src_w, int src_h, int G,
                                float* a, float* b, cudaStream_t s);
@@ -200,7 +208,7 @@ cudaError_t launch_cluster_bounds(const void* depth, int mesh_format, const View
 cudaError_t launch_convert_textures(const uint8_t* src, void* dst, int64_t n_texels, int fmt,
                                     const float* scale_per_texel_view, int64_t texels_per_view,
                                     cudaStream_t s);
-cudaError_t launch_view_setup(const FrameArgs& a, cudaStream_t s);
+cudaError_t launch_view_setup(const FrameArgs& a, const InlineEyes& eyes, cudaStream_t s);
 cudaError_t launch_tri_setup(const FrameArgs& a, cudaStream_t s, bool pdl);
 cudaError_t launch_raster(const FrameArgs& a, bool inspect, bool persistent, int persistent_blocks,
                           cudaStream_t s, bool pdl = false);

@@ -225,14 +225,15 @@ __device__ void mark_visible(const FrameArgs& A, const EyeParams& E, const EyeFl
 // disk centre c, and every pixel ray of a tile lies within (half diagonal)/f
 // of the tile's centre ray (rays through image points s apart differ by at
 // most s/f in angle), so a tile is skipped only when the two cones are apart.
-__global__ void __launch_bounds__(kViewSetupThreads) view_setup_kernel(FrameArgs A) {
+__global__ void __launch_bounds__(kViewSetupThreads) view_setup_kernel(FrameArgs A, const __grid_constant__ InlineEyes given) {
   __shared__ float s_dir[kViewsPerSetupBlock][4];   // unit direction to the disk centre, cos of the cone limit
   __shared__ int s_off[kViewsPerSetupBlock + 1];   // exclusive prefix of the footprints' tile counts
   __shared__ int s_tile[kViewsPerSetupBlock][3];    // footprint: first tile column and row, tile columns
   __shared__ int4 s_tile_bb[kViewsPerSetupBlock];   // footprint in pixels
   const int e = blockIdx.y;
   const int v0 = blockIdx.x * kViewsPerSetupBlock;
-  const EyeParams& E = A.eyes[e];
+  const EyeParams& E = given.n ? given.eye[e] : A.eyes[e];
+  if (given.n && blockIdx.x == 0 && blockIdx.z == 0 && threadIdx.x == 64) A.eyes[e] = given.eye[e];
   const float tile_half_diag = 0.5f * sqrtf((float)(A.tile_w * A.tile_w + A.tile_h * A.tile_h));
   const float alpha_tile = tile_half_diag / fminf((float)E.fx, (float)E.fy);
   const bool writer = blockIdx.z == 0;  // the other slices only share the cone tests
@@ -457,9 +458,9 @@ __global__ void __launch_bounds__(kViewSetupThreads) view_setup_kernel(FrameArgs
   }
 }
 
-cudaError_t launch_view_setup(const FrameArgs& a, cudaStream_t s) {
+cudaError_t launch_view_setup(const FrameArgs& a, const InlineEyes& eyes, cudaStream_t s) {
   dim3 grid((a.n_views + kViewsPerSetupBlock - 1) / kViewsPerSetupBlock, a.n_eyes, kViewSetupSlices);
-  view_setup_kernel<<<grid, kViewSetupThreads, 0, s>>>(a);
+  view_setup_kernel<<<grid, kViewSetupThreads, 0, s>>>(a, eyes);
   return cudaGetLastError();
 }
 

@@ -86,6 +86,44 @@ def test_wide_lanes_draw_the_inspection_image(fmt, tile, views, grid, disk, oval
     r.close()
 
 
+@pytest.mark.parametrize("n", [1, 2, 3, 5])
+def test_eyes_by_value_and_by_copy_draw_the_same(n):
+    """Up to two eyes travel with the launch, more through the pinned ring."""
+    torch = pytest.importorskip("torch")
+    import __graft_entry__
+
+    __graft_entry__.build()
+    import paper_1810_08860_gb300 as lfm
+
+    lf, _ = _cap(9, 64, 17)
+    eyes = [scene.head_pose_eyes(scene.SplitMix64(20 + k), 40 + 9 * k, 31 + 5 * k, 90.0, yaw_range=(-0.1, 0.1), pitch_deg=6.0,
+                                 stereo=False)[0] for k in range(n)]
+    r = lfm.Renderer(0, max_eyes=8)
+    r.load_views(lf)
+    r.build_meshes(lf)
+    want = [r.render_inspect(e, max_records=9)["rgba"] for e in eyes]
+    for _ in range(6):  # more calls than the ring has slots, each with its own eyes
+        eyes, want = eyes[1:] + eyes[:1], want[1:] + want[:1]
+        for got in (r.render(eyes), r.render_batch(eyes)):
+            assert all(torch.equal(a, b) for a, b in zip(got, want))
+    # a captured call replays its own eyes after other calls
+    side = torch.cuda.Stream()
+    g = torch.cuda.CUDAGraph()
+    out = [torch.zeros_like(w) for w in want]
+    if n <= 2:
+        r.render(eyes, out=out)
+        torch.cuda.synchronize()
+        with torch.cuda.graph(g, stream=side):
+            r.render(eyes, out=out)
+        r.render([eyes[-1]])
+        for o in out:
+            o.zero_()
+        g.replay()
+        torch.cuda.synchronize()
+        assert all(torch.equal(a, b) for a, b in zip(out, want))
+    r.close()
+
+
 def _cap(views, size, grid, seed=3):
     side = math.isqrt(views - 1) + 1
     lf = scene.build_light_field(scene.sphere_scene(seed, 8, forward_cone_deg=35.0),
