@@ -75,7 +75,7 @@ struct lf_ctx {
   lf_mesh_format mesh_fmt = LF_MESH_F32_DEPTH;
   Buffer depth, tab_a, tab_b, cluster_z;
   // per-call scratch
-  Buffer eyes, eyes_f, ray_cols, ray_rows, vrecs, masks, pool, pool_owner, bin_offsets, bin_entries, small, active;
+  Buffer eyes, eyes_f, ray_cols, ray_rows, vrecs, masks, pool, pool_owner, pool_box, bin_offsets, bin_entries, small, active;
   EyeParams* pinned = nullptr;  // kRing slots of max_eyes
   cudaEvent_t ring_ev[kRing] = {};
   int ring_next = 0;
@@ -236,7 +236,10 @@ lf_status ensure_scratch(lf_ctx* c, const Layout& L) {
   int64_t cap = c->cfg.tri_capacity;
   LF_CUDA(c, ensure(c->pool, sizeof(TriRec) * (size_t)cap));
   const int ncl = clusters_per_side(c->G);
-  if (ncl * ncl > kSetupPartClusters) LF_CUDA(c, ensure(c->pool_owner, sizeof(int32_t) * (size_t)cap));
+  if (ncl * ncl > kSetupPartClusters) {
+    LF_CUDA(c, ensure(c->pool_owner, sizeof(int32_t) * (size_t)cap));
+    LF_CUDA(c, ensure(c->pool_box, sizeof(int2) * (size_t)cap));
+  }
   LF_CUDA(c, ensure(c->bin_offsets, sizeof(int32_t) * (size_t)bin_offsets_capacity(c, total_tiles)));
   LF_CUDA(c, ensure(c->bin_entries, sizeof(int32_t) * (size_t)bin_entries_capacity(c, total_tiles)));
   if (c->lv.n_fine > 0) {
@@ -321,6 +324,7 @@ FrameArgs frame_args(lf_ctx* c, const Layout& L) {
   a.ray_rows = static_cast<float4*>(c->ray_rows.p);
   a.pool = static_cast<TriRec*>(c->pool.p);
   a.pool_owner = static_cast<int32_t*>(c->pool_owner.p);
+  a.pool_box = static_cast<int2*>(c->pool_box.p);
   a.pool_capacity = c->cfg.tri_capacity;
   a.bin_offsets = static_cast<int32_t*>(c->bin_offsets.p);
   a.bin_offsets_capacity = bin_offsets_capacity(c, L.total_tiles);
@@ -571,7 +575,7 @@ void lf_destroy(lf_ctx* ctx) {
   if (ctx->has_call && ctx->last_stream) cudaStreamSynchronize(ctx->last_stream);
   cudaDeviceSynchronize();
   if (ctx->graph) cudaGraphExecDestroy(ctx->graph);
-  for (Buffer* b : {&ctx->views, &ctx->tex, &ctx->depth, &ctx->tab_a, &ctx->tab_b, &ctx->cluster_z, &ctx->pool_owner, &ctx->eyes, &ctx->eyes_f, &ctx->ray_cols, &ctx->ray_rows,
+  for (Buffer* b : {&ctx->views, &ctx->tex, &ctx->depth, &ctx->tab_a, &ctx->tab_b, &ctx->cluster_z, &ctx->pool_owner, &ctx->pool_box, &ctx->eyes, &ctx->eyes_f, &ctx->ray_cols, &ctx->ray_rows,
                     &ctx->vrecs, &ctx->masks, &ctx->pool, &ctx->bin_offsets, &ctx->bin_entries, &ctx->small,
                     &ctx->active})
     release(*b);
@@ -810,7 +814,7 @@ lf_status lf_render_batch(lf_ctx* c, int32_t n_eyes, const lf_pose* eyes, const 
   std::vector<int64_t> sig = {n_eyes, L.total_tiles, c->n_views, c->G, c->tex_fmt, c->mesh_fmt,
                               (int64_t)(intptr_t)c->eyes.p, (int64_t)(intptr_t)c->eyes_f.p, (int64_t)(intptr_t)c->ray_cols.p, (int64_t)(intptr_t)c->ray_rows.p,
                               (int64_t)(intptr_t)c->bin_offsets.p, (int64_t)(intptr_t)c->bin_entries.p,
-                              (int64_t)(intptr_t)c->vrecs.p, (int64_t)(intptr_t)c->pool_owner.p, (int64_t)(intptr_t)c->cluster_z.p,
+                              (int64_t)(intptr_t)c->vrecs.p, (int64_t)(intptr_t)c->pool_owner.p, (int64_t)(intptr_t)c->pool_box.p, (int64_t)(intptr_t)c->cluster_z.p,
                               (int64_t)(intptr_t)c->masks.p, (int64_t)(intptr_t)c->pool.p,
                               (int64_t)(intptr_t)c->active.p, (int64_t)(intptr_t)c->small.p,
                               (int64_t)(intptr_t)c->tex.p, (int64_t)(intptr_t)c->depth.p, c->persistent_blocks,

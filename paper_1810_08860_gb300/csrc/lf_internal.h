@@ -160,6 +160,7 @@ struct FrameArgs {
   float4* ray_rows;        // per eye from line_base: each row's ray terms (ray_row)
   TriRec* pool;
   int32_t* pool_owner;     // per record its eye * n_views + view (grids set up by several blocks per view)
+  int2* pool_box;          // and its first 8 bytes, the pixel box, once more
   int64_t pool_capacity;
   unsigned long long* pool_counter;
   int32_t* bin_offsets;

@@ -45,10 +45,6 @@ __device__ __forceinline__ bool snap_rn(float x, float y, float z, float fx, flo
   return true;
 }
 
-__device__ __forceinline__ int64_t floor_div256_up(int64_t a) {  // ceil(a / 256)
-  return (a + 255) >> 8;
-}
-
 // ------------------------------------------------------------------ grid tables
 
 __global__ void grid_tables_kernel(const ViewStatic* __restrict__ views, int n_views, int src_w, int src_h,
@@ -504,6 +500,7 @@ cudaError_t launch_cluster_bounds(const void* depth, int mesh_format, const View
 // ------------------------------------------------------------------ triangle set-up
 
 constexpr uint32_t kOcBehind = 16;  // outcode: bit0..3 left/right/above/below the padded footprint, bit4 behind z_near
+constexpr uint32_t kOcFar = 32;     // in front of it, but its snapped coordinates leave the 32-bit range: its triangles are dropped
 
 struct SetupCtx {
   float fx, fy, cx, cy, zn;
@@ -511,29 +508,27 @@ struct SetupCtx {
   int bb0, bb1, bb2, bb3;
 };
 
-// Orient, classify and bound one snapped sub-triangle; false if culled.
-__device__ bool setup_sub(const int32_t* sx, const int32_t* sy, const SetupCtx& C, TriRec& t, int32_t& tl) {
-  int64_t X0 = sx[0], Y0 = sy[0], X1 = sx[1], Y1 = sy[1], X2 = sx[2], Y2 = sy[2];
-  int64_t A = (X1 - X0) * (Y2 - Y0) - (Y1 - Y0) * (X2 - X0);
-  if (A == 0) return false;
-  if (A < 0) {
-    int64_t tx = X1, ty = Y1;
-    X1 = X2; Y1 = Y2; X2 = tx; Y2 = ty;
-  }
-  int64_t minx = min(X0, min(X1, X2)), maxx = max(X0, max(X1, X2));
-  int64_t miny = min(Y0, min(Y1, Y2)), maxy = max(Y0, max(Y1, Y2));
-  int64_t i0 = floor_div256_up(minx - 128), i1 = (maxx - 128) >> 8;
-  int64_t j0 = floor_div256_up(miny - 128), j1 = (maxy - 128) >> 8;
-  i0 = max(i0, (int64_t)C.bb0);
-  j0 = max(j0, (int64_t)C.bb1);
-  i1 = min(i1, (int64_t)C.bb2);
-  j1 = min(j1, (int64_t)C.bb3);
+// Orient, classify and bound one snapped sub-triangle; false if culled.  The
+// coordinates are below kSnapLimit, so differences and boxes are 32-bit; only the
+// area needs 64.
+__device__ __forceinline__ bool setup_sub(const int32_t* sx, const int32_t* sy, const SetupCtx& C, TriRec& t,
+                                          int32_t& tl) {
+  static_assert((int64_t)kSnapLimit + 256 < (int64_t)1 << 30, "differences of snapped coordinates fit 32 bits");
+  const int32_t X0 = sx[0], Y0 = sy[0];
+  const int64_t area = (int64_t)(sx[1] - X0) * (sy[2] - Y0) - (int64_t)(sy[1] - Y0) * (sx[2] - X0);
+  if (area == 0) return false;
+  const bool turn = area < 0;
+  const int32_t X1 = turn ? sx[2] : sx[1], Y1 = turn ? sy[2] : sy[1];
+  const int32_t X2 = turn ? sx[1] : sx[2], Y2 = turn ? sy[1] : sy[2];
+  // the pixel centres of its box: the first at or after the least coordinate, the last at or before the greatest
+  const int32_t i0 = max((min(X0, min(X1, X2)) + 127) >> 8, C.bb0), i1 = min((max(X0, max(X1, X2)) - 128) >> 8, C.bb2);
+  const int32_t j0 = max((min(Y0, min(Y1, Y2)) + 127) >> 8, C.bb1), j1 = min((max(Y0, max(Y1, Y2)) - 128) >> 8, C.bb3);
   if (i0 > i1 || j0 > j1) return false;
   t.bx0 = (int16_t)i0; t.by0 = (int16_t)j0; t.bx1 = (int16_t)i1; t.by1 = (int16_t)j1;
-  t.x[0] = (int32_t)X0; t.y[0] = (int32_t)Y0;
-  t.x[1] = (int32_t)X1; t.y[1] = (int32_t)Y1;
-  t.x[2] = (int32_t)X2; t.y[2] = (int32_t)Y2;
-  const int64_t X[3] = {X0, X1, X2}, Y[3] = {Y0, Y1, Y2};
+  t.x[0] = X0; t.y[0] = Y0;
+  t.x[1] = X1; t.y[1] = Y1;
+  t.x[2] = X2; t.y[2] = Y2;
+  const int32_t X[3] = {X0, X1, X2}, Y[3] = {Y0, Y1, Y2};
   tl = 0;
 #pragma unroll
   for (int k = 0; k < 3; ++k) {
@@ -549,36 +544,29 @@ struct EyeVtx {
   float x, y, z;
 };
 
-// The snapped polygon of a parent triangle after the near clip: np vertices (0:
-// dropped, 3, or 4: two sub-triangles, a fan from the first kept vertex) and the
-// parent's FP32 inverse-depth plane.  The decisions (snap, clip) are taken
-// exactly as the oracle takes them.
-struct SetupPoly {
-  int32_t px[4], py[4];
-  int np;
-  float ia, ib, ic;
-};
-
-__device__ __forceinline__ void setup_poly(const EyeVtx& v0, const EyeVtx& v1, const EyeVtx& v2, uint32_t o0,
-                                           uint32_t o1, uint32_t o2, const SetupCtx& C, SetupPoly& P) {
-  P.np = 0;
-  // FP32 inverse-depth plane of the parent (original vertex order), fixed order.
+// A parent's FP32 inverse-depth plane (original vertex order, fixed order); false if it has none.
+__device__ __forceinline__ bool setup_plane(const EyeVtx& v0, const EyeVtx& v1, const EyeVtx& v2, TriRec& t) {
   const float e1x = __fsub_rn(v1.x, v0.x), e1y = __fsub_rn(v1.y, v0.y), e1z = __fsub_rn(v1.z, v0.z);
   const float e2x = __fsub_rn(v2.x, v0.x), e2y = __fsub_rn(v2.y, v0.y), e2z = __fsub_rn(v2.z, v0.z);
   const float nx = __fsub_rn(__fmul_rn(e1y, e2z), __fmul_rn(e1z, e2y));
   const float ny = __fsub_rn(__fmul_rn(e1z, e2x), __fmul_rn(e1x, e2z));
   const float nz = __fsub_rn(__fmul_rn(e1x, e2y), __fmul_rn(e1y, e2x));
   const float dd = dot3_rn(nx, ny, nz, v0.x, v0.y, v0.z);
-  P.ia = __fdiv_rn(nx, dd); P.ib = __fdiv_rn(ny, dd); P.ic = __fdiv_rn(nz, dd);
-  if (dd == 0.0f || !isfinite(P.ia) || !isfinite(P.ib) || !isfinite(P.ic)) return;
-  if (((o0 | o1 | o2) & kOcBehind) == 0) {
-    if (!snap_rn(v0.x, v0.y, v0.z, C.fx, C.fy, C.cx, C.cy, P.px[0], P.py[0])) return;
-    if (!snap_rn(v1.x, v1.y, v1.z, C.fx, C.fy, C.cx, C.cy, P.px[1], P.py[1])) return;
-    if (!snap_rn(v2.x, v2.y, v2.z, C.fx, C.fy, C.cx, C.cy, P.px[2], P.py[2])) return;
-    P.px[3] = P.px[2]; P.py[3] = P.py[2];
-    P.np = 3;
-    return;
-  }
+  t.ia = __fdiv_rn(nx, dd); t.ib = __fdiv_rn(ny, dd); t.ic = __fdiv_rn(nz, dd);
+  return dd != 0.0f && isfinite(t.ia) && isfinite(t.ib) && isfinite(t.ic);
+}
+
+// The snapped polygon of a parent triangle that crosses the near plane: np
+// vertices (0: dropped, 3, or 4: two sub-triangles, a fan from the first kept
+// vertex).  The decisions (snap, clip) are taken exactly as the oracle takes them.
+struct SetupPoly {
+  int32_t px[4], py[4];
+  int np;
+};
+
+__device__ __forceinline__ void clip_poly(const EyeVtx& v0, const EyeVtx& v1, const EyeVtx& v2, uint32_t o0,
+                                          uint32_t o1, uint32_t o2, const SetupCtx& C, SetupPoly& P) {
+  P.np = 0;
   // Sutherland-Hodgman against z >= z_near, walking v0 -> v1 -> v2 -> v0.
   const float vx[3] = {v0.x, v1.x, v2.x}, vy[3] = {v0.y, v1.y, v2.y}, vz[3] = {v0.z, v1.z, v2.z};
   const bool in[3] = {(o0 & kOcBehind) == 0, (o1 & kOcBehind) == 0, (o2 & kOcBehind) == 0};
@@ -653,19 +641,23 @@ __device__ __forceinline__ TileBox footprint_tiles(const int32_t* bb, int tw, in
   return b;
 }
 
-// f(tile) for each tile of the box (relative to it) that a record's pixel box
-// overlaps; returns false, without calling f, when these are more than max_tiles.
+// The tiles of the box (relative to it) that a record's pixel box overlaps.
 // Shifts, not divisions: set-up of the stereo rig 25 -> 22 us.
+struct RecordTiles {
+  int x0, y0, x1, y1;
+};
+__device__ __forceinline__ RecordTiles record_tiles(int2 bb, const TileBox& b) {
+  return {max(((int)(int16_t)(bb.x & 0xffff) >> b.sw) - b.tx0, 0), max((bb.x >> (16 + b.sh)) - b.ty0, 0),
+          min(((int)(int16_t)(bb.y & 0xffff) >> b.sw) - b.tx0, b.ntx - 1), min((bb.y >> (16 + b.sh)) - b.ty0, b.nty - 1)};
+}
+// f(tile) for each of them; returns false, without calling f, when they are more than max_tiles.
 template <typename F>
 __device__ __forceinline__ bool for_record_tiles(int2 bb, const TileBox& b, int max_tiles, F&& f) {
-  const int x0 = max(((int)(int16_t)(bb.x & 0xffff) >> b.sw) - b.tx0, 0);
-  const int y0 = max((bb.x >> (16 + b.sh)) - b.ty0, 0);
-  const int x1 = min(((int)(int16_t)(bb.y & 0xffff) >> b.sw) - b.tx0, b.ntx - 1);
-  const int y1 = min((bb.y >> (16 + b.sh)) - b.ty0, b.nty - 1);
-  if (x0 > x1 || y0 > y1) return true;
-  if ((x1 - x0 + 1) * (y1 - y0 + 1) > max_tiles) return false;
-  for (int y = y0; y <= y1; ++y)
-    for (int x = x0; x <= x1; ++x) f(y * b.ntx + x);
+  const RecordTiles t = record_tiles(bb, b);
+  if (t.x0 > t.x1 || t.y0 > t.y1) return true;
+  if ((t.x1 - t.x0 + 1) * (t.y1 - t.y0 + 1) > max_tiles) return false;
+  for (int y = t.y0; y <= t.y1; ++y)
+    for (int x = t.x0; x <= t.x1; ++x) f(y * b.ntx + x);
   return true;
 }
 
@@ -890,7 +882,11 @@ __global__ void __launch_bounds__(kSetupBlock, MULTI ? 4 : 3) tri_setup_kernel(F
                         ? __fadd_rn(z0, __half2float(reinterpret_cast<const __half*>(A.depth)[gi]))
                         : __ldg(reinterpret_cast<const float*>(A.depth) + gi);
     const EyeVtx q = to_eye(__ldg(ta + vj), __ldg(tb + vk), z);
-    const uint32_t oc = q.z >= C.zn ? side_bits(q) : kOcBehind;
+    // snapped here, once per vertex, instead of by the up to six triangles around it (with 32-bit boxes and the
+    // plane's divisions for kept triangles only: stereo rig 29.2 -> 27.8 us, ovals 52 -> 50, a 256^2 eye 19.7 -> 18.2)
+    int32_t qx = 0, qy = 0;
+    uint32_t oc = kOcBehind;
+    if (q.z >= C.zn) oc = side_bits(q) | (snap_rn(q.x, q.y, q.z, C.fx, C.fy, C.cx, C.cy, qx, qy) ? 0u : kOcFar);
     EyeVtx p0, p1, p2;
     p0.x = __shfl_sync(0xffffffffu, q.x, l0); p0.y = __shfl_sync(0xffffffffu, q.y, l0); p0.z = __shfl_sync(0xffffffffu, q.z, l0);
     p1.x = __shfl_sync(0xffffffffu, q.x, l1); p1.y = __shfl_sync(0xffffffffu, q.y, l1); p1.z = __shfl_sync(0xffffffffu, q.z, l1);
@@ -899,10 +895,17 @@ __global__ void __launch_bounds__(kSetupBlock, MULTI ? 4 : 3) tri_setup_kernel(F
     const uint32_t o2 = __shfl_sync(0xffffffffu, oc, l2);
     const int j = cl_x * kClusterCells + tcx, k = cl_y * kClusterCells + tcy;
     SetupPoly P;
-    P.np = 0;
+#pragma unroll
+    for (int i = 0; i < 3; ++i) {
+      const int l = i == 0 ? l0 : i == 1 ? l1 : l2;
+      P.px[i] = __shfl_sync(0xffffffffu, qx, l);
+      P.py[i] = __shfl_sync(0xffffffffu, qy, l);
+    }
+    P.px[3] = P.px[2]; P.py[3] = P.py[2];
     // the outcodes only drop triangles that lie wholly behind the near plane or outside
     // the padded disk footprint, whose pixels never see this view
-    if (j < n_cell && k < n_cell && (o0 & o1 & o2) == 0) setup_poly(p0, p1, p2, o0, o1, o2, C, P);
+    P.np = j < n_cell && k < n_cell && (o0 & o1 & o2) == 0 && ((o0 | o1 | o2) & kOcFar) == 0 ? 3 : 0;
+    if (P.np && ((o0 | o1 | o2) & kOcBehind)) clip_poly(p0, p1, p2, o0, o1, o2, C, P);
     const int id = 2 * (k * n_cell + j) + half;
 #pragma unroll
     for (int f = 0; f < 2; ++f) {
@@ -912,7 +915,7 @@ __global__ void __launch_bounds__(kSetupBlock, MULTI ? 4 : 3) tri_setup_kernel(F
       bool kept = false;
       if (P.np >= f + 3) {
         const int32_t sx[3] = {P.px[0], P.px[f + 1], P.px[f + 2]}, sy[3] = {P.py[0], P.py[f + 1], P.py[f + 2]};
-        kept = setup_sub(sx, sy, C, t, tl);
+        kept = setup_sub(sx, sy, C, t, tl) && setup_plane(p0, p1, p2, t);
       }
       const uint32_t m = __ballot_sync(0xffffffffu, kept);
       if (m == 0) continue;
@@ -923,10 +926,12 @@ __global__ void __launch_bounds__(kSetupBlock, MULTI ? 4 : 3) tri_setup_kernel(F
       const bool fits = (int64_t)base + n <= A.pool_capacity;
       const int64_t at = (int64_t)base + __popc(m & below);
       if (kept && at < A.pool_capacity) {
-        t.ia = P.ia; t.ib = P.ib; t.ic = P.ic;
         t.id_tl = (id << 3) | tl;
         A.pool[at] = t;
-        if constexpr (MULTI) A.pool_owner[at] = e * A.n_views + v;
+        if constexpr (MULTI) {
+          A.pool_owner[at] = e * A.n_views + v;
+          A.pool_box[at] = *reinterpret_cast<const int2*>(&t);
+        }
       }
       if (lane == 0) {
         if (!fits) atomicOr(A.error_word, kErrPoolOverflow);
@@ -970,15 +975,23 @@ __global__ void __launch_bounds__(kSetupBlock, MULTI ? 4 : 3) tri_setup_kernel(F
 
 // Records of the call, a thread each (four at a time, their loads together): pass
 // 0 counts the bins' entries, pass 1 (after bin_scan_kernel) scatters the pool
-// indices through the cursors.
-template <int PASS>
+// indices through the cursors.  The boxes lie in an array of their own, 12 bytes
+// per record with the owner instead of a sector of the record and the owner: 64
+// renders of 256^2 meshes (36 M records) count 465 -> 340 us, scatter 695 -> 553,
+// their writing adds 50 us to the set-up.  SHARE: lanes whose records enter the same
+// bin share one addition and write neighbouring entries - for fine meshes, whose
+// neighbours meet in one tile: scatter 553 -> 455 us; counting, whose additions
+// return nothing, 340 -> 373 (kept apart), and triangles of several tiles, which the
+// warp then walks in step, count 35 -> 45 us at 128^2 meshes of a 256^2 eye.
+template <int PASS, bool SHARE>
 __global__ void __launch_bounds__(256) bin_records_kernel(FrameArgs A) {
   constexpr int U = 4;
   griddep_wait();
   griddep_release();
   const int64_t n = min((int64_t)*A.pool_counter, A.pool_capacity), step = (int64_t)gridDim.x * blockDim.x;
   const int sw = __ffs(A.tile_w) - 1, sh = __ffs(A.tile_h) - 1;
-  for (int64_t i0 = blockIdx.x * (int64_t)blockDim.x + threadIdx.x; i0 < n; i0 += U * step) {
+  const int lane = threadIdx.x & 31;
+  for (int64_t i0 = blockIdx.x * (int64_t)blockDim.x + threadIdx.x; i0 - lane < n; i0 += U * step) {
     int2 bb[U];
     int4 bins[U];  // bin_off, btx0 | bty0, bntx | bnty, big_base
 #pragma unroll
@@ -986,18 +999,45 @@ __global__ void __launch_bounds__(256) bin_records_kernel(FrameArgs A) {
       const int64_t i = i0 + u * step;
       bins[u].x = -1;
       if (i >= n) continue;
-      bb[u] = *reinterpret_cast<const int2*>(A.pool + i);
+      bb[u] = A.pool_box[i];
       bins[u] = *reinterpret_cast<const int4*>(&A.vrecs[A.pool_owner[i]].bin_off);
     }
 #pragma unroll
     for (int u = 0; u < U; ++u) {
-      if (bins[u].x < 0) continue;
-      const TileBox b = {(int16_t)(bins[u].y & 0xffff), bins[u].y >> 16, (int16_t)(bins[u].z & 0xffff), bins[u].z >> 16, sw, sh};
-      int* curs = A.bin_offsets + bins[u].x + b.ntx * b.nty + 1;
-      for_record_tiles(bb[u], b, INT32_MAX, [&](int tile) {
-        const int at = atomicAdd(&curs[tile], 1);
-        if (PASS == 1) A.bin_entries[at] = (int)(i0 + u * step);
-      });
+      RecordTiles T = {0, 0, -1, -1};
+      int ntx = 0, curs = 0;
+      if (bins[u].x >= 0) {
+        const TileBox b = {(int16_t)(bins[u].y & 0xffff), bins[u].y >> 16, (int16_t)(bins[u].z & 0xffff), bins[u].z >> 16, sw, sh};
+        T = record_tiles(bb[u], b);
+        ntx = b.ntx;
+        curs = bins[u].x + b.ntx * b.nty + 1;
+      }
+      if constexpr (!SHARE) {
+        for (int y = T.y0; y <= T.y1; ++y)
+          for (int x = T.x0; x <= T.x1; ++x) {
+            const int at = atomicAdd(&A.bin_offsets[curs + y * ntx + x], 1);
+            if (PASS == 1) A.bin_entries[at] = (int)(i0 + u * step);
+          }
+        continue;
+      }
+      int x = T.x0, y = T.y0;
+      bool has = T.x0 <= T.x1 && T.y0 <= T.y1;
+      while (__any_sync(0xffffffffu, has)) {
+        // lanes whose records enter the same bin here share one addition
+        const int key = has ? curs + y * ntx + x : -1 - lane;
+        const uint32_t same = __match_any_sync(0xffffffffu, key);
+        const int first = __ffs(same) - 1;
+        int at = 0;
+        if (has && lane == first) at = atomicAdd(&A.bin_offsets[key], __popc(same));
+        if (PASS == 1) {
+          at = __shfl_sync(0xffffffffu, at, first);
+          if (has) A.bin_entries[at + __popc(same & ((1u << lane) - 1u))] = (int)(i0 + u * step);
+        }
+        if (has && ++x > T.x1) {
+          x = T.x0;
+          has = ++y <= T.y1;
+        }
+      }
     }
   }
 }
@@ -1024,9 +1064,10 @@ cudaError_t launch_tri_setup(const FrameArgs& a, cudaStream_t s, bool pdl) {
   if (parts == 1) return launch_kernel(tri_setup_kernel<false>, grid, block, bytes, s, pdl, a, kBinSmemTiles);
   cudaError_t e = launch_kernel(tri_setup_kernel<true>, grid, block, 0, s, pdl, a, 0);
   const dim3 all(152 * 8);
-  if (e == cudaSuccess) e = launch_kernel(bin_records_kernel<0>, all, dim3(256), 0, s, pdl, a);
+  if (e == cudaSuccess) e = launch_kernel(bin_records_kernel<0, false>, all, dim3(256), 0, s, pdl, a);
   if (e == cudaSuccess) e = launch_kernel(bin_scan_kernel, dim3(a.n_views, a.n_eyes), block, 0, s, pdl, a);
-  if (e == cudaSuccess) e = launch_kernel(bin_records_kernel<1>, all, dim3(256), 0, s, pdl, a);
+  auto scatter = a.fine_mesh ? bin_records_kernel<1, true> : bin_records_kernel<1, false>;
+  if (e == cudaSuccess) e = launch_kernel(scatter, all, dim3(256), 0, s, pdl, a);
   return e;
 }
 

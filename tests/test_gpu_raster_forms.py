@@ -26,6 +26,8 @@ CASES = [
     (9, 64, 5, 1.2, (1100, 900), True),
     (40, 64, 33, 6.0, (90, 70), False),
     (40, 64, 33, 6.0, (24, 20), False),
+    (9, 64, 70, 1.2, (75, 53), False),
+    (9, 64, 70, 1.2, (311, 203), True),
 ]
 
 
@@ -124,23 +126,24 @@ def test_eyes_by_value_and_by_copy_draw_the_same(n):
     r.close()
 
 
-def _cap(views, size, grid, seed=3):
+def _cap(views, size, grid, seed=3, eye=(75, 53)):
     side = math.isqrt(views - 1) + 1
     lf = scene.build_light_field(scene.sphere_scene(seed, 8, forward_cone_deg=35.0),
                                  scene.cap_grid_directions(side, 40.0)[:views], size, size, 90.0, grid)
-    e = scene.head_pose_eyes(scene.SplitMix64(seed), 75, 53, 90.0, yaw_range=(-0.1, 0.1), pitch_deg=6.0, stereo=False)[0]
+    e = scene.head_pose_eyes(scene.SplitMix64(seed), eye[0], eye[1], 90.0, yaw_range=(-0.1, 0.1), pitch_deg=6.0, stereo=False)[0]
     return lf, e
 
 
-@pytest.mark.parametrize("grid,mesh", [(2, "f32"), (6, "f16"), (65, "f32"), (66, "f32"), (70, "f32"), (131, "f32")])
-def test_grids_of_one_and_of_several_parts_cover_as_the_oracle(grid, mesh):
+@pytest.mark.parametrize("grid,mesh,eye", [(2, "f32", (75, 53)), (6, "f16", (75, 53)), (65, "f32", (75, 53)), (66, "f32", (75, 53)),
+                                           (70, "f32", (75, 53)), (131, "f32", (75, 53)), (66, "f32", (311, 203))])
+def test_grids_of_one_and_of_several_parts_cover_as_the_oracle(grid, mesh, eye):
     pytest.importorskip("torch")
     import __graft_entry__
 
     __graft_entry__.build()
     import paper_1810_08860_gb300 as lfm
 
-    lf, e = _cap(9, 64, grid)
+    lf, e = _cap(9, 64, grid, eye=eye)
     if mesh == "f16":  # depths that FP16 offsets hold exactly: the oracle sees the same mesh
         lf.depth = (lf.depth * 8).round().clip(8, 48) / 8
         lf.depth = lf.depth.astype("float32")
