@@ -762,7 +762,14 @@ __device__ void bin_view(const FrameArgs& A, ViewRec& R, const int2* ranges, int
 
 constexpr int kSetupBlock = 256;
 constexpr int kPartClusters = kSetupPartClusters;
-static_assert(kPartClusters == kSetupBlock, "one thread per cluster in the first cull");
+static_assert(kPartClusters <= kSetupBlock, "one thread per cluster in the first cull");
+// A view of one part takes 512 threads where its list of clusters is long: the grid has at least 64 of them and few
+// enough views share the sphere (a footprint holds about a view's share of it).  Microseconds, 256 / 512 threads
+// (1024 in brackets): a batch of 64 eyes, 16 views of 32^2, 200 / 150; ovals, 256 views of 64^2, 50 / 42 (40); 512
+// views 31.5 / 26.6; 640 views 32 / 27.5; a 256^2 eye 18.5 / 17.5 (16.8), 731x517 17.6 / 16.5 (17.7).  Shorter lists
+// leave the second half idle: 1024 views of 64^2 28.2 / 29.8, 26 views of 23^2 14.6 / 15.2.
+constexpr int kWideBlock = 512;
+static bool long_lists(int n_views, int n_clusters) { return n_clusters >= 64 && n_views <= 3 * n_clusters; }
 
 // One block per (eye, view, part) whose disk footprint reaches the eye; a part
 // is kPartClusters clusters of 4x4 cells, the whole view for grids up to 65^2.
@@ -789,9 +796,9 @@ static_assert(kPartClusters == kSetupBlock, "one thread per cluster in the first
 // cluster that counts in the leader's shared memory (distributed shared memory
 // atomics), 256 views and a 400^2 eye took 20 us instead of 29, but the stereo rig
 // 30 to 128 us instead of 22 (1 to 8 blocks per view).
-template <bool MULTI>
-__global__ void __launch_bounds__(kSetupBlock, MULTI ? 4 : 3) tri_setup_kernel(FrameArgs A, int cnt_cap) {
-  constexpr int NW = kSetupBlock / 32;
+template <bool MULTI, int BLOCK>
+__global__ void __launch_bounds__(BLOCK, BLOCK > kSetupBlock ? 1024 / BLOCK : MULTI ? 4 : 3) tri_setup_kernel(FrameArgs A, int cnt_cap) {
+  constexpr int NW = BLOCK / 32;
   const int v = blockIdx.x, e = blockIdx.y;
   const int lane = threadIdx.x & 31, warp = threadIdx.x >> 5;
   // the view set-up has completed (it wrote the view records read below); the
@@ -843,7 +850,7 @@ __global__ void __launch_bounds__(kSetupBlock, MULTI ? 4 : 3) tri_setup_kernel(F
   {
     const int c = blockIdx.z * kPartClusters + threadIdx.x;
     bool keep = false;
-    if (c < ncl * ncl) {
+    if (threadIdx.x < kPartClusters && c < ncl * ncl) {
       const int cl_y = c / ncl, cl_x = c - cl_y * ncl;
       const float2 zr = __ldg(A.cluster_z + (int64_t)v * ncl * ncl + c);
       const int j = cl_x * kClusterCells, k = cl_y * kClusterCells;
@@ -945,7 +952,7 @@ __global__ void __launch_bounds__(kSetupBlock, MULTI ? 4 : 3) tri_setup_kernel(F
   // ---- (3) bins
   if constexpr (!MULTI) {
     if (threadIdx.x == 0) R.tri_count = s_total;
-    if (s_nrange > 0) bin_view<kSetupBlock>(A, R, s_range, s_nrange, reinterpret_cast<int*>(smem), cnt_cap, s_warp);
+    if (s_nrange > 0) bin_view<BLOCK>(A, R, s_range, s_nrange, reinterpret_cast<int*>(smem), cnt_cap, s_warp);
   } else {
     __shared__ int s_last;
     __shared__ long long s_off;
@@ -969,7 +976,7 @@ __global__ void __launch_bounds__(kSetupBlock, MULTI ? 4 : 3) tri_setup_kernel(F
     const TileBox t = footprint_tiles(R.bb, A.tile_w, A.tile_h);
     const int nt = t.ntx * t.nty;
     int* curs = A.bin_offsets + s_off + nt + 1;
-    for (int k = threadIdx.x; k < nt; k += kSetupBlock) curs[k] = 0;
+    for (int k = threadIdx.x; k < nt; k += BLOCK) curs[k] = 0;
   }
 }
 
@@ -1061,8 +1068,10 @@ cudaError_t launch_tri_setup(const FrameArgs& a, cudaStream_t s, bool pdl) {
   const int ncl = clusters_per_side(a.G);
   const int parts = (ncl * ncl + kPartClusters - 1) / kPartClusters;
   const dim3 grid(a.n_views, a.n_eyes, parts), block(kSetupBlock);
-  if (parts == 1) return launch_kernel(tri_setup_kernel<false>, grid, block, bytes, s, pdl, a, kBinSmemTiles);
-  cudaError_t e = launch_kernel(tri_setup_kernel<true>, grid, block, 0, s, pdl, a, 0);
+  if (parts == 1 && long_lists(a.n_views, ncl * ncl))
+    return launch_kernel(tri_setup_kernel<false, kWideBlock>, grid, dim3(kWideBlock), bytes, s, pdl, a, kBinSmemTiles);
+  if (parts == 1) return launch_kernel(tri_setup_kernel<false, kSetupBlock>, grid, block, bytes, s, pdl, a, kBinSmemTiles);
+  cudaError_t e = launch_kernel(tri_setup_kernel<true, kSetupBlock>, grid, block, 0, s, pdl, a, 0);
   const dim3 all(152 * 8);
   if (e == cudaSuccess) e = launch_kernel(bin_records_kernel<0, false>, all, dim3(256), 0, s, pdl, a);
   if (e == cudaSuccess) e = launch_kernel(bin_scan_kernel, dim3(a.n_views, a.n_eyes), block, 0, s, pdl, a);

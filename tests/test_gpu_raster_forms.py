@@ -26,6 +26,7 @@ CASES = [
     (9, 64, 5, 1.2, (1100, 900), True),
     (40, 64, 33, 6.0, (90, 70), False),
     (40, 64, 33, 6.0, (24, 20), False),
+    (200, 16, 33, 1.2, (90, 70), False),
     (9, 64, 70, 1.2, (75, 53), False),
     (9, 64, 70, 1.2, (311, 203), True),
 ]
