@@ -3,7 +3,7 @@
 //
 // A warp owns a screen tile (or one strip of it when a call has few tiles) and
 // draws it by itself, without block barriers, strip by strip: a strip is TW x
-// (2 * 32 / TW) pixels, two vertically adjacent pixels per lane, whose FP32
+// (kPx * 32 / TW) pixels, kPx (two or four) vertically adjacent pixels per lane, whose FP32
 // accumulators of Eq. 2's numerator and denominator stay in registers (the
 // paper's accumulation framebuffer becomes registers, and its second pass
 // becomes the epilogue).
@@ -26,9 +26,9 @@
 //
 // Bound by instruction issue (DRAM traffic is a few per cent of the peak), so
 // what counts is instructions per pixel and view.  Against one warp per strip
-// that listed, gathered and buffered winners by itself: 217 M -> 145 M warp
+// that listed, gathered and buffered winners by itself: 217 M -> 142 M warp
 // instructions on the stereo rig frame (1,024 views, 2 x 1440x1600, FP32), the raster
-// alone 293 -> 200 us; 3,772 -> 1,901 us for a batch of 64 eyes of the cap rig; 144 ->
+// alone 293 -> 205 us; 3,772 -> 1,898 us for a batch of 64 eyes of the cap rig; 144 ->
 // 82 us for a 1921x1083 eye with oval disks and FP8 texels.  Of that, reading a
 // column's slope and a row's terms from tables instead of dividing per pixel gives
 // 2,100 -> 2,011 us on the batch, and five blocks per SM at 96 registers instead of
@@ -96,13 +96,14 @@ template <> struct Texel<LF_TEX_FP8E4M3> {
 constexpr int kViewsPerRound = 32;  // views a warp handles per round (one per lane)
 constexpr int kWindow = 64;         // gathered triangles a warp holds at a time
 // Vertically adjacent pixels per lane: two, or four for a warp that takes a whole
-// tile of 256 pixels of small texels - a view's list, disk, triangles and constants
-// are then read half as often, and the wider accumulators still fit the registers.
-// Raster alone, two / four: BF16 stereo 1081x1203 119 / 109 us, FP8 ovals 1921x1083
-// 91 / 82, u8 stereo rig 214 / 194, FP32 stereo rig 200 / 198 (its texels' registers cancel the gain: two).  A
-// 256^2 eye, a strip per warp, 23 / 34: two.
-template <int TW, int TH, int FMT>
-constexpr int tile_px() { return TW * TH == 256 && FMT != LF_TEX_F32 ? 4 : 2; }
+// tile of 256 pixels - a view's list, disk, triangles and constants are then read
+// half as often.  Raster alone, two / four: BF16 stereo 1081x1203 119 / 109 us, FP8
+// ovals 1921x1083 91 / 82, u8 stereo rig 214 / 194, FP32 stereo rig 217 / 215 (its
+// texels' registers take most of the gain), 640 views of 512^2 in FP32 234 / 220, 256
+// views 204 / 195, the batch of 64 eyes 1,898 / 1,898.  A 256^2 eye, a strip per
+// warp, 23 / 34: two.
+template <int TW, int TH>
+constexpr int tile_px() { return TW * TH == 256 ? 4 : 2; }
 constexpr int kPxMax = 4;
 constexpr int kRasterWarps = 4;     // warps per block, each on its own work item
 // Calls with fewer tiles than the chip holds warps (152 SMs x 24) are split into
@@ -750,7 +751,7 @@ template <int TW, int TH, int FMT, bool OVAL>
 static cudaError_t launch_disk(const FrameArgs& a, bool inspect, bool persistent, int pblocks, cudaStream_t s,
                                bool pdl) {
   const bool whole_tiles = a.total_tiles >= kTileItemTiles;
-  if constexpr (tile_px<TW, TH, FMT>() == 4)
+  if constexpr (tile_px<TW, TH>() == 4)
     if (whole_tiles && !inspect) return launch_px<TW, TH, FMT, OVAL, 4>(a, true, false, persistent, pblocks, s, pdl);
   return launch_px<TW, TH, FMT, OVAL, 2>(a, whole_tiles, inspect, persistent, pblocks, s, pdl);
 }

@@ -61,8 +61,8 @@ def test_every_form_draws_the_inspection_image(views, size, grid, disk, eye, ova
     r.close()
 
 
-# Four pixels per lane: 256-pixel tiles of the narrow texture formats, in eyes of at least 3648 tiles (whole tiles).
-@pytest.mark.parametrize("fmt", ["u8", "bf16", "fp8"])
+# Four pixels per lane: 256-pixel tiles in eyes of at least 3648 tiles (whole tiles).
+@pytest.mark.parametrize("fmt", ["f32", "u8", "bf16", "fp8"])
 @pytest.mark.parametrize("tile", [(16, 16), (32, 8)])
 @pytest.mark.parametrize("views,grid,disk,oval", [(9, 5, 1.2, True), (40, 17, 6.0, False)])
 def test_wide_lanes_draw_the_inspection_image(fmt, tile, views, grid, disk, oval):
