@@ -783,7 +783,7 @@ static bool long_lists(int n_views, int n_clusters) { return n_clusters >= 64 &&
 //     outcodes, sets it up (snap, clip, orientation, fill rule) and the warp
 //     appends the kept records to the pool.
 // (3) MULTI = false (one part): the block bins the view's records.  MULTI = true:
-//     every record notes its (eye, view) in A.pool_owner, the last part of a view
+//     every record notes its (eye, view) and its box once more (A.pool_owner, A.pool_box), the last part of a view
 //     to finish reserves and clears its tile counts, and the bin_* kernels below
 //     count and scatter all records of the call, a thread each.
 // Bound by the latency of its phases (dependent loads, the pool's atomic, the
