@@ -838,15 +838,20 @@ __global__ void __launch_bounds__(BLOCK, BLOCK > kSetupBlock ? 1024 / BLOCK : MU
     q.z = __fmaf_rn(Mf[6], X, __fmaf_rn(Mf[7], Y, __fmaf_rn(Mf[8], z, Mf[11])));
     return q;
   };
-  auto side_bits = [&](const EyeVtx& q) -> uint32_t {
+  auto side_bits = [&](const EyeVtx& q, float mx, float my) -> uint32_t {  // beyond a side by more than a margin
     const float ux = C.fx * q.x, uy = C.fy * q.y;
-    return (ux < oxl * q.z ? 1u : 0u) | (ux > oxr * q.z ? 2u : 0u) | (uy < oyt * q.z ? 4u : 0u) |
-           (uy > oyb * q.z ? 8u : 0u);
+    return (ux < oxl * q.z - mx ? 1u : 0u) | (ux > oxr * q.z + mx ? 2u : 0u) | (uy < oyt * q.z - my ? 4u : 0u) |
+           (uy > oyb * q.z + my ? 8u : 0u);
   };
   __syncthreads();
 
   // ---- (1) clusters that can reach the footprint.  The half-spaces are linear, so
-  // what holds at the eight corners holds for every point between them.
+  // what holds at the eight corners holds for every point between them - but for the
+  // roundings: to_eye is within four of them, 2^-22 of the sum of its terms' sizes,
+  // at a corner and at a vertex, and the crossing of an edge with the near plane and
+  // the sides' products are within ten more.  The corners must be beyond a plane by
+  // 2^-19 of those sums, so that no cluster is dropped of which (2) would keep a triangle.
+  // (Without the margin, clusters whose vertices lie on the near plane within rounding were lost.)
   {
     const int c = blockIdx.z * kPartClusters + threadIdx.x;
     bool keep = false;
@@ -856,11 +861,21 @@ __global__ void __launch_bounds__(BLOCK, BLOCK > kSetupBlock ? 1024 / BLOCK : MU
       const int j = cl_x * kClusterCells, k = cl_y * kClusterCells;
       const float a[2] = {__ldg(ta + j), __ldg(ta + min(j + kClusterCells, n_cell))};
       const float b[2] = {__ldg(tb + k), __ldg(tb + min(k + kClusterCells, n_cell))};
+      const float am = fmaxf(fabsf(a[0]), fabsf(a[1])), bm = fmaxf(fabsf(b[0]), fabsf(b[1]));
+      const float zm = fmaxf(fabsf(zr.x), fabsf(zr.y));
+      float sum[3];  // per eye axis, the size of to_eye's terms
+#pragma unroll
+      for (int r = 0; r < 3; ++r)
+        sum[r] = zm * (fabsf(Mf[3 * r]) * am + fabsf(Mf[3 * r + 1]) * bm + fabsf(Mf[3 * r + 2])) + fabsf(Mf[9 + r]);
+      constexpr float kRound = 1.0f / (1 << 19);
+      const float mx = kRound * (C.fx * sum[0] + fmaxf(fabsf(oxl), fabsf(oxr)) * sum[2]);
+      const float my = kRound * (C.fy * sum[1] + fmaxf(fabsf(oyt), fabsf(oyb)) * sum[2]);
+      const float near = C.zn - kRound * sum[2];
       uint32_t oc = 31u;
 #pragma unroll
       for (int i = 0; i < 8; ++i) {
         const EyeVtx q = to_eye(a[i & 1], b[(i >> 1) & 1], i < 4 ? zr.x : zr.y);
-        oc &= side_bits(q) | (q.z < C.zn ? kOcBehind : 0u);
+        oc &= side_bits(q, mx, my) | (q.z < near ? kOcBehind : 0u);
       }
       keep = oc == 0u;
     }
@@ -893,7 +908,7 @@ __global__ void __launch_bounds__(BLOCK, BLOCK > kSetupBlock ? 1024 / BLOCK : MU
     // plane's divisions for kept triangles only: stereo rig 29.2 -> 27.8 us, ovals 52 -> 50, a 256^2 eye 19.7 -> 18.2)
     int32_t qx = 0, qy = 0;
     uint32_t oc = kOcBehind;
-    if (q.z >= C.zn) oc = side_bits(q) | (snap_rn(q.x, q.y, q.z, C.fx, C.fy, C.cx, C.cy, qx, qy) ? 0u : kOcFar);
+    if (q.z >= C.zn) oc = side_bits(q, 0.0f, 0.0f) | (snap_rn(q.x, q.y, q.z, C.fx, C.fy, C.cx, C.cy, qx, qy) ? 0u : kOcFar);
     EyeVtx p0, p1, p2;
     p0.x = __shfl_sync(0xffffffffu, q.x, l0); p0.y = __shfl_sync(0xffffffffu, q.y, l0); p0.z = __shfl_sync(0xffffffffu, q.z, l0);
     p1.x = __shfl_sync(0xffffffffu, q.x, l1); p1.y = __shfl_sync(0xffffffffu, q.y, l1); p1.z = __shfl_sync(0xffffffffu, q.z, l1);
