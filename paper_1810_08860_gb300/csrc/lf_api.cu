@@ -43,7 +43,7 @@ namespace {
 
 constexpr int kRing = 4;
 // Mesh cells narrower than this on the screen: a raster lane walks a triangle's
-// box (lf_raster.cu).  Raster alone, a lane per pixel / per triangle: 2.0-pixel
+// box (lf_raster_impl.h).  Raster alone, a lane per pixel / per triangle: 2.0-pixel
 // cells (a prefilter's dense model) 5.1 / 2.8 ms; 2.9-pixel cells 71 / 82 us.
 constexpr double kFineCellPx = 2.5;
 constexpr int kHostSlots = LF_HOST_FRAMES_IN_FLIGHT;
@@ -167,15 +167,32 @@ bool valid_tile(int w, int h) { return (w == 16 && h == 16) || (w == 32 && h == 
 
 struct Layout {
   int32_t total_tiles = 0;
+  int32_t fine_eyes = 0;    // eyes drawn a lane per triangle
   int64_t total_lines = 0;  // of the ray tables: per eye room for max(its rows, a quarter of its columns)
   std::vector<EyeParams> eyes;
 };
+
+// FrameArgs::fine_mesh of a call.
+inline int32_t fine_form(const Layout& L) { return L.fine_eyes == 0 ? 0 : L.fine_eyes == (int32_t)L.eyes.size() ? 1 : 2; }
 
 // Lines that an eye takes in the ray tables.
 inline int64_t ray_lines(const EyeParams& P) { return std::max(P.H, (P.W + 3) / 4); }
 
 // RGBA images are read and written as 16-byte texels.
 inline bool aligned16(const void* p) { return (reinterpret_cast<uintptr_t>(p) & 15u) == 0; }
+
+// Whether the loaded mesh's cells are so small on this eye's screen that the
+// raster walks triangles instead of pixels: cell width in eye pixels of a surface
+// seen from about the same distance by the eye and the view.  A value of speed
+// only, so the first view stands for all; but each eye of a call is judged by
+// itself: eyes of 256^2 and 2048^2 in one batch, 129^2 meshes of 16 views (2- and
+// 16-pixel cells), take 259 us, or 307 in the other order; where the first eye
+// decided for both, 440 and 446.
+int32_t fine_cells(const lf_ctx* c, const EyeParams& E) {
+  if (c->views_host.empty() || c->G < 2) return 0;
+  const double cell = (double)c->src_w / (c->G - 1) * E.fx / c->views_host[0].fx;
+  return cell < kFineCellPx ? 1 : 0;
+}
 
 lf_status make_layout(lf_ctx* c, int32_t n_eyes, const lf_pose* eyes, const lf_intrinsics* intr,
                       float* const* out, Layout& L) {
@@ -197,12 +214,13 @@ lf_status make_layout(lf_ctx* c, int32_t n_eyes, const lf_pose* eyes, const lf_i
     P.fx = K.fx; P.fy = K.fy; P.cx = K.cx; P.cy = K.cy;
     P.W = K.width; P.H = K.height;
     P.tiles_x = (K.width + c->cfg.tile_w - 1) / c->cfg.tile_w;
-    P.tiles_y = (K.height + c->cfg.tile_h - 1) / c->cfg.tile_h;
     P.tile_base = (int32_t)base;
     P.out = out[e];
     P.line_base = (int32_t)L.total_lines;
+    P.fine = fine_cells(c, P);
+    L.fine_eyes += P.fine;
     L.total_lines += ray_lines(P);
-    base += (int64_t)P.tiles_x * P.tiles_y;
+    base += (int64_t)P.tiles_x * ((K.height + c->cfg.tile_h - 1) / c->cfg.tile_h);
     if (base > (int64_t)1 << 30) return fail(c, LF_ERR_INVALID_ARG, "too many tiles");
   }
   L.total_tiles = (int32_t)base;
@@ -285,16 +303,6 @@ void use_counters(FrameArgs& a, unsigned char* block) {
   a.bin_entries_counter = reinterpret_cast<unsigned long long*>(block + 24);
 }
 
-// Whether the loaded mesh's cells are so small on this eye's screen that the
-// raster walks triangles instead of pixels (a value of speed only, so the first
-// view and the first eye of a call stand for all): cell width in eye pixels of a
-// surface seen from about the same distance by both.
-int32_t fine_mesh(const lf_ctx* c, const EyeParams& E) {
-  if (c->views_host.empty() || c->G < 2) return 0;
-  const double cell = (double)c->src_w / (c->G - 1) * E.fx / c->views_host[0].fx;
-  return cell < kFineCellPx ? 1 : 0;
-}
-
 FrameArgs frame_args(lf_ctx* c, const Layout& L) {
   FrameArgs a;
   std::memset(&a, 0, sizeof(a));
@@ -336,7 +344,8 @@ FrameArgs frame_args(lf_ctx* c, const Layout& L) {
   a.total_tiles = L.total_tiles;
   a.tile_w = c->cfg.tile_w;
   a.tile_h = c->cfg.tile_h;
-  if (!L.eyes.empty()) a.fine_mesh = fine_mesh(c, L.eyes[0]);
+  a.fine_mesh = fine_form(L);
+  a.fine_most = 2 * L.fine_eyes >= (int32_t)L.eyes.size();
   if (c->lv.n_fine > 0) {
     a.tex_table = static_cast<const void* const*>(c->lv.table.p);
     a.enable_bits = static_cast<uint32_t*>(c->lv.enable.p);
@@ -820,7 +829,7 @@ lf_status lf_render_batch(lf_ctx* c, int32_t n_eyes, const lf_pose* eyes, const 
                               (int64_t)(intptr_t)c->tex.p, (int64_t)(intptr_t)c->depth.p, c->persistent_blocks,
                               c->cfg.tile_w, c->cfg.tile_h, c->cfg.timing, c->disk_mode, c->lv.n_fine,
                               (int64_t)(intptr_t)c->lv.pool.p, (int64_t)(intptr_t)c->lv.enable.p,
-                              (int64_t)(intptr_t)c->lv.visible.p, fine_mesh(c, L.eyes[0])};
+                              (int64_t)(intptr_t)c->lv.visible.p, fine_form(L), 2 * L.fine_eyes >= n_eyes};
   for (int e = 0; e < n_eyes; ++e) { sig.push_back(intr[e].width); sig.push_back(intr[e].height); }
   cudaStream_t s = static_cast<cudaStream_t>(stream);
   if (c->cfg.timing) {
@@ -1119,10 +1128,10 @@ extern "C" lf_status lf_render_static(lf_ctx* c, const lf_pose* eye, const lf_in
   P.fx = K.fx; P.fy = K.fy; P.cx = K.cx; P.cy = K.cy;
   P.W = K.width; P.H = K.height;
   P.tiles_x = (K.width + c->cfg.tile_w - 1) / c->cfg.tile_w;
-  P.tiles_y = (K.height + c->cfg.tile_h - 1) / c->cfg.tile_h;
   P.tile_base = 0;
   P.out = out_rgba;
-  const int64_t tiles = (int64_t)P.tiles_x * P.tiles_y;
+  P.fine = fine_cells(c, P);
+  const int64_t tiles = (int64_t)P.tiles_x * ((K.height + c->cfg.tile_h - 1) / c->cfg.tile_h);
   if (tiles > kStaticMaxTiles)
     return fail(c, LF_ERR_CAPACITY, "lf_render_static: eye view has more than 8192 screen tiles");
   unsigned char* base = nullptr;
@@ -1135,7 +1144,7 @@ extern "C" lf_status lf_render_static(lf_ctx* c, const lf_pose* eye, const lf_in
   FrameArgs a = frame_args(c, none);
   a.n_eyes = 1;
   a.total_tiles = (int32_t)tiles;
-  a.fine_mesh = fine_mesh(c, P);
+  a.fine_mesh = a.fine_most = P.fine;
   a.eyes = reinterpret_cast<EyeParams*>(base + kOffEye);
   a.eyes_f = reinterpret_cast<EyeFloat*>(base + kOffEyeF);
   a.ray_cols = reinterpret_cast<float*>(base + kOffRayCols);

@@ -70,7 +70,8 @@ struct EyeParams {
   double t[3];
   double fx, fy, cx, cy;
   int32_t W, H;
-  int32_t tiles_x, tiles_y;
+  int32_t tiles_x;
+  int32_t fine;         // 1: the mesh cells take few pixels of this eye, a raster lane takes a triangle
   int32_t tile_base;    // first tile index of this eye in the call's flattened tile range
   int32_t line_base;    // first row of this eye in the call's ray rows (and first 4 columns in its ray columns)
   float* out;           // H x W float4
@@ -181,7 +182,8 @@ struct FrameArgs {
   uint32_t* texel_bits;
   // persistent batch raster
   int32_t* work_counter;
-  int32_t fine_mesh;       // 1: mesh cells of a few eye pixels, a raster lane takes a triangle
+  int32_t fine_mesh;       // mesh cells of a few pixels, a raster lane takes a triangle: 0 no eye, 1 every eye, 2 EyeParams::fine
+  int32_t fine_most;       // 1: most eyes' cells are, their bins are filled accordingly
   int32_t strips_per_item; // strips of a tile that a raster warp takes at a time (set by launch_raster)
   // two-level progressive rendering (all null / 0 with one level)
   const void* const* tex_table;  // per view: its texels (a pool page for fine views; null when not resident)

@@ -1090,7 +1090,7 @@ cudaError_t launch_tri_setup(const FrameArgs& a, cudaStream_t s, bool pdl) {
   const dim3 all(152 * 8);
   if (e == cudaSuccess) e = launch_kernel(bin_records_kernel<0, false>, all, dim3(256), 0, s, pdl, a);
   if (e == cudaSuccess) e = launch_kernel(bin_scan_kernel, dim3(a.n_views, a.n_eyes), block, 0, s, pdl, a);
-  auto scatter = a.fine_mesh ? bin_records_kernel<1, true> : bin_records_kernel<1, false>;
+  auto scatter = a.fine_most ? bin_records_kernel<1, true> : bin_records_kernel<1, false>;
   if (e == cudaSuccess) e = launch_kernel(scatter, all, dim3(256), 0, s, pdl, a);
   return e;
 }
