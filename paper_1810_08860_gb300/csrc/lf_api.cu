@@ -167,6 +167,7 @@ bool valid_tile(int w, int h) { return (w == 16 && h == 16) || (w == 32 && h == 
 
 struct Layout {
   int32_t total_tiles = 0;
+  int64_t near_tiles = 0;   // tiles within about 70 degrees of their eye's axis
   int32_t fine_eyes = 0;    // eyes drawn a lane per triangle
   int64_t total_lines = 0;  // of the ray tables: per eye room for max(its rows, a quarter of its columns)
   std::vector<EyeParams> eyes;
@@ -174,6 +175,28 @@ struct Layout {
 
 // FrameArgs::fine_mesh of a call.
 inline int32_t fine_form(const Layout& L) { return L.fine_eyes == 0 ? 0 : L.fine_eyes == (int32_t)L.eyes.size() ? 1 : 2; }
+
+// Tiles of an eye within about 70 degrees of its axis (of tangent 2.75).  Those beyond fill
+// most of a very tall or wide image but see next to nothing.
+inline int64_t near_tiles(const lf_config& cfg, const EyeParams& P) {
+  const auto along = [](double n, double f, int tile) { return (int64_t)std::ceil(std::min(n, 5.5 * f) / tile); };
+  return along(P.W, P.fx, cfg.tile_w) * along(P.H, P.fy, cfg.tile_h);
+}
+
+// FrameArgs::raster_form.  Sharing a tile's lists pays where there are warps enough without
+// splitting it, and several items per warp slot to even the tail out: the chip holds 20
+// raster warps per SM (3,040).  Whole passes, strips / halves / whole tiles (and, before
+// whole tiles were drawn at all, strips of a warp each): 16 views of a cap, FP32, 2,500
+// tiles (800^2) 44.6 / 49.3 / 54.5 us (58.6), 3,844 tiles 52.9 / 49.8 / 58.4 (67.6), 5,625
+// 63.4 / 56.5 / 62.5 (75.8), 10,000 87.0 / 74.6 / 71.8 (99.5); 100 views with wide disks,
+// 3,844 tiles 179 / 210 / 383 (332), 5,625 232 / 235 / 380 (407); 256 views of a sphere,
+// 3,844 tiles 92.5 / 82.2 / 83.9 (118), 5,625 114.4 / 98.3 / 94.0 (144), stereo rig (18,000)
+// 315 / 264 / 243 (368).  16 views, 250x16000 (16,000 tiles, 700 of them near the axis)
+// 73 / 80 / 106 (90).  Whole tiles from 24 per SM on lost to the older form where a few
+// tiles hold most of the work.
+inline int32_t raster_form(int64_t near, int sm_count) {
+  return near >= 36 * (int64_t)sm_count ? kRasterWhole : near >= 24 * (int64_t)sm_count ? kRasterHalves : kRasterStrips;
+}
 
 // Lines that an eye takes in the ray tables.
 inline int64_t ray_lines(const EyeParams& P) { return std::max(P.H, (P.W + 3) / 4); }
@@ -219,6 +242,7 @@ lf_status make_layout(lf_ctx* c, int32_t n_eyes, const lf_pose* eyes, const lf_i
     P.line_base = (int32_t)L.total_lines;
     P.fine = fine_cells(c, P);
     L.fine_eyes += P.fine;
+    L.near_tiles += near_tiles(c->cfg, P);
     L.total_lines += ray_lines(P);
     base += (int64_t)P.tiles_x * ((K.height + c->cfg.tile_h - 1) / c->cfg.tile_h);
     if (base > (int64_t)1 << 30) return fail(c, LF_ERR_INVALID_ARG, "too many tiles");
@@ -344,6 +368,7 @@ FrameArgs frame_args(lf_ctx* c, const Layout& L) {
   a.total_tiles = L.total_tiles;
   a.tile_w = c->cfg.tile_w;
   a.tile_h = c->cfg.tile_h;
+  a.raster_form = raster_form(L.near_tiles, c->sm_count);
   a.fine_mesh = fine_form(L);
   a.fine_most = 2 * L.fine_eyes >= (int32_t)L.eyes.size();
   if (c->lv.n_fine > 0) {
@@ -829,7 +854,8 @@ lf_status lf_render_batch(lf_ctx* c, int32_t n_eyes, const lf_pose* eyes, const 
                               (int64_t)(intptr_t)c->tex.p, (int64_t)(intptr_t)c->depth.p, c->persistent_blocks,
                               c->cfg.tile_w, c->cfg.tile_h, c->cfg.timing, c->disk_mode, c->lv.n_fine,
                               (int64_t)(intptr_t)c->lv.pool.p, (int64_t)(intptr_t)c->lv.enable.p,
-                              (int64_t)(intptr_t)c->lv.visible.p, fine_form(L), 2 * L.fine_eyes >= n_eyes};
+                              (int64_t)(intptr_t)c->lv.visible.p, fine_form(L), 2 * L.fine_eyes >= n_eyes,
+                              raster_form(L.near_tiles, c->sm_count)};
   for (int e = 0; e < n_eyes; ++e) { sig.push_back(intr[e].width); sig.push_back(intr[e].height); }
   cudaStream_t s = static_cast<cudaStream_t>(stream);
   if (c->cfg.timing) {
@@ -1144,6 +1170,7 @@ extern "C" lf_status lf_render_static(lf_ctx* c, const lf_pose* eye, const lf_in
   FrameArgs a = frame_args(c, none);
   a.n_eyes = 1;
   a.total_tiles = (int32_t)tiles;
+  a.raster_form = raster_form(near_tiles(c->cfg, P), c->sm_count);
   a.fine_mesh = a.fine_most = P.fine;
   a.eyes = reinterpret_cast<EyeParams*>(base + kOffEye);
   a.eyes_f = reinterpret_cast<EyeFloat*>(base + kOffEyeF);

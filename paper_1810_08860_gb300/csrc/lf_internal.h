@@ -136,6 +136,10 @@ struct GridTables {
   const float* b;   // n_views x G
 };
 
+// What a raster warp takes: a strip of a tile with two pixels per lane, a strip with four (half a tile of 256
+// pixels), or a whole tile with four.
+enum : int { kRasterStrips = 0, kRasterHalves = 1, kRasterWhole = 2 };
+
 struct FrameArgs {
   EyeParams* eyes;
   int32_t n_eyes;
@@ -184,6 +188,7 @@ struct FrameArgs {
   int32_t* work_counter;
   int32_t fine_mesh;       // mesh cells of a few pixels, a raster lane takes a triangle: 0 no eye, 1 every eye, 2 EyeParams::fine
   int32_t fine_most;       // 1: most eyes' cells are, their bins are filled accordingly
+  int32_t raster_form;     // kRasterStrips ..: what a raster warp takes at a time
   int32_t strips_per_item; // strips of a tile that a raster warp takes at a time (set by launch_raster)
   // two-level progressive rendering (all null / 0 with one level)
   const void* const* tex_table;  // per view: its texels (a pool page for fine views; null when not resident)

@@ -1,7 +1,7 @@
 // lf_raster_impl.h - the fragment stage: rasterise, depth test within each view,
 // fetch, weight, accumulate and normalise (Eq. 2, Sec. 4.2 and 4.2.2).
 //
-// A warp owns a screen tile (or one strip of it when a call has few tiles) and
+// A warp owns a screen tile (or one strip of it when a call has fewer tiles) and
 // draws it by itself, without block barriers, strip by strip: a strip is TW x
 // (kPx * 32 / TW) pixels, kPx (two or four) vertically adjacent pixels per lane, whose FP32
 // accumulators of Eq. 2's numerator and denominator stay in registers (the
@@ -95,23 +95,16 @@ template <> struct Texel<LF_TEX_FP8E4M3> {
 
 constexpr int kViewsPerRound = 32;  // views a warp handles per round (one per lane)
 constexpr int kWindow = 64;         // gathered triangles a warp holds at a time
-// Vertically adjacent pixels per lane: two, or four for a warp that takes a whole
-// tile of 256 pixels - a view's list, disk, triangles and constants are then read
-// half as often.  Raster alone, two / four: BF16 stereo 1081x1203 119 / 109 us, FP8
-// ovals 1921x1083 91 / 82, u8 stereo rig 214 / 194, FP32 stereo rig 217 / 215 (its
-// texels' registers take most of the gain), 640 views of 512^2 in FP32 234 / 220, 256
-// views 204 / 195, the batch of 64 eyes 1,898 / 1,898.  A 256^2 eye, a strip per
-// warp, 23 / 34: two.
+// Vertically adjacent pixels per lane: two, or four where a call has many tiles of 256
+// pixels (FrameArgs::raster_form) - a view's list, disk, triangles and constants are then
+// read half as often.  Whole tiles, raster alone, two / four: BF16 stereo 1081x1203 119 /
+// 109 us, FP8 ovals 1921x1083 91 / 82, u8 stereo rig 214 / 194, FP32 stereo rig 217 / 215
+// (its texels' registers take most of the gain), 640 views of 512^2 in FP32 234 / 220, 256
+// views 204 / 195, the batch of 64 eyes 1,898 / 1,898.
 template <int TW, int TH>
 constexpr int tile_px() { return TW * TH == 256 ? 4 : 2; }
 constexpr int kPxMax = 4;
 constexpr int kRasterWarps = 4;     // warps per block, each on its own work item
-// Calls with fewer tiles than the chip holds warps (152 SMs x 24) are split into
-// strips, one per warp: sharing a tile's lists then costs more than it saves,
-// since warps are missing.  Measured, whole passes, strips / tiles: 256 tiles
-// (256^2 eye) 65 / 118 us; 1,600 tiles (640^2) 100 / 125; 3,249 (900^2) 123 / 125;
-// 5,625 (1200^2) 158 / 146; 18,000 (stereo 1440x1600) 323 / 264.
-constexpr int kTileItemTiles = 152 * 24;
 
 // A warp's private shared memory: its view table and its window of triangles.
 // The triangle arrays are 16-byte columns, so the 32 lanes that store one
@@ -740,10 +733,9 @@ __global__ void __launch_bounds__(kRasterWarps * 32, 5) raster_kernel(FrameArgs 
 }
 
 template <int TW, int TH, int FMT, bool OVAL, int PX>
-static cudaError_t launch_px(FrameArgs a, bool whole_tiles, bool inspect, bool persistent, int pblocks, cudaStream_t s,
-                             bool pdl) {
+static cudaError_t launch_px(FrameArgs a, bool inspect, bool persistent, int pblocks, cudaStream_t s, bool pdl) {
   constexpr int STRIPS = TH / ((32 / TW) * PX);
-  a.strips_per_item = whole_tiles ? STRIPS : 1;
+  a.strips_per_item = a.raster_form == kRasterWhole ? STRIPS : 1;
   const int64_t items = (int64_t)a.total_tiles * (STRIPS / a.strips_per_item);
   const dim3 block(kRasterWarps * 32), grid((unsigned)((items + kRasterWarps - 1) / kRasterWarps));
   if constexpr (PX == 2)  // the inspection form: two pixels per lane only
@@ -755,10 +747,9 @@ static cudaError_t launch_px(FrameArgs a, bool whole_tiles, bool inspect, bool p
 template <int TW, int TH, int FMT, bool OVAL>
 static cudaError_t launch_disk(const FrameArgs& a, bool inspect, bool persistent, int pblocks, cudaStream_t s,
                                bool pdl) {
-  const bool whole_tiles = a.total_tiles >= kTileItemTiles;
   if constexpr (tile_px<TW, TH>() == 4)
-    if (whole_tiles && !inspect) return launch_px<TW, TH, FMT, OVAL, 4>(a, true, false, persistent, pblocks, s, pdl);
-  return launch_px<TW, TH, FMT, OVAL, 2>(a, whole_tiles, inspect, persistent, pblocks, s, pdl);
+    if (a.raster_form != kRasterStrips && !inspect) return launch_px<TW, TH, FMT, OVAL, 4>(a, false, persistent, pblocks, s, pdl);
+  return launch_px<TW, TH, FMT, OVAL, 2>(a, inspect, persistent, pblocks, s, pdl);
 }
 
 template <int TW, int TH, int FMT>
