@@ -1,7 +1,7 @@
 """The share of the image that a raster warp takes changes with the number of tiles near the
 eye's axis: strips of a tile, half tiles, whole tiles.  Rows added far from the axis, where there
-is nothing to see, must not take a multiple of the time (drawing whole tiles in every call of 3,648
-tiles and more made it 1.85 times here, 1.2 times the form before it; about 1.45 are the rows' own)."""
+is nothing to see, must not change the time by more than their writing (1,488 tiles of background,
+a few per cent; drawing whole tiles in every call of 3,648 tiles and more made it 1.46 times here)."""
 import pytest
 
 import scene
@@ -11,7 +11,7 @@ pytestmark = pytest.mark.gpu
 
 
 def test_rows_far_from_the_axis_cost_what_they_write():
-    """2,512 and 16,000 tiles, as much to see in each."""
+    """2,512 and 4,000 tiles, as much to see in each."""
     torch = pytest.importorskip("torch")
     import __graft_entry__
 
@@ -24,7 +24,7 @@ def test_rows_far_from_the_axis_cost_what_they_write():
     r.load_views(lf)
     r.build_meshes(lf)
     ms = []
-    for h in (2500, 16000):
+    for h in (2500, 4000):
         E = _eyes(1, 250, h, 125.0)
         out = [torch.empty((e.height, e.width, 4), device="cuda") for e in E]
         best = float("inf")
@@ -41,7 +41,7 @@ def test_rows_far_from_the_axis_cost_what_they_write():
         ms.append(best)
     r.stats()
     r.close()
-    assert ms[1] < 1.75 * ms[0], ms
+    assert ms[1] < 1.25 * ms[0], ms
 
 
 @pytest.mark.parametrize("tile", [(16, 16), (32, 8), (8, 8)])
