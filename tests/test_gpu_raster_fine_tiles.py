@@ -1,6 +1,6 @@
 """Fine meshes (cells below 2.5 eye pixels: a raster lane takes a triangle) in calls of at least
-3,648 tiles, where a warp draws whole tiles with four pixels per lane: strips that share a resident
-round whose bins exceed a window, several rounds of views, one and several set-up blocks per view,
+3,648 tiles, where a warp draws half tiles with four pixels per lane, and of at least 5,472, where it
+draws whole ones: strips that share a resident round whose bins exceed a window, several rounds of views, one and several set-up blocks per view,
 plain and persistent grids.  The reference is the inspection render, which takes a lane per pixel;
 the arithmetic is the same, so the images are compared bit for bit."""
 import math
@@ -21,13 +21,16 @@ def _eyes(n, w, h, f):
 
 
 # views, grid, disk scale, ovals, eyes (number, width, height, focal length): cells of 2.0 pixels
-# (16 eyes of 4,096 tiles) and 1.9 pixels (one eye of 3,933 tiles; 4,972 of 32 x 8 pixels)
+# (16 eyes of 4,096 tiles, 22 of 5,632) and 1.6 and 1.9 pixels (one eye of 3,933 or 6,688 tiles)
 @pytest.mark.parametrize("views,grid,disk,oval,eyes", [
     (9, 129, 1.2, False, (16, 256, 250, 128.0)),
     (9, 65, 1.2, True, (16, 256, 250, 64.0)),
     (40, 65, 6.0, False, (16, 256, 250, 64.0)),
     (9, 257, 1.2, False, (1, 1100, 901, 240.0)),
-    (40, 129, 6.0, True, (1, 1100, 901, 120.0)),
+    (40, 257, 6.0, True, (1, 1100, 901, 210.0)),
+    (9, 129, 1.2, True, (22, 256, 250, 128.0)),
+    (40, 65, 6.0, False, (22, 256, 250, 64.0)),
+    (9, 257, 1.2, False, (1, 1400, 1203, 240.0)),
 ])
 @pytest.mark.parametrize("tile", [(16, 16), (32, 8)])
 @pytest.mark.parametrize("fmt", ["f32", "u8"])
