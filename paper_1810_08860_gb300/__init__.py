@@ -220,8 +220,12 @@ _EYE_INTR = struct.Struct("4d2i")  # lf_intrinsics
 def _stream_handle(stream):
     import torch
     if stream is None:
-        # the current stream's handle as it is: a torch.cuda.Stream built around it takes 3.6 us a call
-        return ctypes.c_void_p(torch._C._cuda_getCurrentRawStream(torch.cuda.current_device()))
+        # the current stream's handle as it is, where this PyTorch has the call: a torch.cuda.Stream built around it
+        # takes 3.6 us a call
+        raw = getattr(torch._C, "_cuda_getCurrentRawStream", None)
+        if raw is not None:
+            return ctypes.c_void_p(raw(torch.cuda.current_device()))
+        stream = torch.cuda.current_stream()
     return ctypes.c_void_p(stream.cuda_stream)
 
 
