@@ -198,7 +198,8 @@ inline int32_t raster_form(int64_t near, int sm_count) {
   return near >= 36 * (int64_t)sm_count ? kRasterWhole : near >= 24 * (int64_t)sm_count ? kRasterHalves : kRasterStrips;
 }
 
-// Lines that an eye takes in the ray tables.
+// Lines that an eye takes in the ray tables: at most a tile's height (or a quarter of its width) per tile, and kMaxEyeLines.
+constexpr int64_t kMaxEyeLines = 32768;
 inline int64_t ray_lines(const EyeParams& P) { return std::max(P.H, (P.W + 3) / 4); }
 
 // RGBA images are read and written as 16-byte texels.
@@ -267,8 +268,12 @@ int64_t bin_entries_capacity(const lf_ctx* c, int64_t total_tiles) {
 
 lf_status ensure_scratch(lf_ctx* c, const Layout& L) {
   const int32_t n_eyes = (int32_t)L.eyes.size(), total_tiles = L.total_tiles;
-  LF_CUDA(c, ensure(c->ray_cols, sizeof(float) * 4 * (size_t)L.total_lines));
-  LF_CUDA(c, ensure(c->ray_rows, sizeof(float4) * (size_t)L.total_lines));
+  // The ray tables' room follows from eyes and tiles alone, as the other scratch does: a call of no more of either than
+  // one before it allocates nothing, whatever its images' shapes (it can be captured).  At most 1 MB per eye.
+  const int64_t lines = std::min<int64_t>((int64_t)total_tiles * std::max(c->cfg.tile_h, c->cfg.tile_w / 4),
+                                          (int64_t)n_eyes * kMaxEyeLines);
+  LF_CUDA(c, ensure(c->ray_cols, sizeof(float) * 4 * (size_t)lines));
+  LF_CUDA(c, ensure(c->ray_rows, sizeof(float4) * (size_t)lines));
   LF_CUDA(c, ensure(c->eyes, sizeof(EyeParams) * (size_t)c->cfg.max_eyes));
   LF_CUDA(c, ensure(c->eyes_f, sizeof(EyeFloat) * (size_t)c->cfg.max_eyes));
   LF_CUDA(c, ensure(c->vrecs, sizeof(ViewRec) * (size_t)n_eyes * c->n_views));
@@ -1091,8 +1096,7 @@ constexpr size_t align256(size_t x) { return (x + 255) & ~(size_t)255; }
 constexpr size_t kOffCounters = 0;
 constexpr size_t kOffEye = align256(kOffCounters + 64);
 constexpr size_t kOffEyeF = align256(kOffEye + sizeof(EyeParams));
-// ray tables: the widest and the tallest eye of at most 8192 tiles of 32 pixels, or the largest eye
-constexpr size_t kStaticLines = 32768;
+constexpr size_t kStaticLines = kMaxEyeLines;  // ray tables of one eye
 constexpr size_t kOffRayCols = align256(kOffEyeF + sizeof(EyeFloat));
 constexpr size_t kOffRayRows = align256(kOffRayCols + sizeof(float) * 4 * kStaticLines);
 constexpr size_t kOffVrecs = align256(kOffRayRows + sizeof(float4) * kStaticLines);
