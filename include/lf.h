@@ -95,8 +95,9 @@ typedef struct {
   int32_t tile_w, tile_h;   /* screen tile in pixels: 16x16, 32x8 or 8x8 [16x16] */
   int32_t max_eyes;         /* eyes per lf_render / lf_render_batch call [2] */
   int32_t timing;           /* 1: bracket each kernel with CUDA events on the call's stream [0] */
-  int64_t tri_capacity;     /* set-up triangle records per call [8 Mi]; the triangle
-                               bins get max(4 x this, 32 per screen tile) entries */
+  int64_t tri_capacity;     /* set-up triangle records per call [8 Mi]: 48 bytes each, 60 with
+                               mesh grids above 65 x 65; the triangle bins get
+                               max(4 x this, 32 per screen tile) entries */
   float z_near;             /* eye-space near clip plane in metres [0.1] */
   int32_t pad1;
   int64_t wait_limit;       /* bound in nanoseconds (%globaltimer) on each device wait - the

@@ -1,7 +1,7 @@
 // lf_api.cu - host side of the C ABI declared in include/lf.h: context,
 // uploads, per-call parameter staging, kernel sequencing, CUDA-graph replay of
 // batched calls, and statistics.  All arithmetic of the rendering method runs
-// in the kernels of lf_setup.cu and lf_raster.cu.
+// in the kernels of lf_setup.cu and lf_raster_impl.h.
 #include <cuda_runtime.h>
 
 #include <algorithm>

@@ -15,6 +15,8 @@
 //   EyeFloat[n_eyes]              the eye's FP32 constants (rounded once, on the device)
 //   ray columns / ray rows        the eyes' ray slopes by column and ray terms by row
 //   TriRec pool                   set-up (sub-)triangles, in runs of one 4x4-cell cluster
+//   pool owners, pool boxes       grids of more than 256 clusters (65^2 vertices): 12 bytes more
+//                                 per record, its eye and view and its pixel box once more
 //   bin offsets / bin entries     per (eye, view): its triangles binned into the screen
 //                                 tiles of its footprint (pool indices), plus a list of
 //                                 triangles spanning more than bin_max_tiles tiles
@@ -32,7 +34,6 @@
 
 namespace lfk {
 
-constexpr int kMaxTileThreads = 256;
 constexpr int kSnapLimit = 1 << 29;     // |snapped| must stay below 2^29 subpixels
 constexpr int kBigEdge = 1 << 22;       // edge deltas from 2^22 subpixels use the int64 path
 constexpr int kQClamp = 1 << 28;        // clamp of the per-tile edge offset in the int32 path
@@ -100,7 +101,7 @@ struct __align__(16) ViewRec {
   int16_t btx0, bty0, bntx, bnty;  // the tiles of the footprint box
   int32_t big_base;     // entries of the triangles spanning more than kBinMaxTiles tiles
   int32_t big_count;
-  int32_t tri_count;    // its set-up triangles
+  int32_t tri_count;    // its set-up triangles (grids of several parts)
   int32_t parts_done;   // set-up blocks of a grid of several parts that have finished
   int32_t pad;
   int32_t bb[4];        // conservative footprint in pixels, inclusive; bb[0] > bb[2] when empty
@@ -128,7 +129,7 @@ constexpr int kMaxGridForSetup = 257;    // triangle ids and the cluster grid ar
 
 constexpr int kSetupPartClusters = 256;  // clusters a triangle set-up block takes (a view of more is split into parts)
 
-// Clusters per side of a mesh grid, and whether its set-up takes several blocks per view.
+// Clusters per side of a mesh grid.
 __host__ __device__ constexpr int clusters_per_side(int G) { return (G - 1 + kClusterCells - 1) / kClusterCells; }
 
 struct GridTables {

@@ -32,7 +32,9 @@
 // 82 us for a 1921x1083 eye with oval disks and FP8 texels.  Of that, reading a
 // column's slope and a row's terms from tables instead of dividing per pixel gives
 // 2,100 -> 2,011 us on the batch, and five blocks per SM at 96 registers instead of
-// six at 80 (which spill) 2,011 -> 1,901.
+// six at 80 2,011 -> 1,901.  With four pixels per lane 96 registers are too few as well
+// (110 bytes of spills stored and 168 loaded per thread, round disks; 118 and 176 with the
+// batch's work counter; two pixels 8 and 12).
 //
 // Included by the lf_raster_<format>.cu files, a texture format each (compiled side by
 // side), and by lf_raster.cu for what the view selection shares.
@@ -810,6 +812,8 @@ cudaError_t launch_raster_fmt<LF_RASTER_FORMAT>(const FrameArgs& a, bool inspect
   return cudaErrorInvalidValue;
 }
 
+// Both forms of a tile (two and four pixels per lane) have the same launch bounds, 96 registers and the same shared
+// memory, so one answers for the other: five blocks per SM.
 template <int TW, int TH, int FMT>
 static cudaError_t occupancy_tile(int disk_mode, int* n) {
   constexpr int kThreads = kRasterWarps * 32;

@@ -504,7 +504,6 @@ constexpr uint32_t kOcFar = 32;     // in front of it, but its snapped coordinat
 
 struct SetupCtx {
   float fx, fy, cx, cy, zn;
-  int W, H;
   int bb0, bb1, bb2, bb3;
 };
 
@@ -811,7 +810,6 @@ __global__ void __launch_bounds__(BLOCK, BLOCK > kSetupBlock ? 1024 / BLOCK : MU
   if (C.bb0 > C.bb2 || C.bb1 > C.bb3) return;  // disk footprint misses the eye
   // a two-level frame sets up only the views the eye draws
   if (A.enable_bits && !((A.enable_bits[(int64_t)e * A.mask_words + (v >> 5)] >> (v & 31)) & 1u)) return;
-  const EyeParams& E = A.eyes[e];
   const EyeFloat& EF = A.eyes_f[e];
   const int G = A.G, n_cell = G - 1, ncl = clusters_per_side(G);
   extern __shared__ __align__(16) unsigned char smem[];  // the binning's per-tile counts
@@ -821,7 +819,7 @@ __global__ void __launch_bounds__(BLOCK, BLOCK > kSetupBlock ? 1024 / BLOCK : MU
   __shared__ int s_nlist, s_nrange, s_total;
   if (threadIdx.x == 0) s_nlist = s_nrange = s_total = 0;
   C.fx = EF.fx; C.fy = EF.fy; C.cx = EF.cx; C.cy = EF.cy;
-  C.zn = A.z_near; C.W = E.W; C.H = E.H;
+  C.zn = A.z_near;
   // outcode planes in the form fx*x <op> (edge - cx) * z, padded by 2 pixels
   const float oxl = (float)C.bb0 - 2.0f - C.cx, oxr = (float)C.bb2 + 3.0f - C.cx;
   const float oyt = (float)C.bb1 - 2.0f - C.cy, oyb = (float)C.bb3 + 3.0f - C.cy;
@@ -957,7 +955,7 @@ __global__ void __launch_bounds__(BLOCK, BLOCK > kSetupBlock ? 1024 / BLOCK : MU
       }
       if (lane == 0) {
         if (!fits) atomicOr(A.error_word, kErrPoolOverflow);
-        atomicAdd(&s_total, n);
+        if (MULTI) atomicAdd(&s_total, n);
         if (!MULTI && fits) s_range[atomicAdd(&s_nrange, 1)] = make_int2((int)base, n);
       }
     }
@@ -966,7 +964,6 @@ __global__ void __launch_bounds__(BLOCK, BLOCK > kSetupBlock ? 1024 / BLOCK : MU
 
   // ---- (3) bins
   if constexpr (!MULTI) {
-    if (threadIdx.x == 0) R.tri_count = s_total;
     if (s_nrange > 0) bin_view<BLOCK>(A, R, s_range, s_nrange, reinterpret_cast<int*>(smem), cnt_cap, s_warp);
   } else {
     __shared__ int s_last;
@@ -1007,6 +1004,7 @@ __global__ void __launch_bounds__(BLOCK, BLOCK > kSetupBlock ? 1024 / BLOCK : MU
 // warp then walks in step, count 35 -> 45 us at 128^2 meshes of a 256^2 eye.
 template <int PASS, bool SHARE>
 __global__ void __launch_bounds__(256) bin_records_kernel(FrameArgs A) {
+  static_assert(PASS == 1 || !SHARE, "only the scatter shares additions");
   constexpr int U = 4;
   griddep_wait();
   griddep_release();
@@ -1051,10 +1049,8 @@ __global__ void __launch_bounds__(256) bin_records_kernel(FrameArgs A) {
         const int first = __ffs(same) - 1;
         int at = 0;
         if (has && lane == first) at = atomicAdd(&A.bin_offsets[key], __popc(same));
-        if (PASS == 1) {
-          at = __shfl_sync(0xffffffffu, at, first);
-          if (has) A.bin_entries[at + __popc(same & ((1u << lane) - 1u))] = (int)(i0 + u * step);
-        }
+        at = __shfl_sync(0xffffffffu, at, first);
+        if (has) A.bin_entries[at + __popc(same & ((1u << lane) - 1u))] = (int)(i0 + u * step);
         if (has && ++x > T.x1) {
           x = T.x0;
           has = ++y <= T.y1;
