@@ -594,7 +594,7 @@ REFINE_FLOP_PER_PX = 2 * (27 * 32 + 288 * 32 + 288 * 3)  # 21,888: the three con
 # A training step per pixel: the forward pass, dL/d(input) of layers 3 and 2 (layer 1's is not needed),
 # and the three layers' weight gradients, as multiply-adds x 2 (63,936).
 TRAIN_FLOP_PER_PX = 2 * ((27 * 32 + 288 * 32 + 288 * 3) + (27 * 32 + 288 * 32) + (27 * 32 + 288 * 32 + 288 * 3))
-TRAIN_LAUNCHES_PER_STEP = 13  # count, 3 convolutions, 3 weight gradients, 2 backward convolutions, 3 reductions, Adam, pack
+TRAIN_LAUNCHES_PER_STEP = 12  # count, 3 convolutions, 3 weight gradients, 2 backward convolutions, reduction, Adam, pack
 
 
 def measured_tensor_peak():
