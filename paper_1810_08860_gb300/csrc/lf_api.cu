@@ -167,7 +167,7 @@ bool valid_tile(int w, int h) { return (w == 16 && h == 16) || (w == 32 && h == 
 
 struct Layout {
   int32_t total_tiles = 0;
-  int64_t near_tiles = 0;   // tiles within about 70 degrees of their eye's axis
+  int32_t form = kRasterStrips, mixed_items = 0;  // FrameArgs::raster_form, ::mixed_items
   int32_t fine_eyes = 0;    // eyes drawn a lane per triangle
   int64_t total_lines = 0;  // of the ray tables: per eye room for max(its rows, a quarter of its columns)
   std::vector<EyeParams> eyes;
@@ -194,8 +194,43 @@ inline int64_t near_tiles(const lf_config& cfg, const EyeParams& P) {
 // 315 / 264 / 243 (368).  16 views, 250x16000 (16,000 tiles, 700 of them near the axis)
 // 73 / 80 / 106 (90).  Whole tiles from 24 per SM on lost to the older form where a few
 // tiles hold most of the work.
-inline int32_t raster_form(int64_t near, int sm_count) {
-  return near >= 36 * (int64_t)sm_count ? kRasterWhole : near >= 24 * (int64_t)sm_count ? kRasterHalves : kRasterStrips;
+inline int32_t raster_form(double near, int sm_count) {
+  return near >= 36.0 * sm_count ? kRasterWhole : near >= 24.0 * sm_count ? kRasterHalves : kRasterStrips;
+}
+
+// The eyes' forms, and FrameArgs::raster_form and mixed_items.  A tile's work is taken as 1 (its
+// pixels) and its solid angle over kTileAngle (the views and triangles it meets); an eye is
+// judged by how many of its tiles the call's work would make.  By itself, or among its like, that is
+// their number; beside large images, a tile of a small one holds the work of many and, drawn whole,
+// the call would wait for it.  Whole passes, whole tiles for all / by eye (and the older strips of a
+// warp each), 48^2 + 1200^2 pixels: 16 views of a cap 194 / 108 us (221), 256 of a sphere 316 / 126
+// (206); 256^2 + 1200^2: 90 / 60 (73) and 92 / 98 (131); 4 x 256^2 + 4 x 1024^2, 65^2 meshes 210 / 153 (192).
+// Over 300 such calls in all, 0.70 of the time; with 0.006 two were slower than the older form, with
+// 0.002 images of about one size are split needlessly.
+constexpr double kTileAngle = 0.004;
+void set_forms(const lf_ctx* c, Layout& L) {
+  const auto weight = [&](const EyeParams& P) { return 1.0 + c->cfg.tile_w / P.fx * c->cfg.tile_h / P.fy / kTileAngle; };
+  double near = 0, work = 0;
+  for (const EyeParams& P : L.eyes) {
+    const double n = (double)near_tiles(c->cfg, P);
+    near += n;
+    work += n * weight(P);
+  }
+  const int32_t form = raster_form(near, c->sm_count);
+  L.form = form;
+  int64_t items = 0;
+  bool differ = false;
+  for (EyeParams& P : L.eyes) {
+    const int32_t f = std::min(form, raster_form(work / weight(P) * (1 + 1e-9), c->sm_count));
+    P.form = f | (near_tiles(c->cfg, P) <= c->sm_count ? kEyeFew : 0);
+    P.item_base = (int32_t)std::min<int64_t>(items, INT32_MAX);
+    const int64_t tiles = (int64_t)P.tiles_x * ((P.H + c->cfg.tile_h - 1) / c->cfg.tile_h);
+    items += tiles * (f == kRasterStrips ? 4 : f == kRasterHalves ? 2 : 1);
+    differ |= f != form;
+  }
+  if (!differ || c->cfg.tile_w * c->cfg.tile_h != 256 || items > INT32_MAX) return;
+  L.form = kRasterMixed;
+  L.mixed_items = (int32_t)items;
 }
 
 // Lines that an eye takes in the ray tables: at most a tile's height (or a quarter of its width) per tile, and kMaxEyeLines.
@@ -243,12 +278,12 @@ lf_status make_layout(lf_ctx* c, int32_t n_eyes, const lf_pose* eyes, const lf_i
     P.line_base = (int32_t)L.total_lines;
     P.fine = fine_cells(c, P);
     L.fine_eyes += P.fine;
-    L.near_tiles += near_tiles(c->cfg, P);
     L.total_lines += ray_lines(P);
     base += (int64_t)P.tiles_x * ((K.height + c->cfg.tile_h - 1) / c->cfg.tile_h);
     if (base > (int64_t)1 << 30) return fail(c, LF_ERR_INVALID_ARG, "too many tiles");
   }
   L.total_tiles = (int32_t)base;
+  set_forms(c, L);
   return LF_OK;
 }
 
@@ -373,7 +408,8 @@ FrameArgs frame_args(lf_ctx* c, const Layout& L) {
   a.total_tiles = L.total_tiles;
   a.tile_w = c->cfg.tile_w;
   a.tile_h = c->cfg.tile_h;
-  a.raster_form = raster_form(L.near_tiles, c->sm_count);
+  a.raster_form = L.form;
+  a.mixed_items = L.mixed_items;
   a.fine_mesh = fine_form(L);
   a.fine_most = 2 * L.fine_eyes >= (int32_t)L.eyes.size();
   if (c->lv.n_fine > 0) {
@@ -860,7 +896,7 @@ lf_status lf_render_batch(lf_ctx* c, int32_t n_eyes, const lf_pose* eyes, const 
                               c->cfg.tile_w, c->cfg.tile_h, c->cfg.timing, c->disk_mode, c->lv.n_fine,
                               (int64_t)(intptr_t)c->lv.pool.p, (int64_t)(intptr_t)c->lv.enable.p,
                               (int64_t)(intptr_t)c->lv.visible.p, fine_form(L), 2 * L.fine_eyes >= n_eyes,
-                              raster_form(L.near_tiles, c->sm_count)};
+                              L.form, L.mixed_items};
   for (int e = 0; e < n_eyes; ++e) { sig.push_back(intr[e].width); sig.push_back(intr[e].height); }
   cudaStream_t s = static_cast<cudaStream_t>(stream);
   if (c->cfg.timing) {
@@ -1161,6 +1197,8 @@ extern "C" lf_status lf_render_static(lf_ctx* c, const lf_pose* eye, const lf_in
   P.tile_base = 0;
   P.out = out_rgba;
   P.fine = fine_cells(c, P);
+  const int64_t near = near_tiles(c->cfg, P);
+  P.form = raster_form((double)near, c->sm_count) | (near <= c->sm_count ? kEyeFew : 0);
   const int64_t tiles = (int64_t)P.tiles_x * ((K.height + c->cfg.tile_h - 1) / c->cfg.tile_h);
   if (tiles > kStaticMaxTiles)
     return fail(c, LF_ERR_CAPACITY, "lf_render_static: eye view has more than 8192 screen tiles");
@@ -1174,7 +1212,7 @@ extern "C" lf_status lf_render_static(lf_ctx* c, const lf_pose* eye, const lf_in
   FrameArgs a = frame_args(c, none);
   a.n_eyes = 1;
   a.total_tiles = (int32_t)tiles;
-  a.raster_form = raster_form(near_tiles(c->cfg, P), c->sm_count);
+  a.raster_form = P.form & 3;
   a.fine_mesh = a.fine_most = P.fine;
   a.eyes = reinterpret_cast<EyeParams*>(base + kOffEye);
   a.eyes_f = reinterpret_cast<EyeFloat*>(base + kOffEyeF);

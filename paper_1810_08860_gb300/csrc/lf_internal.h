@@ -66,6 +66,10 @@ struct ViewStatic {
   float disk_ext[4];    // oval extents (+u, -u, +v, -v) in metres when ovals are set
 };
 
+// What a raster warp takes: a strip of a tile with two pixels per lane, a strip with four (half a tile of 256
+// pixels), or a whole tile with four; by call, or by eye where the eyes of a call differ (kRasterMixed).
+enum : int { kRasterStrips = 0, kRasterHalves = 1, kRasterWhole = 2, kRasterMixed = 3, kEyeFew = 4 };
+
 struct EyeParams {
   double R[9];
   double t[3];
@@ -75,6 +79,8 @@ struct EyeParams {
   int32_t fine;         // 1: the mesh cells take few pixels of this eye, a raster lane takes a triangle
   int32_t tile_base;    // first tile index of this eye in the call's flattened tile range
   int32_t line_base;    // first row of this eye in the call's ray rows (and first 4 columns in its ray columns)
+  int32_t form;         // kRasterStrips ..: what a raster warp takes of its tiles, | kEyeFew (see lf_raster_impl.h)
+  int32_t item_base;    // its first work item in a kRasterMixed launch
   float* out;           // H x W float4
 };
 
@@ -137,10 +143,6 @@ struct GridTables {
   const float* b;   // n_views x G
 };
 
-// What a raster warp takes: a strip of a tile with two pixels per lane, a strip with four (half a tile of 256
-// pixels), or a whole tile with four.
-enum : int { kRasterStrips = 0, kRasterHalves = 1, kRasterWhole = 2 };
-
 struct FrameArgs {
   EyeParams* eyes;
   int32_t n_eyes;
@@ -189,7 +191,8 @@ struct FrameArgs {
   int32_t* work_counter;
   int32_t fine_mesh;       // mesh cells of a few pixels, a raster lane takes a triangle: 0 no eye, 1 every eye, 2 EyeParams::fine
   int32_t fine_most;       // 1: most eyes' cells are, their bins are filled accordingly
-  int32_t raster_form;     // kRasterStrips ..: what a raster warp takes at a time
+  int32_t raster_form;     // kRasterStrips .. kRasterMixed: what a raster warp takes at a time
+  int32_t mixed_items;     // work items of a kRasterMixed launch
   int32_t strips_per_item; // strips of a tile that a raster warp takes at a time (set by launch_raster)
   // two-level progressive rendering (all null / 0 with one level)
   const void* const* tex_table;  // per view: its texels (a pool page for fine views; null when not resident)

@@ -107,12 +107,11 @@ template <int TW, int TH>
 constexpr int tile_px() { return TW * TH == 256 ? 4 : 2; }
 constexpr int kPxMax = 4;
 constexpr int kRasterWarps = 4;     // warps per block, each on its own work item
-// In calls of at most a tile per SM a warp has its scheduler to itself and waits for each
+// An eye of few tiles near its axis (kEyeFew, lf_api.cu) has few warps, which wait for each
 // view's record, disk test and vote in turn.  Of full rounds of views (a rig of a thousand
-// in an image of 48^2) it tests all disks first and keeps the views that a pixel sees.
+// in an image of 48^2) they test all disks first and keep the views that a pixel sees.
 // Whole passes, without / with: 4,096 views, one pixel 432 / 185 us, 32^2 430 / 351;
 // 1,024 views, 48^2 168 / 142.
-constexpr int kFewTiles = 152;
 
 // A warp's private shared memory: its view table and its window of triangles.
 // The triangle arrays are 16-byte columns, so the 32 lanes that store one
@@ -280,7 +279,7 @@ __device__ __forceinline__ void raster_item(const FrameArgs& A, const int item, 
     w0 = w1 = T = 0;
     stored = 0;
     if constexpr (kPx == 2) {
-      if (nv == kViewsPerRound && A.total_tiles <= kFewTiles) {  // drop the views that no pixel sees
+      if (nv == kViewsPerRound && (E.form & kEyeFew)) {  // drop the views that no pixel sees
         const int v = S.views[lane];
         if constexpr (OVAL) {
           for (int k = 0; k < 4; ++k) S.ov[lane][k] = reinterpret_cast<const float4*>(A.vrecs[vbase + v].ov)[k];
@@ -768,6 +767,42 @@ __global__ void __launch_bounds__(kRasterWarps * 32, 5) raster_kernel(FrameArgs 
   }
 }
 
+// Where the eyes of a call differ in what a warp should take of their tiles (EyeParams::form),
+// both raster_item forms in one kernel, an eye's items from its item_base on.
+template <int TW, int TH, int FMT, bool PERSISTENT, bool OVAL>
+__global__ void __launch_bounds__(kRasterWarps * 32, 5) raster_mixed_kernel(FrameArgs A) {
+  using Smem = typename std::conditional<OVAL, WarpSmemOval, WarpSmem>::type;
+  __shared__ Smem S[kRasterWarps];
+  constexpr int STRIPS2 = TH / ((32 / TW) * 2), STRIPS4 = STRIPS2 / 2;
+  const int warp = threadIdx.x >> 5;
+  griddep_wait();
+  for (int turn = 0;; ++turn) {
+    int item = 0;
+    if constexpr (PERSISTENT) {
+      if ((threadIdx.x & 31) == 0) item = atomicAdd(A.work_counter, 1);
+      item = __shfl_sync(0xffffffffu, item, 0);
+    } else {
+      if (turn) break;
+      item = blockIdx.x * kRasterWarps + warp;
+    }
+    if (item >= A.mixed_items) break;
+    int e = 0;  // the last eye whose first item is <= item
+    for (int hi = A.n_eyes; hi - e > 1;) {
+      const int mid = (e + hi) >> 1;
+      if (A.eyes[mid].item_base <= item) e = mid;
+      else hi = mid;
+    }
+    const EyeParams& E = A.eyes[e];
+    const int i = item - E.item_base, form = E.form & 3;
+    if (form == kRasterStrips) {
+      raster_item<TW, TH, FMT, false, PERSISTENT, OVAL, 2>(A, E.tile_base + i / STRIPS2, i % STRIPS2, i % STRIPS2 + 1, S[warp]);
+    } else {
+      const int per = form == kRasterWhole ? STRIPS4 : 1, groups = STRIPS4 / per, s0 = i % groups * per;
+      raster_item<TW, TH, FMT, false, PERSISTENT, OVAL, 4>(A, E.tile_base + i / groups, s0, s0 + per, S[warp]);
+    }
+  }
+}
+
 template <int TW, int TH, int FMT, bool OVAL, int PX>
 static cudaError_t launch_px(FrameArgs a, bool inspect, bool persistent, int pblocks, cudaStream_t s, bool pdl) {
   constexpr int STRIPS = TH / ((32 / TW) * PX);
@@ -783,8 +818,14 @@ static cudaError_t launch_px(FrameArgs a, bool inspect, bool persistent, int pbl
 template <int TW, int TH, int FMT, bool OVAL>
 static cudaError_t launch_disk(const FrameArgs& a, bool inspect, bool persistent, int pblocks, cudaStream_t s,
                                bool pdl) {
-  if constexpr (tile_px<TW, TH>() == 4)
+  if constexpr (tile_px<TW, TH>() == 4) {
+    if (a.raster_form == kRasterMixed) {
+      const dim3 block(kRasterWarps * 32), grid((unsigned)((a.mixed_items + kRasterWarps - 1) / kRasterWarps));
+      if (persistent) return launch_kernel(raster_mixed_kernel<TW, TH, FMT, true, OVAL>, dim3(pblocks), block, 0, s, pdl, a);
+      return launch_kernel(raster_mixed_kernel<TW, TH, FMT, false, OVAL>, grid, block, 0, s, pdl, a);
+    }
     if (a.raster_form != kRasterStrips && !inspect) return launch_px<TW, TH, FMT, OVAL, 4>(a, false, persistent, pblocks, s, pdl);
+  }
   return launch_px<TW, TH, FMT, OVAL, 2>(a, inspect, persistent, pblocks, s, pdl);
 }
 
