@@ -1002,8 +1002,16 @@ __global__ void __launch_bounds__(BLOCK, BLOCK > kSetupBlock ? 1024 / BLOCK : MU
 // neighbours meet in one tile: scatter 553 -> 455 us; counting, whose additions
 // return nothing, 340 -> 373 (kept apart), and triangles of several tiles, which the
 // warp then walks in step, count 35 -> 45 us at 128^2 meshes of a 256^2 eye.
+// Triangles of many tiles (a telephoto eye over a dense mesh: up to 15,625 of a 2000^2 image each) are
+// walked by all lanes of a warp, and by several warps where the records are no more than the warps.
+// Whole passes of such an eye (focal length 20,000 pixels, 1400x1200; 100,000, 2000^2), the older set-up's
+// blocks / a thread each / so: 64 views of 66^2 meshes 223 / 1,219 / 108 us and 626 / 5,538 / 198; of 129^2
+// 251 / 510 / 110 and 996 / 4,915 / 199.  A prefilter's 36 M records as before (count 340, scatter 445).
+constexpr int kWideTiles = 32;
+constexpr int kBinThreads = 256, kBinBlocks = 152 * 8;
+
 template <int PASS, bool SHARE>
-__global__ void __launch_bounds__(256) bin_records_kernel(FrameArgs A) {
+__global__ void __launch_bounds__(kBinThreads) bin_records_kernel(FrameArgs A) {
   static_assert(PASS == 1 || !SHARE, "only the scatter shares additions");
   constexpr int U = 4;
   griddep_wait();
@@ -1011,6 +1019,36 @@ __global__ void __launch_bounds__(256) bin_records_kernel(FrameArgs A) {
   const int64_t n = min((int64_t)*A.pool_counter, A.pool_capacity), step = (int64_t)gridDim.x * blockDim.x;
   const int sw = __ffs(A.tile_w) - 1, sh = __ffs(A.tile_h) - 1;
   const int lane = threadIdx.x & 31;
+  auto tiles_of = [&](int2 bb, int4 bins, RecordTiles& T, int& ntx, int& curs) {  // bins: bin_off, btx0 | bty0, bntx | bnty
+    const TileBox b = {(int16_t)(bins.y & 0xffff), bins.y >> 16, (int16_t)(bins.z & 0xffff), bins.z >> 16, sw, sh};
+    T = record_tiles(bb, b);
+    ntx = b.ntx;
+    curs = bins.x + b.ntx * b.nty + 1;
+  };
+  auto enter = [&](int bin, int record) {
+    const int at = atomicAdd(&A.bin_offsets[bin], 1);
+    if (PASS == 1) A.bin_entries[at] = record;
+  };
+  // tiles first, first + stride, .. of a record's box
+  auto walk = [&](const RecordTiles& T, int ntx, int curs, int record, int first, int stride) {
+    const int w = T.x1 - T.x0 + 1, count = w * (T.y1 - T.y0 + 1);
+#pragma unroll 4
+    for (int t = first; t < count; t += stride) enter(curs + (T.y0 + t / w) * ntx + T.x0 + t % w, record);
+  };
+  const int64_t warps = step >> 5;
+  if (n <= warps) {  // a warp or more per record
+    const int64_t w = (blockIdx.x * (int64_t)blockDim.x + threadIdx.x) >> 5;
+    const int parts = n > 0 ? (int)min(warps / n, (int64_t)64) : 0;
+    if (w >= n * parts) return;
+    const int64_t i = w % n;
+    const int4 bins = *reinterpret_cast<const int4*>(&A.vrecs[A.pool_owner[i]].bin_off);
+    if (bins.x < 0) return;
+    RecordTiles T;
+    int ntx, curs;
+    tiles_of(A.pool_box[i], bins, T, ntx, curs);
+    if (T.x0 <= T.x1 && T.y0 <= T.y1) walk(T, ntx, curs, (int)i, (int)(w / n) * 32 + lane, parts * 32);
+    return;
+  }
   for (int64_t i0 = blockIdx.x * (int64_t)blockDim.x + threadIdx.x; i0 - lane < n; i0 += U * step) {
     int2 bb[U];
     int4 bins[U];  // bin_off, btx0 | bty0, bntx | bnty, big_base
@@ -1026,18 +1064,19 @@ __global__ void __launch_bounds__(256) bin_records_kernel(FrameArgs A) {
     for (int u = 0; u < U; ++u) {
       RecordTiles T = {0, 0, -1, -1};
       int ntx = 0, curs = 0;
-      if (bins[u].x >= 0) {
-        const TileBox b = {(int16_t)(bins[u].y & 0xffff), bins[u].y >> 16, (int16_t)(bins[u].z & 0xffff), bins[u].z >> 16, sw, sh};
-        T = record_tiles(bb[u], b);
-        ntx = b.ntx;
-        curs = bins[u].x + b.ntx * b.nty + 1;
+      if (bins[u].x >= 0) tiles_of(bb[u], bins[u], T, ntx, curs);
+      const int record = (int)(i0 + u * step);
+      for (uint32_t m = __ballot_sync(0xffffffffu, T.x0 <= T.x1 && T.y0 <= T.y1 && (T.x1 - T.x0 + 1) * (T.y1 - T.y0 + 1) > kWideTiles);
+           m; m &= m - 1) {  // the warp's wide records, one after the other
+        const int l = __ffs(m) - 1;
+        const RecordTiles W = {__shfl_sync(0xffffffffu, T.x0, l), __shfl_sync(0xffffffffu, T.y0, l),
+                               __shfl_sync(0xffffffffu, T.x1, l), __shfl_sync(0xffffffffu, T.y1, l)};
+        walk(W, __shfl_sync(0xffffffffu, ntx, l), __shfl_sync(0xffffffffu, curs, l), __shfl_sync(0xffffffffu, record, l), lane, 32);
+        if (lane == l) T.x1 = T.x0 - 1;
       }
       if constexpr (!SHARE) {
         for (int y = T.y0; y <= T.y1; ++y)
-          for (int x = T.x0; x <= T.x1; ++x) {
-            const int at = atomicAdd(&A.bin_offsets[curs + y * ntx + x], 1);
-            if (PASS == 1) A.bin_entries[at] = (int)(i0 + u * step);
-          }
+          for (int x = T.x0; x <= T.x1; ++x) enter(curs + y * ntx + x, record);
         continue;
       }
       int x = T.x0, y = T.y0;
@@ -1050,7 +1089,7 @@ __global__ void __launch_bounds__(256) bin_records_kernel(FrameArgs A) {
         int at = 0;
         if (has && lane == first) at = atomicAdd(&A.bin_offsets[key], __popc(same));
         at = __shfl_sync(0xffffffffu, at, first);
-        if (has) A.bin_entries[at + __popc(same & ((1u << lane) - 1u))] = (int)(i0 + u * step);
+        if (has) A.bin_entries[at + __popc(same & ((1u << lane) - 1u))] = record;
         if (has && ++x > T.x1) {
           x = T.x0;
           has = ++y <= T.y1;
@@ -1083,11 +1122,11 @@ cudaError_t launch_tri_setup(const FrameArgs& a, cudaStream_t s, bool pdl) {
     return launch_kernel(tri_setup_kernel<false, kWideBlock>, grid, dim3(kWideBlock), bytes, s, pdl, a, kBinSmemTiles);
   if (parts == 1) return launch_kernel(tri_setup_kernel<false, kSetupBlock>, grid, block, bytes, s, pdl, a, kBinSmemTiles);
   cudaError_t e = launch_kernel(tri_setup_kernel<true, kSetupBlock>, grid, block, 0, s, pdl, a, 0);
-  const dim3 all(152 * 8);
-  if (e == cudaSuccess) e = launch_kernel(bin_records_kernel<0, false>, all, dim3(256), 0, s, pdl, a);
+  const dim3 all(kBinBlocks), threads(kBinThreads);
+  if (e == cudaSuccess) e = launch_kernel(bin_records_kernel<0, false>, all, threads, 0, s, pdl, a);
   if (e == cudaSuccess) e = launch_kernel(bin_scan_kernel, dim3(a.n_views, a.n_eyes), block, 0, s, pdl, a);
   auto scatter = a.fine_most ? bin_records_kernel<1, true> : bin_records_kernel<1, false>;
-  if (e == cudaSuccess) e = launch_kernel(scatter, all, dim3(256), 0, s, pdl, a);
+  if (e == cudaSuccess) e = launch_kernel(scatter, all, threads, 0, s, pdl, a);
   return e;
 }
 
