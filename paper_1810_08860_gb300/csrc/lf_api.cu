@@ -216,21 +216,24 @@ void set_forms(const lf_ctx* c, Layout& L) {
     near += n;
     work += n * weight(P);
   }
-  const int32_t form = raster_form(near, c->sm_count);
+  const int32_t least = L.total_tiles > 1 << 28 ? kRasterWhole : kRasterStrips;  // items are counted in 32 bits
+  const int32_t form = std::max(least, raster_form(near, c->sm_count));
   L.form = form;
-  int64_t items = 0;
+  int32_t items = 0;
   bool differ = false;
   for (EyeParams& P : L.eyes) {
-    const int32_t f = std::min(form, raster_form(work / weight(P) * (1 + 1e-9), c->sm_count));
+    const int32_t f = std::max(least, std::min(form, raster_form(work / weight(P) * (1 + 1e-9), c->sm_count)));
     P.form = f | (near_tiles(c->cfg, P) <= c->sm_count ? kEyeFew : 0);
-    P.item_base = (int32_t)std::min<int64_t>(items, INT32_MAX);
-    const int64_t tiles = (int64_t)P.tiles_x * ((P.H + c->cfg.tile_h - 1) / c->cfg.tile_h);
+    P.item_base = items;
+    const int32_t tiles = P.tiles_x * ((P.H + c->cfg.tile_h - 1) / c->cfg.tile_h);
     items += tiles * (f == kRasterStrips ? 4 : f == kRasterHalves ? 2 : 1);
     differ |= f != form;
   }
-  if (!differ || c->cfg.tile_w * c->cfg.tile_h != 256 || items > INT32_MAX) return;
+  // (8 x 8 tiles have one form, whose kernel looks EyeParams::fine up for itself)
+  differ |= fine_form(L) == 2;
+  if (!differ || c->cfg.tile_w * c->cfg.tile_h != 256) return;
   L.form = kRasterMixed;
-  L.mixed_items = (int32_t)items;
+  L.mixed_items = items;
 }
 
 // Lines that an eye takes in the ray tables: at most a tile's height (or a quarter of its width) per tile, and kMaxEyeLines.

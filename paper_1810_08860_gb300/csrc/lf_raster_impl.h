@@ -241,8 +241,9 @@ __device__ __forceinline__ bool covers_wide(const TriRec* tr, int64_t Px, int64_
   return in;
 }
 
-// One warp's work item: strips s0 .. s1 - 1 of tile `item`.
-template <int TW, int TH, int FMT, bool INSPECT, bool MANY_EYES, bool OVAL, int kPx, typename Smem>
+// One warp's work item: strips s0 .. s1 - 1 of tile `item`.  EYE_FINE: the eyes may differ in
+// EyeParams::fine (the look-up costs a batch of 64 like eyes 0.7 per cent of its raster).
+template <int TW, int TH, int FMT, bool INSPECT, bool MANY_EYES, bool OVAL, int kPx, bool EYE_FINE, typename Smem>
 __device__ __forceinline__ void raster_item(const FrameArgs& A, const int item, const int s0, const int s1, Smem& S) {
   constexpr int ROWS = (32 / TW) * kPx;
   constexpr int STRIPS = TH / ROWS;
@@ -261,10 +262,8 @@ __device__ __forceinline__ void raster_item(const FrameArgs& A, const int item, 
   const float px = (float)pi + 0.5f;
   const int64_t vbase = (int64_t)e * A.n_views;
 
-  // The tile's eye decides; it is looked up only where the eyes of a call differ (a flag
-  // held in a register over the loops below made the stereo rig's frame 234 -> 250 us,
-  // the look-up the batch of 64 eyes 1,898 -> 1,911, raster alone).
-  auto fine = [&]() { return !INSPECT && A.fine_mesh && (A.fine_mesh == 1 || E.fine); };
+  // (a flag held in a register over the loops below made the stereo rig's frame 234 -> 250 us)
+  auto fine = [&]() { return !INSPECT && A.fine_mesh && (!EYE_FINE || A.fine_mesh == 1 || E.fine); };
 
   int nv = 0, T = 0;          // the round's views, and their bin entries
   int w0 = 0, w1 = 0;         // the window: entries [w0, w1) are in shared memory
@@ -763,12 +762,12 @@ __global__ void __launch_bounds__(kRasterWarps * 32, 5) raster_kernel(FrameArgs 
     }
     if (item >= n_items) break;
     const int tile = item / groups, s0 = (item - tile * groups) * per;
-    raster_item<TW, TH, FMT, INSPECT, PERSISTENT, OVAL, PX>(A, tile, s0, s0 + per, S[warp]);
+    raster_item<TW, TH, FMT, INSPECT, PERSISTENT, OVAL, PX, tile_px<TW, TH>() == 2>(A, tile, s0, s0 + per, S[warp]);
   }
 }
 
-// Where the eyes of a call differ in what a warp should take of their tiles (EyeParams::form),
-// both raster_item forms in one kernel, an eye's items from its item_base on.
+// Where the eyes of a call differ, in what a warp should take of their tiles (EyeParams::form) or in
+// being fine, both raster_item forms in one kernel, an eye's items from its item_base on.
 template <int TW, int TH, int FMT, bool PERSISTENT, bool OVAL>
 __global__ void __launch_bounds__(kRasterWarps * 32, 5) raster_mixed_kernel(FrameArgs A) {
   using Smem = typename std::conditional<OVAL, WarpSmemOval, WarpSmem>::type;
@@ -795,10 +794,10 @@ __global__ void __launch_bounds__(kRasterWarps * 32, 5) raster_mixed_kernel(Fram
     const EyeParams& E = A.eyes[e];
     const int i = item - E.item_base, form = E.form & 3;
     if (form == kRasterStrips) {
-      raster_item<TW, TH, FMT, false, PERSISTENT, OVAL, 2>(A, E.tile_base + i / STRIPS2, i % STRIPS2, i % STRIPS2 + 1, S[warp]);
+      raster_item<TW, TH, FMT, false, PERSISTENT, OVAL, 2, true>(A, E.tile_base + i / STRIPS2, i % STRIPS2, i % STRIPS2 + 1, S[warp]);
     } else {
       const int per = form == kRasterWhole ? STRIPS4 : 1, groups = STRIPS4 / per, s0 = i % groups * per;
-      raster_item<TW, TH, FMT, false, PERSISTENT, OVAL, 4>(A, E.tile_base + i / groups, s0, s0 + per, S[warp]);
+      raster_item<TW, TH, FMT, false, PERSISTENT, OVAL, 4, true>(A, E.tile_base + i / groups, s0, s0 + per, S[warp]);
     }
   }
 }
