@@ -248,8 +248,8 @@ inline bool aligned16(const void* p) { return (reinterpret_cast<uintptr_t>(p) & 
 // seen from about the same distance by the eye and the view.  A value of speed
 // only, so the first view stands for all; but each eye of a call is judged by
 // itself: eyes of 256^2 and 2048^2 in one batch, 129^2 meshes of 16 views (2- and
-// 16-pixel cells), take 259 us, or 307 in the other order; where the first eye
-// decided for both, 440 and 446.
+// 16-pixel cells), took 440 us where the first eye decided for both, and 259 so
+// (446 and 307 in the other order; 191 and 238 with each eye's form below).
 int32_t fine_cells(const lf_ctx* c, const EyeParams& E) {
   if (c->views_host.empty() || c->G < 2) return 0;
   const double cell = (double)c->src_w / (c->G - 1) * E.fx / c->views_host[0].fx;
